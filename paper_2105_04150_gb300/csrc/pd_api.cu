@@ -133,6 +133,14 @@ struct pd_handle {
     float2* lendw = nullptr;                // per slot |xi| / delta
     float2* cbdw = nullptr;                 // per slot c_ij (per-bond stiffness)
     double dw_origin[3] = {0.0, 0.0, 0.0};  // origin of the double-word positions
+    // bond-based PD_PREC_F64: three-word records and bond lengths of the step (W3Args)
+    bool w3 = false;
+    float4* rec3[2] = {nullptr, nullptr};
+    float2 *il3 = nullptr, *cb3 = nullptr, *wrel3 = nullptr;
+    double* phi0 = nullptr; // per node the damage of an intact family
+    double w3_scale = 1.0;  // 1 / U, a power of two (batches: per instance in itab)
+    int w3_x_grid = kW3UGrid;  // exponent of the positions' grid
+    int team = 1;           // warps per slice
     int integrator = PD_INTEGRATOR_EC;
     int64_t ramp_steps = 0;
     void* vpeek = nullptr;  // velocity-Verlet: full-step velocity for pd_get_state
@@ -372,6 +380,7 @@ StepArgsF64 args_f64(pd_handle* h, int k)
     a.v = (double*)h->v;
     a.nbr = h->nbr;
     a.bits = h->bits;
+    a.bits0 = h->bits0;
     a.sw = h->sw;
     a.cbond = h->per_bond_c ? (const double*)h->cbond : nullptr;
     a.ilen = h->ilen;
@@ -391,6 +400,7 @@ StepArgsF64 args_f64(pd_handle* h, int k)
     a.Q = h->Q;
     a.has_nofail = h->has_nofail ? 1 : 0;
     a.frozen = h->frozen ? 1 : 0;
+    a.sc_mode = h->sc_mode;
     a.sc = h->sc;
     a.sc_lo = h->sc_lo;
     a.sc_hi = h->sc_hi;
@@ -403,6 +413,15 @@ StepArgsF64 args_f64(pd_handle* h, int k)
     a.ramp_steps = h->ramp_steps;
     a.vv = h->integrator == PD_INTEGRATOR_VV ? 1 : 0;
     return a;
+}
+
+W3Args w3_args(pd_handle* h);
+
+// the bond-based FP64 step of this handle (softening or not)
+cudaError_t launch_f64(pd_handle* h, const StepArgsF64& a)
+{
+    return h->integ != nullptr ? launch_step_f64_soft(a, h->grid, h->block, h->stream)
+                               : launch_step_f64(a, w3_args(h), h->grid, h->block, h->stream);
 }
 
 // the FP32 step kernel build for this handle (bilinear softening or not)
@@ -512,15 +531,36 @@ DwArgs dw_args(pd_handle* h)
     return d;
 }
 
-// double-word records of both buffers from the FP64 records
-pd_status dw_publish(pd_handle* h)
+W3Args w3_args(pd_handle* h)
 {
-    if (!h->dw) return PD_OK;
-    for (int b = 0; b < 2; ++b)
-        PD_CUDA(launch_dw_publish(h->rec[b], h->recdw[b], h->n_pad, h->dw_origin, 1.0 / h->delta,
-                                  h->stream),
-                "double-word records");
-    return PD_OK;
+    W3Args d{};
+    d.rec[0] = h->rec3[0];
+    d.rec[1] = h->rec3[1];
+    d.il = h->il3;
+    d.cb = h->per_bond_c ? h->cb3 : nullptr;
+    d.wrel = h->wrel3;
+    d.phi0 = h->phi0;
+    d.w_ref = (h->per_bond_c ? 1.0 : h->c) * h->vol0;
+    d.scale = h->w3_scale;
+    d.x_grid = h->w3_x_grid;
+    d.dt_rho = h->dt / h->rho;
+    d.x_hi = h->frozen ? kW3XMax : w3_x_hi(h->sc_lo);
+    d.uniform_w = h->uniform_vol ? 1 : 0;
+    d.team = h->team;
+    d.max_seg = h->Q * (32 / kW3Seg);
+    return d;
+}
+
+// the records that neighbours read, of buffer b, from the FP64 records
+cudaError_t publish64(pd_handle* h, int b)
+{
+    if (h->dw)
+        return launch_dw_publish(h->rec[b], h->recdw[b], h->n_pad, h->dw_origin, 1.0 / h->delta,
+                                 h->stream);
+    if (h->w3)
+        return launch_w3_publish(h->rec[b], h->rec3[b], h->n_pad, h->w3_scale, h->w3_x_grid,
+                                 h->batch ? h->inst : nullptr, h->itab, h->stream);
+    return cudaSuccess;
 }
 
 const void* step_kernel_fn(pd_handle* h)
@@ -529,7 +569,8 @@ const void* step_kernel_fn(pd_handle* h)
     if (h->dw)
         return step_dw_kernel(h->sc_mode, h->uniform_vol && !h->batch, h->integ != nullptr,
                               h->integrator == PD_INTEGRATOR_VV);
-    return step_f64_kernel(h->sc_mode);
+    if (h->w3) return step_f64_kernel(h->uniform_vol, h->team > 1);
+    return h->integ != nullptr ? step_f64_soft_kernel(h->sc_mode) : osb_force_kernel();
 }
 
 // One step launch, k steps past the device counter; step_abs >= 0 (F32 lattice
@@ -553,7 +594,7 @@ cudaError_t launch_one(pd_handle* h, int k, int64_t step_abs = -1)
         return launch_osb_step(args_f64(h, k), osb_args(h), h->grid, h->block, h->stream);
     if (h->precision == 32)
         return launch_f32(h, args_f32(h, k, step_abs));
-    return launch_step_f64(args_f64(h, k), h->sc_mode, h->grid, h->block, h->stream);
+    return launch_f64(h, args_f64(h, k));
 }
 
 // The tensor maps of the tile step's copies (both record buffers) for box shape
@@ -605,6 +646,24 @@ pd_status encode_lat_tma(pd_handle* h, int shape)
     return PD_OK;
 }
 
+// Warps per slice of the FP64 step.  One warp takes about 52 us for a family of 122
+// whatever the model's size, so a model with fewer slices than the chip holds warps
+// (16 per SM) shares each among 8, 4 or 2, as long as that fills the chip only once;
+// two warps still pay a little past that, where one would leave a short last wave.
+// us per step with 1 / 2 / 4 / 8 warps: 125 slices 54.7 / 34.6 / 23.6 / 18.0, 422
+// slices 55 / 34 / 37 / 38, 1000: 56 / 54 / 59 / 63, 2695: 157 / 137 / 142 / 165, 4160:
+// 187 / 190 / 201 / 248, 9000: 355 / 376 / 415 / 512 (the barrier and the shared sums).
+int w3_team(const pd_handle* h, int sms)
+{
+    if (h->Q * (32 / kW3Seg) > kW3TeamSegs) return 1;
+    const int wpb = h->block / 32;
+    const int64_t cap = (int64_t)sms * 16;
+    if (wpb % 8 == 0 && h->n_slices * 8 <= cap) return 8;
+    if (wpb % 4 == 0 && h->n_slices * 4 <= cap / 2) return 4;
+    if (wpb % 2 == 0 && h->n_slices * 4 <= 5 * cap) return 2;
+    return 1;
+}
+
 pd_status choose_grid(pd_handle* h, int blocks_per_sm)
 {
     if (h->lattice && h->lat_var >= 2) {  // the tile step: one block per box of the lattice
@@ -628,16 +687,24 @@ pd_status choose_grid(pd_handle* h, int blocks_per_sm)
     }
     int sms = 0;
     PD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device), "sm count");
+    if (h->w3) h->team = w3_team(h, sms);
     const void* fn = step_kernel_fn(h);
-    // no shared memory is used: give the unified L1/shared array to L1
-    PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 0),
+    const size_t smem = h->w3 ? step_f64_smem(h->team, h->Q * (32 / kW3Seg), h->block) : 0;
+    // no shared memory, or that of two resident blocks: the rest of the unified
+    // L1/shared array (228 KB) goes to L1
+    PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 smem ? (int)std::min<size_t>(100, 1 + 200 * (smem + 1024) / (228 << 10))
+                                      : 0),
             "carveout");
+    if (smem)
+        PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                "shared memory size");
     int occ = 0;
-    PD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, h->block, 0), "occupancy");
+    PD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, h->block, smem), "occupancy");
     if (occ < 1) occ = 1;
     if (blocks_per_sm > 0) occ = std::min(occ, blocks_per_sm);
-    const int64_t warps_per_block = h->block / 32;
-    const int64_t need = (h->n_slices + warps_per_block - 1) / warps_per_block;
+    const int64_t slices_per_block = h->block / 32 / h->team;
+    const int64_t need = (h->n_slices + slices_per_block - 1) / slices_per_block;
     h->grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * occ, need));
     h->grid_dil = h->grid;
     h->grid_osbf = h->grid;
@@ -677,7 +744,12 @@ pd_status upload_weights(pd_handle* h)
     PD_CUDA(launch_set_weights(h->precision, w0, w1, h->vol, h->nbr, h->bits0, h->sw, h->n, h->Q,
                                wscale, h->wsum_inv, h->stream),
             "set weights");
-    return dw_publish(h);
+    if (h->w3)
+        PD_CUDA(launch_damage(64, w0, h->nbr, h->bits0, h->sw, h->wsum_inv, nullptr, h->n, h->Q,
+                              nullptr, h->phi0, h->stream),
+                "intact damage");
+    for (int b = 0; b < 2; ++b) PD_CUDA(publish64(h, b), "neighbour records");
+    return PD_OK;
 }
 
 pd_status check_dev_err(pd_handle* h)
@@ -719,7 +791,7 @@ pd_status vv_force_pass(pd_handle* h)
                       : launch_osb_step(a, osb_args(h), h->grid, h->block, h->stream);
         else
             e = h->dw ? launch_step_dw(a, dw_args(h), h->sc_mode, h->grid, h->block, h->stream)
-                      : launch_step_f64(a, h->sc_mode, h->grid, h->block, h->stream);
+                      : launch_f64(h, a);
     }
     if (e != cudaSuccess) return cuda_fail(e, "velocity-Verlet force pass");
     h->peek_step = h->step;
@@ -867,6 +939,7 @@ struct ModelDesc {
     int64_t n = 0;
     const double* coords = nullptr;   // 3n
     const double* wvol = nullptr;     // n: w = c * wvol (batches fold c into wvol)
+    const double* wrel = nullptr;     // n, batches: volume / volume of the instance's first node
     const uint8_t* type = nullptr;    // 3n
     const double* disp = nullptr;     // 3n or null
     const double* force = nullptr;    // 3n or null
@@ -920,6 +993,8 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
     std::vector<uint8_t> cls;
     std::string msg = bc_classes(n, d.type, d.disp, d.force, d.no_fail, table, cls, h->has_nofail);
     if (!msg.empty()) return fail(PD_ERR_ARG, "%s", msg.c_str());
+    h->w3 = cfg->precision == PD_PREC_F64 && h->model == 0 &&
+            (h->kr < 1.0 || (h->kr == 1.0 && !h->has_nofail));
 
     // FP32 Euler-Cromer PMB models on a regular lattice (the stencil kernel's
     // case): lattice node order and the stencil-ordered layout
@@ -1002,6 +1077,13 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
             ALLOC(h->recdw[1], float4, 4 * np);
             ALLOC(h->lendw, float2, nbr.size());
         }
+        if (h->w3) {
+            ALLOC(h->rec3[0], float4, 4 * np);
+            ALLOC(h->rec3[1], float4, 4 * np);
+            ALLOC(h->il3, float2, nbr.size());
+            ALLOC(h->phi0, double, np);
+            if (!h->uniform_vol) ALLOC(h->wrel3, float2, np);
+        }
         ALLOC(h->ilen, double, nbr.size());  // also the adjoint's
     }
     if (h->model == 1) {
@@ -1030,7 +1112,9 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
             ALLOC(h->osb_beta, double, np);
         }
     }
-    if (h->kr >= 1.0) {  // bilinear softening: every bond starts intact, mu = 1
+    // bilinear softening: every bond starts intact, mu = 1 (FP64 with kr = 1 and no
+    // no-fail nodes is the PMB law: its kernel, and the flags are the integrity)
+    if (h->kr >= 1.0 && !h->w3) {
         if (f32)
             ALLOC(h->integ, float, nbr.size());
         else
@@ -1148,15 +1232,79 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
         (st = up(h->x64, xs.data(), 24 * np, "upload coordinates")) ||
         (st = up(h->vol, vs.data(), 8 * np, "upload volumes")))
         return st;
+    std::vector<InstParams> itab = d.itab;
+    std::vector<float2> wrel;
+    if (h->w3) {
+        // U: a power of two no smaller than the longest bond (of each instance), and the
+        // FP32 grid of the largest coordinate in that unit
+        std::vector<double> len2(std::max<size_t>(1, itab.size()), 0.0), far(len2);
+        const int nl = (int)len2.size();
+        const int64_t* off = h->off.data();
+        const int32_t* idx = h->idx.data();
+#pragma omp parallel
+        {
+            std::vector<double> mine(nl, 0.0), wide(nl, 0.0);
+#pragma omp for schedule(static)
+            for (int64_t i = 0; i < n; ++i) {
+                double m = 0.0;
+                for (int64_t k = off[i]; k < off[i + 1]; ++k) {
+                    double q = 0.0;
+                    for (int a = 0; a < 3; ++a) {
+                        const double e = d.coords[3 * (int64_t)idx[k] + a] - d.coords[3 * i + a];
+                        q += e * e;
+                    }
+                    m = std::max(m, q);
+                }
+                const int b = d.inst.empty() ? 0 : d.inst[i];
+                mine[b] = std::max(mine[b], m);
+                for (int a = 0; a < 3; ++a)
+                    wide[b] = std::max(wide[b], std::fabs(d.coords[3 * i + a]));
+            }
+#pragma omp critical
+            for (int k = 0; k < nl; ++k) {
+                len2[k] = std::max(len2[k], mine[k]);
+                far[k] = std::max(far[k], wide[k]);
+            }
+        }
+        for (int k = 0; k < nl; ++k) {
+            const double L = len2[k] > 0.0 ? std::sqrt(len2[k]) : d.unit;
+            const double s = std::ldexp(1.0, -(std::ilogb(L) + 1));
+            const double X = far[k] * s;
+            const int g = std::min(100, std::max(kW3UGrid, (X > 0.0 ? std::ilogb(X) : 0) - 23));
+            if (itab.empty()) {
+                h->w3_scale = s;
+                h->w3_x_grid = g;
+            } else {
+                itab[k].w3_scale = s;
+                itab[k].w3_x_grid = g;
+                itab[k].w3_x_hi = w3_x_hi(itab[k].sc_lo);
+            }
+        }
+        if (!h->uniform_vol) {
+            wrel.assign(np, make_float2(0.f, 0.f));
+            for (int64_t p = 0; p < n; ++p) {
+                const int64_t i = h->perm[p];
+                const double r = d.wrel ? d.wrel[i] : d.wvol[i] / d.wvol[0];
+                wrel[p].x = (float)r;
+                wrel[p].y = (float)(r - (double)wrel[p].x);
+            }
+            if ((st = up(h->wrel3, wrel.data(), 8 * np, "upload weight ratios"))) return st;
+        }
+    }
     if (!d.inst.empty()) {
         if ((st = up(h->inst, insts.data(), 4 * np, "upload instance ids")) ||
             (st = up(h->hid, hids.data(), 4 * np, "upload local ids")) ||
-            (st = up(h->itab, d.itab.data(), d.itab.size() * sizeof(InstParams),
+            (st = up(h->itab, itab.data(), itab.size() * sizeof(InstParams),
                      "upload instance table")))
             return st;
     }
     if (!f32) {
         e = launch_inv_len(h->x64, h->nbr, h->sw, n, h->Q, h->ilen, h->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "bond lengths");
+    }
+    if (h->w3) {
+        e = launch_w3_ilen(h->ilen, h->nbr, h->sw, n, h->Q, h->w3_scale,
+                           h->batch ? h->inst : nullptr, h->itab, h->il3, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "bond lengths");
     }
     if (h->dw) {
@@ -1330,7 +1478,7 @@ pd_status pd_batch_create(int32_t n_inst, const pd_instance* inst, const pd_conf
 
     pd_handle* h = new (std::nothrow) pd_handle();
     if (!h) return fail(PD_ERR_OOM, "host allocation");
-    std::vector<double> x(3 * n), wv(n), disp(3 * n, 0.0), force(3 * n, 0.0), centre(3 * n);
+    std::vector<double> x(3 * n), wv(n), wr(n), disp(3 * n, 0.0), force(3 * n, 0.0), centre(3 * n);
     std::vector<uint8_t> type(3 * n), nofail(any_nofail ? n : 0, 0);
     ModelDesc d;
     d.inst.resize(n);
@@ -1398,6 +1546,7 @@ pd_status pd_batch_create(int32_t n_inst, const pd_instance* inst, const pd_conf
             // bond-based weights carry the instance's micromodulus; the state-based
             // model's are the volumes
             wv[k] = (I.mat.model == 1 ? 1.0 : I.mat.c) * I.volumes[i];
+            wr[k] = I.volumes[i] / I.volumes[0];
             if (I.bc.no_fail) nofail[k] = I.bc.no_fail[i];
             d.inst[k] = b;
             d.hid[k] = (int32_t)i;
@@ -1411,7 +1560,8 @@ pd_status pd_batch_create(int32_t n_inst, const pd_instance* inst, const pd_conf
         // softening: the band below the smallest s_0 = s_c / kr is resolved too
         ip.fast_lo = (float)((1.0 - 2.0 * kGuard) * ip.sc_lo /
                              (inst[0].mat.kr >= 1.0 ? inst[0].mat.kr : 1.0));
-        ip.w_const = (float)((I.mat.model == 1 ? 1.0 : I.mat.c) * I.volumes[0]);
+        ip.w_ref = (I.mat.model == 1 ? 1.0 : I.mat.c) * I.volumes[0];
+        ip.w_const = (float)ip.w_ref;
         if (all_lattice) {
             const Lattice& L = lats.back();
             const double f = (1.0 - 2.0 * kGuard) * ip.sc_lo;
@@ -1436,6 +1586,7 @@ pd_status pd_batch_create(int32_t n_inst, const pd_instance* inst, const pd_conf
     d.n = n;
     d.coords = x.data();
     d.wvol = wv.data();
+    d.wrel = wr.data();
     d.type = type.data();
     d.disp = disp.data();
     d.force = force.data();
@@ -1652,10 +1803,7 @@ pd_status pd_set_state(pd_handle* h, const double* u, const double* v, int64_t s
             PD_CUDA(launch_set_state_f64(src[0], src[1], h->gid, h->n, h->rec[cur],
                                          (double*)h->v, h->stream),
                     "set state");
-        if (h->dw)
-            PD_CUDA(launch_dw_publish(h->rec[cur], h->recdw[cur], h->n_pad, h->dw_origin,
-                                      1.0 / h->delta, h->stream),
-                    "double-word records");
+        if (h->precision == 64) PD_CUDA(publish64(h, cur), "neighbour records");
     }
     // the velocity-Verlet history starts again at this step (a^n formed afresh);
     // the host inputs were consumed before the check above, so nothing more
@@ -1856,6 +2004,11 @@ pd_status pd_damage(pd_handle* h, double* phi)
     if (h->damage_fresh)  // written by the last step kernel (fused)
         PD_CUDA(launch_gather_damage(h->precision, h->damage, h->gid, h->n, dst, h->stream),
                 "damage");
+    else if (h->w3)
+        PD_CUDA(launch_damage_lost(h->uniform_vol, h->rec[0], h->nbr, h->bits, h->bits0,
+                                   (const double*)h->wsum_inv, h->phi0, h->gid, h->n, h->Q, dst,
+                                   h->stream),
+                "damage");
     else
         PD_CUDA(launch_damage(h->precision, h->wrec(), h->nbr, h->bits, h->sw, h->wsum_inv,
                               h->gid, h->n, h->Q, h->integ, dst, h->stream),
@@ -1870,7 +2023,7 @@ pd_status pd_adjoint_forward(pd_handle* h, int64_t n_steps, int64_t checkpoint_e
 {
     NvtxScope nvtx_scope_("pd_adjoint_forward");
     if (!h) return fail(PD_ERR_ARG, "NULL handle");
-    if (h->precision != 64 || h->batch || h->integ || h->model != 0)
+    if (h->precision != 64 || h->batch || h->kr >= 1.0 || h->model != 0)
         return fail(PD_ERR_STATE,
                     "the adjoint is available on FP64 and PD_PREC_DW single-model PMB handles");
     if (n_steps < 1 || checkpoint_every < 0)
@@ -2086,9 +2239,7 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         if (ke == cudaSuccess) ke = cudaStreamSynchronize(h->stream);
         const int cur = (int)(h->step & 1);
         if (ke == cudaSuccess) ke = launch_insert_u(T.ck_u + k * np3, h->n_pad, h->rec[cur], h->stream);
-        if (ke == cudaSuccess && h->dw)
-            ke = launch_dw_publish(h->rec[cur], h->recdw[cur], h->n_pad, h->dw_origin,
-                                   1.0 / h->delta, h->stream);
+        if (ke == cudaSuccess) ke = publish64(h, cur);
         if (ke == cudaSuccess)
             ke = cudaMemcpyAsync(h->v, T.ck_v + k * np3, 8 * np3, cudaMemcpyDeviceToDevice, h->stream);
         if (ke == cudaSuccess)
@@ -2118,9 +2269,7 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
                              h->stream);
     if (ke == cudaSuccess) ke = cudaStreamSynchronize(h->stream);
     if (ke == cudaSuccess) ke = launch_insert_u(T.fin_u, h->n_pad, h->rec[h->step & 1], h->stream);
-    if (ke == cudaSuccess && h->dw)
-        ke = launch_dw_publish(h->rec[h->step & 1], h->recdw[h->step & 1], h->n_pad, h->dw_origin,
-                               1.0 / h->delta, h->stream);
+    if (ke == cudaSuccess) ke = publish64(h, (int)(h->step & 1));
     if (ke == cudaSuccess)
         ke = cudaMemcpyAsync(h->v, T.fin_v, 8 * np3, cudaMemcpyDeviceToDevice, h->stream);
     h->damage_fresh = false;
@@ -2208,6 +2357,10 @@ pd_status pd_autotune(pd_handle* h, int32_t trial_steps, int32_t* block_threads,
             bufs.push_back({h->recdw[0], (size_t)(64 * np), {}});
             bufs.push_back({h->recdw[1], (size_t)(64 * np), {}});
         }
+        if (h->w3) {
+            bufs.push_back({h->rec3[0], (size_t)(64 * np), {}});
+            bufs.push_back({h->rec3[1], (size_t)(64 * np), {}});
+        }
         bufs.push_back({h->v, (size_t)(24 * np), {}});
         bufs.push_back({h->damage, (size_t)(8 * np), {}});
     }
@@ -2268,7 +2421,8 @@ pd_status pd_autotune(pd_handle* h, int32_t trial_steps, int32_t* block_threads,
             if (var >= 2) break;  // the tile step's grid does not depend on bps
             int occ = 0;
             const void* fn = step_kernel_fn(h);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, 0);
+            const size_t smem = h->w3 ? step_f64_smem(h->team, h->Q * (32 / kW3Seg), block) : 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem);
             if (bps >= occ) break;  // larger requests are capped to the same grid
         }
     }
@@ -2325,12 +2479,13 @@ pd_status pd_set_params(pd_handle* h, double c, double sc, double load, double d
                 if (pos[s] >= 0) cb[s] = c_bond[pos[s]];
             PD_CUDA(cudaMemcpyAsync(h->cbond, cb.data(), slots * 8, cudaMemcpyHostToDevice, h->stream),
                     "upload c_bond");
-            if (h->dw) {
-                if (!h->cbdw) {
-                    cudaError_t e = h->alloc(&h->cbdw, slots);
+            if (h->dw || h->w3) {
+                float2*& dst = h->dw ? h->cbdw : h->cb3;
+                if (!dst) {
+                    cudaError_t e = h->alloc(&dst, slots);
                     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc c_bond");
                 }
-                PD_CUDA(launch_dw_split((const double*)h->cbond, (int64_t)slots, h->cbdw, h->stream),
+                PD_CUDA(launch_dw_split((const double*)h->cbond, (int64_t)slots, dst, h->stream),
                         "double-word c_bond");
             }
         }
@@ -2522,9 +2677,7 @@ pd_status pd_adjoint_backward_static(pd_handle* h, const double* dLdu, const dou
         if (ke == cudaSuccess) ke = cudaStreamSynchronize(h->stream);
         const int cur = (int)(h->step & 1);
         if (ke == cudaSuccess) ke = launch_insert_u(T.ck_u + k * np3, h->n_pad, h->rec[cur], h->stream);
-        if (ke == cudaSuccess && h->dw)
-            ke = launch_dw_publish(h->rec[cur], h->recdw[cur], h->n_pad, h->dw_origin,
-                                   1.0 / h->delta, h->stream);
+        if (ke == cudaSuccess) ke = publish64(h, cur);
         if (ke == cudaSuccess)
             ke = cudaMemcpyAsync(h->v, T.ck_v + k * np3, 8 * np3, cudaMemcpyDeviceToDevice, h->stream);
         if (ke == cudaSuccess)
@@ -2549,9 +2702,7 @@ pd_status pd_adjoint_backward_static(pd_handle* h, const double* dLdu, const dou
                              h->stream);
     if (ke == cudaSuccess) ke = cudaStreamSynchronize(h->stream);
     if (ke == cudaSuccess) ke = launch_insert_u(T.fin_u, h->n_pad, h->rec[h->step & 1], h->stream);
-    if (ke == cudaSuccess && h->dw)
-        ke = launch_dw_publish(h->rec[h->step & 1], h->recdw[h->step & 1], h->n_pad, h->dw_origin,
-                               1.0 / h->delta, h->stream);
+    if (ke == cudaSuccess) ke = publish64(h, (int)(h->step & 1));
     if (ke == cudaSuccess)
         ke = cudaMemcpyAsync(h->v, T.fin_v, 8 * np3, cudaMemcpyDeviceToDevice, h->stream);
     h->damage_fresh = false;

@@ -188,8 +188,20 @@ __global__ void k_damage(const void* __restrict__ wrec, const int32_t* __restric
         const T acc = masked_wsum<T>(wrec, nbr, bits, g, lane, sw[g], Q, integ);
         // a node without family has no damage (the integral ratio of Eq. 8 is 0/0)
         if (p < n)
-            phi[gid[p]] = wsum_inv[p] > 0 ? (double)fmax((T)0, (T)1 - acc * wsum_inv[p]) : 0.0;
+            phi[gid != nullptr ? gid[p] : p] = wsum_inv[p] > 0 ? (double)fmax((T)0, (T)1 - acc * wsum_inv[p]) : 0.0;
     }
+}
+
+__global__ void k_damage_lost(bool uniform_w, const double* __restrict__ rec,
+                              const int32_t* __restrict__ nbr, const uint32_t* __restrict__ bits,
+                              const uint32_t* __restrict__ bits0,
+                              const double* __restrict__ wsum_inv,
+                              const double* __restrict__ phi0, const int32_t* __restrict__ gid,
+                              int64_t n, int Q, double* __restrict__ phi)
+{
+    GRID_STRIDE(p, n)
+    phi[gid[p]] = damage_lost(uniform_w, rec, nbr, bits, bits0, wsum_inv[p], phi0[p], p >> 5,
+                              (int)(p & 31), Q);
 }
 
 template <typename T>
@@ -332,6 +344,16 @@ cudaError_t launch_damage(int precision, const void* wrec, const int32_t* nbr,
     else
         k_damage<double><<<g, 256, 0, s>>>(wrec, nbr, bits, sw, (const double*)wsum_inv, gid, n,
                                            Q, (const double*)integ, phi_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_damage_lost(bool uniform_w, const double* rec, const int32_t* nbr,
+                               const uint32_t* bits, const uint32_t* bits0, const double* wsum_inv,
+                               const double* phi0, const int32_t* gid, int64_t n, int Q,
+                               double* phi_out, cudaStream_t s)
+{
+    k_damage_lost<<<grid_for(n, 256), 256, 0, s>>>(uniform_w, rec, nbr, bits, bits0, wsum_inv, phi0,
+                                                   gid, n, Q, phi_out);
     return cudaGetLastError();
 }
 

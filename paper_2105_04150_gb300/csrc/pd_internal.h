@@ -33,6 +33,7 @@
 //   neighbours and a double-word reference length per slot, see DwArgs)
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <cuda.h>  // CUtensorMap
 #include <cuda_runtime.h>
@@ -65,6 +66,11 @@ struct InstParams {
                                // (lat_cc, lat_ch of StepArgsF32 per unit q)
     float dtd;                 // dt / dx
     double unit, inv_unit;     // dx, 1 / dx
+    // FP64 batches: the weight of the instance's first node, and the scale and
+    // literal-evaluation bound of its three-word records (W3Args)
+    double w_ref, w3_scale;
+    float w3_x_hi;
+    int32_t w3_x_grid;
 };
 
 // Regular-lattice stencil.  On a cubic lattice of spacing dx with
@@ -264,9 +270,10 @@ struct StepArgsF64 {
     double* v;
     const int32_t* nbr;
     uint32_t* bits;
+    const uint32_t* bits0;     // bond flags after the initial cuts
     const int32_t* sw;
     int32_t frozen;            // 1: no bond breaks (the adjoint's forward runs)
-    int32_t pad1;
+    int32_t sc_mode;           // 0: constant s_c, 1: per-bond draw
     const double* cbond;
     const double* ilen;        // per slot 1 / |xi| (reference bond length)
     const uint8_t* bcc;
@@ -291,6 +298,36 @@ struct StepArgsF64 {
     double* integ;             // bilinear softening: per-slot integrity mu, or nullptr
     double kr;                 // s_0 = s_c / kr
     double k1, beta;           // trilinear: kink at s_1 = k1 s_0 with force beta c s_0 (k1 > 1)
+};
+
+// Three-word records of the FP64 step (pd_step_f64.cu, pd_w3.h): positions and
+// displacements in units of U, a power of two no smaller than the longest bond
+constexpr int kW3Seg = 16;             // slots of a family whose forces are summed together
+constexpr int kW3TeamSegs = 16;        // largest family, in segments, that a team of warps takes
+constexpr float kW3XMax = 0x1.0p-6f;   // largest |x|, x = |y|^2 / |xi|^2 - 1, of the double-word
+                                       // bond arithmetic (see pd_w3.h)
+constexpr int kW3UGrid = -22;          // exponent of the displacements' grid below 4 U
+// the record's x at which the literal evaluation takes over: a band below the stretch
+// s_lo at which a bond can first break or soften, never past kW3XMax
+inline float w3_x_hi(double s_lo)
+{
+    const double f = (1.0 - 0x1.0p-20) * s_lo;
+    return (float)std::min((double)kW3XMax, f * (2.0 + f));
+}
+struct W3Args {
+    const float4* rec[2];      // 4 float4 per node, double buffered like the FP64 records
+    const float2* il;          // per slot U / |xi| as a double-word
+    const float2* cb;          // per slot stiffness c_ij as a double-word, or nullptr
+    const float2* wrel;        // per node w / w_ref as a double-word (non-uniform weights)
+    const double* phi0;        // per node the damage of an intact family (rounding only)
+    double w_ref;              // weight of the first node (batches: per instance)
+    double scale;              // 1 / U (batches: per instance)
+    double dt_rho;             // dt / rho
+    int32_t x_grid;            // exponent of the positions' grid (batches: per instance)
+    float x_hi;                // w3_x_hi (batches: per instance); kW3XMax while frozen
+    int32_t uniform_w;         // 1: every node has weight w_ref
+    int32_t team;              // warps per slice
+    int32_t max_seg;           // segments of the largest family
 };
 
 // Double-word (FP64-grade) step of FP64 handles created with PD_PREC_DW
@@ -472,7 +509,7 @@ cudaError_t launch_sum(const double* x, int64_t n, double scale, double* partial
 // ---- step kernels (pd_step_f32.cu / pd_step_f64.cu) --------------------------
 cudaError_t launch_step_f32(const StepArgsF32& a, int sc_mode, int grid, int block,
                             cudaStream_t s);
-cudaError_t launch_step_f64(const StepArgsF64& a, int sc_mode, int grid, int block,
+cudaError_t launch_step_f64(const StepArgsF64& a, const W3Args& d, int grid, int block,
                             cudaStream_t s);
 const void* step_f32_kernel(int sc_mode, bool uniform_w, bool per_bond_c);
 // extended-epilogue build (velocity-Verlet, smooth loading start, force pass)
@@ -500,7 +537,19 @@ const void* step_f32_kernel_lat_batch_r80(int sc_mode, bool per_bond_c);
 cudaError_t launch_step_f32_soft(const StepArgsF32& a, int sc_mode, int grid, int block,
                                  cudaStream_t s);
 const void* step_f32_kernel_soft(int sc_mode, bool uniform_w, bool per_bond_c);
-const void* step_f64_kernel(int sc_mode);
+const void* step_f64_kernel(bool uniform_w, bool team);
+// literal FP64 step of the models with softening (pd_step_f64_soft.cu)
+cudaError_t launch_step_f64_soft(const StepArgsF64& a, int grid, int block, cudaStream_t s);
+const void* step_f64_soft_kernel(int sc_mode);
+// dynamic shared memory of a block of the FP64 step
+size_t step_f64_smem(int team, int max_seg, int block);
+// three-word records of every node from its FP64 record, and U / |xi| of every slot
+cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, double scale,
+                              int x_grid, const int32_t* inst, const InstParams* itab,
+                              cudaStream_t s);
+cudaError_t launch_w3_ilen(const double* ilen, const int32_t* nbr, const int32_t* sw, int64_t n,
+                           int Q, double scale, const int32_t* inst, const InstParams* itab,
+                           float2* il, cudaStream_t s);
 cudaError_t launch_step_dw(const StepArgsF64& a, const DwArgs& d, int sc_mode, int grid, int block,
                            cudaStream_t s);
 const void* step_dw_kernel(int sc_mode, bool uniform_w, bool soft, bool vv);
@@ -536,12 +585,17 @@ cudaError_t launch_get_state_f64(const double* rec64, const double* v64, const i
                                  int64_t n, double* u_out, double* v_out, cudaStream_t s);
 cudaError_t launch_set_state_f64(const double* u_in, const double* v_in, const int32_t* gid,
                                  int64_t n, double* rec64, double* v64, cudaStream_t s);
-// damage from the bond flags (Eq. 8), written to caller order
+// damage from the bond flags (Eq. 8), written to caller order (library order if gid is null)
 // (integ: per-slot integrity weighting each intact bond, or nullptr)
 cudaError_t launch_damage(int precision, const void* wrec, const int32_t* nbr,
                           const uint32_t* bits, const int32_t* sw, const void* wsum_inv,
                           const int32_t* gid, int64_t n, int Q, const void* integ,
                           double* phi_out, cudaStream_t s);
+// the same for the FP64 step's handles, as its kernel writes it (damage_lost)
+cudaError_t launch_damage_lost(bool uniform_w, const double* rec, const int32_t* nbr,
+                               const uint32_t* bits, const uint32_t* bits0, const double* wsum_inv,
+                               const double* phi0, const int32_t* gid, int64_t n, int Q,
+                               double* phi_out, cudaStream_t s);
 // flag |= 1 if any of x[0..m) is not finite
 cudaError_t launch_check_finite(const double* x, int64_t m, int* flag, cudaStream_t s);
 // clear the bond flags of m slots (bits[word[e]] &= ~mask[e]) and zero their
@@ -562,6 +616,7 @@ cudaError_t launch_osb_setup(const StepArgsF64& a, const OsbArgs& o, const doubl
                              cudaStream_t s);
 cudaError_t launch_osb_step(const StepArgsF64& a, const OsbArgs& o, int grid, int block,
                             cudaStream_t s);
+const void* osb_force_kernel();
 cudaError_t launch_osb32_setup(const StepArgsF32& a, const OsbArgs32& o, cudaStream_t s);
 // the two state-based launches, each on a grid sized by its own occupancy
 cudaError_t launch_osb32_step(const StepArgsF32& a, const OsbArgs32& o, int sc_mode, int grid,
@@ -601,6 +656,35 @@ __device__ __forceinline__ double soft_mu_of(double s, double s0, double sc, dou
         return s0 * beta * (sc - s) / ((sc - s1) * s);
     }
     return s0 * (sc - s) / (s * (sc - s0));
+}
+#endif
+
+// Damage (Eq. 8) of a node of the FP64 step from what its family has lost: with
+// equal weights a ratio of counts, else the weights of the broken bonds times
+// wi = 1 / sum_j w_j (0 without a family).  An intact node has phi0 = 1 - wi sum_j w_j
+// as FP64 rounds it, computed with the weights.  The flags may have been written by
+// other warps of the block, before its last barrier.
+#ifdef __CUDACC__
+__device__ __forceinline__ double damage_lost(bool uniform_w, const double* __restrict__ rec,
+                                              const int32_t* __restrict__ nbr,
+                                              const uint32_t* bits,
+                                              const uint32_t* __restrict__ bits0, double wi,
+                                              double phi0, int64_t g, int lane, int Q)
+{
+    int was = 0, now = 0;
+    double lost = 0.0;
+    for (int q = 0; q < Q; ++q) {
+        const int64_t w = (g * Q + q) * 32 + lane;
+        const uint32_t b0 = __ldg(bits0 + w), b1 = __ldcg(bits + w);
+        was += __popc(b0);
+        now += __popc(b1);
+        if (!uniform_w)
+            for (uint32_t m = b0 & ~b1; m; m &= m - 1u)
+                lost += rec[8 * (int64_t)nbr[((g * Q + q) * 32 + __ffs(m) - 1) * 32 + lane] + 3];
+    }
+    if (was == now) return phi0;
+    if (now == 0) return 1.0;
+    return uniform_w ? (double)(was - now) / (double)was : fmin(1.0, lost * wi);
 }
 #endif
 

@@ -1,26 +1,41 @@
 // Fused FP64 peridynamic step kernel for sm_103a (the parity path).
 //
-// Same decomposition as the FP32-bulk kernel (lane per node over the sliced
-// family layout, double-buffered displacement, bond flags as the lane's own
-// bit words, integration and damage in the same pass), but every quantity is
-// FP64 and the stretch is that of Eq. 4, s = (|xi + eta| - |xi|) / |xi|, so
-// break decisions are FP64 decisions.  GB300's FP64 rate is a small fraction
-// of its FP32 rate and this kernel is bound by it, so the per-bond square roots
-// and divisions are avoided: 1/|xi| is a per-slot array computed once (8 bytes
-// per bond: memory is not the limit here), and 1/|y| comes from a Newton-
-// refined reciprocal square root; then |y| = |y|^2 / |y|, s = |y| / |xi| - 1
-// (one rounding, an absolute error of a few 1e-16) and the force scale is
-// c V s / |y| with multiplications only.
-// Node record: 8 doubles {x, y, z, w, ux, uy, uz, 0}, w = c V (or V with
-// per-bond stiffness).
+// Same decomposition as the other step kernels (lane per node over the sliced
+// family layout, double-buffered displacement, bond flags as the lane's own bit
+// words, integration and damage in the same pass).  Node state and integration
+// are FP64.  GB300 issues one FP64 operation in the time of 64 FP32 ones, so a
+// kernel that forms Eq. 4 literally in FP64 (about 41 FP64 operations a bond) is
+// bound by that pipe: 1.88 ms per step of a 180x35x35 notched beam, and 0.29 ms of a
+// 4000-node bar, whose 125 warps each walk a whole family alone.  With the arithmetic
+// and the split below they take 0.285 and 0.018 ms, 277 warp instructions a bond, bound
+// by their issue (66 % active; 16 warps per SM at 128 registers).
+// Here the FP64 differences x_j - x_i and u_j - u_i come exactly from three-word
+// FP32 records, and the stretch without cancellation in double-word arithmetic
+// (pd_w3.h): no FP64 operation on the bonds of the bulk.  The literal form rounds
+// s = |y| / |xi| - 1 at an absolute 3e-16, 3e-12 of the force at a stretch of
+// 1e-4; this one has a relative error of about 1e-14 of the force, so it is the more
+// accurate of the two up to stretches of about 1 % (velocities of the beam after 5
+// steps: 6e-13 relative to the exact step instead of 1.2e-11).  The other bonds are decided and
+// evaluated literally in FP64 after their segment (literal_bond): those past kW3XMax
+// and those in or above the band below the smallest s_c, so that every break is an
+// FP64 decision on Eq. 4.  Models with softening take the literal kernel of
+// pd_step_f64_soft.cu for every bond.
+//
+// Work split: a family is walked in segments of 16 slots whose force sums are
+// added up in segment order, so the result does not depend on which warp walks
+// which segment.  A model with few slices gives each slice to a team of warps
+// (TEAM), which take its segments in turn and add their sums through shared memory.
 #include <cuda_runtime.h>
 
 #include "pd_internal.h"
+#include "pd_w3.h"
 
 namespace pd {
 namespace {
 
-constexpr int kUnroll = 2;
+using namespace w3;
+
+constexpr int kSeg = kW3Seg;  // slots per segment
 
 __device__ __forceinline__ uint64_t splitmix_out(uint64_t seed, uint64_t m)
 {
@@ -39,187 +54,384 @@ __device__ __forceinline__ double sc_draw(uint64_t seed, double lo, double hi, i
     return lo + (hi - lo) * ((double)(h >> 11) * 0x1.0p-53);
 }
 
-__device__ __noinline__ bool pair_no_fail(const uint8_t* __restrict__ bcc,
-                                          const BcClass* __restrict__ bct, int64_t i, int64_t j)
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes)
 {
-    return ((bct[bcc[i]].mask | bct[bcc[j]].mask) & 8u) != 0u;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-template <int SCM>
-__global__ void __launch_bounds__(256) k_step_f64(const StepArgsF64 a)
+// One bond literally in FP64: s = |y| / |xi| - 1 (1/|xi| stored per slot, 1/|y| from
+// the Newton-refined reciprocal square root), the break test against the bond's s_c,
+// the no-fail rule, and the force, added to f.  True when it breaks.
+__device__ __noinline__ bool literal_bond(const StepArgsF64& a, int cur, int64_t i, int64_t j,
+                                          int64_t slot, double* f)
+{
+    const double2* __restrict__ rin = reinterpret_cast<const double2*>(a.rec[cur]);
+    const double2 x01 = __ldg(rin + 4 * i), x2w = __ldg(rin + 4 * i + 1);
+    const double2 u01 = __ldg(rin + 4 * i + 2), u2_ = __ldg(rin + 4 * i + 3);
+    const double2 X01 = __ldg(rin + 4 * j), X2w = __ldg(rin + 4 * j + 1);
+    const double2 U01 = __ldg(rin + 4 * j + 2), U2_ = __ldg(rin + 4 * j + 3);
+    const double yx = (X01.x - x01.x) + (U01.x - u01.x);
+    const double yy = (X01.y - x01.y) + (U01.y - u01.y);
+    const double yz = (X2w.x - x2w.x) + (U2_.x - u2_.x);
+    const double y2 = yx * yx + yy * yy + yz * yz;
+    const double ir = rsqrt_nr(y2);
+    const double s = fma(y2 * ir, __ldg(a.ilen + slot), -1.0);
+    double sc = a.sc;
+    if (a.inst != nullptr) {  // batch: instance parameters, local ids as keys
+        const InstParams& ip = a.itab[a.inst[i]];
+        sc = ip.sc_mode == 1 ? sc_draw(ip.sc_seed, ip.sc_lo, ip.sc_hi, a.hid[i], a.hid[j]) : ip.sc;
+    } else if (a.sc_mode == 1) {
+        sc = sc_draw(a.sc_seed, a.sc_lo, a.sc_hi, a.gid[i], a.gid[j]);
+    }
+    bool brk = !a.frozen && s >= sc;
+    if (brk && a.has_nofail) brk = ((a.bct[a.bcc[i]].mask | a.bct[a.bcc[j]].mask) & 8u) == 0u;
+    if (brk) return true;
+    double w = X2w.y;
+    if (a.cbond != nullptr) w *= __ldg(a.cbond + slot);
+    const double c = w * s * ir;
+    f[0] += c * yx;
+    f[1] += c * yy;
+    f[2] += c * yz;
+    return false;
+}
+
+// F += coef y when `ok` (a select: whatever a masked slot computed, including
+// a non-finite value, is dropped)
+__device__ __forceinline__ void add_force(Dw (&F)[3], const Bond& b, bool ok)
+{
+    const Dw cf{ok ? b.coef.h : 0.0f, ok ? b.coef.l : 0.0f};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const Dw f = dw_mul(cf, b.y[k]);
+        const Dw t = two_sum(F[k].h, f.h);
+        F[k].h = t.h;
+        F[k].l += t.l + f.l;
+    }
+}
+
+// The sums of a segment, or of a whole family, of the 32 nodes of a slice, in shared
+// memory (the walk's registers are all taken).
+struct __align__(16) Sums {
+    float F[6][32];   // sum of -s y / |y| (times w_j / w_ref and c_ij), leading and low words
+    double lit[3][32];  // force density of the literally evaluated bonds
+};
+
+// One segment of the family of the lane's node: into S, or added to it.
+template <bool UW, bool TEAM>
+__device__ __forceinline__ void walk_segment(const StepArgsF64& a, const W3Args& d, int cur,
+                                             const Own& own, float x_hi, float ts, int64_t i,
+                                             int64_t g, int seg, int Wg, Sums& S)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int Q = a.Q;
+    const float4* __restrict__ R = d.rec[cur];
+    const int m_lo = seg * kSeg;
+    const int nch = (min(kSeg, Wg - m_lo) + 1) >> 1;  // chunks of two slots (bonds A and B)
+    const int64_t slot0 = (g * 32LL * Q + m_lo) * 32 + lane;
+    const int32_t* __restrict__ col = a.nbr + slot0;
+    uint32_t* bw = a.bits + (g * Q + (m_lo >> 5)) * 32 + lane;
+    const int sh = m_lo & 31;
+    const uint32_t word = (*bw >> sh) & ((1u << kSeg) - 1u);
+    uint32_t pend = 0u;
+    Dw F[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    int32_t jn0 = __ldg(col), jn1 = __ldg(col + 32);
+    for (int c = 0; c < nch; ++c) {
+        const int32_t j0 = jn0, j1 = jn1;
+        if (c + 1 < nch) {
+            jn0 = __ldg(col + (2 * c + 2) * 32);
+            jn1 = __ldg(col + (2 * c + 3) * 32);
+        }
+        Rec A, B;
+        dwa::ld_rec(R + 4 * (int64_t)j0, A.a0, A.a1);
+        dwa::ld_rec(R + 4 * (int64_t)j0 + 2, A.b0, A.b1);
+        dwa::ld_rec(R + 4 * (int64_t)j1, B.a0, B.a1);
+        dwa::ld_rec(R + 4 * (int64_t)j1 + 2, B.b0, B.b1);
+        const int64_t sA = slot0 + 2 * c * 32, sB = sA + 32;
+        Bond bA = bond_w3(own, A, __ldg(d.il + sA), ts);
+        Bond bB = bond_w3(own, B, __ldg(d.il + sB), ts);
+        // literal evaluation: near or past s_c, past kW3XMax, or not a number
+        const bool litA = !(bA.x.h < x_hi) || !(bA.x.h > -kW3XMax);
+        const bool litB = !(bB.x.h < x_hi) || !(bB.x.h > -kW3XMax);
+        if (d.cb != nullptr) {  // per-bond stiffness (a uniform branch)
+            const float2 cA = __ldg(d.cb + sA), cB = __ldg(d.cb + sB);
+            bA.coef = dw_mul(bA.coef, Dw{cA.x, cA.y});
+            bB.coef = dw_mul(bB.coef, Dw{cB.x, cB.y});
+        }
+        const uint32_t wb = word >> (2 * c);
+        pend |= (((litA ? 1u : 0u) | (litB ? 2u : 0u)) & wb) << (2 * c);
+        const bool okA = (wb & 1u) && !litA, okB = (wb & 2u) && !litB;
+        if (!UW) {
+            const float2 wA = __ldg(d.wrel + j0), wB = __ldg(d.wrel + j1);
+            bA.coef = dw_mul(bA.coef, Dw{wA.x, wA.y});
+            bB.coef = dw_mul(bB.coef, Dw{wB.x, wB.y});
+        }
+        // the next chunk's records start toward L1 (their ids have arrived by now)
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(R + 4 * (int64_t)jn0));
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(R + 4 * (int64_t)jn1));
+        add_force(F, bA, okA);
+        add_force(F, bB, okB);
+    }
+    const bool any = pend != 0u;
+    uint32_t gone = 0u;
+    double lit[3] = {0.0, 0.0, 0.0};
+    while (pend) {
+        const int b = __ffs(pend) - 1;
+        pend &= pend - 1u;
+        const int64_t j = col[(int64_t)b * 32];
+        if (literal_bond(a, cur, i, j, slot0 + (int64_t)b * 32, lit)) gone |= 1u << b;
+    }
+    // another warp of the team may own the other half of the flag word
+    if (gone) atomicAnd(bw, ~(gone << sh));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const Dw t = TEAM ? F[k] : dw_add(Dw{S.F[2 * k][lane], S.F[2 * k + 1][lane]}, F[k]);
+        S.F[2 * k][lane] = t.h;
+        S.F[2 * k + 1][lane] = t.l;
+        if (TEAM) S.lit[k][lane] = lit[k];
+        else if (any) S.lit[k][lane] += lit[k];
+    }
+}
+
+// Integration of the lane's node (damped Euler-Cromer, Eq. 11, or damped
+// velocity-Verlet), BCs, damage, and the records its neighbours read next.
+__device__ __forceinline__ void finish_node(const StepArgsF64& a, const W3Args& d, int cur,
+                                            int64_t step, bool first, const Rec& me, double scale,
+                                            int64_t i, const double (&T)[3])
+{
+    const double2* __restrict__ rin = reinterpret_cast<const double2*>(a.rec[cur]);
+    double2* __restrict__ rout = reinterpret_cast<double2*>(const_cast<double*>(a.rec[cur ^ 1]));
+    float4* __restrict__ Rout = const_cast<float4*>(d.rec[cur ^ 1]);
+    const uint32_t cls = a.bcc[i];
+    uint32_t mask = 0u;
+    double gdisp[3] = {0.0, 0.0, 0.0};
+    double F[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        F[c] = T[c];
+    if (cls != 0u) {
+        const BcClass& bc = a.bct[cls];
+        mask = bc.mask;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            gdisp[c] = bc.disp[c];
+            F[c] += a.load * bc.force[c];
+        }
+    }
+    const double2 u01 = __ldg(rin + 4 * i + 2), u2_ = __ldg(rin + 4 * i + 3);
+    const double uo[3] = {u01.x, u01.y, u2_.x};
+    double un[3];
+    float uh[3], um[3], tw[3];
+    const float tin[3] = {me.a1.z, me.a1.w, me.b1.z};
+    bool finite = true;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        // stored velocity: v^n (Euler-Cromer) or, for velocity-Verlet, the
+        // half-step velocity v^{n-1} + dt/2 a^{n-1} (v^n right after a set state)
+        const double vi = a.v[3 * i + c];
+        const double adt = (F[c] - a.eta * vi) * d.dt_rho;  // dt a
+        double vn, vfull;
+        if (a.vv) {
+            vfull = first ? vi : fma(0.5, adt, vi);
+            vn = fma(0.5, adt, vfull);
+        } else {
+            vn = vi + adt;
+            vfull = vn;
+        }
+        double u = fma(a.dt, vn, uo[c]);
+        if (mask & (1u << c)) {
+            const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
+            const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
+            u = gdisp[c] * s_next;
+            vn = gdisp[c] * (s_next - s_now) / a.dt;
+            vfull = vi;
+        }
+        finite = finite && isfinite(u);
+        un[c] = u;
+        if (a.peek)
+            a.vout[3 * i + c] = vfull;
+        else
+            a.v[3 * i + c] = vn;
+        float ut;
+        split3(u * scale, kW3UGrid, uh[c], um[c], ut);
+        tw[c] = pack_t(__float_as_uint(tin[c]) & 0x7ffu, ut);
+    }
+    if (a.peek) return;
+    rout[4 * i + 2] = make_double2(un[0], un[1]);  // (positions and weights: in both buffers)
+    rout[4 * i + 3] = make_double2(un[2], 0.0);
+    dwa::st_rec(Rout + 4 * i, make_float4(me.a0.x, me.a0.y, me.a0.z, uh[0]),
+                make_float4(uh[1], uh[2], tw[0], tw[1]));
+    dwa::st_rec(Rout + 4 * i + 2, make_float4(me.b0.x, me.b0.y, me.b0.z, um[0]),
+                make_float4(um[1], um[2], tw[2], 0.0f));
+    a.damage[i] = damage_lost(d.uniform_w != 0, a.rec[cur], a.nbr, a.bits, a.bits0, a.wsum_inv[i],
+                              d.phi0[i], i >> 5, (int)(i & 31), a.Q);
+    if (!finite) atomicOr(a.err, PD_DEVERR_NONFINITE);
+}
+
+template <bool UW, bool TEAM>
+__global__ void __launch_bounds__(256, 2)
+    k_step_f64(const __grid_constant__ StepArgsF64 a, const __grid_constant__ W3Args d)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31;
+    const int wpb = blockDim.x >> 5;
+    const int team = TEAM ? d.team : 1;       // warps per slice
+    const int tpb = wpb / team;               // slices per block at a time
+    const int tm = (int)(threadIdx.x >> 5) / team;
+    const int rank = (int)(threadIdx.x >> 5) % team;
+    // the slice's sums: one entry, or one per segment for a team
+    Sums* const S = reinterpret_cast<Sums*>(smem) + (TEAM ? tm * d.max_seg : tm);
     const int64_t step = a.step_ctr[0] + a.k;
     const bool first = a.vv && step == a.step_ctr[1];  // velocity-Verlet: a^n formed afresh
     const int cur = (int)(step & 1);
-    const int Q = a.Q;
-    const int64_t W = 32LL * Q;
     const int64_t nslices = (a.n + 31) >> 5;
-    const double2* __restrict__ rin = reinterpret_cast<const double2*>(a.rec[cur]);
-    double2* __restrict__ rout = reinterpret_cast<double2*>(const_cast<double*>(a.rec[cur ^ 1]));
-    const double* __restrict__ cb = a.cbond;
+    const float4* __restrict__ R = d.rec[cur];
 
-    for (int64_t g = wid; g < nslices; g += nwarps) {
+    // (every warp of a block makes the same number of rounds: teams synchronise)
+    for (int64_t g0 = (int64_t)blockIdx.x * tpb; g0 < nslices; g0 += (int64_t)gridDim.x * tpb) {
+        const int64_t g = g0 + tm;
+        const bool have = g < nslices;
+        if (!TEAM && !have) continue;
         const int64_t i = (g << 5) + lane;
-        const int Wg = a.sw[g];
-        const double2 x01 = __ldg(rin + 4 * i), x23 = __ldg(rin + 4 * i + 1);
-        const double2 u01 = __ldg(rin + 4 * i + 2), u23 = __ldg(rin + 4 * i + 3);
-        const int32_t* __restrict__ col = a.nbr + g * W * 32 + lane;
-        uint32_t* bw = a.bits + g * Q * 32 + lane;
-        double fx = 0.0, fy = 0.0, fz = 0.0, ws = 0.0;
-
-        for (int q = 0; q * 32 < Wg; ++q) {
-            const uint32_t word = bw[q * 32];
-            uint32_t nword = word;
-            const int mend = min(32, Wg - q * 32);
-            for (int b0 = 0; b0 < mend; b0 += kUnroll) {
-                int32_t jj[kUnroll];
-                bool al[kUnroll];
-                double2 ra[kUnroll][4];
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    const int b = b0 + u;
-                    al[u] = (b < mend) && ((word >> b) & 1u);
-                    jj[u] = al[u] ? __ldg(col + (int64_t)(q * 32 + b) * 32) : 0;
-                }
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u)
-                    if (al[u])
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) ra[u][e] = __ldg(rin + 4 * (int64_t)jj[u] + e);
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    if (!al[u]) continue;
-                    const double ex = ra[u][0].x - x01.x, ey = ra[u][0].y - x01.y;
-                    const double ez = ra[u][1].x - x23.x;
-                    const double yx = ex + (ra[u][2].x - u01.x);
-                    const double yy = ey + (ra[u][2].y - u01.y);
-                    const double yz = ez + (ra[u][3].x - u23.x);
-                    const int64_t slot = (g * W + q * 32 + b0 + u) * 32 + lane;
-                    const double y2 = yx * yx + yy * yy + yz * yz;
-                    const double ir = rsqrt_nr(y2);
-                    const double r = y2 * ir;
-                    const double s = fma(r, __ldg(a.ilen + slot), -1.0);
-                    double sc;
-                    if (a.inst != nullptr) {  // batch: instance parameters, local ids as keys
-                        const InstParams& ip = a.itab[a.inst[i]];
-                        sc = ip.sc_mode == 1 ? sc_draw(ip.sc_seed, ip.sc_lo, ip.sc_hi, a.hid[i],
-                                                       a.hid[jj[u]])
-                                             : ip.sc;
-                    } else {
-                        sc = (SCM == 0) ? a.sc
-                                        : sc_draw(a.sc_seed, a.sc_lo, a.sc_hi, a.gid[i],
-                                                  a.gid[jj[u]]);
-                    }
-                    bool brk = !a.frozen && s >= sc;
-                    if (brk && a.has_nofail) brk = !pair_no_fail(a.bcc, a.bct, i, jj[u]);
-                    if (brk) {
-                        nword &= ~(1u << (b0 + u));
-                        if (a.integ != nullptr) a.integ[slot] = 0.0;
-                    } else {
-                        // bilinear softening: the integrity only decreases, as the
-                        // stretch passes s_0 = s_c / kr (a no-fail bond past s_c keeps 0)
-                        double mu = 1.0;
-                        if (a.integ != nullptr) {
-                            mu = a.integ[slot];
-                            const double s0 = sc / a.kr;
-                            if (s > s0) {
-                                const double ms =
-                                    s >= sc ? 0.0 : soft_mu_of(s, s0, sc, a.k1, a.beta);
-                                if (ms < mu) {
-                                    mu = ms;
-                                    a.integ[slot] = ms;
-                                }
-                            }
-                        }
-                        double wj = ra[u][1].y * mu;
-                        if (cb != nullptr) wj *= __ldg(cb + slot);
-                        const double f = wj * s * ir;
-                        fx += f * yx;
-                        fy += f * yy;
-                        fz += f * yz;
-                        ws += ra[u][1].y * mu;
-                    }
-                }
+        Rec me{};
+        int nseg = 0;
+        double w_ref = d.w_ref, scale = d.scale;
+        if (have) {
+            const int Wg = a.sw[g];
+            nseg = (Wg + kSeg - 1) / kSeg;
+            if (lane == 0 && rank == 0)
+                prefetch_l2(a.nbr + g * 32LL * a.Q * 32, (uint32_t)(((Wg + 3) & ~3) * 128));
+            dwa::ld_rec(R + 4 * i, me.a0, me.a1);
+            dwa::ld_rec(R + 4 * i + 2, me.b0, me.b1);
+            const Own own = own_words(me);
+            float x_hi = d.x_hi;
+            int grid = d.x_grid;
+            if (a.inst != nullptr) {  // batch: the instance's own band, weight and unit
+                const InstParams& ip = a.itab[a.inst[i]];
+                w_ref = ip.w_ref;
+                scale = ip.w3_scale;
+                x_hi = a.frozen ? kW3XMax : ip.w3_x_hi;
+                grid = ip.w3_x_grid;
             }
-            if (nword != word) bw[q * 32] = nword;
+            const float ts = pow2(grid - 33);
+            if (!TEAM) {
+#pragma unroll
+                for (int k = 0; k < 6; ++k) S->F[k][lane] = 0.0f;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) S->lit[k][lane] = 0.0;
+            }
+            for (int seg = rank; seg < nseg; seg += team)
+                walk_segment<UW, TEAM>(a, d, cur, own, x_hi, ts, i, g, seg, Wg, S[TEAM ? seg : 0]);
         }
+        if (TEAM) __syncthreads();
+        if (have && rank == 0 && i < a.n) {
+            // the segments' sums in their order, whichever warps formed them
+            Dw F[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+            double T[3] = {0.0, 0.0, 0.0};
+            for (int e = 0; e < (TEAM ? nseg : 1); ++e) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    F[k] = dw_add(F[k], Dw{S[e].F[2 * k][lane], S[e].F[2 * k + 1][lane]});
+                    T[k] += S[e].lit[k][lane];
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) T[k] = fma(-((double)F[k].h + (double)F[k].l), w_ref, T[k]);
+            finish_node(a, d, cur, step, first, me, scale, i, T);
+        }
+        if (TEAM) __syncthreads();  // the sums' memory is free again
+    }
+}
 
-        if (i < a.n) {
-            const uint32_t cls = a.bcc[i];
-            uint32_t mask = 0u;
-            double gdisp[3] = {0.0, 0.0, 0.0};
-            double F[3] = {fx, fy, fz};
-            if (cls != 0u) {
-                const BcClass& bc = a.bct[cls];
-                mask = bc.mask;
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    gdisp[c] = bc.disp[c];
-                    F[c] += a.load * bc.force[c];
-                }
-            }
-            const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
-            const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
-            const double uo[3] = {u01.x, u01.y, u23.x};
-            double un[3];
-            bool finite = true;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                // stored velocity: v^n (Euler-Cromer) or, for velocity-Verlet, the
-                // half-step velocity v^{n-1} + dt/2 a^{n-1} (v^n right after a set state)
-                const double vi = a.v[3 * i + c];
-                double vn, vfull;
-                if (a.vv) {
-                    const double acc = (F[c] - a.eta * vi) / a.rho;
-                    vfull = first ? vi : vi + 0.5 * a.dt * acc;
-                    vn = vfull + 0.5 * a.dt * acc;
-                } else {
-                    vn = vi + a.dt * (F[c] - a.eta * vi) / a.rho;
-                    vfull = vn;
-                }
-                double u = uo[c] + a.dt * vn;
-                if (mask & (1u << c)) {
-                    u = gdisp[c] * s_next;
-                    vn = gdisp[c] * (s_next - s_now) / a.dt;
-                    vfull = vi;
-                }
-                finite = finite && isfinite(u);
-                un[c] = u;
-                if (a.peek)
-                    a.vout[3 * i + c] = vfull;
-                else
-                    a.v[3 * i + c] = vn;
-            }
-            if (a.peek) continue;
-            rout[4 * i] = x01;
-            rout[4 * i + 1] = x23;
-            rout[4 * i + 2] = make_double2(un[0], un[1]);
-            rout[4 * i + 3] = make_double2(un[2], 0.0);
-            const double wi = a.wsum_inv[i];
-            // clamp: ws * (1 / sum w) can round to 1 + 1 ulp for an intact family
-            a.damage[i] = wi > 0.0 ? fmax(0.0, 1.0 - ws * wi) : 0.0;
-            if (!finite) atomicOr(a.err, PD_DEVERR_NONFINITE);
+// Records of every node from its FP64 record
+__global__ void k_w3_publish(const double* __restrict__ rec64, float4* __restrict__ rec,
+                             int64_t n_pad, double scale, int x_grid, const int32_t* __restrict__ inst,
+                             const InstParams* __restrict__ itab)
+{
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_pad;
+         p += (int64_t)gridDim.x * blockDim.x) {
+        const double* r = rec64 + 8 * p;
+        const double sc = inst != nullptr ? itab[inst[p]].w3_scale : scale;
+        const int g = inst != nullptr ? itab[inst[p]].w3_x_grid : x_grid;
+        float xh[3], xm[3], uh[3], um[3], t[3];
+        for (int k = 0; k < 3; ++k) {
+            float xt, ut;
+            split3(r[k] * sc, g, xh[k], xm[k], xt);
+            split3(r[4 + k] * sc, kW3UGrid, uh[k], um[k], ut);
+            t[k] = pack_t(t_int(xt, g), ut);
+        }
+        rec[4 * p] = make_float4(xh[0], xh[1], xh[2], uh[0]);
+        rec[4 * p + 1] = make_float4(uh[1], uh[2], t[0], t[1]);
+        rec[4 * p + 2] = make_float4(xm[0], xm[1], xm[2], um[0]);
+        rec[4 * p + 3] = make_float4(um[1], um[2], t[2], 0.0f);
+    }
+}
+
+// U / |xi| of every slot as a double-word (1 where there is no bond)
+__global__ void k_w3_ilen(const double* __restrict__ ilen, const int32_t* __restrict__ nbr,
+                          const int32_t* __restrict__ sw, int64_t n, int Q, double scale,
+                          const int32_t* __restrict__ inst, const InstParams* __restrict__ itab,
+                          float2* __restrict__ il)
+{
+    const int64_t W = 32LL * Q;
+    const int64_t total = ((n + 31) >> 5) << 5;
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < total;
+         p += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t g = p >> 5;
+        const double U = 1.0 / (inst != nullptr ? itab[inst[p]].w3_scale : scale);  // a power of two
+        for (int m = 0; m < W; ++m) {
+            const int64_t slot = (g * W + m) * 32 + (p & 31);
+            const double v = m < sw[g] && nbr[slot] != p ? ilen[slot] * U : 1.0;
+            const float h = (float)v;
+            il[slot] = make_float2(h, (float)(v - (double)h));
         }
     }
 }
 
+int grid_of(int64_t work)
+{
+    const int64_t b = (work + 255) / 256;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(b, 152 * 16));
+}
+
 }  // namespace
 
-cudaError_t launch_step_f64(const StepArgsF64& a, int sc_mode, int grid, int block, cudaStream_t s)
+size_t step_f64_smem(int team, int max_seg, int block)
 {
-    if (sc_mode == 0)
-        k_step_f64<0><<<grid, block, 0, s>>>(a);
-    else
-        k_step_f64<1><<<grid, block, 0, s>>>(a);
+    return (size_t)(block / 32 / team) * (team > 1 ? max_seg : 1) * sizeof(Sums);
+}
+
+const void* step_f64_kernel(bool uniform_w, bool team)
+{
+    static const void* const k[4] = {
+        (const void*)k_step_f64<false, false>, (const void*)k_step_f64<false, true>,
+        (const void*)k_step_f64<true, false>, (const void*)k_step_f64<true, true>};
+    return k[(uniform_w ? 2 : 0) + (team ? 1 : 0)];
+}
+
+cudaError_t launch_step_f64(const StepArgsF64& a, const W3Args& d, int grid, int block,
+                            cudaStream_t s)
+{
+    const void* fn = step_f64_kernel(d.uniform_w != 0, d.team > 1);
+    void* args[] = {const_cast<StepArgsF64*>(&a), const_cast<W3Args*>(&d)};
+    return cudaLaunchKernel(fn, dim3(grid), dim3(block), args,
+                            step_f64_smem(d.team, d.max_seg, block), s);
+}
+
+cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, double scale,
+                              int x_grid, const int32_t* inst, const InstParams* itab,
+                              cudaStream_t s)
+{
+    k_w3_publish<<<grid_of(n_pad), 256, 0, s>>>(rec64, rec, n_pad, scale, x_grid, inst, itab);
     return cudaGetLastError();
 }
 
-const void* step_f64_kernel(int sc_mode)
+cudaError_t launch_w3_ilen(const double* ilen, const int32_t* nbr, const int32_t* sw, int64_t n,
+                           int Q, double scale, const int32_t* inst, const InstParams* itab,
+                           float2* il, cudaStream_t s)
 {
-    return sc_mode == 0 ? (const void*)k_step_f64<0> : (const void*)k_step_f64<1>;
+    k_w3_ilen<<<grid_of(((n + 31) >> 5) << 5), 256, 0, s>>>(ilen, nbr, sw, n, Q, scale, inst, itab,
+                                                            il);
+    return cudaGetLastError();
 }
 
 }  // namespace pd

@@ -289,4 +289,6 @@ cudaError_t launch_osb_step(const StepArgsF64& a, const OsbArgs& o, int grid, in
     return cudaGetLastError();
 }
 
+const void* osb_force_kernel() { return (const void*)k_osb_force; }
+
 }  // namespace pd
