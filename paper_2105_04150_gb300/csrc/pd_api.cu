@@ -186,6 +186,10 @@ struct pd_handle {
         // per-slot gradient accumulator
         float4 *rrec = nullptr, *wrec = nullptr;
         float2* gcdw = nullptr;
+        // FP64 reverse sweep (pd_adjoint_w3.cu): w in FP64 records, xi / |xi|^(3/2) per
+        // slot, the seeds' largest component
+        double *w64 = nullptr, *e = nullptr;
+        unsigned long long* wmax = nullptr;
     } tape;
     // regular lattice (FP32 Euler-Cromer PMB models): stencil-ordered layout,
     // FP64 displacement and FP32 published records with a halo of lat_halo
@@ -2123,6 +2127,15 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
             (e = h->alloc(&T.gcdw, (size_t)slots)) != cudaSuccess)
             return cuda_fail(e, "cudaMalloc double-word adjoint buffers");
     }
+    if (h->w3 && !T.e) {
+        if ((e = h->alloc(&T.rrec, (size_t)(4 * h->n_pad))) != cudaSuccess ||
+            (e = h->alloc(&T.wrec, (size_t)(2 * h->n_pad))) != cudaSuccess ||
+            (e = h->alloc(&T.w64, (size_t)(4 * h->n_pad))) != cudaSuccess ||
+            (e = h->alloc(&T.wmax, 1)) != cudaSuccess ||
+            (e = h->alloc(&T.e, (size_t)(3 * slots))) != cudaSuccess)
+            return cuda_fail(e, "cudaMalloc adjoint records");
+        PD_CUDA(launch_adj_e(h->rec[0], h->nbr, h->n_slices, h->Q, T.e, h->stream), "bond vectors");
+    }
     // seed: dL/du^N, dL/dv^N in library order
     auto to_lib = [&](const double* src, double* dst) -> pd_status {
         if (!src) {
@@ -2146,28 +2159,46 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
     PD_CUDA(cudaMemsetAsync(T.gc, 0, 8 * slots, h->stream), "memset");
     PD_CUDA(cudaMemsetAsync(T.gl, 0, 8 * h->n_pad, h->stream), "memset");
     if (h->dw) PD_CUDA(cudaMemsetAsync(T.gcdw, 0, 8 * slots, h->stream), "memset");
+    if (h->w3)
+        PD_CUDA(launch_adj_scale_w3(T.ub[0], T.vb[0], np3, h->dt, T.wmax, h->stream),
+                "gradient scale");
 
     int sms = 0;
     PD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device), "sm count");
     const int agrid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * 8,
                                                                   (h->n_slices + 7) / 8));
-    AdjArgs A{};
-    A.x64 = h->x64;
-    A.nbr = h->nbr;
-    A.bits = h->bits;
-    A.sw = h->sw;
-    A.Q = h->Q;
-    A.vol = h->vol;
-    A.cbond = h->per_bond_c ? (const double*)h->cbond : nullptr;
-    A.ilen = h->ilen;
-    A.c = h->c;
-    A.gc = T.gc;
-    A.gl = T.gl;
-    A.bcc = h->bcc;
-    A.bct = h->bct;
-    A.dt_rho = h->dt / h->rho;
-    A.damp = 1.0 - h->dt * h->eta / h->rho;
-    A.n = h->n;
+    const double dt_rho = h->dt / h->rho;
+    AdjW3Args A{};
+    if (h->w3) {
+        A.x64 = h->rec[0];
+        A.rec = T.rrec;
+        A.w64 = T.w64;
+        A.wdw = T.wrec;
+        A.ubm = T.ubm;
+        A.wmax = T.wmax;
+        A.nbr = h->nbr;
+        A.bits = h->bits;
+        A.sw = h->sw;
+        A.Q = h->Q;
+        A.uniform_w = h->uniform_vol ? 1 : 0;
+        A.x_grid = h->w3_x_grid;
+        A.vol = h->vol;
+        A.wrel = h->wrel3;
+        A.cbond = h->per_bond_c ? (const double*)h->cbond : nullptr;
+        A.cb = h->cb3;
+        A.ilen = h->ilen;
+        A.e = T.e;
+        A.il = h->il3;
+        A.gc = (float2*)T.gc;
+        A.gl = T.gl;
+        A.bcc = h->bcc;
+        A.bct = h->bct;
+        A.scale = h->w3_scale;
+        A.w_ref = (h->per_bond_c ? 1.0 : h->c) * h->vol0;
+        A.inv_vref = 1.0 / h->vol0;
+        A.dt_rho = dt_rho;
+        A.n = h->n;
+    }
     AdjDwArgs D{};
     if (h->dw) {
         D.rec = T.rrec;
@@ -2188,8 +2219,7 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         D.n = h->n;
         D.bcc = h->bcc;
         D.bct = h->bct;
-        D.dt_rho = A.dt_rho;
-        D.damp = A.damp;
+        D.dt_rho = dt_rho;
         D.inv_delta = 1.0 / h->delta;
         D.vol0 = h->vol0;
     }
@@ -2202,27 +2232,23 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
     // velocity) between a half kick at its first step and a half kick that
     // forms the full-step velocity it ends with: ws = 1/2 there, and
     // damp = 1 + (1 - dt eta / rho) so that damp ws = 1 - dt eta / (2 rho)
-    const double damp_full = A.damp;
+    const double damp_full = 1.0 - h->dt * h->eta / h->rho;
     auto reverse_step = [&](const double* un, double dtw, double ws, double damp) {
-        A.un = un;
-        A.w = T.w;
-        A.ubm = T.ubm;
-        A.ub_out = T.ub[cb ^ 1];
-        A.vb_out = T.vb[cb ^ 1];
-        A.damp = damp;
         cudaError_t r;
         if (h->dw) {
             r = launch_adj_mask_publish_dw(T.ub[cb], T.vb[cb], h->bcc, h->bct, dtw, ws,
                                            h->recdw[0], un, h->vol, h->n_pad, 1.0 / h->delta,
                                            T.ubm, T.w, T.rrec, T.wrec, h->stream);
-            D.ub_out = A.ub_out;
-            D.vb_out = A.vb_out;
+            D.ub_out = T.ub[cb ^ 1];
+            D.vb_out = T.vb[cb ^ 1];
             D.damp = damp;
             if (r == cudaSuccess) r = launch_adj_step_dw(D, agrid, 256, h->stream);
         } else {
-            r = launch_adj_mask(T.ub[cb], T.vb[cb], h->bcc, h->bct, h->n_pad, dtw, ws, T.ubm, T.w,
-                                h->stream);
-            if (r == cudaSuccess) r = launch_adj_step(A, agrid, 256, h->stream);
+            A.un = un;
+            A.ub_out = T.ub[cb ^ 1];
+            A.vb_out = T.vb[cb ^ 1];
+            A.damp = damp;
+            r = launch_adj_step_w3(A, T.ub[cb], T.vb[cb], h->rec3[0], dtw, ws, h->n_pad, h->stream);
         }
         cb ^= 1;
         return r;
@@ -2258,8 +2284,9 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
                               half ? 1.0 + damp_full : damp_full);
         }
     }
-    if (h->dw && ke == cudaSuccess)
-        ke = launch_adj_merge_dw(T.gcdw, slots, A.dt_rho, T.gc, h->stream);
+    if (ke == cudaSuccess)
+        ke = h->dw ? launch_adj_merge_dw(T.gcdw, slots, dt_rho, T.gc, h->stream)
+                   : launch_adj_merge_w3(T.gc, slots, dt_rho * h->vol0, T.wmax, h->stream);
     h->frozen = false;
     h->drop_graph();
     // restore the final state u^N, v^N
@@ -2278,7 +2305,7 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
 
     // outputs
     if (dL_dload) {
-        PD_CUDA(launch_sum(T.gl, h->n, A.dt_rho, T.partial, T.n_partial, T.out, h->stream),
+        PD_CUDA(launch_sum(T.gl, h->n, dt_rho, T.partial, T.n_partial, T.out, h->stream),
                 "load gradient");
         PD_CUDA(cudaMemcpyAsync(dL_dload, T.out, sizeof(double), cudaMemcpyDeviceToHost, h->stream),
                 "copy load gradient");

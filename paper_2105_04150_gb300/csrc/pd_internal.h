@@ -477,6 +477,54 @@ struct AdjDwArgs {
     double dt_rho, damp, inv_delta, vol0;
 };
 
+// Reverse step of bond-based FP64 handles (pd_adjoint_w3.cu)
+struct AdjW3Args {
+    const double* x64;         // the FP64 step records (8 doubles per node, positions first)
+    const double* un;          // u^n, the state the forward step n -> n+1 read
+    float4* rec;               // 4 float4 per node: three-word record of x and u^n
+    double* w64;               // 4 doubles per node: w, 0
+    float4* wdw;               // 2 float4 per node: w as double-words, scaled
+    double* ubm;               // ubar of step n+1, controlled components zeroed
+    const unsigned long long* wmax;  // bits of the seeds' largest component (sets the scale)
+    double* ub_out;            // ubar^n
+    double* vb_out;            // vbar^n
+    const int32_t* nbr;
+    const uint32_t* bits;      // frozen bond flags
+    const int32_t* sw;
+    int32_t Q;
+    int32_t uniform_w;         // 1: every node has volume V_ref
+    int32_t x_grid;            // W3Args::x_grid
+    int32_t pad0;
+    const double* vol;
+    const float2* wrel;        // per node V / V_ref as a double-word (non-uniform volumes)
+    const double* cbond;       // per-slot stiffness, or nullptr for the constant c
+    const float2* cb;          // the same as double-words
+    const double* ilen;        // per slot 1 / |xi|
+    const double* e;           // per slot xi / |xi|^(3/2), rows of 32 lanes per component
+    const float2* il;          // per slot U / |xi| as a double-word
+    float2* gc;                // per-slot dL/dc accumulator (merged to FP64 in place)
+    double* gl;                // per-node accumulator of force . w
+    const uint8_t* bcc;
+    const BcClass* bct;
+    double scale;              // 1 / U
+    double w_ref;              // V_ref, times the constant c without per-bond stiffness
+    double inv_vref;           // 1 / V_ref
+    double dt_rho;             // dt / rho
+    double damp;               // 1 - dt eta / rho
+    int64_t n;
+};
+// the scale of the double-word w from the seeds (once per sweep), the records of one
+// reverse step and the step itself, e of every slot, and the FP64 gradient
+cudaError_t launch_adj_scale_w3(const double* ub, const double* vb, int64_t n3, double dt,
+                                unsigned long long* wmax, cudaStream_t s);
+cudaError_t launch_adj_e(const double* x64, const int32_t* nbr, int64_t n_slices, int Q, double* e,
+                         cudaStream_t s);
+cudaError_t launch_adj_step_w3(const AdjW3Args& a, const double* ub, const double* vb,
+                               const float4* fwd, double dt, double ws, int64_t n_pad,
+                               cudaStream_t s);
+cudaError_t launch_adj_merge_w3(double* gc, int64_t count, double scale,
+                                const unsigned long long* wmax, cudaStream_t s);
+
 cudaError_t launch_adj_mask_publish_dw(const double* ub, const double* vb, const uint8_t* bcc,
                                        const BcClass* bct, double dt, double ws,
                                        const float4* fwd, const double* un, const double* vol,

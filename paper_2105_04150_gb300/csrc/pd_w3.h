@@ -111,14 +111,15 @@ __device__ __forceinline__ Dw diff3(float jh, float jm, float ih, float im, floa
     return {s, fmaf(dt, ts, dm - (s - dh))};
 }
 
-struct Bond {
-    Dw x;     // |y|^2 / |xi|^2 - 1
-    Dw coef;  // -s / |y| (in 1 / U)
-    Dw y[3];  // deformed bond vector (in U)
+// One bond of the lane's node (in units of U).
+struct Geo {
+    Dw xi[3], et[3];  // xi = x_j - x_i, eta = u_j - u_i
+    Dw y[3];          // xi + eta
+    Dw x;             // |y|^2 / |xi|^2 - 1
+    Dw z;             // |xi| / |y| - 1
 };
 
-// One bond of the lane's node; il: the slot's U / |xi| as a double-word; ts: the
-// unit of the positions' t.
+// il: the slot's U / |xi| as a double-word; ts: the unit of the positions' t.
 // num = eta . (2 xi + eta) = |y|^2 - |xi|^2 without cancellation, x = num / |xi|^2,
 // and with r = sqrt(1 + x) = |y| / |xi|: s / |y| = (1 - 1/r) / |xi|.  z = 1/r - 1 is
 // a small number, so it is formed by itself: seeded in FP32 as -x / (r (1 + r))
@@ -126,19 +127,19 @@ struct Bond {
 // (2z + z^2 + x) + x (2z + z^2) is taken in double-word arithmetic (its leading
 // terms cancel exactly).  23 operations, against 45 for the double-word square
 // root, reciprocal and quotient of the direct form; relative error < 2^-44.
-__device__ __forceinline__ Bond bond_w3(const Own& o, const Rec& j, const float2 il, float ts)
+__device__ __forceinline__ Geo bond_geo(const Own& o, const Rec& j, const float2 il, float ts)
 {
     const float jxh[3] = {j.a0.x, j.a0.y, j.a0.z}, juh[3] = {j.a0.w, j.a1.x, j.a1.y};
     const float jxm[3] = {j.b0.x, j.b0.y, j.b0.z}, jum[3] = {j.b0.w, j.b1.x, j.b1.y};
     const float jt[3] = {j.a1.z, j.a1.w, j.b1.z};
-    Bond out;
+    Geo out;
     Dw nm[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const Dw xi = diff3(jxh[c], jxm[c], o.xh[c], o.xm[c], k_of(jt[c]) - o.xk[c], ts);
-        const Dw et = diff3(juh[c], jum[c], o.uh[c], o.um[c], ut_of(jt[c]) - o.ut[c], 1.0f);
-        out.y[c] = dw_add(xi, et);
-        nm[c] = dw_mul(et, dw_add(xi, out.y[c]));  // eta_c (2 xi_c + eta_c)
+        out.xi[c] = diff3(jxh[c], jxm[c], o.xh[c], o.xm[c], k_of(jt[c]) - o.xk[c], ts);
+        out.et[c] = diff3(juh[c], jum[c], o.uh[c], o.um[c], ut_of(jt[c]) - o.ut[c], 1.0f);
+        out.y[c] = dw_add(out.xi[c], out.et[c]);
+        nm[c] = dw_mul(out.et[c], dw_add(out.xi[c], out.y[c]));  // eta_c (2 xi_c + eta_c)
     }
     Dw num = two_sum(nm[0].h, nm[1].h);
     num.l += nm[0].l + nm[1].l;
@@ -153,10 +154,21 @@ __device__ __forceinline__ Bond bond_w3(const Own& o, const Rec& j, const float2
     const Dw p{ph, (zz - fmaf(-2.0f, z0, ph)) + fmaf(z0, z0, -zz)};
     const Dw xp = dw_mul(x, p);
     const float R = ((ph + x.h) + xp.h) + ((p.l + x.l) + xp.l);
-    const Dw z{z0, R * fmaf(z0, -0.5f, -0.5f)};
     out.x = x;
-    out.coef = dw_mul(z, iL);
+    out.z = Dw{z0, R * fmaf(z0, -0.5f, -0.5f)};
     return out;
+}
+
+struct Bond {
+    Dw x;     // |y|^2 / |xi|^2 - 1
+    Dw coef;  // -s / |y| (in 1 / U)
+    Dw y[3];  // deformed bond vector (in U)
+};
+
+__device__ __forceinline__ Bond bond_w3(const Own& o, const Rec& j, const float2 il, float ts)
+{
+    const Geo g = bond_geo(o, j, il, ts);
+    return {g.x, dw_mul(g.z, Dw{il.x, il.y}), {g.y[0], g.y[1], g.y[2]}};
 }
 
 }  // namespace w3

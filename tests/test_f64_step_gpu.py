@@ -93,3 +93,54 @@ def test_result_does_not_depend_on_the_split(shape, jitter):
     for o in out[1:]:
         for a, b in zip(out[0], o):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n_shape", [(5, 4, 3), (13, 7, 6)])
+@pytest.mark.parametrize("jitter", [0.0, 0.2])       # equal and unequal volumes
+@pytest.mark.parametrize("per_bond", [False, True])
+@pytest.mark.parametrize("strain,angle", [(1e-5, 0.0), (2e-3, 4e-3), (1e-3, 0.3), (2e-2, 0.0)])
+@pytest.mark.parametrize("seed_scale", [1.0, 1e-60, 1e50])
+def test_reverse_step_against_oracle(n_shape, jitter, per_bond, strain, angle, seed_scale):
+    # one reverse step: dL/du0 = gu + dt/rho sum c K d with w = gv + dt gu, formed by the
+    # oracle literally in FP64.  |K d| <= 2 |d| / L and both sides round a dozen
+    # operations a bond and the sum: 200 2^-53 of the terms' sum bounds the difference.
+    # dL/dc = dt/rho s V_j (y/|y|).w: the oracle's s carries 8 2^-53, the kernel's 2^-44
+    # of itself, the other factors a few roundings.
+    w = _body(n_shape, jitter, 4, 0.0, 3.01)
+    rng = np.random.default_rng(9)
+    c, s = np.cos(angle), np.sin(angle)
+    A = np.array([[c, -s, 0], [s, c, 0], [0, 0, 1]]) @ (np.eye(3) * (1 + strain)) - np.eye(3)
+    u0 = (w.coords - w.coords.mean(0)) @ A.T + rng.uniform(-0.05, 0.05, (w.n, 3)) * strain * w.dx
+    v0 = np.zeros((w.n, 3))
+    off, idx = oracle.cut_family(w.coords, w.horizon, w.cuts_array())
+    c0 = oracle.micromodulus(w.bulk_modulus, w.horizon)
+    cb = np.full(len(idx), c0)
+    if per_bond:
+        cb = workloads.bond_stiffness_grf(w, off, idx, c0, 3)
+        rev = workloads.reverse_bond(w.n, off, idx)
+        cb = 0.5 * (cb + cb[rev])
+    gu = rng.normal(size=(w.n, 3)) * seed_scale
+    gv = rng.normal(size=(w.n, 3)) * 1e-7 * seed_scale
+    om = oracle.Model.from_workload(w, off, idx, c=c0, c_bond=cb)
+    gc_o, gl_o, gu_o, gv_o = oracle.adjoint(om, 0, 1, u0, v0, om.fresh_bonds(), gu, gv)
+    m = pdgb.Model.from_workload(w, precision=pdgb.PD_PREC_F64, c=c0)
+    if per_bond:
+        m.set_params(c0, w.sc, w.load, w.disp_rate, cb)
+    m.set_state(u0, v0, step=0)
+    pdgb.pd_adjoint_forward(m.h, 1)
+    gc, gl, gu0, gv0 = pdgb.pd_adjoint_backward(m.h, gu, gv)
+    m.close()
+    rows = np.repeat(np.arange(w.n), np.diff(off))
+    xi = w.coords[idx] - w.coords[rows]
+    L = np.linalg.norm(xi, axis=1)
+    s = np.abs(np.linalg.norm(xi + u0[idx] - u0[rows], axis=1) / L - 1.0)
+    ww = gv + w.dt * gu
+    wa = np.linalg.norm(ww, axis=1)
+    dr = w.dt / w.density
+    tol = np.zeros(w.n)
+    np.add.at(tol, rows, 2 * cb / L * (w.volumes[rows] * wa[idx] + w.volumes[idx] * wa[rows]))
+    tol = 200 * 2.0 ** -53 * (dr * tol + np.abs(gu).max(1))
+    assert (np.abs(gu0 - gu_o).max(1) <= tol).all()
+    assert np.abs(gv0 - gv_o).max() <= 8 * 2.0 ** -53 * np.abs(gv_o).max()
+    tolc = dr * w.volumes[idx] * wa[rows] * (8 * 2.0 ** -53 + (2.0 ** -44 + 16 * 2.0 ** -53) * s)
+    assert (np.abs(gc - gc_o) <= tolc).all()
