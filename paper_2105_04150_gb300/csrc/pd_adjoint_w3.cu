@@ -108,10 +108,10 @@ __global__ void k_adj_prep_w3(const AdjW3Args a, const double* __restrict__ ub,
         double2* wr = reinterpret_cast<double2*>(a.w64 + 4 * p);
         wr[0] = make_double2(w[0], w[1]);
         wr[1] = make_double2(w[2], 0.0);
-        a.rec[4 * p] = make_float4(a0.x, a0.y, a0.z, uh[0]);
-        a.rec[4 * p + 1] = make_float4(uh[1], uh[2], t[0], t[1]);
-        a.rec[4 * p + 2] = make_float4(b0.x, b0.y, b0.z, um[0]);
-        a.rec[4 * p + 3] = make_float4(um[1], um[2], t[2], 0.0f);
+        a.rec[4 * p] = make_float4(a0.x, a0.y, uh[0], uh[1]);
+        a.rec[4 * p + 1] = make_float4(a1.x, uh[2], t[0], t[1]);
+        a.rec[4 * p + 2] = make_float4(b0.x, b0.y, um[0], um[1]);
+        a.rec[4 * p + 3] = make_float4(b1.x, um[2], t[2], 0.0f);
         a.wdw[2 * p] = make_float4(wh[0], wh[1], wh[2], wl[0]);
         a.wdw[2 * p + 1] = make_float4(wl[1], wl[2], 0.0f, 0.0f);
     }
@@ -188,7 +188,8 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         const D4 wj = ld_d4(a.w64 + 4 * j);
         float4 v0, v1;
         dwa::ld_rec(a.wdw + 2 * j, v0, v1);
-        const float2 il = __ldg(a.il + slot);
+        const float4 il2 = __ldg(a.il + (slot - lane) / 64 * 32 + lane);
+        const float2 il = b & 1 ? make_float2(il2.y, il2.w) : make_float2(il2.x, il2.z);
         // e is kept by rows of 32 lanes: x, y, z of slot b of the slice
         const double* ep = a.e + 3 * (slot - lane) + lane;
         const double e0 = __ldg(ep), e1 = __ldg(ep + 32), e2 = __ldg(ep + 64);

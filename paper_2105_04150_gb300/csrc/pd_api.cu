@@ -136,8 +136,10 @@ struct pd_handle {
     // bond-based PD_PREC_F64: three-word records and bond lengths of the step (W3Args)
     bool w3 = false;
     float4* rec3[2] = {nullptr, nullptr};
-    float2 *il3 = nullptr, *cb3 = nullptr, *wrel3 = nullptr;
+    float4* il3 = nullptr;
+    float2 *cb3 = nullptr, *wrel3 = nullptr;
     double* phi0 = nullptr; // per node the damage of an intact family
+    int32_t* fam3 = nullptr;  // per node its bonds
     double w3_scale = 1.0;  // 1 / U, a power of two (batches: per instance in itab)
     int w3_x_grid = kW3UGrid;  // exponent of the positions' grid
     int team = 1;           // warps per slice
@@ -548,6 +550,7 @@ W3Args w3_args(pd_handle* h)
     d.cb = h->per_bond_c ? h->cb3 : nullptr;
     d.wrel = h->wrel3;
     d.phi0 = h->phi0;
+    d.fam = h->fam3;
     d.w_ref = (h->per_bond_c ? 1.0 : h->c) * h->vol0;
     d.scale = h->w3_scale;
     d.x_grid = h->w3_x_grid;
@@ -654,22 +657,24 @@ pd_status encode_lat_tma(pd_handle* h, int shape)
     return PD_OK;
 }
 
-// Warps per slice of the FP64 step.  One warp takes about 52 us for a family of 122
+// Warps per slice of the FP64 step.  One warp takes about 43 us for a family of 122
 // whatever the model's size, so a model with fewer slices than the chip holds warps
-// (16 per SM) shares each among 8, 4 or 2, as long as that fills the chip only once;
-// two warps still pay a little past that, where one would leave a short last wave.
-// us per step with 1 / 2 / 4 / 8 warps: 125 slices 54.7 / 34.6 / 23.6 / 18.0, 422
-// slices 55 / 34 / 37 / 38, 1000: 56 / 54 / 59 / 63, 2695: 157 / 137 / 142 / 165, 4160:
-// 187 / 190 / 201 / 248, 9000: 355 / 376 / 415 / 512 (the barrier and the shared sums).
+// (16 per SM) shares each among 8, 4 or 2 as long as that fills the chip only once.
+// Past that, two warps per slice where they leave a last wave that one would not fill.
+// us per step with 1 / 2 / 4 / 8 warps: 125 slices 45.6 / 29.3 / 18.0 / 12.5, 422
+// slices 45 / 29 / 26 / 30, 1000: 46 / 45 / 48 / 53, 2695: 120 / 110 / 126 / 130, 4160:
+// 159 / 181 / 175 / 200, 6075: 241 / 228 / 250 / 286, 9000: 320 / 329 / 371 / 421 (the
+// barrier and the shared sums).
 int w3_team(const pd_handle* h, int sms)
 {
     if (h->Q * (32 / kW3Seg) > kW3TeamSegs) return 1;
     const int wpb = h->block / 32;
-    const int64_t cap = (int64_t)sms * 16;
-    if (wpb % 8 == 0 && h->n_slices * 8 <= cap) return 8;
-    if (wpb % 4 == 0 && h->n_slices * 4 <= cap / 2) return 4;
-    if (wpb % 2 == 0 && h->n_slices * 2 <= 3 * cap) return 2;
-    return 1;
+    const int64_t cap = (int64_t)sms * 16, n = h->n_slices;
+    for (int t : {8, 4, 2})
+        if (wpb % t == 0 && n * t <= cap) return t;
+    // half waves of two warps per slice against two half waves of one
+    const int64_t w1 = 2 * ((n + cap - 1) / cap), w2 = (2 * n + cap - 1) / cap;
+    return wpb % 2 == 0 && 10 * w2 < 9 * w1 ? 2 : 1;
 }
 
 pd_status choose_grid(pd_handle* h, int blocks_per_sm)
@@ -1088,8 +1093,9 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
         if (h->w3) {
             ALLOC(h->rec3[0], float4, 4 * np);
             ALLOC(h->rec3[1], float4, 4 * np);
-            ALLOC(h->il3, float2, nbr.size());
+            ALLOC(h->il3, float4, nbr.size() / 2);
             ALLOC(h->phi0, double, np);
+            ALLOC(h->fam3, int32_t, np);
             if (!h->uniform_vol) ALLOC(h->wrel3, float2, np);
         }
         ALLOC(h->ilen, double, nbr.size());  // also the adjoint's
@@ -1242,6 +1248,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
         return st;
     std::vector<InstParams> itab = d.itab;
     std::vector<float2> wrel;
+    std::vector<int32_t> fam;
     if (h->w3) {
         // U: a power of two no smaller than the longest bond (of each instance), and the
         // FP32 grid of the largest coordinate in that unit
@@ -1288,6 +1295,10 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
                 itab[k].w3_x_hi = w3_x_hi(itab[k].sc_lo);
             }
         }
+        fam.assign(np, 0);
+        for (int64_t p = 0; p < n; ++p)
+            fam[p] = (int32_t)(h->off[h->perm[p] + 1] - h->off[h->perm[p]]);
+        if ((st = up(h->fam3, fam.data(), 4 * np, "upload family sizes"))) return st;
         if (!h->uniform_vol) {
             wrel.assign(np, make_float2(0.f, 0.f));
             for (int64_t p = 0; p < n; ++p) {

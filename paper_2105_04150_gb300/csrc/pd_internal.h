@@ -43,6 +43,34 @@
 
 namespace pd {
 
+// Programmatic dependent launch: a kernel launched with launch_pdl starts while its
+// predecessor in the stream runs (once all of that one's blocks have called
+// pdl_launch), and reads what the predecessor writes only after pdl_wait, which waits
+// for its completion.  It hides the launch latency and the kernel's first instruction,
+// constant and static-array misses.
+inline cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, void** args, size_t smem,
+                              cudaStream_t s)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 struct BcClass {
     uint32_t mask;     // bit a (0..2): component a displacement-controlled; bit 3: no-fail
     uint32_t pad;
@@ -303,7 +331,7 @@ struct StepArgsF64 {
 // Three-word records of the FP64 step (pd_step_f64.cu, pd_w3.h): positions and
 // displacements in units of U, a power of two no smaller than the longest bond
 constexpr int kW3Seg = 16;             // slots of a family whose forces are summed together
-constexpr int kW3TeamSegs = 16;        // largest family, in segments, that a team of warps takes
+constexpr int kW3TeamSegs = 256 / kW3Seg;  // largest family, in segments, that a team takes
 constexpr float kW3XMax = 0x1.0p-6f;   // largest |x|, x = |y|^2 / |xi|^2 - 1, of the double-word
                                        // bond arithmetic (see pd_w3.h)
 constexpr int kW3UGrid = -22;          // exponent of the displacements' grid below 4 U
@@ -316,10 +344,11 @@ inline float w3_x_hi(double s_lo)
 }
 struct W3Args {
     const float4* rec[2];      // 4 float4 per node, double buffered like the FP64 records
-    const float2* il;          // per slot U / |xi| as a double-word
+    const float4* il;          // per pair of slots U / |xi| as double-words {h, h', l, l'}
     const float2* cb;          // per slot stiffness c_ij as a double-word, or nullptr
     const float2* wrel;        // per node w / w_ref as a double-word (non-uniform weights)
     const double* phi0;        // per node the damage of an intact family (rounding only)
+    const int32_t* fam;        // per node the bonds of the intact family
     double w_ref;              // weight of the first node (batches: per instance)
     double scale;              // 1 / U (batches: per instance)
     double dt_rho;             // dt / rho
@@ -501,7 +530,7 @@ struct AdjW3Args {
     const float2* cb;          // the same as double-words
     const double* ilen;        // per slot 1 / |xi|
     const double* e;           // per slot xi / |xi|^(3/2), rows of 32 lanes per component
-    const float2* il;          // per slot U / |xi| as a double-word
+    const float4* il;          // W3Args::il
     float2* gc;                // per-slot dL/dc accumulator (merged to FP64 in place)
     double* gl;                // per-node accumulator of force . w
     const uint8_t* bcc;
@@ -597,7 +626,7 @@ cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, d
                               cudaStream_t s);
 cudaError_t launch_w3_ilen(const double* ilen, const int32_t* nbr, const int32_t* sw, int64_t n,
                            int Q, double scale, const int32_t* inst, const InstParams* itab,
-                           float2* il, cudaStream_t s);
+                           float4* il, cudaStream_t s);
 cudaError_t launch_step_dw(const StepArgsF64& a, const DwArgs& d, int sc_mode, int grid, int block,
                            cudaStream_t s);
 const void* step_dw_kernel(int sc_mode, bool uniform_w, bool soft, bool vv);
@@ -713,6 +742,10 @@ __device__ __forceinline__ double soft_mu_of(double s, double s0, double sc, dou
 // as FP64 rounds it, computed with the weights.  The flags may have been written by
 // other warps of the block, before its last barrier.
 #ifdef __CUDACC__
+__device__ __forceinline__ double damage_ratio(int was, int now)
+{
+    return (double)(was - now) / (double)was;
+}
 __device__ __forceinline__ double damage_lost(bool uniform_w, const double* __restrict__ rec,
                                               const int32_t* __restrict__ nbr,
                                               const uint32_t* bits,
@@ -731,8 +764,8 @@ __device__ __forceinline__ double damage_lost(bool uniform_w, const double* __re
                 lost += rec[8 * (int64_t)nbr[((g * Q + q) * 32 + __ffs(m) - 1) * 32 + lane] + 3];
     }
     if (was == now) return phi0;
-    if (now == 0) return 1.0;
-    return uniform_w ? (double)(was - now) / (double)was : fmin(1.0, lost * wi);
+    if (uniform_w) return damage_ratio(was, now);
+    return now == 0 ? 1.0 : fmin(1.0, lost * wi);
 }
 #endif
 

@@ -7,8 +7,9 @@
 // kernel that forms Eq. 4 literally in FP64 (about 41 FP64 operations a bond) is
 // bound by that pipe: 1.88 ms per step of a 180x35x35 notched beam, and 0.29 ms of a
 // 4000-node bar, whose 125 warps each walk a whole family alone.  With the arithmetic
-// and the split below they take 0.285 and 0.018 ms, 277 warp instructions a bond, bound
-// by their issue (66 % active; 16 warps per SM at 128 registers).
+// and the split below they take 0.25 and 0.0125 ms, 195 warp instructions a bond (277
+// without the paired instructions, 0.285 ms), 55 % of the issue slots with the FMA
+// pipe occupied twice by each pair and 16 warps per SM (128 registers).
 // Here the FP64 differences x_j - x_i and u_j - u_i come exactly from three-word
 // FP32 records, and the stretch without cancellation in double-word arithmetic
 // (pd_w3.h): no FP64 operation on the bonds of the bulk.  The literal form rounds
@@ -62,7 +63,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes)
 // One bond literally in FP64: s = |y| / |xi| - 1 (1/|xi| stored per slot, 1/|y| from
 // the Newton-refined reciprocal square root), the break test against the bond's s_c,
 // the no-fail rule, and the force, added to f.  True when it breaks.
-__device__ __noinline__ bool literal_bond(const StepArgsF64& a, int cur, int64_t i, int64_t j,
+__device__ __forceinline__ bool literal_bond(const StepArgsF64& a, int cur, int64_t i, int64_t j,
                                           int64_t slot, double* f)
 {
     const double2* __restrict__ rin = reinterpret_cast<const double2*>(a.rec[cur]);
@@ -95,18 +96,24 @@ __device__ __noinline__ bool literal_bond(const StepArgsF64& a, int cur, int64_t
     return false;
 }
 
-// F += coef y when `ok` (a select: whatever a masked slot computed, including
-// a non-finite value, is dropped)
-__device__ __forceinline__ void add_force(Dw (&F)[3], const Bond& b, bool ok)
+// The lane's force sum: (x, y) and z.
+struct Force {
+    Dw2 xy;
+    Dw z;
+};
+
+// F += c y when `ok` (a select: whatever a masked slot computed, including a
+// non-finite value, is dropped)
+__device__ __forceinline__ void add_force(Force& F, float ch, float cl, const Kin& b, bool ok)
 {
-    const Dw cf{ok ? b.coef.h : 0.0f, ok ? b.coef.l : 0.0f};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const Dw f = dw_mul(cf, b.y[k]);
-        const Dw t = two_sum(F[k].h, f.h);
-        F[k].h = t.h;
-        F[k].l += t.l + f.l;
-    }
+    ch = ok ? ch : 0.0f;
+    cl = ok ? cl : 0.0f;
+    const Dw2 f = dw_mul2(Dw2{both(ch), both(cl)}, b.y);
+    const Dw fz = dw_mul(Dw{ch, cl}, b.yz);
+    const Dw2 t = two_sum2(F.xy.h, f.h);
+    F.xy = Dw2{t.h, add2(F.xy.l, add2(t.l, f.l))};
+    const Dw tz = two_sum(F.z.h, fz.h);
+    F.z = Dw{tz.h, F.z.l + (tz.l + fz.l)};
 }
 
 // The sums of a segment, or of a whole family, of the 32 nodes of a slice, in shared
@@ -114,102 +121,185 @@ __device__ __forceinline__ void add_force(Dw (&F)[3], const Bond& b, bool ok)
 struct __align__(16) Sums {
     float F[6][32];   // sum of -s y / |y| (times w_j / w_ref and c_ij), leading and low words
     double lit[3][32];  // force density of the literally evaluated bonds
+    int info[32];       // intact bonds, + kLit if lit is not zero
 };
+constexpr int kLit = 1 << 16;
 
-// One segment of the family of the lane's node: into S, or added to it.
+// The segment's bonds `pend` literally: their breaks and their forces, in slot order.
+// Returns the broken ones.
+__device__ __noinline__ uint32_t literal_segment(const StepArgsF64& a, int cur, int64_t i, int64_t g,
+                                             int m_lo, uint32_t pend, uint32_t* bw, Sums& S)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t slot0 = (g * 32LL * a.Q + m_lo) * 32 + lane;
+    uint32_t gone = 0u;
+    double lit[3] = {0.0, 0.0, 0.0};
+    for (; pend; pend &= pend - 1u) {
+        const int b = __ffs(pend) - 1;
+        const int64_t slot = slot0 + (int64_t)b * 32;
+        if (literal_bond(a, cur, i, a.nbr[slot], slot, lit)) gone |= 1u << b;
+    }
+    // another warp of the team may own the other half of the flag word
+    if (gone) atomicAnd(bw + (m_lo >> 5) * 32, ~(gone << (m_lo & 31)));
+    for (int k = 0; k < 3; ++k) S.lit[k][lane] += lit[k];
+    return gone;
+}
+
+// The segments of a family that the warp takes, `rank`, rank + team, ...: into their
+// entries of S (TEAM), or added up in it.  The neighbours' records come from L2 as
+// often as from L1 and nothing else hides that latency (16 warps per SM, and a
+// prefetch to L1 has no effect), so the walk is software-pipelined across segments:
+// a record's registers are free after kin(), and the next chunk's loads go out
+// there, behind them the coefficients and forces of the current one.
 template <bool UW, bool TEAM>
-__device__ __forceinline__ void walk_segment(const StepArgsF64& a, const W3Args& d, int cur,
-                                             const Own& own, float x_hi, float ts, int64_t i,
-                                             int64_t g, int seg, int Wg, Sums& S)
+__device__ __forceinline__ void walk(const StepArgsF64& a, const W3Args& d, int cur,
+                                     const Own2& own, float x_hi, float ts, int64_t i, int64_t g,
+                                     int rank, int team, int Wg, Sums* S)
 {
     const int lane = threadIdx.x & 31;
     const int Q = a.Q;
     const float4* __restrict__ R = d.rec[cur];
-    const int m_lo = seg * kSeg;
-    const int nch = (min(kSeg, Wg - m_lo) + 1) >> 1;  // chunks of two slots (bonds A and B)
-    const int64_t slot0 = (g * 32LL * Q + m_lo) * 32 + lane;
-    const int32_t* __restrict__ col = a.nbr + slot0;
-    uint32_t* bw = a.bits + (g * Q + (m_lo >> 5)) * 32 + lane;
-    const int sh = m_lo & 31;
-    const uint32_t word = (*bw >> sh) & ((1u << kSeg) - 1u);
-    uint32_t pend = 0u;
-    Dw F[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-    int32_t jn0 = __ldg(col), jn1 = __ldg(col + 32);
-    for (int c = 0; c < nch; ++c) {
-        const int32_t j0 = jn0, j1 = jn1;
-        if (c + 1 < nch) {
-            jn0 = __ldg(col + (2 * c + 2) * 32);
-            jn1 = __ldg(col + (2 * c + 3) * 32);
+    const int32_t* __restrict__ col = a.nbr + g * 32LL * Q * 32 + lane;
+    const float4* __restrict__ ilp = d.il + g * 16LL * Q * 32 + lane;
+    uint32_t* const bw = a.bits + g * Q * 32 + lane;
+    // first slot of the chunk after the one at m: within a segment, then the team's next
+    auto after = [&](int m) { return ((m + 2) & (kSeg - 1)) ? m + 2 : m + 2 + (team - 1) * kSeg; };
+
+    int m = rank * kSeg;
+    if (m >= Wg) return;
+    int mn = after(m);
+    int32_t j0 = __ldg(col + m * 32), j1 = __ldg(col + m * 32 + 32);
+    int32_t n0 = 0, n1 = 0;  // the next chunk's neighbours
+    if (mn < Wg) {
+        n0 = __ldg(col + mn * 32);
+        n1 = __ldg(col + mn * 32 + 32);
+    }
+    Rec A, B;
+    dwa::ld_rec(R + 4 * (int64_t)j0, A.a0, A.a1);
+    dwa::ld_rec(R + 4 * (int64_t)j0 + 2, A.b0, A.b1);
+    dwa::ld_rec(R + 4 * (int64_t)j1, B.a0, B.a1);
+    dwa::ld_rec(R + 4 * (int64_t)j1 + 2, B.b0, B.b1);
+    float4 il = __ldg(ilp + m * 16);
+    uint32_t word = 0u, pend = 0u;
+    Force F{Dw2{both(0.0f), both(0.0f)}, Dw{0.0f, 0.0f}};
+    while (true) {
+        const bool more = mn < Wg;
+        const int b = m & (kSeg - 1);
+        if (b == 0) word = (bw[(m >> 5) * 32] >> (m & 31)) & ((1u << kSeg) - 1u);
+        const Kin bA = kin(own, A, both(ts), make_float2(ts, 1.0f));
+        if (more) {
+            dwa::ld_rec(R + 4 * (int64_t)n0, A.a0, A.a1);
+            dwa::ld_rec(R + 4 * (int64_t)n0 + 2, A.b0, A.b1);
         }
-        Rec A, B;
-        dwa::ld_rec(R + 4 * (int64_t)j0, A.a0, A.a1);
-        dwa::ld_rec(R + 4 * (int64_t)j0 + 2, A.b0, A.b1);
-        dwa::ld_rec(R + 4 * (int64_t)j1, B.a0, B.a1);
-        dwa::ld_rec(R + 4 * (int64_t)j1 + 2, B.b0, B.b1);
-        const int64_t sA = slot0 + 2 * c * 32, sB = sA + 32;
-        Bond bA = bond_w3(own, A, __ldg(d.il + sA), ts);
-        Bond bB = bond_w3(own, B, __ldg(d.il + sB), ts);
+        const Kin bB = kin(own, B, both(ts), make_float2(ts, 1.0f));
+        const float4 ilc = il;
+        const int32_t c0 = j0, c1 = j1;
+        const int mc = m;
+        if (more) {
+            dwa::ld_rec(R + 4 * (int64_t)n1, B.a0, B.a1);
+            dwa::ld_rec(R + 4 * (int64_t)n1 + 2, B.b0, B.b1);
+            il = __ldg(ilp + mn * 16);
+            m = mn;
+            mn = after(m);
+            if (!UW) {
+                j0 = n0;
+                j1 = n1;
+            }
+            if (mn < Wg) {
+                n0 = __ldg(col + mn * 32);
+                n1 = __ldg(col + mn * 32 + 32);
+            }
+        }
+        Coef2 cf = coef2(bA.num, bB.num, ilc);
         // literal evaluation: near or past s_c, past kW3XMax, or not a number
-        const bool litA = !(bA.x.h < x_hi) || !(bA.x.h > -kW3XMax);
-        const bool litB = !(bB.x.h < x_hi) || !(bB.x.h > -kW3XMax);
+        const bool litA = !(cf.x.x < x_hi) || !(cf.x.x > -kW3XMax);
+        const bool litB = !(cf.x.y < x_hi) || !(cf.x.y > -kW3XMax);
         if (d.cb != nullptr) {  // per-bond stiffness (a uniform branch)
-            const float2 cA = __ldg(d.cb + sA), cB = __ldg(d.cb + sB);
-            bA.coef = dw_mul(bA.coef, Dw{cA.x, cA.y});
-            bB.coef = dw_mul(bB.coef, Dw{cB.x, cB.y});
+            const float2* cb = d.cb + (g * 32LL * Q + mc) * 32 + lane;
+            const float2 cA = __ldg(cb), cB = __ldg(cb + 32);
+            cf.c = dw_mul2(cf.c, Dw2{make_float2(cA.x, cB.x), make_float2(cA.y, cB.y)});
         }
-        const uint32_t wb = word >> (2 * c);
-        pend |= (((litA ? 1u : 0u) | (litB ? 2u : 0u)) & wb) << (2 * c);
-        const bool okA = (wb & 1u) && !litA, okB = (wb & 2u) && !litB;
         if (!UW) {
-            const float2 wA = __ldg(d.wrel + j0), wB = __ldg(d.wrel + j1);
-            bA.coef = dw_mul(bA.coef, Dw{wA.x, wA.y});
-            bB.coef = dw_mul(bB.coef, Dw{wB.x, wB.y});
+            const float2 wA = __ldg(d.wrel + c0), wB = __ldg(d.wrel + c1);
+            cf.c = dw_mul2(cf.c, Dw2{make_float2(wA.x, wB.x), make_float2(wA.y, wB.y)});
         }
-        // the next chunk's records start toward L1 (their ids have arrived by now)
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(R + 4 * (int64_t)jn0));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(R + 4 * (int64_t)jn1));
-        add_force(F, bA, okA);
-        add_force(F, bB, okB);
-    }
-    const bool any = pend != 0u;
-    uint32_t gone = 0u;
-    double lit[3] = {0.0, 0.0, 0.0};
-    while (pend) {
-        const int b = __ffs(pend) - 1;
-        pend &= pend - 1u;
-        const int64_t j = col[(int64_t)b * 32];
-        if (literal_bond(a, cur, i, j, slot0 + (int64_t)b * 32, lit)) gone |= 1u << b;
-    }
-    // another warp of the team may own the other half of the flag word
-    if (gone) atomicAnd(bw, ~(gone << sh));
+        const uint32_t wb = word >> b;
+        pend |= (((litA ? 1u : 0u) | (litB ? 2u : 0u)) & wb) << b;
+        add_force(F, cf.c.h.x, cf.c.l.x, bA, (wb & 1u) && !litA);
+        add_force(F, cf.c.h.y, cf.c.l.y, bB, (wb & 2u) && !litB);
+
+        if (b == kSeg - 2 || !more) {  // the segment's end
+            const int m_lo = mc & ~(kSeg - 1);
+            Sums& T = S[TEAM ? m_lo / kSeg : 0];
+            const Dw Fk[3] = {{F.xy.h.x, F.xy.l.x}, {F.xy.h.y, F.xy.l.y}, F.z};
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const Dw t = TEAM ? F[k] : dw_add(Dw{S.F[2 * k][lane], S.F[2 * k + 1][lane]}, F[k]);
-        S.F[2 * k][lane] = t.h;
-        S.F[2 * k + 1][lane] = t.l;
-        if (TEAM) S.lit[k][lane] = lit[k];
-        else if (any) S.lit[k][lane] += lit[k];
+            for (int k = 0; k < 3; ++k) {
+                const Dw t = TEAM ? Fk[k] : dw_add(Dw{T.F[2 * k][lane], T.F[2 * k + 1][lane]}, Fk[k]);
+                T.F[2 * k][lane] = t.h;
+                T.F[2 * k + 1][lane] = t.l;
+            }
+            F = Force{Dw2{both(0.0f), both(0.0f)}, Dw{0.0f, 0.0f}};
+            int info = TEAM ? 0 : T.info[lane];
+            if (pend) {
+                if (TEAM)
+                    for (int k = 0; k < 3; ++k) T.lit[k][lane] = 0.0;
+                word &= ~literal_segment(a, cur, i, g, m_lo, pend, bw, T);
+                info |= kLit;
+                pend = 0u;
+            }
+            T.info[lane] = info + __popc(word);
+        }
+        if (!more) break;
     }
+}
+
+// What the end of a node's step reads, loaded before the team's barrier.
+struct Node {
+    double2 u01, u2_;
+    double v[3];
+    double phi0;
+    uint32_t cls;
+    int fam;  // bonds of the intact family
+};
+__device__ __forceinline__ Node load_node(const StepArgsF64& a, const W3Args& d, int cur, int64_t i)
+{
+    const double2* __restrict__ rin = reinterpret_cast<const double2*>(a.rec[cur]);
+    Node n;
+    n.u01 = __ldg(rin + 4 * i + 2);
+    n.u2_ = __ldg(rin + 4 * i + 3);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) n.v[c] = a.v[3 * i + c];
+    n.phi0 = __ldg(d.phi0 + i);
+    n.cls = a.bcc[i];
+    n.fam = __ldg(d.fam + i);
+    return n;
+}
+
+// Displacement and velocity of a controlled component.  A call, because inlined its
+// FP64 operations (about 150 with the smooth start and the divisions) are moved in front
+// of the node loop, where every warp of a team executes them: 10 of the 16 us of a step of
+// the 4000-node bar.
+__device__ __noinline__ double2 controlled(const StepArgsF64& a, double g, int64_t step)
+{
+    const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
+    const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
+    return make_double2(g * s_next, g * (s_next - s_now) / a.dt);
 }
 
 // Integration of the lane's node (damped Euler-Cromer, Eq. 11, or damped
 // velocity-Verlet), BCs, damage, and the records its neighbours read next.
 __device__ __forceinline__ void finish_node(const StepArgsF64& a, const W3Args& d, int cur,
-                                            int64_t step, bool first, const Rec& me, double scale,
-                                            int64_t i, const double (&T)[3])
+                                            int64_t step, const Rec& me, const Node& nd,
+                                            double scale, int64_t i, const double (&T)[3], int alive)
 {
-    const double2* __restrict__ rin = reinterpret_cast<const double2*>(a.rec[cur]);
     double2* __restrict__ rout = reinterpret_cast<double2*>(const_cast<double*>(a.rec[cur ^ 1]));
     float4* __restrict__ Rout = const_cast<float4*>(d.rec[cur ^ 1]);
-    const uint32_t cls = a.bcc[i];
+    const bool first = a.vv && step == a.step_ctr[1];  // velocity-Verlet: a^n formed afresh
     uint32_t mask = 0u;
     double gdisp[3] = {0.0, 0.0, 0.0};
-    double F[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-        F[c] = T[c];
-    if (cls != 0u) {
-        const BcClass& bc = a.bct[cls];
+    double F[3] = {T[0], T[1], T[2]};
+    if (nd.cls != 0u) {
+        const BcClass& bc = a.bct[nd.cls];
         mask = bc.mask;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -217,8 +307,7 @@ __device__ __forceinline__ void finish_node(const StepArgsF64& a, const W3Args& 
             F[c] += a.load * bc.force[c];
         }
     }
-    const double2 u01 = __ldg(rin + 4 * i + 2), u2_ = __ldg(rin + 4 * i + 3);
-    const double uo[3] = {u01.x, u01.y, u2_.x};
+    const double uo[3] = {nd.u01.x, nd.u01.y, nd.u2_.x};
     double un[3];
     float uh[3], um[3], tw[3];
     const float tin[3] = {me.a1.z, me.a1.w, me.b1.z};
@@ -227,7 +316,7 @@ __device__ __forceinline__ void finish_node(const StepArgsF64& a, const W3Args& 
     for (int c = 0; c < 3; ++c) {
         // stored velocity: v^n (Euler-Cromer) or, for velocity-Verlet, the
         // half-step velocity v^{n-1} + dt/2 a^{n-1} (v^n right after a set state)
-        const double vi = a.v[3 * i + c];
+        const double vi = nd.v[c];
         const double adt = (F[c] - a.eta * vi) * d.dt_rho;  // dt a
         double vn, vfull;
         if (a.vv) {
@@ -239,10 +328,9 @@ __device__ __forceinline__ void finish_node(const StepArgsF64& a, const W3Args& 
         }
         double u = fma(a.dt, vn, uo[c]);
         if (mask & (1u << c)) {
-            const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
-            const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
-            u = gdisp[c] * s_next;
-            vn = gdisp[c] * (s_next - s_now) / a.dt;
+            const double2 uv = controlled(a, gdisp[c], step);
+            u = uv.x;
+            vn = uv.y;
             vfull = vi;
         }
         finite = finite && isfinite(u);
@@ -258,12 +346,17 @@ __device__ __forceinline__ void finish_node(const StepArgsF64& a, const W3Args& 
     if (a.peek) return;
     rout[4 * i + 2] = make_double2(un[0], un[1]);  // (positions and weights: in both buffers)
     rout[4 * i + 3] = make_double2(un[2], 0.0);
-    dwa::st_rec(Rout + 4 * i, make_float4(me.a0.x, me.a0.y, me.a0.z, uh[0]),
-                make_float4(uh[1], uh[2], tw[0], tw[1]));
-    dwa::st_rec(Rout + 4 * i + 2, make_float4(me.b0.x, me.b0.y, me.b0.z, um[0]),
-                make_float4(um[1], um[2], tw[2], 0.0f));
-    a.damage[i] = damage_lost(d.uniform_w != 0, a.rec[cur], a.nbr, a.bits, a.bits0, a.wsum_inv[i],
-                              d.phi0[i], i >> 5, (int)(i & 31), a.Q);
+    dwa::st_rec(Rout + 4 * i, make_float4(me.a0.x, me.a0.y, uh[0], uh[1]),
+                make_float4(me.a1.x, uh[2], tw[0], tw[1]));
+    dwa::st_rec(Rout + 4 * i + 2, make_float4(me.b0.x, me.b0.y, um[0], um[1]),
+                make_float4(me.b1.x, um[2], tw[2], 0.0f));
+    double phi = nd.phi0;
+    if (alive != nd.fam)
+        phi = d.uniform_w != 0
+                  ? damage_ratio(nd.fam, alive)
+                  : damage_lost(false, a.rec[cur], a.nbr, a.bits, a.bits0, a.wsum_inv[i], nd.phi0,
+                                i >> 5, (int)(i & 31), a.Q);
+    a.damage[i] = phi;
     if (!finite) atomicOr(a.err, PD_DEVERR_NONFINITE);
 }
 
@@ -274,16 +367,26 @@ __global__ void __launch_bounds__(256, 2)
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
-    const int team = TEAM ? d.team : 1;       // warps per slice
-    const int tpb = wpb / team;               // slices per block at a time
-    const int tm = (int)(threadIdx.x >> 5) / team;
-    const int rank = (int)(threadIdx.x >> 5) % team;
+    const int team = TEAM ? d.team : 1;       // warps per slice (a power of two)
+    const int sh = TEAM ? __ffs(team) - 1 : 0;
+    const int tpb = wpb >> sh;                // slices per block at a time
+    const int tm = (int)(threadIdx.x >> 5) >> sh;
+    const int rank = (int)(threadIdx.x >> 5) & (team - 1);
     // the slice's sums: one entry, or one per segment for a team
     Sums* const S = reinterpret_cast<Sums*>(smem) + (TEAM ? tm * d.max_seg : tm);
-    const int64_t step = a.step_ctr[0] + a.k;
-    const bool first = a.vv && step == a.step_ctr[1];  // velocity-Verlet: a^n formed afresh
-    const int cur = (int)(step & 1);
     const int64_t nslices = (a.n + 31) >> 5;
+
+    // before the previous kernel is done (programmatic launch): nothing it writes is read
+    if (lane == 0 && rank == 0 && (int64_t)blockIdx.x * tpb + tm < nslices) {
+        const int64_t g = (int64_t)blockIdx.x * tpb + tm;
+        const int Wg = a.sw[g];
+        prefetch_l2(a.nbr + g * 32LL * a.Q * 32, (uint32_t)(((Wg + 3) & ~3) * 128));
+        if (TEAM) prefetch_l2(d.il + g * 16LL * a.Q * 32, (uint32_t)(((Wg + 3) & ~3) * 256));
+    }
+    pdl_wait();
+    pdl_launch();
+    const int64_t step = a.step_ctr[0] + a.k;
+    const int cur = (int)(step & 1);
     const float4* __restrict__ R = d.rec[cur];
 
     // (every warp of a block makes the same number of rounds: teams synchronise)
@@ -293,16 +396,17 @@ __global__ void __launch_bounds__(256, 2)
         if (!TEAM && !have) continue;
         const int64_t i = (g << 5) + lane;
         Rec me{};
+        Node nd{};
         int nseg = 0;
         double w_ref = d.w_ref, scale = d.scale;
         if (have) {
             const int Wg = a.sw[g];
             nseg = (Wg + kSeg - 1) / kSeg;
-            if (lane == 0 && rank == 0)
+            if (lane == 0 && rank == 0 && g0 != (int64_t)blockIdx.x * tpb)
                 prefetch_l2(a.nbr + g * 32LL * a.Q * 32, (uint32_t)(((Wg + 3) & ~3) * 128));
             dwa::ld_rec(R + 4 * i, me.a0, me.a1);
             dwa::ld_rec(R + 4 * i + 2, me.b0, me.b1);
-            const Own own = own_words(me);
+            const Own2 own = own_pairs(me);
             float x_hi = d.x_hi;
             int grid = d.x_grid;
             if (a.inst != nullptr) {  // batch: the instance's own band, weight and unit
@@ -318,25 +422,31 @@ __global__ void __launch_bounds__(256, 2)
                 for (int k = 0; k < 6; ++k) S->F[k][lane] = 0.0f;
 #pragma unroll
                 for (int k = 0; k < 3; ++k) S->lit[k][lane] = 0.0;
+                S->info[lane] = 0;
             }
-            for (int seg = rank; seg < nseg; seg += team)
-                walk_segment<UW, TEAM>(a, d, cur, own, x_hi, ts, i, g, seg, Wg, S[TEAM ? seg : 0]);
+            walk<UW, TEAM>(a, d, cur, own, x_hi, ts, i, g, rank, team, Wg, S);
+            if (rank == 0) nd = load_node(a, d, cur, i);  // (node arrays are padded)
         }
         if (TEAM) __syncthreads();
         if (have && rank == 0 && i < a.n) {
             // the segments' sums in their order, whichever warps formed them
             Dw F[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
             double T[3] = {0.0, 0.0, 0.0};
+            int alive = 0;
             for (int e = 0; e < (TEAM ? nseg : 1); ++e) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
+                for (int k = 0; k < 3; ++k)
                     F[k] = dw_add(F[k], Dw{S[e].F[2 * k][lane], S[e].F[2 * k + 1][lane]});
-                    T[k] += S[e].lit[k][lane];
+                const int info = S[e].info[lane];
+                alive += info & (kLit - 1);
+                if (info >= kLit) {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) T[k] += S[e].lit[k][lane];
                 }
             }
 #pragma unroll
             for (int k = 0; k < 3; ++k) T[k] = fma(-((double)F[k].h + (double)F[k].l), w_ref, T[k]);
-            finish_node(a, d, cur, step, first, me, scale, i, T);
+            finish_node(a, d, cur, step, me, nd, scale, i, T, alive);
         }
         if (TEAM) __syncthreads();  // the sums' memory is free again
     }
@@ -359,18 +469,19 @@ __global__ void k_w3_publish(const double* __restrict__ rec64, float4* __restric
             split3(r[4 + k] * sc, kW3UGrid, uh[k], um[k], ut);
             t[k] = pack_t(t_int(xt, g), ut);
         }
-        rec[4 * p] = make_float4(xh[0], xh[1], xh[2], uh[0]);
-        rec[4 * p + 1] = make_float4(uh[1], uh[2], t[0], t[1]);
-        rec[4 * p + 2] = make_float4(xm[0], xm[1], xm[2], um[0]);
-        rec[4 * p + 3] = make_float4(um[1], um[2], t[2], 0.0f);
+        rec[4 * p] = make_float4(xh[0], xh[1], uh[0], uh[1]);
+        rec[4 * p + 1] = make_float4(xh[2], uh[2], t[0], t[1]);
+        rec[4 * p + 2] = make_float4(xm[0], xm[1], um[0], um[1]);
+        rec[4 * p + 3] = make_float4(xm[2], um[2], t[2], 0.0f);
     }
 }
 
-// U / |xi| of every slot as a double-word (1 where there is no bond)
+// U / |xi| of every slot as a double-word (1 where there is no bond), by pairs of slots:
+// {h, h', l, l'} of slots m and m + 1
 __global__ void k_w3_ilen(const double* __restrict__ ilen, const int32_t* __restrict__ nbr,
                           const int32_t* __restrict__ sw, int64_t n, int Q, double scale,
                           const int32_t* __restrict__ inst, const InstParams* __restrict__ itab,
-                          float2* __restrict__ il)
+                          float4* __restrict__ il)
 {
     const int64_t W = 32LL * Q;
     const int64_t total = ((n + 31) >> 5) << 5;
@@ -378,11 +489,15 @@ __global__ void k_w3_ilen(const double* __restrict__ ilen, const int32_t* __rest
          p += (int64_t)gridDim.x * blockDim.x) {
         const int64_t g = p >> 5;
         const double U = 1.0 / (inst != nullptr ? itab[inst[p]].w3_scale : scale);  // a power of two
-        for (int m = 0; m < W; ++m) {
-            const int64_t slot = (g * W + m) * 32 + (p & 31);
-            const double v = m < sw[g] && nbr[slot] != p ? ilen[slot] * U : 1.0;
-            const float h = (float)v;
-            il[slot] = make_float2(h, (float)(v - (double)h));
+        for (int m = 0; m < W; m += 2) {
+            float h[2], l[2];
+            for (int k = 0; k < 2; ++k) {
+                const int64_t slot = (g * W + m + k) * 32 + (p & 31);
+                const double v = m + k < sw[g] && nbr[slot] != p ? ilen[slot] * U : 1.0;
+                h[k] = (float)v;
+                l[k] = (float)(v - (double)h[k]);
+            }
+            il[(g * W / 2 + m / 2) * 32 + (p & 31)] = make_float4(h[0], h[1], l[0], l[1]);
         }
     }
 }
@@ -413,8 +528,7 @@ cudaError_t launch_step_f64(const StepArgsF64& a, const W3Args& d, int grid, int
 {
     const void* fn = step_f64_kernel(d.uniform_w != 0, d.team > 1);
     void* args[] = {const_cast<StepArgsF64*>(&a), const_cast<W3Args*>(&d)};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(block), args,
-                            step_f64_smem(d.team, d.max_seg, block), s);
+    return launch_pdl(fn, dim3(grid), dim3(block), args, step_f64_smem(d.team, d.max_seg, block), s);
 }
 
 cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, double scale,
@@ -427,7 +541,7 @@ cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, d
 
 cudaError_t launch_w3_ilen(const double* ilen, const int32_t* nbr, const int32_t* sw, int64_t n,
                            int Q, double scale, const int32_t* inst, const InstParams* itab,
-                           float2* il, cudaStream_t s)
+                           float4* il, cudaStream_t s)
 {
     k_w3_ilen<<<grid_of(((n + 31) >> 5) << 5), 256, 0, s>>>(ilen, nbr, sw, n, Q, scale, inst, itab,
                                                             il);

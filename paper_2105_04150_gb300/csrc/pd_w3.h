@@ -20,10 +20,15 @@
 // words, whose grids differ) and keeps only 2^-48 of |v|.
 //
 // Record: two 32-byte sectors, each one 256-bit load
-//   {xh.x, xh.y, xh.z, uh.x | uh.y, uh.z, t.x, t.y}
-//   {xm.x, xm.y, xm.z, um.x | um.y, um.z, t.z, 0}
+//   {xh.x, xh.y, uh.x, uh.y | xh.z, uh.z, t.x, t.y}
+//   {xm.x, xm.y, um.x, um.y | xm.z, um.z, t.z, 0}
 // word t.c holds the integer t of x_c, biased, in its low 11 bits and above them
 // the leading 21 bits of the t of u_c, an FP32 number.
+//
+// Paired arithmetic: sm_103a's paired FP32 instructions do two operations in one
+// issue slot.  A bond's (x, y) components, and z of xi and of eta, are adjacent in the
+// record for that; from num on the two bonds of a chunk are a pair (the slots'
+// U / |xi| are stored by pairs of slots).  Each half is rounded as the scalar operation.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -64,10 +69,10 @@ __device__ __forceinline__ float ut_of(float w)
 __device__ __forceinline__ Own own_words(const Rec& r)
 {
     Own o;
-    o.xh[0] = r.a0.x; o.xh[1] = r.a0.y; o.xh[2] = r.a0.z;
-    o.uh[0] = r.a0.w; o.uh[1] = r.a1.x; o.uh[2] = r.a1.y;
-    o.xm[0] = r.b0.x; o.xm[1] = r.b0.y; o.xm[2] = r.b0.z;
-    o.um[0] = r.b0.w; o.um[1] = r.b1.x; o.um[2] = r.b1.y;
+    o.xh[0] = r.a0.x; o.xh[1] = r.a0.y; o.xh[2] = r.a1.x;
+    o.uh[0] = r.a0.z; o.uh[1] = r.a0.w; o.uh[2] = r.a1.y;
+    o.xm[0] = r.b0.x; o.xm[1] = r.b0.y; o.xm[2] = r.b1.x;
+    o.um[0] = r.b0.z; o.um[1] = r.b0.w; o.um[2] = r.b1.y;
     const float t[3] = {r.a1.z, r.a1.w, r.b1.z};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -129,8 +134,8 @@ struct Geo {
 // root, reciprocal and quotient of the direct form; relative error < 2^-44.
 __device__ __forceinline__ Geo bond_geo(const Own& o, const Rec& j, const float2 il, float ts)
 {
-    const float jxh[3] = {j.a0.x, j.a0.y, j.a0.z}, juh[3] = {j.a0.w, j.a1.x, j.a1.y};
-    const float jxm[3] = {j.b0.x, j.b0.y, j.b0.z}, jum[3] = {j.b0.w, j.b1.x, j.b1.y};
+    const float jxh[3] = {j.a0.x, j.a0.y, j.a1.x}, juh[3] = {j.a0.z, j.a0.w, j.a1.y};
+    const float jxm[3] = {j.b0.x, j.b0.y, j.b1.x}, jum[3] = {j.b0.z, j.b0.w, j.b1.y};
     const float jt[3] = {j.a1.z, j.a1.w, j.b1.z};
     Geo out;
     Dw nm[3];
@@ -159,16 +164,120 @@ __device__ __forceinline__ Geo bond_geo(const Own& o, const Rec& j, const float2
     return out;
 }
 
-struct Bond {
-    Dw x;     // |y|^2 / |xi|^2 - 1
-    Dw coef;  // -s / |y| (in 1 / U)
-    Dw y[3];  // deformed bond vector (in U)
-};
+// ---- two bonds at a time ----------------------------------------------------
 
-__device__ __forceinline__ Bond bond_w3(const Own& o, const Rec& j, const float2 il, float ts)
+// two double-words, one per half
+struct Dw2 {
+    float2 h, l;
+};
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+// a - b (a product by -1 is exact, so this is one rounding)
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, both(-1.0f), a); }
+
+__device__ __forceinline__ Dw2 two_sum2(float2 a, float2 b)
 {
-    const Geo g = bond_geo(o, j, il, ts);
-    return {g.x, dw_mul(g.z, Dw{il.x, il.y}), {g.y[0], g.y[1], g.y[2]}};
+    const float2 s = add2(a, b);
+    const float2 bb = sub2(s, a);
+    return {s, add2(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+__device__ __forceinline__ Dw2 dw_add2(Dw2 a, Dw2 b)
+{
+    Dw2 t = two_sum2(a.h, b.h);
+    t.l = add2(t.l, add2(a.l, b.l));
+    return t;
+}
+__device__ __forceinline__ Dw2 dw_mul2(Dw2 a, Dw2 b)
+{
+    const float2 p = mul2(a.h, b.h);
+    const float2 e = make_float2(fmaf(a.h.x, b.h.x, -p.x), fmaf(a.h.y, b.h.y, -p.y));
+    return {p, fma2(a.h, b.l, fma2(a.l, b.h, e))};
+}
+// the difference of two records' pairs, as diff3
+__device__ __forceinline__ Dw2 diff3_2(float2 jh, float2 jm, float2 nh, float2 nm, float2 dt,
+                                       float2 ts)
+{
+    const float2 dh = add2(jh, nh), dm = add2(jm, nm);
+    const float2 s = add2(dh, dm);
+    return {s, fma2(dt, ts, sub2(dm, sub2(s, dh)))};
+}
+
+// The lane's own words, negated, in the pairs of the record.
+struct Own2 {
+    float2 xh, uh, zh, xm, um, zm;  // (x, y) of x and u; (x_z, u_z)
+    float2 xk, ut, zt;              // the third words likewise
+};
+__device__ __forceinline__ Own2 own_pairs(const Rec& r)
+{
+    Own2 o;
+    o.xh = make_float2(-r.a0.x, -r.a0.y);
+    o.uh = make_float2(-r.a0.z, -r.a0.w);
+    o.zh = make_float2(-r.a1.x, -r.a1.y);
+    o.xm = make_float2(-r.b0.x, -r.b0.y);
+    o.um = make_float2(-r.b0.z, -r.b0.w);
+    o.zm = make_float2(-r.b1.x, -r.b1.y);
+    o.xk = make_float2(-k_of(r.a1.z), -k_of(r.a1.w));
+    o.ut = make_float2(-ut_of(r.a1.z), -ut_of(r.a1.w));
+    o.zt = make_float2(-k_of(r.b1.z), -ut_of(r.b1.z));
+    return o;
+}
+
+// y = xi + eta and num = eta . (2 xi + eta) of one bond
+struct Kin {
+    Dw2 y;   // x, y components
+    Dw yz;
+    Dw num;
+};
+__device__ __forceinline__ Kin kin(const Own2& o, const Rec& j, float2 ts2, float2 tsz)
+{
+    const Dw2 xi = diff3_2(make_float2(j.a0.x, j.a0.y), make_float2(j.b0.x, j.b0.y), o.xh, o.xm,
+                           add2(make_float2(k_of(j.a1.z), k_of(j.a1.w)), o.xk), ts2);
+    const float2 dt = add2(make_float2(ut_of(j.a1.z), ut_of(j.a1.w)), o.ut);
+    Dw2 et;
+    {
+        const float2 dh = add2(make_float2(j.a0.z, j.a0.w), o.uh);
+        const float2 dm = add2(make_float2(j.b0.z, j.b0.w), o.um);
+        const float2 s = add2(dh, dm);
+        et = Dw2{s, add2(dt, sub2(dm, sub2(s, dh)))};
+    }
+    const Dw2 zz = diff3_2(make_float2(j.a1.x, j.a1.y), make_float2(j.b1.x, j.b1.y), o.zh, o.zm,
+                           add2(make_float2(k_of(j.b1.z), ut_of(j.b1.z)), o.zt), tsz);
+    const Dw xz{zz.h.x, zz.l.x}, ez{zz.h.y, zz.l.y};
+    Kin k;
+    k.y = dw_add2(xi, et);
+    k.yz = dw_add(xz, ez);
+    const Dw2 n2 = dw_mul2(et, dw_add2(xi, k.y));
+    const Dw nz = dw_mul(ez, dw_add(xz, k.yz));
+    Dw num = two_sum(n2.h.x, n2.h.y);
+    num.l += n2.l.x + n2.l.y;
+    k.num = dw_add(num, nz);
+    return k;
+}
+
+// x = |y|^2 / |xi|^2 - 1 of two bonds and (1 / |xi|) z = -s / |y| (see bond_geo)
+struct Coef2 {
+    float2 x;  // leading words
+    Dw2 c;
+};
+__device__ __forceinline__ Coef2 coef2(Dw a, Dw b, const float4 il)
+{
+    const Dw2 num{make_float2(a.h, b.h), make_float2(a.l, b.l)};
+    const Dw2 iL{make_float2(il.x, il.y), make_float2(il.z, il.w)};
+    const Dw2 x = dw_mul2(dw_mul2(num, iL), iL);
+    const float2 x1 = add2(both(1.0f), x.h);
+    const float2 r = mul2(x1, make_float2(dwa::rsqrt_seed(x1.x), dwa::rsqrt_seed(x1.y)));
+    const float2 den = fma2(r, r, r);
+    const float2 nx = mul2(x.h, both(-1.0f));
+    const float2 z0 = mul2(nx, make_float2(dwa::rcp_seed(den.x), dwa::rcp_seed(den.y)));
+    const float2 zz = mul2(z0, z0), ph = fma2(both(2.0f), z0, zz);
+    const float2 e = make_float2(fmaf(z0.x, z0.x, -zz.x), fmaf(z0.y, z0.y, -zz.y));
+    const Dw2 p{ph, add2(sub2(zz, fma2(both(-2.0f), z0, ph)), e)};
+    const Dw2 xp = dw_mul2(x, p);
+    const float2 R = add2(add2(add2(ph, x.h), xp.h), add2(add2(p.l, x.l), xp.l));
+    const Dw2 z{z0, mul2(R, fma2(z0, both(-0.5f), both(-0.5f)))};
+    return {x.h, dw_mul2(z, iL)};
 }
 
 }  // namespace w3
