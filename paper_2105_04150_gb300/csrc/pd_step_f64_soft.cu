@@ -45,12 +45,42 @@ __device__ __noinline__ bool pair_no_fail(const uint8_t* __restrict__ bcc,
     return ((bct[bcc[i]].mask | bct[bcc[j]].mask) & 8u) != 0u;
 }
 
+// Displacement and velocity of a controlled component (a call, so that its FP64
+// operations are not moved before the node loop)
+__device__ __noinline__ double2 controlled(const StepArgsF64& a, double g, int64_t step)
+{
+    const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
+    const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
+    return make_double2(g * s_next, g * (s_next - s_now) / a.dt);
+}
+
+// rsqrt_nr with the halvings and the seed's conversion to FP64 as integer operations on
+// the exponent field (the same bits; they keep three operations a bond off the FP64 pipe)
+__device__ __forceinline__ double half_of(double y)
+{
+    return __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y));
+}
+__device__ __forceinline__ double rsqrt_nr_int(double x)
+{
+    const float xf = (float)x;
+    if (!(xf > 0x1.0p-100f) || xf > 0x1.0p100f) return rsqrt_nr(x);
+    const uint32_t b = __float_as_uint(rsqrtf(xf));  // in [2^-50, 2^50]
+    double y = __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
+    double t = x * y;
+    y = fma(half_of(y), fma(-t, y, 1.0), y);
+    t = x * y;
+    y = fma(half_of(y), fma(-t, y, 1.0), y);
+    return y;
+}
+
 template <int SCM>
 __global__ void __launch_bounds__(256) k_step_f64_soft(const StepArgsF64 a)
 {
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_wait();
+    pdl_launch();
     const int64_t step = a.step_ctr[0] + a.k;
     const bool first = a.vv && step == a.step_ctr[1];  // velocity-Verlet: a^n formed afresh
     const int cur = (int)(step & 1);
@@ -69,6 +99,9 @@ __global__ void __launch_bounds__(256) k_step_f64_soft(const StepArgsF64 a)
         const int32_t* __restrict__ col = a.nbr + g * W * 32 + lane;
         uint32_t* bw = a.bits + g * Q * 32 + lane;
         double fx = 0.0, fy = 0.0, fz = 0.0, ws = 0.0;
+        // high word of the smallest s_0 the node's bonds can have, less a band for rounding
+        const double s_lo = a.inst != nullptr ? a.itab[a.inst[i]].sc_lo : SCM == 0 ? a.sc : a.sc_lo;
+        const int s0_hi = __double2hiint((1.0 - 0x1.0p-20) * s_lo / a.kr);
 
         for (int q = 0; q * 32 < Wg; ++q) {
             const uint32_t word = bw[q * 32];
@@ -99,49 +132,53 @@ __global__ void __launch_bounds__(256) k_step_f64_soft(const StepArgsF64 a)
                     const double yz = ez + (ra[u][3].x - u23.x);
                     const int64_t slot = (g * W + q * 32 + b0 + u) * 32 + lane;
                     const double y2 = yx * yx + yy * yy + yz * yz;
-                    const double ir = rsqrt_nr(y2);
+                    const double ir = rsqrt_nr_int(y2);
                     const double r = y2 * ir;
                     const double s = fma(r, __ldg(a.ilen + slot), -1.0);
-                    double sc;
-                    if (a.inst != nullptr) {  // batch: instance parameters, local ids as keys
-                        const InstParams& ip = a.itab[a.inst[i]];
-                        sc = ip.sc_mode == 1 ? sc_draw(ip.sc_seed, ip.sc_lo, ip.sc_hi, a.hid[i],
-                                                       a.hid[jj[u]])
-                                             : ip.sc;
-                    } else {
-                        sc = (SCM == 0) ? a.sc
-                                        : sc_draw(a.sc_seed, a.sc_lo, a.sc_hi, a.gid[i],
-                                                  a.gid[jj[u]]);
-                    }
-                    bool brk = !a.frozen && s >= sc;
-                    if (brk && a.has_nofail) brk = !pair_no_fail(a.bcc, a.bct, i, jj[u]);
-                    if (brk) {
-                        nword &= ~(1u << (b0 + u));
-                        if (a.integ != nullptr) a.integ[slot] = 0.0;
-                    } else {
-                        // bilinear softening: the integrity only decreases, as the
-                        // stretch passes s_0 = s_c / kr (a no-fail bond past s_c keeps 0)
-                        double mu = 1.0;
-                        if (a.integ != nullptr) {
-                            mu = a.integ[slot];
-                            const double s0 = sc / a.kr;
-                            if (s > s0) {
-                                const double ms =
-                                    s >= sc ? 0.0 : soft_mu_of(s, s0, sc, a.k1, a.beta);
-                                if (ms < mu) {
-                                    mu = ms;
-                                    a.integ[slot] = ms;
-                                }
+                    // s_0 of the bond, the smallest the slice's bonds can have when
+                    // s_c is drawn per bond: below it, by the high words (an integer
+                    // comparison; not-a-numbers and ties go on), nothing changes
+                    double mu = __ldg(a.integ + slot);
+                    if (__double2hiint(s) >= s0_hi) {
+                        double sc = a.sc;
+                        if (a.inst != nullptr) {  // batch: instance parameters, local ids
+                            const InstParams& ip = a.itab[a.inst[i]];
+                            sc = ip.sc_mode == 1 ? sc_draw(ip.sc_seed, ip.sc_lo, ip.sc_hi,
+                                                           a.hid[i], a.hid[jj[u]])
+                                                 : ip.sc;
+                        } else if (SCM != 0) {
+                            sc = sc_draw(a.sc_seed, a.sc_lo, a.sc_hi, a.gid[i], a.gid[jj[u]]);
+                        }
+                        bool brk = !a.frozen && s >= sc;
+                        if (brk && a.has_nofail) brk = !pair_no_fail(a.bcc, a.bct, i, jj[u]);
+                        if (brk) {
+                            nword &= ~(1u << (b0 + u));
+                            a.integ[slot] = 0.0;
+                            continue;
+                        }
+                        // the integrity only decreases, as the stretch passes
+                        // s_0 = s_c / kr (a no-fail bond past s_c keeps 0)
+                        const double s0 = sc / a.kr;
+                        if (s > s0) {
+                            const double ms = s >= sc ? 0.0 : soft_mu_of(s, s0, sc, a.k1, a.beta);
+                            if (ms < mu) {
+                                mu = ms;
+                                a.integ[slot] = ms;
                             }
                         }
-                        double wj = ra[u][1].y * mu;
-                        if (cb != nullptr) wj *= __ldg(cb + slot);
-                        const double f = wj * s * ir;
-                        fx += f * yx;
-                        fy += f * yy;
-                        fz += f * yz;
-                        ws += ra[u][1].y * mu;
                     }
+                    double wj = ra[u][1].y;
+                    if (mu != 1.0) {
+                        wj *= mu;
+                        ws = fma(ra[u][1].y, mu, ws);
+                    } else {
+                        ws += wj;
+                    }
+                    if (cb != nullptr) wj *= __ldg(cb + slot);
+                    const double f = wj * s * ir;
+                    fx += f * yx;
+                    fy += f * yy;
+                    fz += f * yz;
                 }
             }
             if (nword != word) bw[q * 32] = nword;
@@ -161,8 +198,6 @@ __global__ void __launch_bounds__(256) k_step_f64_soft(const StepArgsF64 a)
                     F[c] += a.load * bc.force[c];
                 }
             }
-            const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
-            const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
             const double uo[3] = {u01.x, u01.y, u23.x};
             double un[3];
             bool finite = true;
@@ -182,8 +217,9 @@ __global__ void __launch_bounds__(256) k_step_f64_soft(const StepArgsF64 a)
                 }
                 double u = uo[c] + a.dt * vn;
                 if (mask & (1u << c)) {
-                    u = gdisp[c] * s_next;
-                    vn = gdisp[c] * (s_next - s_now) / a.dt;
+                    const double2 uv = controlled(a, gdisp[c], step);
+                    u = uv.x;
+                    vn = uv.y;
                     vfull = vi;
                 }
                 finite = finite && isfinite(u);
@@ -210,11 +246,8 @@ __global__ void __launch_bounds__(256) k_step_f64_soft(const StepArgsF64 a)
 
 cudaError_t launch_step_f64_soft(const StepArgsF64& a, int grid, int block, cudaStream_t s)
 {
-    if (a.sc_mode == 0)
-        k_step_f64_soft<0><<<grid, block, 0, s>>>(a);
-    else
-        k_step_f64_soft<1><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+    void* args[] = {const_cast<StepArgsF64*>(&a)};
+    return launch_pdl(step_f64_soft_kernel(a.sc_mode), dim3(grid), dim3(block), args, 0, s);
 }
 
 const void* step_f64_soft_kernel(int sc_mode)
