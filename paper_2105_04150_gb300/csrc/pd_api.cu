@@ -1008,6 +1008,11 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
     if (!msg.empty()) return fail(PD_ERR_ARG, "%s", msg.c_str());
     h->w3 = cfg->precision == PD_PREC_F64 && h->model == 0 &&
             (h->kr < 1.0 || (h->kr == 1.0 && !h->has_nofail));
+    // The literal FP64 step is bound by each SM's FP64 pipe, so its slices have to be
+    // spread evenly: one warp per block (a 962-slice model fills 121 SMs with 8 slices
+    // each in blocks of 256, 152 with 6 or 7 so).
+    if (cfg->precision == PD_PREC_F64 && h->model == 0 && !h->w3 && !cfg->block_threads)
+        h->block = 32;
 
     // FP32 Euler-Cromer PMB models on a regular lattice (the stencil kernel's
     // case): lattice node order and the stencil-ordered layout
