@@ -434,6 +434,14 @@ cudaError_t launch_f64(pd_handle* h, const StepArgsF64& a)
                                : launch_step_f64(a, w3_args(h), h->grid, h->block, h->stream);
 }
 
+// The lattice step's form with four warps per slice, a block (and 62 KB of terms) each: as
+// long as all blocks are resident at once, three per SM.  us per step, one warp / four:
+// 16 slices 8.7 / 5.8, 125: 9.7 / 7.1, 422: 10.2 / 7.9, 1000: 10.1 / 16.7.
+bool lat_team(const pd_handle* h)
+{
+    return h->lattice && !h->batch && h->model == 0 && h->lat_var == 0 && h->n_slices <= 3 * 152;
+}
+
 // the FP32 step kernel build for this handle (bilinear softening or not)
 cudaError_t launch_f32(pd_handle* h, const StepArgsF32& a)
 {
@@ -446,6 +454,7 @@ cudaError_t launch_f32(pd_handle* h, const StepArgsF32& a)
         return h->lat_var == 1
                    ? launch_step_f32_lat_batch_r80(a, h->sc_mode, h->grid, h->block, h->stream)
                    : launch_step_f32_lat_batch(a, h->sc_mode, h->grid, h->block, h->stream);
+    if (h->lattice && lat_team(h)) return launch_step_f32_lat_team(a, h->sc_mode, h->stream);
     if (h->lattice)
         return h->lat_var == 1
                    ? launch_step_f32_lat_r80(a, h->sc_mode, h->grid, h->block, h->stream)
@@ -463,6 +472,7 @@ const void* f32_kernel(pd_handle* h)
     if (h->lattice && h->batch)
         return h->lat_var == 1 ? step_f32_kernel_lat_batch_r80(h->sc_mode, h->per_bond_c)
                                : step_f32_kernel_lat_batch(h->sc_mode, h->per_bond_c);
+    if (h->lattice && lat_team(h)) return step_f32_kernel_lat_team(h->sc_mode, h->per_bond_c);
     if (h->lattice)
         return h->lat_var == 1 ? step_f32_kernel_lat_r80(h->sc_mode, h->per_bond_c)
                                : step_f32_kernel_lat(h->sc_mode, h->per_bond_c);
@@ -701,6 +711,17 @@ pd_status choose_grid(pd_handle* h, int blocks_per_sm)
     int sms = 0;
     PD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device), "sm count");
     if (h->w3) h->team = w3_team(h, sms);
+    if (lat_team(h)) {  // a block of four warps per slice
+        const void* fn = step_kernel_fn(h);
+        PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)step_f32_lat_team_smem()),
+                "shared memory size");
+        PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     (int)cudaSharedmemCarveoutMaxShared),
+                "carveout");
+        h->grid = h->grid_dil = h->grid_osbf = (int)h->n_slices;
+        return PD_OK;
+    }
     const void* fn = step_kernel_fn(h);
     const size_t smem = h->w3 ? step_f64_smem(h->team, h->Q * (32 / kW3Seg), h->block) : 0;
     // no shared memory, or that of two resident blocks: the rest of the unified

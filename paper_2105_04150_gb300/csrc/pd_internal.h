@@ -44,9 +44,8 @@
 namespace pd {
 
 // Programmatic dependent launch: a kernel launched with launch_pdl starts while its
-// predecessor in the stream runs (once all of that one's blocks have called
-// pdl_launch), and reads what the predecessor writes only after pdl_wait, which waits
-// for its completion.  It hides the launch latency and the kernel's first instruction,
+// predecessor in the stream runs (once all of that one's blocks have let it), and reads what the predecessor writes only after pdl_begin, which
+// waits for its completion.  It hides the launch latency and the kernel's first instruction,
 // constant and static-array misses.
 inline cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, void** args, size_t smem,
                               cudaStream_t s)
@@ -65,9 +64,14 @@ inline cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, void** args
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch()
+// The successor is let go as the blocks exit, or (`early`, grids of at most a block per SM)
+// at once: blocks that start early behind a larger grid take the slots of the less loaded
+// SMs and leave the successor unevenly spread (a state-based step of a 4160-slice model
+// 48.5 instead of 37.5 us).
+__device__ __forceinline__ void pdl_begin(bool early = false)
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait();
+    if (early && gridDim.x <= 152u) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 #endif
 
@@ -598,6 +602,10 @@ const void* step_f32_kernel_ext(int sc_mode, bool uniform_w, bool per_bond_c);
 cudaError_t launch_step_f32_lat(const StepArgsF32& a, int sc_mode, int grid, int block,
                                 cudaStream_t s);
 const void* step_f32_kernel_lat(int sc_mode, bool per_bond_c);
+// the same for models with few slices: a block of four warps per slice
+cudaError_t launch_step_f32_lat_team(const StepArgsF32& a, int sc_mode, cudaStream_t s);
+const void* step_f32_kernel_lat_team(int sc_mode, bool per_bond_c);
+size_t step_f32_lat_team_smem();
 // the same for a batch of lattice models (pd_step_f32_lat_batch.cu)
 cudaError_t launch_step_f32_lat_batch(const StepArgsF32& a, int sc_mode, int grid, int block,
                                       cudaStream_t s);
@@ -717,6 +725,25 @@ __device__ __forceinline__ double bc_scale(double rate, int64_t T, int64_t k)
     if (k >= T) return rate * ((double)k - 0.6 * (double)T);
     const double t = (double)k / (double)T;
     return rate * (double)T * (t * t * t * t - 0.6 * t * t * t * t * t);
+}
+
+// Displacement and velocity of a controlled component with prescribed value g per unit
+// scale; the second for the linear ramp.  Calls: inlined, their FP64 operations (about
+// 150 with the smooth start and the divisions, each 16 cycles of the SM's FP64 pipe) are
+// moved before the node loop, where every warp executes them.
+static __device__ __noinline__ double2 bc_controlled(double rate, int64_t T, double dt, double g,
+                                                     int64_t step)
+{
+    const double s_now = bc_scale(rate, T, step);
+    const double s_next = bc_scale(rate, T, step + 1);
+    return make_double2(g * s_next, g * (s_next - s_now) / dt);
+}
+static __device__ __noinline__ double2 bc_controlled_linear(double rate, double dt, double g,
+                                                            int64_t step)
+{
+    const double s_now = rate * (double)step;
+    const double s_next = rate * (double)(step + 1);
+    return make_double2(g * s_next, g * (s_next - s_now) / dt);
 }
 #endif
 

@@ -215,6 +215,7 @@ __global__ void __launch_bounds__(256, PD_DW_MIN_BLOCKS)
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     const int64_t step = a.step_ctr[0] + a.k;
     const int cur = (int)(step & 1);
     const int Q = a.Q;
@@ -353,8 +354,6 @@ __global__ void __launch_bounds__(256, PD_DW_MIN_BLOCKS)
                     Fn[k] += a.load * bc.force[k];
                 }
             }
-            const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
-            const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
             const double2 u01 = rin[4 * i + 2], u23 = rin[4 * i + 3];
             const double uo[3] = {u01.x, u01.y, u23.x};
             // velocity-Verlet: a^n is formed afresh at the step the state was set
@@ -378,8 +377,10 @@ __global__ void __launch_bounds__(256, PD_DW_MIN_BLOCKS)
                 }
                 double u = uo[k] + a.dt * vn;
                 if (mask & (1u << k)) {
-                    u = gdisp[k] * s_next;
-                    vn = gdisp[k] * (s_next - s_now) / a.dt;
+                    const double2 uv =
+                        bc_controlled(a.disp_rate, a.ramp_steps, a.dt, gdisp[k], step);
+                    u = uv.x;
+                    vn = uv.y;
                     vfull = vi;
                 }
                 finite = finite && isfinite(u);
@@ -511,7 +512,7 @@ cudaError_t launch_step_dw(const StepArgsF64& a, const DwArgs& d, int sc_mode, i
     const void* fn = step_dw_kernel(sc_mode, d.uniform_w != 0, a.integ != nullptr,
                                     a.vv != 0 || a.peek != 0);
     void* args[] = {const_cast<StepArgsF64*>(&a), const_cast<DwArgs*>(&d)};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, 0, s);
+    return launch_pdl(fn, dim3(grid), dim3(block), args, 0, s);
 }
 
 cudaError_t launch_dw_publish(const double* rec64, float4* rec, int64_t n_pad, const double* origin,

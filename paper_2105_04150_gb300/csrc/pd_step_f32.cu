@@ -365,6 +365,7 @@ __global__ void __launch_bounds__(256, PD_F32_MIN_BLOCKS)
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     const int64_t step = a.step_ctr[0] + a.k;
     const int cur = (int)(step & 1);
     const int Q = a.Q;
@@ -502,10 +503,10 @@ __global__ void __launch_bounds__(256, PD_F32_MIN_BLOCKS)
                     float vn = vi + dtf * (F[c] - etaf * vi) / rhof;
                     ff_add(H[c], L[c], vn * dtd);
                     if (mask & (1u << c)) {
-                        const double s_now = a.disp_rate * (double)step;
-                        const double s_next = a.disp_rate * (double)(step + 1);
-                        ff_set(bc->disp[c] * s_next * a.inv_delta, H[c], L[c]);
-                        vn = (float)(bc->disp[c] * (s_next - s_now) / a.dt);
+                        const double2 uv =
+                            bc_controlled_linear(a.disp_rate, a.dt, bc->disp[c], step);
+                        ff_set(uv.x * a.inv_delta, H[c], L[c]);
+                        vn = (float)uv.y;
                     }
                     finite = finite && isfinite(H[c]);
                     a.v[3 * i + c] = vn;
@@ -521,10 +522,10 @@ __global__ void __launch_bounds__(256, PD_F32_MIN_BLOCKS)
                     }
                     ff_add(H[c], L[c], vn * dtd);
                     if (mask & (1u << c)) {
-                        const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
-                        const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
-                        ff_set(bc->disp[c] * s_next * a.inv_delta, H[c], L[c]);
-                        vn = (float)(bc->disp[c] * (s_next - s_now) / a.dt);
+                        const double2 uv = bc_controlled(a.disp_rate, a.ramp_steps, a.dt,
+                                                         bc->disp[c], step);
+                        ff_set(uv.x * a.inv_delta, H[c], L[c]);
+                        vn = (float)uv.y;
                         vfull = vi;
                     }
                     finite = finite && isfinite(H[c]);
@@ -549,8 +550,8 @@ __global__ void __launch_bounds__(256, PD_F32_MIN_BLOCKS)
 template <int SCM, bool UW>
 cudaError_t launch_v(const StepArgsF32& a, int grid, int block, cudaStream_t s)
 {
-    k_step_f32<SCM, UW><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+    void* args[] = {const_cast<StepArgsF32*>(&a)};
+    return launch_pdl((const void*)k_step_f32<SCM, UW>, dim3(grid), dim3(block), args, 0, s);
 }
 
 }  // namespace

@@ -249,6 +249,7 @@ struct LatNode {
     int64_t slot0;      // index of slot 0 of this node in per-slot arrays
     float2 fx, fy, fz;  // force sums over the first and the second bonds of the pairs
     uint32_t word[4];   // bond flags (stencil slot order)
+    float2* term;       // team: where the next pair's terms go (shared memory)
     uint32_t pend;      // near-s_c candidates of the current flag word
     int alive;          // intact bonds after this step's decisions
 };
@@ -305,7 +306,8 @@ struct SrcTile {
 // Every quantity of the two bonds sits in one register pair and goes through
 // paired FP32 instructions, each half rounded as the scalar operation, so each
 // bond's terms are those of the one-bond formulas (lat_resolve re-forms them).
-template <class Src, int QXY, int K0, int K1, int ZX, int ZY, bool PBC>
+// TERM: the pair's coefficient and y are stored instead of added to the sums.
+template <class Src, int QXY, int K0, int K1, int ZX, int ZY, bool PBC, bool TERM>
 __device__ __forceinline__ void lat_pair_bond(const StepArgsF32& a, const float2 xix,
                                               const float2 xiy, const float2 xi2x,
                                               const float2 xi2y, const float4* P0,
@@ -353,13 +355,21 @@ __device__ __forceinline__ void lat_pair_bond(const StepArgsF32& a, const float2
         rp0 |= fabsf(d.x) >= a.lat_ch[Q] ? (1u << K0) : 0u;
         rp1 |= fabsf(d.y) >= a.lat_ch[Q] ? (1u << K1) : 0u;
     }
-    s.fx = __ffma2_rn(coef, yx, s.fx);
-    s.fy = __ffma2_rn(coef, yy, s.fy);
-    s.fz = __ffma2_rn(coef, yz, s.fz);
+    if constexpr (TERM) {
+        s.term[0] = coef;
+        s.term[32] = yx;
+        s.term[64] = yy;
+        s.term[96] = yz;
+        s.term += 4 * 32;
+    } else {
+        s.fx = __ffma2_rn(coef, yx, s.fx);
+        s.fy = __ffma2_rn(coef, yy, s.fy);
+        s.fz = __ffma2_rn(coef, yz, s.fz);
+    }
 }
 
 // Rows R and R + 1 (compile-time) of segment SG, unrolled, their offsets fixed
-template <class Src, bool PBC, int SG, int R, int... K>
+template <class Src, bool PBC, int SG, bool TERM, int R, int... K>
 __device__ __forceinline__ void lat_rowpair_fixed(const StepArgsF32& a, const float4* Pi,
                                                   LatNode& s, std::integer_sequence<int, K...>)
 {
@@ -378,24 +388,24 @@ __device__ __forceinline__ void lat_rowpair_fixed(const StepArgsF32& a, const fl
     const float2 xiy = make_float2(a.lat_xi[o0.y + 3], a.lat_xi[o1.y + 3]);
     const float2 xi2x = make_float2(a.lat_xi2[o0.x + 3], a.lat_xi2[o1.x + 3]);
     const float2 xi2y = make_float2(a.lat_xi2[o0.y + 3], a.lat_xi2[o1.y + 3]);
-    (lat_pair_bond<Src, sg.qxy, K, K, o0.x == 0 && o1.x == 0, o0.y == 0 && o1.y == 0, PBC>(
+    (lat_pair_bond<Src, sg.qxy, K, K, o0.x == 0 && o1.x == 0, o0.y == 0 && o1.y == 0, PBC, TERM>(
          a, xix, xiy, xi2x, xi2y, P0, P1, cb0, cb1, rb0, rb1, rp0, rp1, s),
      ...);
     s.pend |= (rp0 | (rp1 << len)) << b0;
 }
 
-template <class Src, bool PBC, int SG, int... R>
+template <class Src, bool PBC, int SG, bool TERM, int... R>
 __device__ __forceinline__ void lat_rows_fixed(const StepArgsF32& a, const float4* Pi, LatNode& s,
                                                std::integer_sequence<int, R...>)
 {
-    (lat_rowpair_fixed<Src, PBC, SG, 2 * R>(
+    (lat_rowpair_fixed<Src, PBC, SG, TERM, 2 * R>(
          a, Pi, s, std::make_integer_sequence<int, stencil_row_len(stencil_seg(SG).qxy)>{}),
      ...);
 }
 
 // The o_x = o_y = 0 row (a segment of one row, o_z = -3..-1, 1..3): its
 // positions K and len - 1 - K (o_z and -o_z) as pairs
-template <class Src, bool PBC, int SG, int... K>
+template <class Src, bool PBC, int SG, bool TERM, int... K>
 __device__ __forceinline__ void lat_row_mirror(const StepArgsF32& a, const float4* Pi, LatNode& s,
                                                std::integer_sequence<int, K...>)
 {
@@ -406,7 +416,7 @@ __device__ __forceinline__ void lat_row_mirror(const StepArgsF32& a, const float
     const float* cb = PBC ? a.cbond + s.slot0 + 32 * (32 * sg.word + sg.bit0) : nullptr;
     uint32_t rp = 0u;
     const float2 z = make_float2(0.f, 0.f);
-    (lat_pair_bond<Src, sg.qxy, K, len - 1 - K, 1, 1, PBC>(a, z, z, z, z, Pi, Pi, cb, cb, rb, rb,
+    (lat_pair_bond<Src, sg.qxy, K, len - 1 - K, 1, 1, PBC, TERM>(a, z, z, z, z, Pi, Pi, cb, cb, rb, rb,
                                                           rp, rp, s),
      ...);
     s.pend |= rp << sg.bit0;
@@ -414,7 +424,7 @@ __device__ __forceinline__ void lat_row_mirror(const StepArgsF32& a, const float
 
 // Segment SG as a loop over its rows, two rows per iteration (offsets of a row
 // unrolled)
-template <class Src, bool PBC, int SG, int... K>
+template <class Src, bool PBC, int SG, bool TERM, int... K>
 __device__ __forceinline__ void lat_rows_loop(const StepArgsF32& a, const float4* Pi, LatNode& s,
                                               std::integer_sequence<int, K...>)
 {
@@ -432,7 +442,7 @@ __device__ __forceinline__ void lat_rows_loop(const StepArgsF32& a, const float4
         const float* cb0 = PBC ? a.cbond + s.slot0 + 32 * (32 * sg.word + b0) : nullptr;
         const float* cb1 = PBC ? cb0 + 32 * len : nullptr;
         uint32_t rp0 = 0u, rp1 = 0u;
-        (lat_pair_bond<Src, sg.qxy, K, K, sg.zx, sg.zy, PBC>(
+        (lat_pair_bond<Src, sg.qxy, K, K, sg.zx, sg.zy, PBC, TERM>(
              a, make_float2(xa.x, xa.y), make_float2(xa.z, xa.w), make_float2(xb.x, xb.y),
              make_float2(xb.z, xb.w), P0, P1, cb0, cb1, rb0, rb1, rp0, rp1, s),
          ...);
@@ -440,17 +450,17 @@ __device__ __forceinline__ void lat_rows_loop(const StepArgsF32& a, const float4
     }
 }
 
-template <class Src, bool PBC, int SG>
+template <class Src, bool PBC, int SG, bool TERM = false>
 __device__ __forceinline__ void lat_seg(const StepArgsF32& a, const float4* Pi, LatNode& s)
 {
     constexpr StencilSeg sg = stencil_seg(SG);
     constexpr int len = stencil_row_len(sg.qxy);
     if constexpr (!sg.unroll)
-        lat_rows_loop<Src, PBC, SG>(a, Pi, s, std::make_integer_sequence<int, len>{});
+        lat_rows_loop<Src, PBC, SG, TERM>(a, Pi, s, std::make_integer_sequence<int, len>{});
     else if constexpr (sg.nrows == 1)
-        lat_row_mirror<Src, PBC, SG>(a, Pi, s, std::make_integer_sequence<int, len / 2>{});
+        lat_row_mirror<Src, PBC, SG, TERM>(a, Pi, s, std::make_integer_sequence<int, len / 2>{});
     else
-        lat_rows_fixed<Src, PBC, SG>(a, Pi, s, std::make_integer_sequence<int, sg.nrows / 2>{});
+        lat_rows_fixed<Src, PBC, SG, TERM>(a, Pi, s, std::make_integer_sequence<int, sg.nrows / 2>{});
 }
 
 // After the last segment of flag word W: decide the word's near-s_c candidates.
@@ -479,28 +489,39 @@ __device__ __forceinline__ void lat_word_end(const StepArgsF32& a, int cur, LatN
 
 // the walk over the stencil: the segments of each flag word, then the word's
 // near-s_c candidates (the segment and word layout of stencil_seg)
+template <class Src, int SCM, bool PBC, int W>
+__device__ __forceinline__ void lat_walk_word(const StepArgsF32& a, int cur, const float4* Pi,
+                                              LatNode& s)
+{
+    if constexpr (W == 0) {
+        lat_seg<Src, PBC, 0>(a, Pi, s);
+        lat_seg<Src, PBC, 1>(a, Pi, s);
+        lat_seg<Src, PBC, 2>(a, Pi, s);
+    } else if constexpr (W == 1) {
+        lat_seg<Src, PBC, 3>(a, Pi, s);
+        lat_seg<Src, PBC, 4>(a, Pi, s);
+        lat_seg<Src, PBC, 5>(a, Pi, s);
+    } else if constexpr (W == 2) {
+        lat_seg<Src, PBC, 6>(a, Pi, s);
+        lat_seg<Src, PBC, 7>(a, Pi, s);
+        lat_seg<Src, PBC, 8>(a, Pi, s);
+    } else {
+        lat_seg<Src, PBC, 9>(a, Pi, s);
+    }
+    lat_word_end<SCM, PBC, W>(a, cur, s);
+}
 template <class Src, int SCM, bool PBC>
 __device__ __forceinline__ void lat_walk(const StepArgsF32& a, int cur, const float4* Pi,
                                          LatNode& s)
 {
-    lat_seg<Src, PBC, 0>(a, Pi, s);
-    lat_seg<Src, PBC, 1>(a, Pi, s);
-    lat_seg<Src, PBC, 2>(a, Pi, s);
-    lat_word_end<SCM, PBC, 0>(a, cur, s);
-    lat_seg<Src, PBC, 3>(a, Pi, s);
-    lat_seg<Src, PBC, 4>(a, Pi, s);
-    lat_seg<Src, PBC, 5>(a, Pi, s);
-    lat_word_end<SCM, PBC, 1>(a, cur, s);
-    lat_seg<Src, PBC, 6>(a, Pi, s);
-    lat_seg<Src, PBC, 7>(a, Pi, s);
-    lat_seg<Src, PBC, 8>(a, Pi, s);
-    lat_word_end<SCM, PBC, 2>(a, cur, s);
-    lat_seg<Src, PBC, 9>(a, Pi, s);
-    lat_word_end<SCM, PBC, 3>(a, cur, s);
+    lat_walk_word<Src, SCM, PBC, 0>(a, cur, Pi, s);
+    lat_walk_word<Src, SCM, PBC, 1>(a, cur, Pi, s);
+    lat_walk_word<Src, SCM, PBC, 2>(a, cur, Pi, s);
+    lat_walk_word<Src, SCM, PBC, 3>(a, cur, Pi, s);
 }
 static_assert(stencil_seg(2).word == 0 && stencil_seg(3).word == 1 && stencil_seg(5).word == 1 &&
                   stencil_seg(6).word == 2 && stencil_seg(8).word == 2 && stencil_seg(9).word == 3,
-              "lat_walk follows the segment layout");
+              "lat_walk_word follows the segment layout");
 
 // The node's update: damped Euler-Cromer (Eq. 11) with the force in FP32 and
 // u accumulated in FP64, the linear displacement ramp, damage (Eq. 8) from the
@@ -536,10 +557,9 @@ __device__ __forceinline__ void lat_update(const StepArgsF32& a, const LatNode& 
         float vn = vi + a.dt_f * (F[c] - a.eta_f * vi) / a.rho_f;
         un[c] = fma((double)vn, (double)dtd, U[3 * i + c]);
         if (mask & (1u << c)) {
-            const double s_now = a.disp_rate * (double)step;
-            const double s_next = a.disp_rate * (double)(step + 1);
-            un[c] = bc->disp[c] * s_next * inv_unit;
-            vn = (float)(bc->disp[c] * (s_next - s_now) / a.dt);
+            const double2 uv = bc_controlled_linear(a.disp_rate, a.dt, bc->disp[c], step);
+            un[c] = uv.x * inv_unit;
+            vn = (float)uv.y;
         }
         finite = finite && isfinite(un[c]);
         a.v[3 * i + c] = vn;
@@ -559,6 +579,7 @@ __global__ void __launch_bounds__(PD_LAT_THREADS, PD_LAT_MIN_BLOCKS)
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     const int64_t step = lat_step_of(a);
     lat_advance_counter(a);
     const int cur = (int)(step & 1);
@@ -594,7 +615,110 @@ __global__ void __launch_bounds__(PD_LAT_THREADS, PD_LAT_MIN_BLOCKS)
     }
 }
 
+#if !PD_LAT_HELPERS && !PD_LAT_BATCH && PD_LAT_MIN_BLOCKS == 4
+// A model with few slices: a block per slice, each of its four warps forming the terms
+// (coefficient and y) of one flag word's pairs of bonds (16, 15, 15, 15) in shared
+// memory; the first warp then adds them in k_step_f32_lat's order and decides the
+// candidates after each word, so the bits are that kernel's.  The sum is a chain of 61
+// paired multiply-adds per component; the rest of the walk, which takes one warp about
+// 8 us whatever the model's size, is shared.  4000-node bar (125 slices): 9.7 -> 7.1 us a
+// step, of which the chain takes about 2.
+constexpr int kTeamPairs = 61;
+template <int SCM, bool PBC>
+__global__ void __launch_bounds__(128)
+    k_step_f32_lat_team(const __grid_constant__ StepArgsF32 a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    float2* const terms = reinterpret_cast<float2*>(smem);  // [pair][c, x, y, z][lane]
+    __shared__ uint32_t spend[4][32];
+    const int lane = threadIdx.x & 31, rank = threadIdx.x >> 5;
+    const int64_t g = blockIdx.x;
+    pdl_begin(true);
+    const int64_t step = lat_step_of(a);
+    lat_advance_counter(a);
+    const int cur = (int)(step & 1);
+    const float4* __restrict__ P = a.lat_pub[cur];
+    LatNode s;
+    s.i = (g << 5) + lane;
+    s.slot0 = g * 128 * 32 + lane;
+    lat_node_begin(s, ld_pub(P + s.i));
+    uint32_t* bw = a.bits + g * 4 * 32 + lane;
+    uint32_t w0[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w0[q] = s.word[q] = bw[q * 32];
+    const float4* Pi = P + s.i;
+    float2* out = terms + (rank == 0 ? 0 : 16 + 15 * (rank - 1)) * 4 * 32 + lane;
+    s.term = out;
+    if (rank == 0) {
+        lat_seg<SrcGlobal, PBC, 0, true>(a, Pi, s);
+        lat_seg<SrcGlobal, PBC, 1, true>(a, Pi, s);
+        lat_seg<SrcGlobal, PBC, 2, true>(a, Pi, s);
+    } else if (rank == 1) {
+        lat_seg<SrcGlobal, PBC, 3, true>(a, Pi, s);
+        lat_seg<SrcGlobal, PBC, 4, true>(a, Pi, s);
+        lat_seg<SrcGlobal, PBC, 5, true>(a, Pi, s);
+    } else if (rank == 2) {
+        lat_seg<SrcGlobal, PBC, 6, true>(a, Pi, s);
+        lat_seg<SrcGlobal, PBC, 7, true>(a, Pi, s);
+        lat_seg<SrcGlobal, PBC, 8, true>(a, Pi, s);
+    } else {
+        lat_seg<SrcGlobal, PBC, 9, true>(a, Pi, s);
+    }
+    spend[rank][lane] = s.pend;
+    __syncthreads();
+    if (rank != 0) return;
+    const float2* in = terms + lane;
+    auto sum = [&](int pairs) {
+#pragma unroll
+        for (int p = 0; p < pairs; ++p, in += 4 * 32) {
+            const float2 c = in[0];
+            s.fx = __ffma2_rn(c, in[32], s.fx);
+            s.fy = __ffma2_rn(c, in[64], s.fy);
+            s.fz = __ffma2_rn(c, in[96], s.fz);
+        }
+    };
+    sum(16);
+    s.pend = spend[0][lane];
+    lat_word_end<SCM, PBC, 0>(a, cur, s);
+    sum(15);
+    s.pend = spend[1][lane];
+    lat_word_end<SCM, PBC, 1>(a, cur, s);
+    sum(15);
+    s.pend = spend[2][lane];
+    lat_word_end<SCM, PBC, 2>(a, cur, s);
+    sum(15);
+    s.pend = spend[3][lane];
+    lat_word_end<SCM, PBC, 3>(a, cur, s);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (s.word[q] != w0[q]) bw[q * 32] = s.word[q];
+    if (s.i >= a.n) return;
+    lat_update(a, s, step, a.lat_u[cur], a.lat_u[cur ^ 1], const_cast<float4*>(a.lat_pub[cur ^ 1]));
+}
+#endif
+
 }  // namespace
+
+#if !PD_LAT_HELPERS && !PD_LAT_BATCH && PD_LAT_MIN_BLOCKS == 4
+size_t step_f32_lat_team_smem() { return (size_t)kTeamPairs * 4 * 32 * sizeof(float2); }
+
+const void* step_f32_kernel_lat_team(int sc_mode, bool per_bond_c)
+{
+    if (per_bond_c)
+        return sc_mode == 0 ? (const void*)k_step_f32_lat_team<0, true>
+                            : (const void*)k_step_f32_lat_team<1, true>;
+    return sc_mode == 0 ? (const void*)k_step_f32_lat_team<0, false>
+                        : (const void*)k_step_f32_lat_team<1, false>;
+}
+
+cudaError_t launch_step_f32_lat_team(const StepArgsF32& a, int sc_mode, cudaStream_t s)
+{
+    void* args[] = {const_cast<StepArgsF32*>(&a)};
+    return launch_pdl(step_f32_kernel_lat_team(sc_mode, a.cbond != nullptr),
+                      dim3((unsigned)((a.n + 31) / 32)), dim3(128), args,
+                      step_f32_lat_team_smem(), s);
+}
+#endif
 
 #if !PD_LAT_HELPERS
 // entry points of this build: single model or batch, register budget
@@ -621,15 +745,9 @@ const void* PD_LAT_KERNEL_OF(int sc_mode, bool per_bond_c)
 
 cudaError_t PD_LAT_LAUNCH(const StepArgsF32& a, int sc_mode, int grid, int block, cudaStream_t s)
 {
-    const bool pbc = a.cbond != nullptr;
-    if (sc_mode == 0) {
-        if (pbc) k_step_f32_lat<0, true><<<grid, block, 0, s>>>(a);
-        else k_step_f32_lat<0, false><<<grid, block, 0, s>>>(a);
-    } else {
-        if (pbc) k_step_f32_lat<1, true><<<grid, block, 0, s>>>(a);
-        else k_step_f32_lat<1, false><<<grid, block, 0, s>>>(a);
-    }
-    return cudaGetLastError();
+    void* args[] = {const_cast<StepArgsF32*>(&a)};
+    return launch_pdl(PD_LAT_KERNEL_OF(sc_mode, a.cbond != nullptr), dim3(grid), dim3(block), args,
+                      0, s);
 }
 #endif  // !PD_LAT_HELPERS
 

@@ -492,6 +492,7 @@ __global__ void __launch_bounds__(PD_LAT_THREADS, PD_LAT_MIN_BLOCKS)
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     // a direct launch's counter still holds this step (the step's force kernel advances it)
     const int64_t step = a.step_ctr[0] + a.k;
     const int cur = (int)(step & 1);
@@ -539,6 +540,7 @@ __global__ void __launch_bounds__(PD_LAT_THREADS, 3)
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     const int64_t step = lat_step_of(a);
     lat_advance_counter(a);  // the step's last kernel
     const int cur = (int)(step & 1);
@@ -595,10 +597,9 @@ __global__ void __launch_bounds__(PD_LAT_THREADS, 3)
             float vn = vi + a.dt_f * (F[c] - a.eta_f * vi) / a.rho_f;
             un[c] = fma((double)vn, (double)a.dtd_f, U[3 * i + c]);
             if (mask & (1u << c)) {
-                const double s_now = a.disp_rate * (double)step;
-                const double s_next = a.disp_rate * (double)(step + 1);
-                un[c] = bc->disp[c] * s_next * a.inv_delta;
-                vn = (float)(bc->disp[c] * (s_next - s_now) / a.dt);
+                const double2 uv = bc_controlled_linear(a.disp_rate, a.dt, bc->disp[c], step);
+                un[c] = uv.x * a.inv_delta;
+                vn = (float)uv.y;
             }
             finite = finite && isfinite(un[c]);
             a.v[3 * i + c] = vn;
@@ -620,12 +621,12 @@ const void* osb_lat_dilation_kernel(int sc_mode)
 cudaError_t launch_osb_lat_step(const StepArgsF32& a, const OsbLatArgs& o, int sc_mode, int grid,
                                 int grid_force, int block, cudaStream_t s)
 {
-    if (sc_mode == 0)
-        k_osb_lat_dilation<0><<<grid, block, 0, s>>>(a, o);
-    else
-        k_osb_lat_dilation<1><<<grid, block, 0, s>>>(a, o);
-    if (cudaPeekAtLastError() == cudaSuccess) k_osb_lat_force<<<grid_force, block, 0, s>>>(a, o);
-    return cudaGetLastError();
+    void* args[] = {const_cast<StepArgsF32*>(&a), const_cast<OsbLatArgs*>(&o)};
+    const cudaError_t e = launch_pdl(osb_lat_dilation_kernel(sc_mode), dim3(grid), dim3(block),
+                                     args, 0, s);
+    return e != cudaSuccess ? e
+                            : launch_pdl(osb_lat_force_kernel(), dim3(grid_force), dim3(block),
+                                         args, 0, s);
 }
 
 }  // namespace pd

@@ -109,9 +109,6 @@ __global__ void __launch_bounds__(BZ * BY * BX, PD_LAT_MIN_BLOCKS)
     float4* tile = reinterpret_cast<float4*>(base);
     uint64_t* bar = reinterpret_cast<uint64_t*>(base + kBytes);
 
-    const int64_t step = lat_step_of(a);
-    lat_advance_counter(a);
-    const int cur = (int)(step & 1);
     const int b = blockIdx.x;
     const int bz = b % t.tiles_z, by = (b / t.tiles_z) % t.tiles_y, bx = b / (t.tiles_z * t.tiles_y);
     const int z0 = bz * BZ, y0 = by * BY, x0 = bx * BX;
@@ -119,6 +116,10 @@ __global__ void __launch_bounds__(BZ * BY * BX, PD_LAT_MIN_BLOCKS)
         mbar_init(bar, 1);
         mbar_fence_init();
     }
+    pdl_begin();
+    const int64_t step = lat_step_of(a);
+    lat_advance_counter(a);
+    const int cur = (int)(step & 1);
     __syncthreads();
     if (threadIdx.x == 0) {
         mbar_arrive_expect_tx(bar, kBytes + (uint32_t)t.extra_tx);
@@ -160,20 +161,6 @@ const void* tma_kernel(int sc_mode, bool pbc)
                         : (const void*)k_step_f32_lat_tma<1, false, BZ, BY, BX>;
 }
 
-template <int BZ, int BY, int BX>
-void tma_launch(const StepArgsF32& a, const LatTmaArgs& t, int sc_mode, bool pbc, int grid,
-                size_t smem, cudaStream_t s)
-{
-    constexpr int threads = BZ * BY * BX;
-    if (sc_mode == 0) {
-        if (pbc) k_step_f32_lat_tma<0, true, BZ, BY, BX><<<grid, threads, smem, s>>>(a, t);
-        else k_step_f32_lat_tma<0, false, BZ, BY, BX><<<grid, threads, smem, s>>>(a, t);
-    } else {
-        if (pbc) k_step_f32_lat_tma<1, true, BZ, BY, BX><<<grid, threads, smem, s>>>(a, t);
-        else k_step_f32_lat_tma<1, false, BZ, BY, BX><<<grid, threads, smem, s>>>(a, t);
-    }
-}
-
 }  // namespace
 
 const void* step_f32_kernel_lat_tma(int shape, int sc_mode, bool per_bond_c)
@@ -188,14 +175,10 @@ const void* step_f32_kernel_lat_tma(int shape, int sc_mode, bool per_bond_c)
 cudaError_t launch_step_f32_lat_tma(const StepArgsF32& a, const LatTmaArgs& t, int shape,
                                     int sc_mode, int grid, cudaStream_t s)
 {
-    const bool pbc = a.cbond != nullptr;
-    const size_t smem = lat_tma_smem_bytes(shape);
-    switch (shape) {
-    case 0: tma_launch<16, 2, 8>(a, t, sc_mode, pbc, grid, smem, s); break;
-    case 1: tma_launch<8, 4, 8>(a, t, sc_mode, pbc, grid, smem, s); break;
-    default: tma_launch<32, 2, 4>(a, t, sc_mode, pbc, grid, smem, s); break;
-    }
-    return cudaGetLastError();
+    const int threads = lat_tma_dim(shape, 0) * lat_tma_dim(shape, 1) * lat_tma_dim(shape, 2);
+    void* args[] = {const_cast<StepArgsF32*>(&a), const_cast<LatTmaArgs*>(&t)};
+    return launch_pdl(step_f32_kernel_lat_tma(shape, sc_mode, a.cbond != nullptr), dim3(grid),
+                      dim3(threads), args, lat_tma_smem_bytes(shape), s);
 }
 
 }  // namespace pd

@@ -57,10 +57,10 @@ __device__ __forceinline__ void integrate_osb_f32(const StepArgsF32& a, int64_t 
         }
         ff_add(H[c], L[c], vn * dtd);
         if (mask & (1u << c)) {
-            const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
-            const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
-            ff_set(bc->disp[c] * s_next * a.inv_delta, H[c], L[c]);
-            vn = (float)(bc->disp[c] * (s_next - s_now) / a.dt);
+            const double2 uv =
+                bc_controlled(a.disp_rate, a.ramp_steps, a.dt, bc->disp[c], step);
+            ff_set(uv.x * a.inv_delta, H[c], L[c]);
+            vn = (float)uv.y;
             vfull = vi;
         }
         finite = finite && isfinite(H[c]);
@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(256) k_osb32_dilation(const __grid_constant__ 
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     const int64_t step = a.step_ctr[0] + a.k;
     const int cur = (int)(step & 1);
     const float4* __restrict__ R = a.rec[cur];
@@ -177,6 +178,7 @@ __global__ void __launch_bounds__(256, 3) k_osb32_force(const __grid_constant__ 
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     const int64_t step = a.step_ctr[0] + a.k;
     const int cur = (int)(step & 1);
     const float4* __restrict__ R = a.rec[cur];
@@ -278,9 +280,12 @@ template <int SCM, bool UW>
 cudaError_t osb32_step(const StepArgsF32& a, const OsbArgs32& o, int grid, int grid_dil,
                        int block, cudaStream_t s)
 {
-    k_osb32_dilation<SCM, UW><<<grid_dil, block, 0, s>>>(a, o);
-    if (cudaPeekAtLastError() == cudaSuccess) k_osb32_force<SCM, UW><<<grid, block, 0, s>>>(a, o);
-    return cudaGetLastError();
+    void* args[] = {const_cast<StepArgsF32*>(&a), const_cast<OsbArgs32*>(&o)};
+    const cudaError_t e = launch_pdl((const void*)k_osb32_dilation<SCM, UW>, dim3(grid_dil),
+                                     dim3(block), args, 0, s);
+    return e != cudaSuccess ? e
+                            : launch_pdl((const void*)k_osb32_force<SCM, UW>, dim3(grid),
+                                         dim3(block), args, 0, s);
 }
 }  // namespace
 

@@ -275,17 +275,6 @@ __device__ __forceinline__ Node load_node(const StepArgsF64& a, const W3Args& d,
     return n;
 }
 
-// Displacement and velocity of a controlled component.  A call, because inlined its
-// FP64 operations (about 150 with the smooth start and the divisions) are moved in front
-// of the node loop, where every warp of a team executes them: 10 of the 16 us of a step of
-// the 4000-node bar.
-__device__ __noinline__ double2 controlled(const StepArgsF64& a, double g, int64_t step)
-{
-    const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
-    const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
-    return make_double2(g * s_next, g * (s_next - s_now) / a.dt);
-}
-
 // Integration of the lane's node (damped Euler-Cromer, Eq. 11, or damped
 // velocity-Verlet), BCs, damage, and the records its neighbours read next.
 __device__ __forceinline__ void finish_node(const StepArgsF64& a, const W3Args& d, int cur,
@@ -328,7 +317,7 @@ __device__ __forceinline__ void finish_node(const StepArgsF64& a, const W3Args& 
         }
         double u = fma(a.dt, vn, uo[c]);
         if (mask & (1u << c)) {
-            const double2 uv = controlled(a, gdisp[c], step);
+            const double2 uv = bc_controlled(a.disp_rate, a.ramp_steps, a.dt, gdisp[c], step);
             u = uv.x;
             vn = uv.y;
             vfull = vi;
@@ -383,8 +372,7 @@ __global__ void __launch_bounds__(256, 2)
         prefetch_l2(a.nbr + g * 32LL * a.Q * 32, (uint32_t)(((Wg + 3) & ~3) * 128));
         if (TEAM) prefetch_l2(d.il + g * 16LL * a.Q * 32, (uint32_t)(((Wg + 3) & ~3) * 256));
     }
-    pdl_wait();
-    pdl_launch();
+    pdl_begin(TEAM);
     const int64_t step = a.step_ctr[0] + a.k;
     const int cur = (int)(step & 1);
     const float4* __restrict__ R = d.rec[cur];

@@ -45,15 +45,6 @@ __device__ __noinline__ bool pair_no_fail(const uint8_t* __restrict__ bcc,
     return ((bct[bcc[i]].mask | bct[bcc[j]].mask) & 8u) != 0u;
 }
 
-// Displacement and velocity of a controlled component (a call, so that its FP64
-// operations are not moved before the node loop)
-__device__ __noinline__ double2 controlled(const StepArgsF64& a, double g, int64_t step)
-{
-    const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
-    const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
-    return make_double2(g * s_next, g * (s_next - s_now) / a.dt);
-}
-
 // rsqrt_nr with the halvings and the seed's conversion to FP64 as integer operations on
 // the exponent field (the same bits; they keep three operations a bond off the FP64 pipe)
 __device__ __forceinline__ double half_of(double y)
@@ -79,8 +70,7 @@ __global__ void __launch_bounds__(256) k_step_f64_soft(const StepArgsF64 a)
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    pdl_wait();
-    pdl_launch();
+    pdl_begin();
     const int64_t step = a.step_ctr[0] + a.k;
     const bool first = a.vv && step == a.step_ctr[1];  // velocity-Verlet: a^n formed afresh
     const int cur = (int)(step & 1);
@@ -217,7 +207,7 @@ __global__ void __launch_bounds__(256) k_step_f64_soft(const StepArgsF64 a)
                 }
                 double u = uo[c] + a.dt * vn;
                 if (mask & (1u << c)) {
-                    const double2 uv = controlled(a, gdisp[c], step);
+                    const double2 uv = bc_controlled(a.disp_rate, a.ramp_steps, a.dt, gdisp[c], step);
                     u = uv.x;
                     vn = uv.y;
                     vfull = vi;

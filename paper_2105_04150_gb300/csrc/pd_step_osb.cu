@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(256) k_osb_dilation(const StepArgsF64 a, OsbAr
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     const int64_t step = a.step_ctr[0] + a.k;
     const double2* __restrict__ rin = reinterpret_cast<const double2*>(a.rec[step & 1]);
     const int64_t W = 32LL * a.Q;
@@ -146,6 +147,7 @@ __global__ void __launch_bounds__(256) k_osb_force(const StepArgsF64 a, OsbArgs 
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     const int64_t step = a.step_ctr[0] + a.k;
     const int cur = (int)(step & 1);
     const double2* __restrict__ rin = reinterpret_cast<const double2*>(a.rec[cur]);
@@ -194,8 +196,6 @@ __global__ void __launch_bounds__(256) k_osb_force(const StepArgsF64 a, OsbArgs 
                 F[c] += a.load * bc.force[c];
             }
         }
-        const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
-        const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
         const double uo[3] = {u01.x, u01.y, u23.x};
         // velocity-Verlet: a^n is formed afresh at the step the state was set
         const bool first = a.vv && step == a.step_ctr[1];
@@ -217,8 +217,10 @@ __global__ void __launch_bounds__(256) k_osb_force(const StepArgsF64 a, OsbArgs 
             }
             double u = uo[c] + a.dt * vn;
             if (mask & (1u << c)) {
-                u = gdisp[c] * s_next;
-                vn = gdisp[c] * (s_next - s_now) / a.dt;
+                const double2 uv =
+                    bc_controlled(a.disp_rate, a.ramp_steps, a.dt, gdisp[c], step);
+                u = uv.x;
+                vn = uv.y;
                 vfull = vi;
             }
             finite = finite && isfinite(u);
@@ -282,11 +284,10 @@ cudaError_t launch_osb_setup(const StepArgsF64& a, const OsbArgs& o, const doubl
 cudaError_t launch_osb_step(const StepArgsF64& a, const OsbArgs& o, int grid, int block,
                             cudaStream_t s)
 {
-    k_osb_dilation<<<grid, block, 0, s>>>(a, o);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_osb_force<<<grid, block, 0, s>>>(a, o);
-    return cudaGetLastError();
+    void* args[] = {const_cast<StepArgsF64*>(&a), const_cast<OsbArgs*>(&o)};
+    const cudaError_t e = launch_pdl((const void*)k_osb_dilation, dim3(grid), dim3(block), args, 0, s);
+    return e != cudaSuccess ? e
+                            : launch_pdl((const void*)k_osb_force, dim3(grid), dim3(block), args, 0, s);
 }
 
 const void* osb_force_kernel() { return (const void*)k_osb_force; }

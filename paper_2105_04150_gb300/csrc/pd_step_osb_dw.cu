@@ -144,6 +144,7 @@ __global__ void __launch_bounds__(256, 2)
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     const int64_t step = a.step_ctr[0] + a.k;
     const float4* __restrict__ R = d.rec[step & 1];
     const int Q = a.Q;
@@ -243,6 +244,7 @@ __global__ void __launch_bounds__(256, 2)
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    pdl_begin();
     const int64_t step = a.step_ctr[0] + a.k;
     const int cur = (int)(step & 1);
     const float4* __restrict__ R = d.rec[cur];
@@ -329,8 +331,6 @@ __global__ void __launch_bounds__(256, 2)
                 Fn[k] += a.load * bc.force[k];
             }
         }
-        const double s_now = bc_scale(a.disp_rate, a.ramp_steps, step);
-        const double s_next = bc_scale(a.disp_rate, a.ramp_steps, step + 1);
         const double2 u01 = rin[4 * i + 2], u23 = rin[4 * i + 3];
         const double uo[3] = {u01.x, u01.y, u23.x};
         const bool first = a.vv && step == a.step_ctr[1];
@@ -351,8 +351,10 @@ __global__ void __launch_bounds__(256, 2)
             }
             double u = uo[k] + a.dt * vn;
             if (mask & (1u << k)) {
-                u = gdisp[k] * s_next;
-                vn = gdisp[k] * (s_next - s_now) / a.dt;
+                const double2 uv =
+                    bc_controlled(a.disp_rate, a.ramp_steps, a.dt, gdisp[k], step);
+                u = uv.x;
+                vn = uv.y;
                 vfull = vi;
             }
             finite = finite && isfinite(u);
@@ -396,14 +398,12 @@ cudaError_t launch_osb_dw_setup(const StepArgsF64& a, const OsbDwArgs& o, cudaSt
 cudaError_t launch_osb_dw_step(const StepArgsF64& a, const DwArgs& d, const OsbDwArgs& o, int grid,
                                int block, cudaStream_t s)
 {
-    k_osb_dw_dilation<<<grid, block, 0, s>>>(a, d, o);
-    cudaError_t e = cudaGetLastError();
+    void* args[] = {const_cast<StepArgsF64*>(&a), const_cast<DwArgs*>(&d), const_cast<OsbDwArgs*>(&o)};
+    const cudaError_t e = launch_pdl((const void*)k_osb_dw_dilation, dim3(grid), dim3(block), args,
+                                     0, s);
     if (e != cudaSuccess) return e;
-    if (d.uniform_w)
-        k_osb_dw_force<true><<<grid, block, 0, s>>>(a, d, o);
-    else
-        k_osb_dw_force<false><<<grid, block, 0, s>>>(a, d, o);
-    return cudaGetLastError();
+    const void* fn = d.uniform_w ? (const void*)k_osb_dw_force<true> : (const void*)k_osb_dw_force<false>;
+    return launch_pdl(fn, dim3(grid), dim3(block), args, 0, s);
 }
 
 }  // namespace pd
