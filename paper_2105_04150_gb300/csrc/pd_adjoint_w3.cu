@@ -1,5 +1,5 @@
-// Reverse step of the FP64 adjoint with most of its work off the FP64 pipe
-// (sm_103a); it computes what k_adj_step (pd_adjoint.cu) computes:
+// Reverse step of the adjoint with most of its work off the FP64 pipe (sm_103a); it
+// computes what k_adj_step (pd_adjoint.cu) computes:
 //
 //   ubar^n_m = ubar_m + (dt/rho) sum_j c_mj K_mj d_mj,  d_mj = V_m w_j - V_j w_m
 //   vbar^n_m = (1 - dt eta/rho) w_m
@@ -75,45 +75,57 @@ __device__ __forceinline__ double unit_scale(const unsigned long long* m)
     return v > 0.0 && v < 1e300 ? scalbn(1.0, -ilogb(v)) : 1.0;
 }
 
-// Start of a reverse step for node p: w = ws (vbar + dt ubar) with the controlled
-// components of ubar and vbar zeroed (as k_adj_mask), and the records the bond loop
-// reads: the three-word one of x (from the forward run's) and u^n, w in FP64
-// ({w, 0}) and w as double-words in units of 1 / unit_scale ({wh, wl.x} {wl.y, wl.z, 0, 0}).
-__global__ void k_adj_prep_w3(const AdjW3Args a, const double* __restrict__ ub,
-                              const double* __restrict__ vb, const float4* __restrict__ fwd,
-                              double dt, double ws, int64_t n_pad, double scale)
+// The records of a reverse step for node p, from its ubar, vbar and u^n: w = ws (vbar + dt
+// ubar) with the controlled components of ubar and vbar zeroed (as k_adj_mask), the
+// three-word record of x (its words from `fwd`) and u^n, w in FP64 ({w, 0}) and w as
+// double-words in units of 1 / unit_scale ({wh, wl.x} {wl.y, wl.z, 0, 0}).
+__device__ __forceinline__ void adj_records(const AdjW3Args& a, int64_t p, uint32_t mask,
+                                            const double (&ub)[3], const double (&vb)[3],
+                                            const double* un, double dt, double ws, double us,
+                                            const Rec& fwd, float4* rec, double* w64, float4* wdw)
+{
+    const float tin[3] = {fwd.a1.z, fwd.a1.w, fwd.b1.z};
+    float uh[3], um[3], t[3], wh[3], wl[3];
+    double w[3];
+    for (int k = 0; k < 3; ++k) {
+        const bool ctl = (mask >> k) & 1u;
+        const double u = ctl ? 0.0 : ub[k];
+        const double v = ctl ? 0.0 : vb[k];
+        w[k] = ws * (v + dt * u);
+        a.ubm[3 * p + k] = u;
+        float ut;
+        split3(un[3 * p + k] * a.scale, kW3UGrid, uh[k], um[k], ut);
+        t[k] = pack_t(__float_as_uint(tin[k]) & 0x7ffu, ut);
+        const double v1 = w[k] * us;
+        wh[k] = (float)v1;
+        wl[k] = (float)(v1 - (double)wh[k]);
+    }
+    double2* wr = reinterpret_cast<double2*>(w64 + 4 * p);
+    wr[0] = make_double2(w[0], w[1]);
+    wr[1] = make_double2(w[2], 0.0);
+    dwa::st_rec(rec + 4 * p, make_float4(fwd.a0.x, fwd.a0.y, uh[0], uh[1]),
+                make_float4(fwd.a1.x, uh[2], t[0], t[1]));
+    dwa::st_rec(rec + 4 * p + 2, make_float4(fwd.b0.x, fwd.b0.y, um[0], um[1]),
+                make_float4(fwd.b1.x, um[2], t[2], 0.0f));
+    dwa::st_rec(wdw + 2 * p, make_float4(wh[0], wh[1], wh[2], wl[0]),
+                make_float4(wl[1], wl[2], 0.0f, 0.0f));
+}
+
+__global__ void k_adj_prep_w3(const __grid_constant__ AdjW3Args a, double dt, double ws, int64_t n_pad)
 {
     const double us = unit_scale(a.wmax);
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_pad;
          p += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t cls = a.bcc[p];
-        const uint32_t mask = cls ? a.bct[cls].mask : 0u;
-        const float4 a0 = fwd[4 * p], a1 = fwd[4 * p + 1], b0 = fwd[4 * p + 2], b1 = fwd[4 * p + 3];
-        const float tin[3] = {a1.z, a1.w, b1.z};
-        float uh[3], um[3], t[3], wh[3], wl[3];
-        double w[3];
-        for (int k = 0; k < 3; ++k) {
-            const bool ctl = (mask >> k) & 1u;
-            const double u = ctl ? 0.0 : ub[3 * p + k];
-            const double v = ctl ? 0.0 : vb[3 * p + k];
-            w[k] = ws * (v + dt * u);
-            a.ubm[3 * p + k] = u;
-            float ut;
-            split3(a.un[3 * p + k] * scale, kW3UGrid, uh[k], um[k], ut);
-            t[k] = pack_t(__float_as_uint(tin[k]) & 0x7ffu, ut);
-            const double v1 = w[k] * us;
-            wh[k] = (float)v1;
-            wl[k] = (float)(v1 - (double)wh[k]);
-        }
-        double2* wr = reinterpret_cast<double2*>(a.w64 + 4 * p);
-        wr[0] = make_double2(w[0], w[1]);
-        wr[1] = make_double2(w[2], 0.0);
-        a.rec[4 * p] = make_float4(a0.x, a0.y, uh[0], uh[1]);
-        a.rec[4 * p + 1] = make_float4(a1.x, uh[2], t[0], t[1]);
-        a.rec[4 * p + 2] = make_float4(b0.x, b0.y, um[0], um[1]);
-        a.rec[4 * p + 3] = make_float4(b1.x, um[2], t[2], 0.0f);
-        a.wdw[2 * p] = make_float4(wh[0], wh[1], wh[2], wl[0]);
-        a.wdw[2 * p + 1] = make_float4(wl[1], wl[2], 0.0f, 0.0f);
+        Rec f;
+        f.a0 = a.fwd[4 * p];
+        f.a1 = a.fwd[4 * p + 1];
+        f.b0 = a.fwd[4 * p + 2];
+        f.b1 = a.fwd[4 * p + 3];
+        const double ub[3] = {a.ub[3 * p], a.ub[3 * p + 1], a.ub[3 * p + 2]};
+        const double vb[3] = {a.vb[3 * p], a.vb[3 * p + 1], a.vb[3 * p + 2]};
+        adj_records(a, p, cls ? a.bct[cls].mask : 0u, ub, vb, a.un, dt, ws, us, f, a.rec, a.w64,
+                    a.wdw);
     }
 }
 
@@ -153,6 +165,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
     const int lane = threadIdx.x & 31, rank = threadIdx.x >> 5;
     const int Q = a.Q;
     const int64_t g = blockIdx.x;
+    pdl_begin();
     const int64_t m = (g << 5) + lane;
     const int Wg = a.sw[g];
     const int64_t slot0 = g * 32LL * Q * 32 + lane;
@@ -285,6 +298,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
     __syncthreads();
     if (rank == 0 && m < a.n) {
         const double w3[3] = {wm.x, wm.y, wm.z};
+        double ub[3], vb[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             double s = 0.0;
@@ -294,14 +308,22 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
                 c = dw_add(c, Dw{sf[r][2 * k][lane], sf[r][2 * k + 1][lane]});
             }
             s += ((double)c.h + (double)c.l) * (a.scale / us);
-            a.ub_out[3 * m + k] = a.ubm[3 * m + k] + (a.dt_rho * a.w_ref) * s;
-            a.vb_out[3 * m + k] = a.damp * w3[k];
+            ub[k] = a.ubm[3 * m + k] + (a.dt_rho * a.w_ref) * s;
+            vb[k] = a.damp * w3[k];
+            a.ub_out[3 * m + k] = ub[k];
+            a.vb_out[3 * m + k] = vb[k];
         }
         const uint32_t cls = a.bcc[m];
+        uint32_t mask = 0u;
         if (cls) {
             const BcClass& bc = a.bct[cls];
+            mask = bc.mask;
             a.gl[m] += bc.force[0] * w3[0] + bc.force[1] * w3[1] + bc.force[2] * w3[2];
         }
+        // the next reverse step's records: everything they need is this node's
+        if (a.next_un != nullptr)
+            adj_records(a, m, mask, ub, vb, a.next_un, a.next_dt, a.next_ws, us, me, a.next_rec,
+                        a.next_w64, a.next_wdw);
     }
 }
 
@@ -384,17 +406,18 @@ cudaError_t launch_adj_e(const double* x64, const int32_t* nbr, int64_t n_slices
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_step_w3(const AdjW3Args& a, const double* ub, const double* vb,
-                               const float4* fwd, double dt, double ws, int64_t n_pad,
+cudaError_t launch_adj_prep_w3(const AdjW3Args& a, double dt, double ws, int64_t n_pad,
                                cudaStream_t s)
 {
-    k_adj_prep_w3<<<grid_of(n_pad), 256, 0, s>>>(a, ub, vb, fwd, dt, ws, n_pad, a.scale);
-    const int blocks = (int)((a.n + 31) / 32);
-    if (a.uniform_w)
-        k_adj_step_w3<true><<<blocks, 32 * kTeam, 0, s>>>(a);
-    else
-        k_adj_step_w3<false><<<blocks, 32 * kTeam, 0, s>>>(a);
+    k_adj_prep_w3<<<grid_of(n_pad), 256, 0, s>>>(a, dt, ws, n_pad);
     return cudaGetLastError();
+}
+
+cudaError_t launch_adj_step_w3(const AdjW3Args& a, cudaStream_t s)
+{
+    const void* fn = a.uniform_w ? (const void*)k_adj_step_w3<true> : (const void*)k_adj_step_w3<false>;
+    void* args[] = {const_cast<AdjW3Args*>(&a)};
+    return launch_pdl(fn, dim3((unsigned)((a.n + 31) / 32)), dim3(32 * kTeam), args, 0, s);
 }
 
 cudaError_t launch_adj_merge_w3(double* gc, int64_t count, double scale,

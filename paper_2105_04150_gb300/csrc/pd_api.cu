@@ -133,7 +133,8 @@ struct pd_handle {
     float2* lendw = nullptr;                // per slot |xi| / delta
     float2* cbdw = nullptr;                 // per slot c_ij (per-bond stiffness)
     double dw_origin[3] = {0.0, 0.0, 0.0};  // origin of the double-word positions
-    // bond-based PD_PREC_F64: three-word records and bond lengths of the step (W3Args)
+    // bond-based PD_PREC_F64 and PD_PREC_DW without softening: three-word records and bond
+    // lengths of the step (W3Args)
     bool w3 = false;
     float4* rec3[2] = {nullptr, nullptr};
     float4* il3 = nullptr;
@@ -184,13 +185,10 @@ struct pd_handle {
         double *ub[2] = {nullptr, nullptr}, *vb[2] = {nullptr, nullptr}, *ubm = nullptr,
                *w = nullptr, *gc = nullptr, *gl = nullptr, *partial = nullptr, *out = nullptr;
         int n_partial = 0;
-        // double-word reverse sweep (PD_PREC_DW): records of u^n and w, and the
-        // per-slot gradient accumulator
-        float4 *rrec = nullptr, *wrec = nullptr;
-        float2* gcdw = nullptr;
-        // FP64 reverse sweep (pd_adjoint_w3.cu): w in FP64 records, xi / |xi|^(3/2) per
-        // slot, the seeds' largest component
-        double *w64 = nullptr, *e = nullptr;
+        // the reverse sweep's records (pd_adjoint_w3.cu), double buffered: u^n, w in
+        // double-words and in FP64; xi / |xi|^(3/2) per slot, the seeds' largest component
+        float4 *rrec[2] = {nullptr, nullptr}, *wrec[2] = {nullptr, nullptr};
+        double *w64[2] = {nullptr, nullptr}, *e = nullptr;
         unsigned long long* wmax = nullptr;
         // dL/dc in canonical order: the family on the device, and the result
         int64_t* fam_off = nullptr;
@@ -575,7 +573,7 @@ W3Args w3_args(pd_handle* h)
 // the records that neighbours read, of buffer b, from the FP64 records
 cudaError_t publish64(pd_handle* h, int b)
 {
-    if (h->dw)
+    if (h->dw && !h->w3)
         return launch_dw_publish(h->rec[b], h->recdw[b], h->n_pad, h->dw_origin, 1.0 / h->delta,
                                  h->stream);
     if (h->w3)
@@ -587,10 +585,10 @@ cudaError_t publish64(pd_handle* h, int b)
 const void* step_kernel_fn(pd_handle* h)
 {
     if (h->precision == 32) return f32_kernel(h);
-    if (h->dw)
-        return step_dw_kernel(h->sc_mode, h->uniform_vol && !h->batch, h->integ != nullptr,
-                              h->integrator == PD_INTEGRATOR_VV);
     if (h->w3) return step_f64_kernel(h->uniform_vol, h->team > 1);
+    if (h->dw)
+        return step_dw_kernel(h->sc_mode, h->uniform_vol && !h->batch,
+                              h->integrator == PD_INTEGRATOR_VV);
     return h->integ != nullptr ? step_f64_soft_kernel(h->sc_mode) : osb_force_kernel();
 }
 
@@ -602,7 +600,7 @@ cudaError_t launch_one(pd_handle* h, int k, int64_t step_abs = -1)
     if (h->dw && h->model == 1)
         return launch_osb_dw_step(args_f64(h, k), dw_args(h), osbdw_args(h), h->grid, h->block,
                                   h->stream);
-    if (h->dw)
+    if (h->dw && !h->w3)
         return launch_step_dw(args_f64(h, k), dw_args(h), h->sc_mode, h->grid, h->block,
                               h->stream);
     if (h->model == 1 && h->precision == 32)
@@ -824,8 +822,9 @@ pd_status vv_force_pass(pd_handle* h)
                                            h->stream)
                       : launch_osb_step(a, osb_args(h), h->grid, h->block, h->stream);
         else
-            e = h->dw ? launch_step_dw(a, dw_args(h), h->sc_mode, h->grid, h->block, h->stream)
-                      : launch_f64(h, a);
+            e = h->dw && !h->w3
+                    ? launch_step_dw(a, dw_args(h), h->sc_mode, h->grid, h->block, h->stream)
+                    : launch_f64(h, a);
     }
     if (e != cudaSuccess) return cuda_fail(e, "velocity-Verlet force pass");
     h->peek_step = h->step;
@@ -1027,7 +1026,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
     std::vector<uint8_t> cls;
     std::string msg = bc_classes(n, d.type, d.disp, d.force, d.no_fail, table, cls, h->has_nofail);
     if (!msg.empty()) return fail(PD_ERR_ARG, "%s", msg.c_str());
-    h->w3 = cfg->precision == PD_PREC_F64 && h->model == 0 &&
+    h->w3 = cfg->precision != PD_PREC_F32 && h->model == 0 &&
             (h->kr < 1.0 || (h->kr == 1.0 && !h->has_nofail));
     // The literal FP64 step is bound by each SM's FP64 pipe, so its slices have to be
     // spread evenly: one warp per block (a 962-slice model fills 121 SMs with 8 slices
@@ -1111,7 +1110,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
         ALLOC(h->v, double, 3 * np);
         ALLOC(h->wsum_inv, double, np);
         ALLOC(h->damage, double, np);
-        if (h->dw) {
+        if (h->dw && !h->w3) {
             ALLOC(h->recdw[0], float4, 4 * np);
             ALLOC(h->recdw[1], float4, 4 * np);
             ALLOC(h->lendw, float2, nbr.size());
@@ -1152,8 +1151,9 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
             ALLOC(h->osb_beta, double, np);
         }
     }
-    // bilinear softening: every bond starts intact, mu = 1 (FP64 with kr = 1 and no
-    // no-fail nodes is the PMB law: its kernel, and the flags are the integrity)
+    // bilinear softening: every bond starts intact, mu = 1 (FP64 and double-word with
+    // kr = 1 and no no-fail nodes is the PMB law: its kernel, and the flags are the
+    // integrity)
     if (h->kr >= 1.0 && !h->w3) {
         if (f32)
             ALLOC(h->integ, float, nbr.size());
@@ -1198,7 +1198,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
                 hi[a] = std::max(hi[a], d.coords[3 * i + a]);
             }
         for (int a = 0; a < 3; ++a) gctr[a] = 0.5 * (lo[a] + hi[a]);
-        if (h->dw) {
+        if (h->dw && !h->w3) {
             // double-word positions start B horizons above zero, B above the
             // largest coordinate difference of any bond: then for every bond
             // x_j / x_i is in [1/2, 2] per component, and the difference of the
@@ -1352,7 +1352,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
                            h->batch ? h->inst : nullptr, h->itab, h->il3, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "bond lengths");
     }
-    if (h->dw) {
+    if (h->dw && !h->w3) {
         e = launch_dw_len(h->x64, h->nbr, n, h->Q, 1.0 / h->delta, h->lendw, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "bond lengths");
     }
@@ -2162,17 +2162,13 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         if ((e = h->alloc(&T.partial, (size_t)T.n_partial)) != cudaSuccess)
             return cuda_fail(e, "cudaMalloc reduction scratch");
     }
-    if (h->dw && !T.gcdw) {
-        if ((e = h->alloc(&T.rrec, (size_t)(4 * h->n_pad))) != cudaSuccess ||
-            (e = h->alloc(&T.wrec, (size_t)(2 * h->n_pad))) != cudaSuccess ||
-            (e = h->alloc(&T.gcdw, (size_t)slots)) != cudaSuccess)
-            return cuda_fail(e, "cudaMalloc double-word adjoint buffers");
-    }
-    if (h->w3 && !T.e) {
-        if ((e = h->alloc(&T.rrec, (size_t)(4 * h->n_pad))) != cudaSuccess ||
-            (e = h->alloc(&T.wrec, (size_t)(2 * h->n_pad))) != cudaSuccess ||
-            (e = h->alloc(&T.w64, (size_t)(4 * h->n_pad))) != cudaSuccess ||
-            (e = h->alloc(&T.wmax, 1)) != cudaSuccess ||
+    if (!T.e) {
+        for (int k = 0; k < 2; ++k)
+            if ((e = h->alloc(&T.rrec[k], (size_t)(4 * h->n_pad))) != cudaSuccess ||
+                (e = h->alloc(&T.wrec[k], (size_t)(2 * h->n_pad))) != cudaSuccess ||
+                (e = h->alloc(&T.w64[k], (size_t)(4 * h->n_pad))) != cudaSuccess)
+                return cuda_fail(e, "cudaMalloc adjoint records");
+        if ((e = h->alloc(&T.wmax, 1)) != cudaSuccess ||
             (e = h->alloc(&T.e, (size_t)(3 * slots))) != cudaSuccess)
             return cuda_fail(e, "cudaMalloc adjoint records");
         PD_CUDA(launch_adj_e(h->rec[0], h->nbr, h->n_slices, h->Q, T.e, h->stream), "bond vectors");
@@ -2199,22 +2195,13 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
     if ((st = to_lib(dLdu, T.ub[0])) != PD_OK || (st = to_lib(dLdv, T.vb[0])) != PD_OK) return st;
     PD_CUDA(cudaMemsetAsync(T.gc, 0, 8 * slots, h->stream), "memset");
     PD_CUDA(cudaMemsetAsync(T.gl, 0, 8 * h->n_pad, h->stream), "memset");
-    if (h->dw) PD_CUDA(cudaMemsetAsync(T.gcdw, 0, 8 * slots, h->stream), "memset");
-    if (h->w3)
-        PD_CUDA(launch_adj_scale_w3(T.ub[0], T.vb[0], np3, h->dt, T.wmax, h->stream),
-                "gradient scale");
+    PD_CUDA(launch_adj_scale_w3(T.ub[0], T.vb[0], np3, h->dt, T.wmax, h->stream), "gradient scale");
 
-    int sms = 0;
-    PD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device), "sm count");
-    const int agrid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * 8,
-                                                                  (h->n_slices + 7) / 8));
     const double dt_rho = h->dt / h->rho;
     AdjW3Args A{};
-    if (h->w3) {
+    {
         A.x64 = h->rec[0];
-        A.rec = T.rrec;
-        A.w64 = T.w64;
-        A.wdw = T.wrec;
+        A.fwd = h->rec3[0];
         A.ubm = T.ubm;
         A.wmax = T.wmax;
         A.nbr = h->nbr;
@@ -2240,31 +2227,6 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         A.dt_rho = dt_rho;
         A.n = h->n;
     }
-    AdjDwArgs D{};
-    if (h->dw) {
-        D.rec = T.rrec;
-        D.wrec = T.wrec;
-        D.len = h->lendw;
-        D.cb = h->per_bond_c ? h->cbdw : nullptr;
-        const float ch = (float)h->c;
-        D.c = make_float2(ch, (float)(h->c - (double)ch));
-        D.gc = T.gcdw;
-        D.w = T.w;
-        D.ubm = T.ubm;
-        D.gl = T.gl;
-        D.nbr = h->nbr;
-        D.bits = h->bits;
-        D.sw = h->sw;
-        D.Q = h->Q;
-        D.uniform_w = h->uniform_vol ? 1 : 0;
-        D.n = h->n;
-        D.bcc = h->bcc;
-        D.bct = h->bct;
-        D.dt_rho = dt_rho;
-        D.inv_delta = 1.0 / h->delta;
-        D.vol0 = h->vol0;
-    }
-
     h->frozen = true;
     h->drop_graph();
     int cb = 0;
@@ -2274,32 +2236,44 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
     // forms the full-step velocity it ends with: ws = 1/2 there, and
     // damp = 1 + (1 - dt eta / rho) so that damp ws = 1 - dt eta / (2 rho)
     const double damp_full = 1.0 - h->dt * h->eta / h->rho;
-    auto reverse_step = [&](const double* un, double dtw, double ws, double damp) {
-        cudaError_t r;
-        if (h->dw) {
-            r = launch_adj_mask_publish_dw(T.ub[cb], T.vb[cb], h->bcc, h->bct, dtw, ws,
-                                           h->recdw[0], un, h->vol, h->n_pad, 1.0 / h->delta,
-                                           T.ubm, T.w, T.rrec, T.wrec, h->stream);
-            D.ub_out = T.ub[cb ^ 1];
-            D.vb_out = T.vb[cb ^ 1];
-            D.damp = damp;
-            if (r == cudaSuccess) r = launch_adj_step_dw(D, agrid, 256, h->stream);
-        } else {
-            A.un = un;
-            A.ub_out = T.ub[cb ^ 1];
-            A.vb_out = T.vb[cb ^ 1];
-            A.damp = damp;
-            r = launch_adj_step_w3(A, T.ub[cb], T.vb[cb], h->rec3[0], dtw, ws, h->n_pad, h->stream);
-        }
+    // The records of a step come from the one before it (next, at the state it steps back
+    // from) or, for the first of a segment, from a kernel of their own (prepared false).
+    struct Rev {
+        const double* un;
+        double dtw, ws, damp;
+    };
+    int rb = 0;  // the records' buffer
+    bool prepared = false;
+    auto reverse_step = [&](const Rev& r, const Rev* next) {
+        A.un = r.un;
+        A.ub = T.ub[cb];
+        A.vb = T.vb[cb];
+        A.ub_out = T.ub[cb ^ 1];
+        A.vb_out = T.vb[cb ^ 1];
+        A.damp = r.damp;
+        A.rec = T.rrec[rb];
+        A.w64 = T.w64[rb];
+        A.wdw = T.wrec[rb];
+        cudaError_t ce = prepared ? cudaSuccess : launch_adj_prep_w3(A, r.dtw, r.ws, h->n_pad, h->stream);
+        A.next_un = next ? next->un : nullptr;
+        A.next_dt = next ? next->dtw : 0.0;
+        A.next_ws = next ? next->ws : 0.0;
+        A.next_rec = T.rrec[rb ^ 1];
+        A.next_w64 = T.w64[rb ^ 1];
+        A.next_wdw = T.wrec[rb ^ 1];
+        if (ce == cudaSuccess) ce = launch_adj_step_w3(A, h->stream);
+        prepared = next != nullptr;
+        rb ^= 1;
         cb ^= 1;
-        return r;
+        return ce;
     };
     cudaError_t ke = cudaSuccess;
-    if (T.vv && dLdv) ke = reverse_step(T.fin_u, 0.0, 0.5, 1.0 + damp_full);
+    if (T.vv && dLdv) ke = reverse_step(Rev{T.fin_u, 0.0, 0.5, 1.0 + damp_full}, nullptr);
     for (int64_t k = T.nck - 1; k >= 0 && ke == cudaSuccess; --k) {
         const int64_t start = k * T.C;
         const int64_t len = std::min(T.C, T.N - start);
-        // recompute u^start .. u^{start+len-1} from checkpoint k
+        // recompute u^start .. u^{start+len-1} from checkpoint k (the step kernel writes each
+        // into the segment too; the counter is set, not advanced)
         h->step = T.step0 + start;
         ke = cudaMemcpyAsync(h->step_ctr, &h->step, sizeof(int64_t), cudaMemcpyHostToDevice,
                              h->stream);
@@ -2312,22 +2286,22 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         if (ke == cudaSuccess)
             ke = cudaMemcpyAsync(T.seg, T.ck_u + k * np3, 8 * np3, cudaMemcpyDeviceToDevice, h->stream);
         for (int64_t t = 1; t < len && ke == cudaSuccess; ++t) {
-            ke = launch_one(h, 0);
-            if (ke == cudaSuccess) ke = launch_advance(h->step_ctr, 1, h->stream);
-            h->step += 1;
-            if (ke == cudaSuccess)
-                ke = launch_extract_u(h->rec[h->step & 1], h->n_pad, T.seg + t * np3, h->stream);
+            StepArgsF64 a = args_f64(h, (int)(t - 1));
+            a.uout = T.seg + t * np3;
+            ke = launch_f64(h, a);
         }
         // reverse through the segment
-        for (int64_t t = len - 1; t >= 0 && ke == cudaSuccess; --t) {
+        auto rev = [&](int64_t t) {
             const bool half = T.vv && start + t == 0;
-            ke = reverse_step(T.seg + t * np3, h->dt, half ? 0.5 : 1.0,
-                              half ? 1.0 + damp_full : damp_full);
+            return Rev{T.seg + t * np3, h->dt, half ? 0.5 : 1.0, half ? 1.0 + damp_full : damp_full};
+        };
+        for (int64_t t = len - 1; t >= 0 && ke == cudaSuccess; --t) {
+            const Rev next = rev(std::max<int64_t>(t - 1, 0));
+            ke = reverse_step(rev(t), t > 0 ? &next : nullptr);
         }
     }
     if (ke == cudaSuccess)
-        ke = h->dw ? launch_adj_merge_dw(T.gcdw, slots, dt_rho, T.gc, h->stream)
-                   : launch_adj_merge_w3(T.gc, slots, dt_rho * h->vol0, T.wmax, h->stream);
+        ke = launch_adj_merge_w3(T.gc, slots, dt_rho * h->vol0, T.wmax, h->stream);
     h->frozen = false;
     h->drop_graph();
     // restore the final state u^N, v^N
@@ -2435,7 +2409,7 @@ pd_status pd_autotune(pd_handle* h, int32_t trial_steps, int32_t* block_threads,
     } else {
         bufs.push_back({h->rec[0], (size_t)(64 * np), {}});
         bufs.push_back({h->rec[1], (size_t)(64 * np), {}});
-        if (h->dw) {
+        if (h->dw && !h->w3) {
             bufs.push_back({h->recdw[0], (size_t)(64 * np), {}});
             bufs.push_back({h->recdw[1], (size_t)(64 * np), {}});
         }
@@ -2562,7 +2536,7 @@ pd_status pd_set_params(pd_handle* h, double c, double sc, double load, double d
             PD_CUDA(cudaMemcpyAsync(h->cbond, cb.data(), slots * 8, cudaMemcpyHostToDevice, h->stream),
                     "upload c_bond");
             if (h->dw || h->w3) {
-                float2*& dst = h->dw ? h->cbdw : h->cb3;
+                float2*& dst = h->w3 ? h->cb3 : h->cbdw;
                 if (!dst) {
                     cudaError_t e = h->alloc(&dst, slots);
                     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc c_bond");

@@ -327,6 +327,7 @@ struct StepArgsF64 {
     int32_t vv;                // 1: damped velocity-Verlet, 0: damped Euler-Cromer
     int32_t peek;              // 1: forces and full-step velocity into vout only
     double* vout;              // peek: 3 doubles per node (library order)
+    double* uout;              // three-word kernel: u^(n+1) here too (3 per node), or nullptr
     double* integ;             // bilinear softening: per-slot integrity mu, or nullptr
     double kr;                 // s_0 = s_c / kr
     double k1, beta;           // trilinear: kink at s_1 = k1 s_0 with force beta c s_0 (k1 > 1)
@@ -485,39 +486,22 @@ struct AdjArgs {
     int64_t n;
 };
 
-// Reverse step of PD_PREC_DW handles (pd_adjoint_dw.cu): double-word records
-// of u^n and w for the neighbours, FP64 node outputs
-struct AdjDwArgs {
-    const float4* rec;         // 4 float4 per node: positions, u^n / delta, V
-    const float4* wrec;        // 2 float4 per node: w
-    const float2* len;         // per slot |xi| / delta
-    const float2* cb;          // per slot c_ij, or nullptr for the constant c
-    float2 c;                  // the constant c as a double-word
-    float2* gc;                // per slot dL/dc accumulator, without dt/rho
-    const double* w;           // w (FP64)
-    const double* ubm;         // ubar of step n+1, controlled components zeroed
-    double* ub_out;            // ubar^n
-    double* vb_out;            // vbar^n
-    double* gl;                // per-node accumulator of force . w
-    const int32_t* nbr;
-    const uint32_t* bits;      // frozen bond flags
-    const int32_t* sw;
-    int32_t Q;
-    int32_t uniform_w;         // 1: every node has volume vol0
-    int64_t n;
-    const uint8_t* bcc;
-    const BcClass* bct;
-    double dt_rho, damp, inv_delta, vol0;
-};
-
-// Reverse step of bond-based FP64 handles (pd_adjoint_w3.cu)
+// Reverse step (pd_adjoint_w3.cu)
 struct AdjW3Args {
     const double* x64;         // the FP64 step records (8 doubles per node, positions first)
     const double* un;          // u^n, the state the forward step n -> n+1 read
+    const float4* fwd;         // the forward step's three-word records (positions)
     float4* rec;               // 4 float4 per node: three-word record of x and u^n
     double* w64;               // 4 doubles per node: w, 0
     float4* wdw;               // 2 float4 per node: w as double-words, scaled
+    const double* ub;          // ubar, vbar of step n+1
+    const double* vb;
     double* ubm;               // ubar of step n+1, controlled components zeroed
+    const double* next_un;     // u^(n-1), whose step's records this one writes, or nullptr
+    double next_dt, next_ws;
+    float4* next_rec;
+    double* next_w64;
+    float4* next_wdw;
     const unsigned long long* wmax;  // bits of the seeds' largest component (sets the scale)
     double* ub_out;            // ubar^n
     double* vb_out;            // vbar^n
@@ -552,20 +536,11 @@ cudaError_t launch_adj_scale_w3(const double* ub, const double* vb, int64_t n3, 
                                 unsigned long long* wmax, cudaStream_t s);
 cudaError_t launch_adj_e(const double* x64, const int32_t* nbr, int64_t n_slices, int Q, double* e,
                          cudaStream_t s);
-cudaError_t launch_adj_step_w3(const AdjW3Args& a, const double* ub, const double* vb,
-                               const float4* fwd, double dt, double ws, int64_t n_pad,
+cudaError_t launch_adj_prep_w3(const AdjW3Args& a, double dt, double ws, int64_t n_pad,
                                cudaStream_t s);
+cudaError_t launch_adj_step_w3(const AdjW3Args& a, cudaStream_t s);
 cudaError_t launch_adj_merge_w3(double* gc, int64_t count, double scale,
                                 const unsigned long long* wmax, cudaStream_t s);
-
-cudaError_t launch_adj_mask_publish_dw(const double* ub, const double* vb, const uint8_t* bcc,
-                                       const BcClass* bct, double dt, double ws,
-                                       const float4* fwd, const double* un, const double* vol,
-                                       int64_t n_pad, double inv_delta, double* ubm, double* w,
-                                       float4* rec, float4* wrec, cudaStream_t s);
-cudaError_t launch_adj_step_dw(const AdjDwArgs& a, int grid, int block, cudaStream_t s);
-cudaError_t launch_adj_merge_dw(const float2* acc, int64_t count, double scale, double* gc,
-                                cudaStream_t s);
 
 cudaError_t launch_adj_mask(const double* ub, const double* vb, const uint8_t* bcc,
                             const BcClass* bct, int64_t n, double dt, double ws, double* ubm,
@@ -637,7 +612,7 @@ cudaError_t launch_w3_ilen(const double* ilen, const int32_t* nbr, const int32_t
                            float4* il, cudaStream_t s);
 cudaError_t launch_step_dw(const StepArgsF64& a, const DwArgs& d, int sc_mode, int grid, int block,
                            cudaStream_t s);
-const void* step_dw_kernel(int sc_mode, bool uniform_w, bool soft, bool vv);
+const void* step_dw_kernel(int sc_mode, bool uniform_w, bool vv);
 // double-word records from the FP64 records (positions relative to origin[3])
 cudaError_t launch_dw_publish(const double* rec64, float4* rec, int64_t n_pad, const double* origin,
                               double inv_delta, cudaStream_t s);

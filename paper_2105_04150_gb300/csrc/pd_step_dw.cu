@@ -147,7 +147,7 @@ __device__ __forceinline__ void add_force(Dw (&F)[3], const BondDw& b, bool ok)
 // A bond whose leading stretch word reached the band below the smallest s_c:
 // recomputed with the same arithmetic and decided in FP64 against its s_c,
 // then the no-fail rule.
-template <int SCM, bool UW, bool SOFT>
+template <int SCM, bool UW>
 __device__ __noinline__ BondDw resolve_dw(const StepArgsF64& a, const DwArgs& d, int cur,
                                           int64_t i, int64_t j, int64_t slot, bool* broken,
                                           double* mu_out)
@@ -172,7 +172,7 @@ __device__ __noinline__ BondDw resolve_dw(const StepArgsF64& a, const DwArgs& d,
     if (brk && a.has_nofail) brk = ((a.bct[a.bcc[i]].mask | a.bct[a.bcc[j]].mask) & 8u) == 0u;
     *broken = brk;
     double mu = 1.0;
-    if (SOFT) {
+    {
         // the integrity only decreases, as the stretch passes s_0 = s_c / kr (a
         // no-fail bond past s_c keeps 0); the force is scaled by it
         if (brk) {
@@ -208,7 +208,7 @@ __device__ __forceinline__ double soften(BondDw& b, const double* integ, int64_t
     return mu - 1.0;
 }
 
-template <int SCM, bool UW, bool SOFT>
+template <int SCM, bool UW>
 __global__ void __launch_bounds__(256, PD_DW_MIN_BLOCKS)
     k_step_dw(const __grid_constant__ StepArgsF64 a, const __grid_constant__ DwArgs d)
 {
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256, PD_DW_MIN_BLOCKS)
         // batch: both ends of a bond belong to the same instance)
         const float fast_lo = a.inst != nullptr
                                   ? (float)((1.0 - 0x1.0p-20) * a.itab[a.inst[i]].sc_lo /
-                                            (SOFT ? a.kr : 1.0))
+                                            a.kr)
                                   : d.fast_lo;
         // force sums of the A and B halves, and (non-uniform weights) the sum of
         // w_j over intact bonds
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(256, PD_DW_MIN_BLOCKS)
             }
             const bool candA = bA.s.h >= fast_lo, candB = bB.s.h >= fast_lo;
             const bool okA = (wb & 1u) && !candA, okB = ((wb >> 1) & 1u) && !candB;
-            if (SOFT) {
+            {
                 const double dA = soften(bA, a.integ, (g * W + m0) * 32 + lane);
                 const double dB = soften(bB, a.integ, (g * W + m0 + 1) * 32 + lane);
                 if (okA && dA != 0.0)
@@ -315,19 +315,19 @@ __global__ void __launch_bounds__(256, PD_DW_MIN_BLOCKS)
                     const int64_t j = col[(int64_t)(q * 32 + b) * 32];
                     bool broken;
                     double mu;
-                    const BondDw f = resolve_dw<SCM, UW, SOFT>(a, d, cur, i, j, slot, &broken, &mu);
+                    const BondDw f = resolve_dw<SCM, UW>(a, d, cur, i, j, slot, &broken, &mu);
                     if (broken) {
                         nword &= ~(1u << b);
                     } else {
                         add_force(F, f, true);
                         float4 c0, c1;
-                        if (!UW || (SOFT && mu != 1.0)) ld_rec(R + 4 * j, c0, c1);
+                        if (!UW || mu != 1.0) ld_rec(R + 4 * j, c0, c1);
                         if (!UW) {
                             const Dw t = two_sum(ws.h, c1.z);
                             ws.h = t.h;
                             ws.l += t.l + c1.w;
                         }
-                        if (SOFT && mu != 1.0)
+                        if (mu != 1.0)
                             wsoft += (mu - 1.0) * (UW ? 1.0 : (double)c1.z + (double)c1.w);
                     }
                 }
@@ -485,32 +485,28 @@ int grid_of(int64_t work)
 #else
 #define PD_DW_KERNELS step_dw_kernels_ec
 #endif
-// the kernel variants of this build: [sc_mode][uniform weights][softening]
-const void* PD_DW_KERNELS(int sc_mode, bool uniform_w, bool soft)
+// the kernel variants of this build: [sc_mode][uniform weights]
+const void* PD_DW_KERNELS(int sc_mode, bool uniform_w)
 {
-    static const void* const k[8] = {
-        (const void*)k_step_dw<0, false, false>, (const void*)k_step_dw<0, false, true>,
-        (const void*)k_step_dw<0, true, false>,  (const void*)k_step_dw<0, true, true>,
-        (const void*)k_step_dw<1, false, false>, (const void*)k_step_dw<1, false, true>,
-        (const void*)k_step_dw<1, true, false>,  (const void*)k_step_dw<1, true, true>};
-    return k[(sc_mode ? 4 : 0) + (uniform_w ? 2 : 0) + (soft ? 1 : 0)];
+    static const void* const k[4] = {
+        (const void*)k_step_dw<0, false>, (const void*)k_step_dw<0, true>,
+        (const void*)k_step_dw<1, false>, (const void*)k_step_dw<1, true>};
+    return k[(sc_mode ? 2 : 0) + (uniform_w ? 1 : 0)];
 }
 #undef PD_DW_KERNELS
 
 #if !PD_DW_VV
-const void* step_dw_kernels_vv(int sc_mode, bool uniform_w, bool soft);
+const void* step_dw_kernels_vv(int sc_mode, bool uniform_w);
 
-const void* step_dw_kernel(int sc_mode, bool uniform_w, bool soft, bool vv)
+const void* step_dw_kernel(int sc_mode, bool uniform_w, bool vv)
 {
-    return vv ? step_dw_kernels_vv(sc_mode, uniform_w, soft)
-              : step_dw_kernels_ec(sc_mode, uniform_w, soft);
+    return vv ? step_dw_kernels_vv(sc_mode, uniform_w) : step_dw_kernels_ec(sc_mode, uniform_w);
 }
 
 cudaError_t launch_step_dw(const StepArgsF64& a, const DwArgs& d, int sc_mode, int grid, int block,
                            cudaStream_t s)
 {
-    const void* fn = step_dw_kernel(sc_mode, d.uniform_w != 0, a.integ != nullptr,
-                                    a.vv != 0 || a.peek != 0);
+    const void* fn = step_dw_kernel(sc_mode, d.uniform_w != 0, a.vv != 0 || a.peek != 0);
     void* args[] = {const_cast<StepArgsF64*>(&a), const_cast<DwArgs*>(&d)};
     return launch_pdl(fn, dim3(grid), dim3(block), args, 0, s);
 }

@@ -335,6 +335,8 @@ __device__ __forceinline__ void finish_node(const StepArgsF64& a, const W3Args& 
     if (a.peek) return;
     rout[4 * i + 2] = make_double2(un[0], un[1]);  // (positions and weights: in both buffers)
     rout[4 * i + 3] = make_double2(un[2], 0.0);
+    if (a.uout != nullptr)  // the adjoint's recomputed segment
+        for (int c = 0; c < 3; ++c) a.uout[3 * i + c] = un[c];
     dwa::st_rec(Rout + 4 * i, make_float4(me.a0.x, me.a0.y, uh[0], uh[1]),
                 make_float4(me.a1.x, uh[2], tw[0], tw[1]));
     dwa::st_rec(Rout + 4 * i + 2, make_float4(me.b0.x, me.b0.y, um[0], um[1]),
