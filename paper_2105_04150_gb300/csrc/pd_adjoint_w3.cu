@@ -15,7 +15,8 @@
 //   A = xi.d, B = eta.d,
 //
 // e is a constant of the slot, stored (24 bytes streamed cost less than the five
-// operations that form it: 0.34 ms a step with xi and 1 / L^3).  The second line is smaller than the first by |eta| / L, 1e-4 to 1e-2, so the
+// operations that form it: 0.34 ms a step of the 100k plate with xi and 1 / L^3; 0.32 now,
+// the FP64 pipe 60 % busy).  The second line is smaller than the first by |eta| / L, 1e-4 to 1e-2, so the
 // double-word arithmetic of pd_w3.h (relative 1e-14) gives it to FP64's rounding
 // of the whole; it runs on the FP32 pipe beside the FP64 one.  dL/dc needs the
 // stretch, which is more accurate in double-words than in the literal FP64 form
@@ -187,31 +188,46 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
 
     double acc[3] = {0.0, 0.0, 0.0};
     Dw cor[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-    uint32_t word = 0u;
-    int32_t jn = rank < Wg ? __ldg(col + rank * 32) : 0;
-    for (int b = rank; b < Wg; b += kTeam) {
-        if ((b & 31) < kTeam) word = a.bits[(g * Q + (b >> 5)) * 32 + lane];
-        const int64_t j = jn;
-        if (b + kTeam < Wg) jn = __ldg(col + (b + kTeam) * 32);
-        if (!((word >> (b & 31)) & 1u)) continue;
-        const int64_t slot = slot0 + b * 32;
+    // Software-pipelined as the forward walk: a bond's loads go out when the previous one's
+    // words are consumed.
+    struct In {
         Rec nb;
-        dwa::ld_rec(a.rec + 4 * j, nb.a0, nb.a1);
-        dwa::ld_rec(a.rec + 4 * j + 2, nb.b0, nb.b1);
-        const D4 wj = ld_d4(a.w64 + 4 * j);
+        D4 wj;
         float4 v0, v1;
-        dwa::ld_rec(a.wdw + 2 * j, v0, v1);
-        const float4 il2 = __ldg(a.il + (slot - lane) / 64 * 32 + lane);
-        const float2 il = b & 1 ? make_float2(il2.y, il2.w) : make_float2(il2.x, il2.z);
-        // e is kept by rows of 32 lanes: x, y, z of slot b of the slice
-        const double* ep = a.e + 3 * (slot - lane) + lane;
-        const double e0 = __ldg(ep), e1 = __ldg(ep + 32), e2 = __ldg(ep + 64);
-        const float2 old = a.gc[slot];
+        float4 il2;
+        double e0, e1, e2;
+        float2 gc;
+    } in;
+    auto load = [&](int b, int64_t j) {
+        const int64_t row = g * 32LL * Q + b;  // of 32 slots
+        dwa::ld_rec(a.rec + 4 * j, in.nb.a0, in.nb.a1);
+        dwa::ld_rec(a.rec + 4 * j + 2, in.nb.b0, in.nb.b1);
+        dwa::ld_rec(a.wdw + 2 * j, in.v0, in.v1);
+        in.wj = ld_d4(a.w64 + 4 * j);
+        in.il2 = __ldg(a.il + (row >> 1) * 32 + lane);
+        const double* ep = a.e + row * 96 + lane;  // x, y, z rows
+        in.e0 = __ldg(ep);
+        in.e1 = __ldg(ep + 32);
+        in.e2 = __ldg(ep + 64);
+        in.gc = a.gc[row * 32 + lane];
+    };
+    uint32_t word = 0u;
+    int32_t jc = 0, jn = 0;
+    if (rank < Wg) {
+        jc = __ldg(col + rank * 32);
+        if (rank + kTeam < Wg) jn = __ldg(col + (rank + kTeam) * 32);
+        load(rank, jc);
+        word = a.bits[g * Q * 32 + lane];
+    }
+    for (int b = rank; b < Wg; b += kTeam) {
+        const bool alive = (word >> (b & 31)) & 1u;
+        const int64_t j = jc, slot = slot0 + b * 32;
+        const float2 il = b & 1 ? make_float2(in.il2.y, in.il2.w) : make_float2(in.il2.x, in.il2.z);
+        const float2 old = in.gc;
         float2 rj = make_float2(1.0f, 0.0f);
         if (!UW) rj = __ldg(a.wrel + j);
-
-        const Geo geo = bond_geo(own, nb, il, ts);
-        const Dw wn[3] = {{v0.x, v0.w}, {v0.y, v1.x}, {v0.z, v1.y}};
+        const Geo geo = bond_geo(own, in.nb, il, ts);
+        const Dw wn[3] = {{in.v0.x, in.v0.w}, {in.v0.y, in.v1.x}, {in.v0.z, in.v1.y}};
         Dw d[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -223,10 +239,31 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
                 d[k] = dw_add(p, Dw{-q.h, -q.l});
             }
         }
+        // the undeformed part in FP64
+        double d0, d1, d2;
+        if (UW) {
+            d0 = in.wj.x - wm.x;
+            d1 = in.wj.y - wm.y;
+            d2 = in.wj.z - wm.z;
+        } else {
+            const double vj = (double)rj.x + (double)rj.y;
+            d0 = vm * in.wj.x - vj * wm.x;
+            d1 = vm * in.wj.y - vj * wm.y;
+            d2 = vm * in.wj.z - vj * wm.z;
+        }
+        const double e0 = in.e0, e1 = in.e1, e2 = in.e2;
+        double ed = fma(e0, d0, fma(e1, d1, e2 * d2));
+        if (b + kTeam < Wg) {
+            load(b + kTeam, jn);
+            jc = jn;
+            if (((b + kTeam) & 31) < kTeam) word = a.bits[(g * Q + ((b + kTeam) >> 5)) * 32 + lane];
+            if (b + 2 * kTeam < Wg) jn = __ldg(col + (b + 2 * kTeam) * 32);
+        }
         const Dw A = dot3(geo.xi, d), B = dot3(geo.et, d);
         const Dw AB = dw_add(A, B);
         const float eta = fmaxf(fmaxf(fabsf(geo.et[0].h), fabsf(geo.et[1].h)), fabsf(geo.et[2].h));
         const bool ok = fabsf(geo.x.h) < kW3XMax && eta * il.x < 0x1.0p-6f && fabsf(AB.h) < 1e30f;
+        if (!alive) continue;
         Dw gs;  // the bond's dL/dc in units of V_ref / unit_scale
         if (ok) {
             const Dw iL{il.x, il.y};
@@ -244,13 +281,15 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             gs = dw_mul(zL, yw);
             if (!UW) gs = dw_mul(gs, Dw{rj.x, rj.y});
             gs = Dw{-gs.h, -gs.l};
-            double cij = 1.0;
             if (a.cbond != nullptr) {  // per-bond stiffness (a uniform branch)
                 const float2 cv = __ldg(a.cb + slot);
                 i3 = dw_mul(i3, Dw{cv.x, cv.y});
                 zc = dw_mul(zc, Dw{cv.x, cv.y});
-                cij = __ldg(a.cbond + slot);
+                ed *= __ldg(a.cbond + slot);
             }
+            acc[0] = fma(ed, e0, acc[0]);
+            acc[1] = fma(ed, e1, acc[1]);
+            acc[2] = fma(ed, e2, acc[2]);
             const Dw al = dw_mul(dw_add(B, qAB), i3), be = dw_mul(dw_add(AB, qAB), i3);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
@@ -259,23 +298,6 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
                                     Dw{-zd.h, -zd.l});
                 cor[k] = dw_add(cor[k], f);
             }
-            // the undeformed part in FP64
-            double d0, d1, d2;
-            if (UW) {
-                d0 = wj.x - wm.x;
-                d1 = wj.y - wm.y;
-                d2 = wj.z - wm.z;
-            } else {
-                const double vj = (double)rj.x + (double)rj.y;
-                d0 = vm * wj.x - vj * wm.x;
-                d1 = vm * wj.y - vj * wm.y;
-                d2 = vm * wj.z - vj * wm.z;
-            }
-            double k = fma(e0, d0, fma(e1, d1, e2 * d2));
-            if (a.cbond != nullptr) k *= cij;
-            acc[0] = fma(k, e0, acc[0]);
-            acc[1] = fma(k, e1, acc[1]);
-            acc[2] = fma(k, e2, acc[2]);
         } else {
             double f[3];
             const double gd = literal_adj(a, m, j, slot, f) * us;

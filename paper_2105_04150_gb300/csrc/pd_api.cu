@@ -2297,7 +2297,9 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         };
         for (int64_t t = len - 1; t >= 0 && ke == cudaSuccess; --t) {
             const Rev next = rev(std::max<int64_t>(t - 1, 0));
-            ke = reverse_step(rev(t), t > 0 ? &next : nullptr);
+            // (one warp of each block does it: a kernel of its own costs less once the blocks
+            // fill the chip several times)
+            ke = reverse_step(rev(t), t > 0 && h->n_slices <= 1216 ? &next : nullptr);
         }
     }
     if (ke == cudaSuccess)
