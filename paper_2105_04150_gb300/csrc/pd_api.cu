@@ -722,10 +722,11 @@ pd_status choose_grid(pd_handle* h, int blocks_per_sm)
     }
     const void* fn = step_kernel_fn(h);
     const size_t smem = h->w3 ? step_f64_smem(h->team, h->Q * (32 / kW3Seg), h->block) : 0;
-    // no shared memory, or that of two resident blocks: the rest of the unified
-    // L1/shared array (228 KB) goes to L1
+    // no shared memory, or that of 16 resident warps: the rest of the unified L1/shared
+    // array (228 KB) goes to L1
+    const size_t resident = (size_t)(512 / h->block) * (smem + 1024);
     PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 smem ? (int)std::min<size_t>(100, 1 + 200 * (smem + 1024) / (228 << 10))
+                                 smem ? (int)std::min<size_t>(100, 1 + 100 * resident / (228 << 10))
                                       : 0),
             "carveout");
     if (smem)
