@@ -1,13 +1,15 @@
-// Double-word arithmetic for the FP64-grade kernels (pd_step_dw.cu,
-// pd_adjoint_dw.cu), device code only.
+// Double-word arithmetic for the FP64-grade kernels (pd_step_f64.cu, pd_adjoint_w3.cu,
+// pd_step_dw.cu, pd_step_osb_dw.cu), device code only.
 //
 // A double-word is an unevaluated sum h + l of two FP32 numbers (Dekker 1971;
 // Knuth's two-sum; the products and error bounds of Joldes, Muller & Popescu,
 // ACM TOMS 2017), about 48 significant bits.  The operations below leave their
 // result unnormalised (|l| up to a few ulp(h)) wherever the next operation
 // takes that, which keeps ~46-bit accuracy for far fewer FP32 operations than
-// renormalising after each step.  GB300's FP32 pipe is the limit of these
-// kernels, so the code is scalar: negated operands cost nothing.
+// renormalising after each step.  Products and sums whose rounding error is taken
+// later are written with the _rn intrinsics, which the compiler does not contract: in
+// s = a b + c, bb = s - a b a fused form of the second would count the product's
+// rounding error twice, and the result would have 2^-25 of it.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -51,9 +53,9 @@ struct Dw {
 // exact sum (Knuth)
 __device__ __forceinline__ Dw two_sum(float a, float b)
 {
-    const float s = a + b;
-    const float bb = s - a;
-    return {s, (a - (s - bb)) + (b - bb)};
+    const float s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
 }
 
 // a + b: the leading words summed exactly, everything else in FP32
@@ -68,7 +70,7 @@ __device__ __forceinline__ Dw dw_add(Dw a, Dw b)
 // (Joldes, Muller & Popescu's DWTimesDW without the final renormalisation)
 __device__ __forceinline__ Dw dw_mul(Dw a, Dw b)
 {
-    const float p = a.h * b.h;
+    const float p = __fmul_rn(a.h, b.h);
     return {p, fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p)))};
 }
 
@@ -79,7 +81,7 @@ __device__ __forceinline__ void dw_norm(Dw y2, Dw& r, Dw& ir)
 {
     float r0 = rsqrt_seed(y2.h);
     r0 = r0 * fmaf(-(0.5f * y2.h) * r0, r0, 1.5f);
-    const float rh = y2.h * r0;
+    const float rh = __fmul_rn(y2.h, r0);
     r = Dw{rh, (fmaf(-rh, rh, y2.h) + y2.l) * r0 * 0.5f};
     ir = Dw{r0, r0 * fmaf(-r.l, r0, fmaf(-r.h, r0, 1.0f))};
 }
@@ -91,7 +93,7 @@ __device__ __forceinline__ Dw dw_div(Dw num, Dw den)
     float q = rcp_seed(den.h);
     q = fmaf(q, fmaf(-den.h, q, 1.0f), q);
     const float q0 = num.h * q;
-    const float ph = den.h * q0;
+    const float ph = __fmul_rn(den.h, q0);
     const float pl = fmaf(den.l, q0, fmaf(den.h, q0, -ph));
     return Dw{q0, (((num.h - ph) - pl) + num.l) * q};
 }

@@ -48,7 +48,7 @@ using dwa::two_sum;
 // Bonds with |x| = ||y|^2 / |xi|^2 - 1| past kW3XMax (a stretch of 0.78 %) are left
 // to the literal FP64 evaluation of Eq. 4, which has the smaller error there: its
 // stretch carries an absolute rounding error of about 3e-16, i.e. 3e-16 / s of the
-// bond's force, against the 1e-14 of bond_w3.
+// bond's force, against the 1e-14 of the form below.
 
 struct Own {
     float xh[3], xm[3], xk[3], uh[3], um[3], ut[3];
@@ -155,10 +155,10 @@ __device__ __forceinline__ Geo bond_geo(const Own& o, const Rec& j, const float2
     const float r = x1 * dwa::rsqrt_seed(x1);
     const float z0 = -x.h * dwa::rcp_seed(fmaf(r, r, r));
     // p = 2 z0 + z0^2 as a double-word
-    const float zz = z0 * z0, ph = fmaf(2.0f, z0, zz);
+    const float zz = __fmul_rn(z0, z0), ph = fmaf(2.0f, z0, zz);
     const Dw p{ph, (zz - fmaf(-2.0f, z0, ph)) + fmaf(z0, z0, -zz)};
     const Dw xp = dw_mul(x, p);
-    const float R = ((ph + x.h) + xp.h) + ((p.l + x.l) + xp.l);
+    const float R = __fadd_rn(__fadd_rn(ph, x.h), xp.h) + ((p.l + x.l) + xp.l);
     out.x = x;
     out.z = Dw{z0, R * fmaf(z0, -0.5f, -0.5f)};
     return out;
