@@ -721,16 +721,17 @@ pd_status choose_grid(pd_handle* h, int blocks_per_sm)
         return PD_OK;
     }
     const void* fn = step_kernel_fn(h);
-    const size_t smem = h->w3 ? step_f64_smem(h->team, h->Q * (32 / kW3Seg), h->block) : 0;
-    // no shared memory, or that of 16 resident warps: the rest of the unified L1/shared
-    // array (228 KB) goes to L1
-    const size_t resident = (size_t)(512 / h->block) * (smem + 1024);
+    // Kernels without shared memory leave the unified L1/shared array to L1.  The FP64 step's
+    // carveout is this handle's, for the occupancy below and given with every launch; its
+    // limit is the same for all handles, which share the function.
+    const int max_seg = h->Q * (32 / kW3Seg);
+    const size_t smem = h->w3 ? step_f64_smem(h->team, max_seg, h->block) : 0;
     PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 smem ? (int)std::min<size_t>(100, 1 + 100 * resident / (228 << 10))
-                                      : 0),
+                                 h->w3 ? step_f64_carveout(h->team, max_seg, h->block) : 0),
             "carveout");
-    if (smem)
-        PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+    if (h->w3 && h->team > 1)
+        PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)step_f64_smem_max()),
                 "shared memory size");
     int occ = 0;
     PD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, h->block, smem), "occupancy");

@@ -44,22 +44,26 @@
 namespace pd {
 
 // Programmatic dependent launch: a kernel launched with launch_pdl starts while its
-// predecessor in the stream runs (once all of that one's blocks have let it), and reads what the predecessor writes only after pdl_begin, which
-// waits for its completion.  It hides the launch latency and the kernel's first instruction,
-// constant and static-array misses.
+// predecessor in the stream runs (once all of that one's blocks have let it), and reads
+// what the predecessor writes only after pdl_begin, which waits for its completion.  It
+// hides the launch latency and the kernel's first instruction, constant and static-array
+// misses.  `carveout` (percent, -1: the function's) is the launch's own split of the
+// L1/shared array: a function's attribute is shared by every handle that launches it.
 inline cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, void** args, size_t smem,
-                              cudaStream_t s)
+                              cudaStream_t s, int carveout = -1)
 {
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[1].val.sharedMemCarveout = (unsigned)(carveout < 0 ? 0 : carveout);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = carveout < 0 ? 1 : 2;
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 #ifdef __CUDACC__
@@ -603,6 +607,8 @@ cudaError_t launch_step_f64_soft(const StepArgsF64& a, int grid, int block, cuda
 const void* step_f64_soft_kernel(int sc_mode);
 // dynamic shared memory of a block of the FP64 step
 size_t step_f64_smem(int team, int max_seg, int block);
+size_t step_f64_smem_max();  // over every team, family and block size
+int step_f64_carveout(int team, int max_seg, int block);
 // three-word records of every node from its FP64 record, and U / |xi| of every slot
 cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, double scale,
                               int x_grid, const int32_t* inst, const InstParams* itab,

@@ -26,6 +26,8 @@
 // added up in segment order, so the result does not depend on which warp walks
 // which segment.  A model with few slices gives each slice to a team of warps
 // (TEAM), which take its segments in turn and add their sums through shared memory.
+#include <algorithm>
+
 #include <cuda_runtime.h>
 
 #include "pd_internal.h"
@@ -505,6 +507,16 @@ size_t step_f64_smem(int team, int max_seg, int block)
     return (size_t)(block / 32 / team) * (team > 1 ? max_seg : 1) * sizeof(Sums);
 }
 
+size_t step_f64_smem_max() { return step_f64_smem(2, kW3TeamSegs, 256); }
+
+// Percent of the unified L1/shared array (228 KB) that the sums of 16 resident warps
+// take; the rest is the records' L1.
+int step_f64_carveout(int team, int max_seg, int block)
+{
+    const size_t resident = (size_t)(512 / block) * (step_f64_smem(team, max_seg, block) + 1024);
+    return (int)std::min<size_t>(100, 1 + 100 * resident / (228 << 10));
+}
+
 const void* step_f64_kernel(bool uniform_w, bool team)
 {
     static const void* const k[4] = {
@@ -518,7 +530,8 @@ cudaError_t launch_step_f64(const StepArgsF64& a, const W3Args& d, int grid, int
 {
     const void* fn = step_f64_kernel(d.uniform_w != 0, d.team > 1);
     void* args[] = {const_cast<StepArgsF64*>(&a), const_cast<W3Args*>(&d)};
-    return launch_pdl(fn, dim3(grid), dim3(block), args, step_f64_smem(d.team, d.max_seg, block), s);
+    return launch_pdl(fn, dim3(grid), dim3(block), args, step_f64_smem(d.team, d.max_seg, block), s,
+                      step_f64_carveout(d.team, d.max_seg, block));
 }
 
 cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, double scale,

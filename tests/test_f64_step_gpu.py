@@ -144,3 +144,53 @@ def test_reverse_step_against_oracle(n_shape, jitter, per_bond, strain, angle, s
     assert np.abs(gv0 - gv_o).max() <= 8 * 2.0 ** -53 * np.abs(gv_o).max()
     tolc = dr * w.volumes[idx] * wa[rows] * (8 * 2.0 ** -53 + (2.0 ** -44 + 16 * 2.0 ** -53) * s)
     assert (np.abs(gc - gc_o) <= tolc).all()
+
+
+def test_handles_that_share_a_kernel_do_not_disturb_each_other():
+    # the step's shared memory depends on the model (104 KB a block for families of 256
+    # with two warps per slice, 13 KB for the small bar): a handle keeps stepping after one
+    # with other needs was made
+    big = _body((32, 30, 30), 0.1, 2, 0.0, 3.8)
+    small = _body((12, 8, 8), 0.1, 2, 0.0, 3.01)
+    out = []
+    for between in (False, True):
+        m = pdgb.Model.from_workload(big, precision=pdgb.PD_PREC_F64)
+        u = 1e-5 * (big.coords - big.coords.mean(0)) ** 2 / big.dx
+        m.set_state(u, np.zeros_like(u), 0)
+        m.step(2)
+        if between:
+            k = pdgb.Model.from_workload(small, precision=pdgb.PD_PREC_F64)
+            k.step(2)
+        m.step(3)
+        if between:
+            k.step(2)
+            assert np.isfinite(k.state()[0]).all()
+            k.close()
+        out.append(m.state())
+        m.close()
+    assert np.abs(out[0][0]).max() > 0
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("jitter", [0.0, 0.2])
+@pytest.mark.parametrize("vv", [False, True])
+def test_pmb_forms_of_both_precisions_take_the_same_step(jitter, vv):
+    # PD_PREC_F64 and PD_PREC_DW without softening, and with kr = 1 (the PMB law), run the
+    # same kernel: the same bits, bonds that break included
+    out = []
+    for prec in (pdgb.PD_PREC_F64, pdgb.PD_PREC_DW):
+        for kr in (0.0, 1.0):
+            w = _body((13, 9, 8), jitter, 6, 0.0, 3.01)
+            w.sc, w.kr = 1.2e-4, kr
+            rng = np.random.default_rng(2)
+            u = 1e-4 * (w.coords - w.coords.mean(0)) + rng.uniform(-1, 1, (w.n, 3)) * 2e-5 * w.dx
+            kw = dict(integrator=pdgb.PD_INTEGRATOR_VV) if vv else {}
+            m = pdgb.Model.from_workload(w, precision=prec, **kw)
+            m.set_state(u, np.zeros((w.n, 3)), 0)
+            m.step(6)
+            out.append((*m.state(), m.bonds(), m.damage()))
+            m.close()
+    assert 0 < (out[0][2] == 0).sum() < out[0][2].size
+    for o in out[1:]:
+        for a, b in zip(out[0], o):
+            assert np.array_equal(a, b)
