@@ -44,13 +44,13 @@ import workloads  # noqa: E402
 # velocity 12 B read + 12 B written, damage 4 B written, BC class 1 B.
 BYTES_PER_BOND = 4.125
 BYTES_PER_NODE = {32: 93.0, 64: 136.0}
-# The FP64 step is bound by GB300's FP64 arithmetic, not by HBM.  Algorithmic
-# FP64 work per bond (Eqs. 4-5 as written): xi, eta, y (9), |xi|^2 and |y|^2
-# (10), two square roots and the stretch's division (3), c V s / |y| (3), the
+# Algorithmic FP64 work per bond (Eqs. 4-5 as written): xi, eta, y (9), |xi|^2 and
+# |y|^2 (10), two square roots and the stretch's division (3), c V s / |y| (3), the
 # force accumulation (6 as 3 fused multiply-adds) = 31 flops, counting a square
-# root or a division as one.  Peak: FP64 fused multiply-add throughput measured
-# on a GB300 of this pool with a plain dependent-chain probe, 1.20 TFLOP/s
-# (nominal 1.25).
+# root or a division as one.  The softening and state-based FP64 steps evaluate it
+# literally and are bound by GB300's FP64 pipe.  Peak: FP64 fused multiply-add
+# throughput measured on a GB300 of this machine with a plain dependent-chain probe,
+# 1.20 TFLOP/s (nominal 1.25).
 FP64_FLOPS_PER_BOND = 31.0
 FP64_PEAK_TFLOPS = 1.20
 # Ordinary state-based step, both loops: the dilation loop (xi, eta, y 9; |y|^2
@@ -58,18 +58,27 @@ FP64_PEAK_TFLOPS = 1.20
 # 5; root 1; e 1; t_ij 5; t_ji 8; the sum, V / |y| 3; accumulation 6 = 38):
 # 57 flops per bond.
 OSB_FLOPS_PER_BOND = 57.0
-# The double-word step (precision 48) is bound by the FP32 pipe.  FP32
-# operations per bond of its arithmetic (pd_step_dw.cu, uniform weights; an add,
-# multiply or fused multiply-add each counted once): xi 2, eta 8, y 8 and
-# 2 xi + eta 8 and their product 4 per component (90); the sum num 16; L^2 and
-# |y|^2 12; the refined 1/|y| seed 4, |y| 5, 1/|y| 3; den 12; the quotient 10;
-# s / |y| 4; the force term and its double-word accumulation 12 per component
-# (36) = 192, plus two hardware reciprocal(-square-root) seeds.  Peak: FP32 FMA
-# lane rate measured by a probe on this machine's GB300, 35.1 T/s (70.2 TFLOP/s
-# counting an FMA as two).
+# The bond-based step of FP64 and double-word models without softening is bound by the
+# FP32 pipe.  FP32 operations per bond of its double-word arithmetic (pd_w3.h,
+# pd_step_f64.cu, uniform weights; an add, multiply or fused multiply-add each counted
+# once, a paired instruction as two): xi and eta 7, y 8, 2 xi + eta 8 and their product
+# 4 per component (102); the sum num 16; x 8, the seed of z 7, its residual 13 and
+# z / |xi| 6; the force term and its double-word accumulation 12 per component (36)
+# = 188, plus two hardware reciprocal(-square-root) seeds.
+W3_FP32_OPS_PER_BOND = 188.0
+W3_FP32_OPS_PER_BOND_NODE_W = W3_FP32_OPS_PER_BOND + 4.0  # the coefficient times w_j
+# per node: the three-word record 64 B read + 64 B written, u of the FP64 record 32 + 32,
+# FP64 velocity 24 + 24, intact damage 8, family size 4, damage 8, BC class 1; per bond
+# 8 B of U / |xi|
+W3_BYTES_PER_NODE = 261.0
+W3_BYTES_PER_BOND = BYTES_PER_BOND + 8.0
+# The double-word softening step (precision 48, pd_step_dw.cu, uniform weights): xi 2,
+# eta 8, y 8 and 2 xi + eta 8 and their product 4 per component (90); the sum num 16;
+# L^2 and |y|^2 12; the refined 1/|y| seed 4, |y| 5, 1/|y| 3; den 12; the quotient 10;
+# s / |y| 4; the force term and its double-word accumulation 12 per component (36)
+# = 192, plus two seeds.  Peak: FP32 FMA lane rate measured by a probe on this machine's
+# GB300, 35.1 T/s (70.2 TFLOP/s counting an FMA as two).
 DW_FP32_OPS_PER_BOND = 192.0
-# per-node weights (batches): the coefficient times w_j (4) and the weight sum (8)
-DW_FP32_OPS_PER_BOND_NODE_W = DW_FP32_OPS_PER_BOND + 12.0
 # double-word state-based step (pd_step_osb_dw.cu), both loops: the bond's
 # stretch, y and 1/|y| (152) in each; the dilation term and its sum (20); the
 # force scalar (36), s V / |y| (8) and the force and its sum (36) = 404
@@ -80,9 +89,10 @@ FP32_PEAK_TOPS = 35.1
 # 8 B, wsum_inv 8 B, BC class 1 B; per bond 8 B of double-word |xi| on top
 BYTES_PER_NODE[48] = 305.0
 DW_BYTES_PER_BOND = BYTES_PER_BOND + 8.0
-STEP_SRC = {32: ["pd_step_f32.cu"], 64: ["pd_step_f64.cu"], 48: ["pd_step_dw.cu"],
+STEP_SRC = {32: ["pd_step_f32.cu"], 64: ["pd_step_f64.cu", "pd_w3.h"],
+            48: ["pd_step_f64.cu", "pd_w3.h"],
             "lat": ["pd_step_f32_lat.cu"], "lat_tma": ["pd_step_f32_lat_tma.cu", "pd_step_f32_lat.cu"]}
-STEP_TAG = {32: "f32", 64: "f64", 48: "dw", "lat": "f32_lat", "lat_tma": "f32_lat_tma"}
+STEP_TAG = {32: "f32", 64: "f64", 48: "f64", "lat": "f32_lat", "lat_tma": "f32_lat_tma"}
 TMA_BOX = ["16x2x8", "8x4x8", "32x2x4"]  # pd_config.lat_variant 2, 3, 4
 # Device memory one FP32 lattice step touches per node: FP64 displacement 24 B
 # read + 24 B written (double-buffered), the published record 16 B read + 16 B
@@ -101,7 +111,7 @@ def step_footprint(n_nodes, n_bonds, precision, lattice, osb=False):
     the kernel streams one)."""
     if lattice:
         return n_nodes * (LAT_OSB_FOOTPRINT_PER_NODE if osb else LAT_FOOTPRINT_PER_NODE)
-    per_bond = DW_BYTES_PER_BOND if precision == 48 else BYTES_PER_BOND
+    per_bond = BYTES_PER_BOND if precision == 32 else W3_BYTES_PER_BOND
     return n_bonds * per_bond + n_nodes * BYTES_PER_NODE[precision]
 
 
@@ -536,7 +546,10 @@ def run_ours(args):
     if args.precision == 48:
         per_bond = DW_BYTES_PER_BOND + (8.0 if args.kr else 0.0)
     osb = args.state_based is not None
+    w3 = args.precision != 32 and not osb and not args.kr
     alg_bytes = n_bonds * per_bond + w.n * BYTES_PER_NODE[args.precision]
+    if w3:
+        alg_bytes = n_bonds * W3_BYTES_PER_BOND + w.n * W3_BYTES_PER_NODE
     if osb and args.precision == 32:
         # two passes over the family (ids and flags twice), and per node the
         # weighted volume, dilation and (alpha', beta') besides the step's node data
@@ -558,28 +571,28 @@ def run_ours(args):
         roofline["note"] = ("algorithmic bytes of the stored-family step (4.125 B per directed "
                             "bond, 93 B per node); the lattice stencil kernel reads no neighbour "
                             "ids, so its DRAM traffic is below them")
-    if args.precision == 64:
+    if args.precision == 64 and not w3:
         fpb = OSB_FLOPS_PER_BOND if args.state_based is not None else FP64_FLOPS_PER_BOND
         tf = fpb * n_bonds / (ms_step * 1e-3) / 1e12
         roofline = {"bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                     "frac": tf / FP64_PEAK_TFLOPS,
-                    "traffic": None if args.state_based is not None
-                    else profiled_traffic(64, args.workload),
+                    "traffic": None,
                     "peak_source": "FP64 FMA throughput measured by a probe on this pool's GB300 "
                                    "(nominal 1.25 TFLOP/s)",
                     "algorithmic_flops_per_bond": fpb,
                     "hbm": {"achieved": achieved, "peak": peak, "unit": "GB/s",
                             "frac": achieved / peak},
                     "kernel": "k_osb_dilation + k_osb_force" if args.state_based is not None
-                    else "k_step_f64"}
-    if args.precision == 48:
-        ops = DW_OSB_FP32_OPS_PER_BOND if osb else DW_FP32_OPS_PER_BOND
+                    else "k_step_f64_soft"}
+    if args.precision == 48 or w3:
+        ops = (DW_OSB_FP32_OPS_PER_BOND if osb
+               else W3_FP32_OPS_PER_BOND if w3 else DW_FP32_OPS_PER_BOND)
         f64 = OSB_FLOPS_PER_BOND if osb else FP64_FLOPS_PER_BOND
         tops = ops * n_bonds / (ms_step * 1e-3) / 1e12
         tf64 = f64 * n_bonds / (ms_step * 1e-3) / 1e12
         roofline = {"bound": "alu", "achieved": tops, "peak": FP32_PEAK_TOPS, "unit": "TFLOP/s",
                     "frac": tops / FP32_PEAK_TOPS,
-                    "traffic": None if osb else profiled_traffic(48, args.workload),
+                    "traffic": profiled_traffic(args.precision, args.workload) if w3 else None,
                     "peak_source": "FP32 operations (add, multiply or fma each counted once) "
                                    "against the FP32 FMA lane rate measured by a probe on this "
                                    "pool's GB300 (70.2 TFLOP/s counting an FMA as two)",
@@ -589,7 +602,8 @@ def run_ours(args):
                                         "flops_per_bond": f64},
                     "hbm": {"achieved": achieved, "peak": peak, "unit": "GB/s",
                             "frac": achieved / peak},
-                    "kernel": "k_osb_dw_dilation + k_osb_dw_force" if osb else "k_step_dw"}
+                    "kernel": "k_osb_dw_dilation + k_osb_dw_force" if osb
+                    else "k_step_f64" if w3 else "k_step_dw"}
     cpu = None
     if world == 1 and not args.no_cpu_baseline:
         import oracle
@@ -735,10 +749,11 @@ def measure_batch(args, steps, warmup, with_cpu, with_e2e):
     reps = max(1, min(steps, 20) // GL)
     ms_l, lay_l = loop_graph_ms(pdgb, torch, ws, args.precision, True, stream, GL, reps)
     ms_ll, lay_ll = loop_graph_ms(pdgb, torch, ws, args.precision, False, stream, GL, reps)
-    # roofline: the step's algorithmic bytes over all instances (FP32, FP64), or
-    # the double-word step's FP32 operations
-    per_bond = DW_BYTES_PER_BOND if args.precision == 48 else BYTES_PER_BOND
-    alg_bytes = n_bonds * per_bond + n_nodes * BYTES_PER_NODE[args.precision]
+    # roofline: the step's algorithmic bytes over all instances (FP32), or the FP32
+    # operations of the double-word arithmetic (FP64 and double-word)
+    w3 = args.precision != 32
+    alg_bytes = n_bonds * (W3_BYTES_PER_BOND if w3 else BYTES_PER_BOND) + n_nodes * (
+        W3_BYTES_PER_NODE if w3 else BYTES_PER_NODE[32])
     peak, peak_kind = hbm_peak()
     achieved = alg_bytes / (ms_b * 1e-3) / 1e9
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
@@ -751,15 +766,17 @@ def measure_batch(args, steps, warmup, with_cpu, with_e2e):
     if lat:
         roofline["note"] = ("algorithmic bytes of the stored-family step; the lattice stencil "
                             "kernel reads no neighbour ids")
-    if args.precision == 48:
-        tops = DW_FP32_OPS_PER_BOND_NODE_W * n_bonds / (ms_b * 1e-3) / 1e12
+    if w3:
+        uniform = all(float(w.volumes.min()) == float(w.volumes.max()) for w in ws)
+        ops = W3_FP32_OPS_PER_BOND if uniform else W3_FP32_OPS_PER_BOND_NODE_W
+        tops = ops * n_bonds / (ms_b * 1e-3) / 1e12
         roofline = {"bound": "alu", "achieved": tops, "peak": FP32_PEAK_TOPS,
                     "unit": "TFLOP/s", "frac": tops / FP32_PEAK_TOPS, "traffic": None,
                     "peak_source": "FP32 operations against the measured FP32 FMA lane rate",
-                    "algorithmic_flops_per_bond": DW_FP32_OPS_PER_BOND_NODE_W,
+                    "algorithmic_flops_per_bond": ops,
                     "hbm": {"achieved": achieved, "peak": peak, "unit": "GB/s",
                             "frac": achieved / peak},
-                    "kernel": "k_step_dw (batch, per-node weights)"}
+                    "kernel": "k_step_f64 (batch)"}
     # the oracle over whole instances, in order, for about 10 s of host time
     cpu = None
     if with_cpu:

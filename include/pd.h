@@ -63,15 +63,16 @@ typedef enum {
                             high word and a bf16 rounding of the low word) */
 #define PD_PREC_DW 48    /* FP64-grade step from FP32 double-word arithmetic: node
                             state (u, v) and integration in FP64 exactly as with
-                            PD_PREC_F64; every bond quantity (xi, eta, y, the
-                            stretch of Eq. 4, |y|, the force of Eq. 5) carried as an
-                            unevaluated sum of two FP32 numbers (~48-bit significand,
-                            bond-force relative error ~1e-13), and the break test
-                            decided against the FP64 s_c.  Everything PD_PREC_F64
-                            offers: both integrators, per-bond stiffness,
-                            softening, batches, the state-based model and the
-                            adjoint, which runs in double-word arithmetic
-                            as well (see pd_adjoint_forward).
+                            PD_PREC_F64.  Bond-based models without softening run
+                            PD_PREC_F64's step and adjoint (the same results); on
+                            softening and state-based models every bond quantity (xi,
+                            eta, y, the stretch of Eq. 4, |y|, the force of Eq. 5) is
+                            carried as an unevaluated sum of two FP32 numbers (~48-bit
+                            significand, bond-force relative error ~1e-13), and the
+                            break test decided against the FP64 s_c, where PD_PREC_F64
+                            is literal FP64.  Everything PD_PREC_F64 offers: both
+                            integrators, per-bond stiffness, softening, batches, the
+                            state-based model and the adjoint.
                             pd_get_info reports 48. */
 #define PD_MAX_FAMILY 1024
 #define PD_MAX_BC_CLASSES 256
@@ -85,7 +86,8 @@ typedef struct {
     int32_t check_dt;     /* 1 = refuse a dt above the bound of Silling & Askari (2005) */
     int32_t device;       /* CUDA device ordinal */
     void* stream;         /* cudaStream_t to queue work on; NULL = library-owned stream */
-    int32_t block_threads;/* threads per block of the step kernel; 0 = default (256) */
+    int32_t block_threads;/* threads per block of the step kernel; 0 = default (256;
+                             32 on PD_PREC_F64 models with softening) */
     int32_t blocks_per_sm;/* resident blocks per SM for the step grid; 0 = default */
     int32_t reorder;      /* 0 = keep the caller's node order (best for lattices given
                              row-major); 1 = sort nodes by horizon-sized cells */
@@ -388,10 +390,10 @@ pd_status pd_set_params(pd_handle* h, double c, double sc, double load, double d
  * handles.  A velocity-Verlet run must start where the state was set
  * (pd_set_state, or creation), so that its acceleration is formed afresh from
  * (u^0, v^0); then dL_dv0 is the derivative with respect to that velocity and
- * dLdv refers to the full-step velocity v^N that pd_get_state reports.  On PD_PREC_DW handles the recorded and
- * recomputed forward runs use the double-word step and pd_adjoint_backward's
- * reverse sweep is in double-word arithmetic too (FP64-grade; the same outputs
- * to ~1e-10); pd_adjoint_backward_static keeps the FP64 reverse sweep.
+ * dLdv refers to the full-step velocity v^N that pd_get_state reports.  The
+ * reverse sweep of pd_adjoint_backward forms each bond's undeformed part in FP64 and
+ * the remainder in double-word arithmetic (FP64-grade); the one of
+ * pd_adjoint_backward_static is literal FP64 (the same outputs to ~1e-10).
  *
  * pd_adjoint_forward - advance n_steps (>= 1) from the current state with the
  *   bond flags frozen (no bond breaks, so the run is a smooth function of the

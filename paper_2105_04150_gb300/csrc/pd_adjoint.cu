@@ -1,5 +1,7 @@
-// Hand-written adjoint of the damped Euler-Cromer run with frozen bond flags
-// (FP64).  One reverse step n+1 -> n is two launches:
+// Hand-written adjoint of the damped Euler-Cromer run with frozen bond flags, in
+// literal FP64: the reverse step of pd_adjoint_backward_static, whose caller gives the
+// memory (pd_adjoint_backward runs k_adj_step_w3, 3.5 times as fast, with 24 bytes a
+// slot more).  One reverse step n+1 -> n is two launches:
 //   k_adj_mask  w = ws (vbar + dt ubar) with the controlled components of ubar
 //               and vbar zeroed (a prescribed component does not depend on the
 //               previous state); ws = 1 for an Euler-Cromer step, 1/2 for the

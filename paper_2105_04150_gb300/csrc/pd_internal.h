@@ -29,8 +29,9 @@
 // FP64 path:
 //   rec[2] 8 doubles per node {x, y, z, w, ux, uy, uz, 0}, double buffered
 //   v      double velocity, 3 per node
-//   (PD_PREC_DW handles add 64-byte double-word copies of the records for the
-//   neighbours and a double-word reference length per slot, see DwArgs)
+//   Bond-based handles without softening (and PD_PREC_DW ones) add 64-byte three-word
+//   copies of the records for the neighbours and U / |xi| per slot, see W3Args; the other
+//   PD_PREC_DW handles 64-byte double-word copies and |xi| per slot, see DwArgs.
 #pragma once
 
 #include <algorithm>

@@ -1,16 +1,16 @@
-// FP64-grade peridynamic step from double-word FP32 arithmetic (sm_103a).
+// FP64-grade step of the PD_PREC_DW models with softening, from double-word FP32
+// arithmetic (sm_103a).  (Without softening they run k_step_f64.)
 //
-// GB300 issues FP32 operations at about 58 times its FP64 rate, and the FP64
-// step kernel is bound by the FP64 pipe.  This kernel computes the same step
+// GB300 issues FP32 operations at about 58 times its FP64 rate, and the literal FP64
+// softening step is bound by the FP64 pipe.  This kernel computes the same step
 // (Eq. 4 stretch, Eq. 6 breaking, Eq. 5/10 force, Eq. 11 update, Eq. 8
 // damage) with every bond quantity carried as an unevaluated sum of two FP32
 // numbers (double-word arithmetic, pd_dw.h), about 48 significant bits: the
 // relative accuracy of a bond force is ~1e-13, far inside the FP64 parity bar,
-// for about two hundred FP32 operations instead of ~30 FP64 ones.  Variants:
-// sc_mode, uniform or per-node weights (batches take the latter), softening
-// (the stored FP64 integrity scales the force; bonds near s_0 are resolved in
-// FP64), per-bond stiffness (a run-time branch), velocity-Verlet (its own
-// translation unit, below).
+// for about two hundred FP32 operations instead of ~30 FP64 ones.  The stored FP64
+// integrity scales the force; bonds near s_0 are resolved in FP64.  Variants:
+// sc_mode, uniform or per-node weights (batches take the latter), per-bond stiffness
+// (a run-time branch), velocity-Verlet (its own translation unit, below).
 //
 // Work decomposition, bond flags, node order and the double-buffered records
 // are those of the FP32 kernel (lane per node over the sliced family).
