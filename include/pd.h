@@ -86,8 +86,8 @@ typedef struct {
     int32_t check_dt;     /* 1 = refuse a dt above the bound of Silling & Askari (2005) */
     int32_t device;       /* CUDA device ordinal */
     void* stream;         /* cudaStream_t to queue work on; NULL = library-owned stream */
-    int32_t block_threads;/* threads per block of the step kernel; 0 = default (256;
-                             32 on PD_PREC_F64 models with softening) */
+    int32_t block_threads;/* threads per block of the step kernel; 0 = default (256,
+                             128 or 32, by the model) */
     int32_t blocks_per_sm;/* resident blocks per SM for the step grid; 0 = default */
     int32_t reorder;      /* 0 = keep the caller's node order (best for lattices given
                              row-major); 1 = sort nodes by horizon-sized cells */

@@ -736,10 +736,22 @@ pd_status choose_grid(pd_handle* h, int blocks_per_sm)
     int occ = 0;
     PD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, h->block, smem), "occupancy");
     if (occ < 1) occ = 1;
+    const int full = occ;
     if (blocks_per_sm > 0) occ = std::min(occ, blocks_per_sm);
     const int64_t slices_per_block = h->block / 32 / h->team;
     const int64_t need = (h->n_slices + slices_per_block - 1) / slices_per_block;
     h->grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * occ, need));
+    // A walk of a slice takes 10 to 45 us, so resident blocks that each take the same number
+    // of slices leave the chip idle in the last round.  The lattice kernels and the
+    // three-word kernels get a block per few slices instead, given to the SMs as they
+    // become free.  us per step, resident / on demand: FP32 beam of 31538 slices 118.3 /
+    // 109.6, plate of 62829 243.7 / 215.2; FP64 step of 6891 slices 266 / 259, 15000: 534 /
+    // 501; state-based lattice step of 31538 slices
+    // 228.9 / 209.6, 7657: 64.8 / 62.6, but 4219: 38.1 / 39.8, hence its limit of two rounds
+    // of its force loop.  (The general FP32 kernel keeps resident blocks: 107.6 / 110.0.)
+    const bool on_demand = (blocks_per_sm <= 0 || blocks_per_sm >= full) &&
+                           (h->w3 || (h->lattice && (h->model == 0 || h->n_slices > 48LL * sms)));
+    if (on_demand) h->grid = (int)std::max<int64_t>(1, need);
     h->grid_dil = h->grid;
     h->grid_osbf = h->grid;
     if (h->model == 1 && h->precision == 32 && h->lattice) {  // the force loop's own grid
@@ -750,6 +762,7 @@ pd_status choose_grid(pd_handle* h, int blocks_per_sm)
         PD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, ff, h->block, 0), "occupancy");
         if (blocks_per_sm > 0) o = std::min(o, blocks_per_sm);
         h->grid_osbf = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * std::max(o, 1), need));
+        if (on_demand) h->grid_osbf = h->grid;
     }
     if (h->model == 1 && h->precision == 32 && !h->lattice) {  // the state-based kernels' own grids
         auto grid_of_kernel = [&](const void* fn, int& out) -> pd_status {
@@ -1402,6 +1415,23 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
         return fail(PD_ERR_ARG, "the tile step (lat_variant 2..4) takes single models");
     h->lat_var = cfg->lat_variant;
     h->blocks_per_sm = cfg->blocks_per_sm;
+    // Threads per block.  The three-word kernels: the smallest block that holds a team and
+    // keeps 16 warps per SM in few blocks (a block's slot is free when its slowest slice is
+    // done, and a team's barrier waits for the block); us per step with 128 / 256 threads:
+    // 750 slices 54.6 / 62.2, 6891: 259 / 260, 9025: 319 / 334, 15000: 501 / 519; one round
+    // of single warps shares L1 better in larger blocks (1953: 92.8 / 87.1).  The
+    // state-based lattice step up to two rounds: 750 slices 19.4 / 20.2, 4219: 38.1 / 39.8,
+    // 7657: 62.0 / 62.6, but 31538: 216.3 / 209.6.
+    if (!cfg->block_threads && (h->w3 || (h->lattice && h->model == 1))) {
+        int sms = 0;
+        PD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device), "sm count");
+        bool small = h->n_slices <= 64LL * sms;
+        if (h->w3) {
+            const int team = w3_team(h, sms);
+            small = team != 8 && (team > 1 || h->n_slices > 16LL * sms);
+        }
+        if (small) h->block = 128;
+    }
     if ((st = choose_grid(h, h->blocks_per_sm)) != PD_OK) return st;
     e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "synchronize");
