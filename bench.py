@@ -47,8 +47,8 @@ BYTES_PER_NODE = {32: 93.0, 64: 136.0}
 # Algorithmic FP64 work per bond (Eqs. 4-5 as written): xi, eta, y (9), |xi|^2 and
 # |y|^2 (10), two square roots and the stretch's division (3), c V s / |y| (3), the
 # force accumulation (6 as 3 fused multiply-adds) = 31 flops, counting a square
-# root or a division as one.  The softening and state-based FP64 steps evaluate it
-# literally and are bound by GB300's FP64 pipe.  Peak: FP64 fused multiply-add
+# root or a division as one.  The softening FP64 step evaluates it literally and is
+# bound by GB300's FP64 pipe.  Peak: FP64 fused multiply-add
 # throughput measured on a GB300 of this machine with a plain dependent-chain probe,
 # 1.20 TFLOP/s (nominal 1.25).
 FP64_FLOPS_PER_BOND = 31.0
@@ -79,10 +79,10 @@ W3_BYTES_PER_BOND = BYTES_PER_BOND + 8.0
 # = 192, plus two seeds.  Peak: FP32 FMA lane rate measured by a probe on this machine's
 # GB300, 35.1 T/s (70.2 TFLOP/s counting an FMA as two).
 DW_FP32_OPS_PER_BOND = 192.0
-# double-word state-based step (pd_step_osb_dw.cu), both loops: the bond's
-# stretch, y and 1/|y| (152) in each; the dilation term and its sum (20); the
-# force scalar (36), s V / |y| (8) and the force and its sum (36) = 404
-DW_OSB_FP32_OPS_PER_BOND = 404.0
+# state-based step of FP64 and double-word models (pd_step_osb_w3.cu), both loops: xi, eta,
+# y, num and z as above (152) in each; the dilation term (23) and its sum (8); the force
+# scalar (20) and the force and its sum (36) = 391
+W3_OSB_FP32_OPS_PER_BOND = 391.0
 FP32_PEAK_TOPS = 35.1
 # per node: the double-word record 64 B read + 64 B written, the FP64 record
 # (x, w copied, u) 56 B read + 56 B written, FP64 velocity 24 + 24 B, damage
@@ -546,9 +546,11 @@ def run_ours(args):
     if args.precision == 48:
         per_bond = DW_BYTES_PER_BOND + (8.0 if args.kr else 0.0)
     osb = args.state_based is not None
-    w3 = args.precision != 32 and not osb and not args.kr
+    w3 = args.precision != 32 and not args.kr
     alg_bytes = n_bonds * per_bond + w.n * BYTES_PER_NODE[args.precision]
-    if w3:
+    if w3 and osb:  # the family twice; alpha and gamma 16 B, alpha and beta 16 B, m 8 B
+        alg_bytes = n_bonds * 2 * W3_BYTES_PER_BOND + w.n * (W3_BYTES_PER_NODE + 64 + 88)
+    elif w3:
         alg_bytes = n_bonds * W3_BYTES_PER_BOND + w.n * W3_BYTES_PER_NODE
     if osb and args.precision == 32:
         # two passes over the family (ids and flags twice), and per node the
@@ -572,7 +574,7 @@ def run_ours(args):
                             "bond, 93 B per node); the lattice stencil kernel reads no neighbour "
                             "ids, so its DRAM traffic is below them")
     if args.precision == 64 and not w3:
-        fpb = OSB_FLOPS_PER_BOND if args.state_based is not None else FP64_FLOPS_PER_BOND
+        fpb = FP64_FLOPS_PER_BOND
         tf = fpb * n_bonds / (ms_step * 1e-3) / 1e12
         roofline = {"bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                     "frac": tf / FP64_PEAK_TFLOPS,
@@ -582,17 +584,17 @@ def run_ours(args):
                     "algorithmic_flops_per_bond": fpb,
                     "hbm": {"achieved": achieved, "peak": peak, "unit": "GB/s",
                             "frac": achieved / peak},
-                    "kernel": "k_osb_dilation + k_osb_force" if args.state_based is not None
-                    else "k_step_f64_soft"}
+                    "kernel": "k_step_f64_soft"}
     if args.precision == 48 or w3:
-        ops = (DW_OSB_FP32_OPS_PER_BOND if osb
+        ops = (W3_OSB_FP32_OPS_PER_BOND if osb
                else W3_FP32_OPS_PER_BOND if w3 else DW_FP32_OPS_PER_BOND)
         f64 = OSB_FLOPS_PER_BOND if osb else FP64_FLOPS_PER_BOND
         tops = ops * n_bonds / (ms_step * 1e-3) / 1e12
         tf64 = f64 * n_bonds / (ms_step * 1e-3) / 1e12
         roofline = {"bound": "alu", "achieved": tops, "peak": FP32_PEAK_TOPS, "unit": "TFLOP/s",
                     "frac": tops / FP32_PEAK_TOPS,
-                    "traffic": profiled_traffic(args.precision, args.workload) if w3 else None,
+                    "traffic": profiled_traffic(args.precision, args.workload) if w3 and not osb
+                    else None,
                     "peak_source": "FP32 operations (add, multiply or fma each counted once) "
                                    "against the FP32 FMA lane rate measured by a probe on this "
                                    "pool's GB300 (70.2 TFLOP/s counting an FMA as two)",
@@ -602,7 +604,7 @@ def run_ours(args):
                                         "flops_per_bond": f64},
                     "hbm": {"achieved": achieved, "peak": peak, "unit": "GB/s",
                             "frac": achieved / peak},
-                    "kernel": "k_osb_dw_dilation + k_osb_dw_force" if osb
+                    "kernel": "k_osb_w3_dilation + k_osb_w3_force" if osb
                     else "k_step_f64" if w3 else "k_step_dw"}
     cpu = None
     if world == 1 and not args.no_cpu_baseline:

@@ -133,8 +133,8 @@ struct pd_handle {
     float2* lendw = nullptr;                // per slot |xi| / delta
     float2* cbdw = nullptr;                 // per slot c_ij (per-bond stiffness)
     double dw_origin[3] = {0.0, 0.0, 0.0};  // origin of the double-word positions
-    // bond-based PD_PREC_F64 and PD_PREC_DW without softening: three-word records and bond
-    // lengths of the step (W3Args)
+    // PD_PREC_F64 and PD_PREC_DW without softening: three-word records and bond lengths of
+    // the step (W3Args)
     bool w3 = false;
     float4* rec3[2] = {nullptr, nullptr};
     float4* il3 = nullptr;
@@ -156,12 +156,9 @@ struct pd_handle {
     void* integ = nullptr;  // softening: per-slot integrity (float / double)
     int model = 0;          // 1: ordinary state-based linear solid (FP64)
     double osb_K = 0.0, osb_G = 0.0;
-    double* osb_len = nullptr;    // per slot |xi|
     double* osb_mvol = nullptr;   // per node weighted volume
-    double* osb_theta = nullptr;  // per node dilation
-    double* osb_alpha = nullptr;  // per node force-scalar coefficients (see pd_step_osb.cu)
-    double* osb_beta = nullptr;
-    float4* osbdw_ab = nullptr;   // double-word state-based: per node alpha~, beta~
+    double2* osb_ab64 = nullptr;  // per node force-scalar coefficients (see pd_step_osb_w3.cu)
+    float4* osb_ab = nullptr;
     float *osb32_mvol = nullptr, *osb32_theta = nullptr;  // FP32 state-based arrays
     float2* osb32_ab = nullptr;
     float4* osblat_coef = nullptr;  // FP32 state-based lattice models (pd_step_f32_lat_osb.cu)
@@ -478,28 +475,13 @@ const void* f32_kernel(pd_handle* h)
                                : step_f32_kernel(h->sc_mode, h->uniform_vol, h->per_bond_c);
 }
 
-OsbArgs osb_args(pd_handle* h)
+OsbW3Args osbw3_args(pd_handle* h)
 {
-    OsbArgs o{};
-    o.len = h->osb_len;
+    OsbW3Args o{};
     o.vol = h->vol;
     o.mvol = h->osb_mvol;
-    o.theta = h->osb_theta;
-    o.alpha = h->osb_alpha;
-    o.beta = h->osb_beta;
-    o.K = h->osb_K;
-    o.G = h->osb_G;
-    return o;
-}
-
-OsbDwArgs osbdw_args(pd_handle* h)
-{
-    OsbDwArgs o{};
-    o.len = h->lendw;
-    o.vol = h->vol;
-    o.mvol = h->osb_mvol;
-    o.theta = h->osb_theta;
-    o.ab = h->osbdw_ab;
+    o.ab64 = h->osb_ab64;
+    o.ab = h->osb_ab;
     o.K = h->osb_K;
     o.G = h->osb_G;
     return o;
@@ -536,7 +518,7 @@ DwArgs dw_args(pd_handle* h)
     d.len = h->lendw;
     d.cb = h->per_bond_c ? h->cbdw : nullptr;
     d.inv_delta = 1.0 / h->delta;
-    d.w_const = ((h->per_bond_c || h->model == 1) ? 1.0 : h->c) * h->vol0;
+    d.w_const = (h->per_bond_c ? 1.0 : h->c) * h->vol0;
     d.dt_rho = h->dt / h->rho;
     // the leading word of a double-word stretch is within 2^-23 of it: below
     // this band the break test cannot be near any s_c of the model
@@ -559,7 +541,7 @@ W3Args w3_args(pd_handle* h)
     d.wrel = h->wrel3;
     d.phi0 = h->phi0;
     d.fam = h->fam3;
-    d.w_ref = (h->per_bond_c ? 1.0 : h->c) * h->vol0;
+    d.w_ref = ((h->per_bond_c || h->model == 1) ? 1.0 : h->c) * h->vol0;
     d.scale = h->w3_scale;
     d.x_grid = h->w3_x_grid;
     d.dt_rho = h->dt / h->rho;
@@ -585,11 +567,12 @@ cudaError_t publish64(pd_handle* h, int b)
 const void* step_kernel_fn(pd_handle* h)
 {
     if (h->precision == 32) return f32_kernel(h);
+    if (h->model == 1) return osb_w3_force_kernel(h->uniform_vol);
     if (h->w3) return step_f64_kernel(h->uniform_vol, h->team > 1);
     if (h->dw)
         return step_dw_kernel(h->sc_mode, h->uniform_vol && !h->batch,
                               h->integrator == PD_INTEGRATOR_VV);
-    return h->integ != nullptr ? step_f64_soft_kernel(h->sc_mode) : osb_force_kernel();
+    return step_f64_soft_kernel(h->sc_mode);
 }
 
 // One step launch, k steps past the device counter; step_abs >= 0 (F32 lattice
@@ -597,9 +580,6 @@ const void* step_kernel_fn(pd_handle* h)
 // counter itself
 cudaError_t launch_one(pd_handle* h, int k, int64_t step_abs = -1)
 {
-    if (h->dw && h->model == 1)
-        return launch_osb_dw_step(args_f64(h, k), dw_args(h), osbdw_args(h), h->grid, h->block,
-                                  h->stream);
     if (h->dw && !h->w3)
         return launch_step_dw(args_f64(h, k), dw_args(h), h->sc_mode, h->grid, h->block,
                               h->stream);
@@ -610,7 +590,8 @@ cudaError_t launch_one(pd_handle* h, int k, int64_t step_abs = -1)
                    : launch_osb32_step(args_f32(h, k), osb32_args(h), h->sc_mode, h->grid_osbf, h->grid_dil, h->block,
                                  h->stream);
     if (h->model == 1)
-        return launch_osb_step(args_f64(h, k), osb_args(h), h->grid, h->block, h->stream);
+        return launch_osb_w3_step(args_f64(h, k), w3_args(h), osbw3_args(h), h->grid, h->block,
+                                  h->stream);
     if (h->precision == 32)
         return launch_f32(h, args_f32(h, k, step_abs));
     return launch_f64(h, args_f64(h, k));
@@ -708,7 +689,7 @@ pd_status choose_grid(pd_handle* h, int blocks_per_sm)
     }
     int sms = 0;
     PD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device), "sm count");
-    if (h->w3) h->team = w3_team(h, sms);
+    if (h->w3 && h->model == 0) h->team = w3_team(h, sms);
     if (lat_team(h)) {  // a block of four warps per slice
         const void* fn = step_kernel_fn(h);
         PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -725,9 +706,10 @@ pd_status choose_grid(pd_handle* h, int blocks_per_sm)
     // carveout is this handle's, for the occupancy below and given with every launch; its
     // limit is the same for all handles, which share the function.
     const int max_seg = h->Q * (32 / kW3Seg);
-    const size_t smem = h->w3 ? step_f64_smem(h->team, max_seg, h->block) : 0;
+    const bool sums = h->w3 && h->model == 0;
+    const size_t smem = sums ? step_f64_smem(h->team, max_seg, h->block) : 0;
     PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 h->w3 ? step_f64_carveout(h->team, max_seg, h->block) : 0),
+                                 sums ? step_f64_carveout(h->team, max_seg, h->block) : 0),
             "carveout");
     if (h->w3 && h->team > 1)
         PD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -746,7 +728,7 @@ pd_status choose_grid(pd_handle* h, int blocks_per_sm)
     // three-word kernels get a block per few slices instead, given to the SMs as they
     // become free.  us per step, resident / on demand: FP32 beam of 31538 slices 118.3 /
     // 109.6, plate of 62829 243.7 / 215.2; FP64 step of 6891 slices 266 / 259, 15000: 534 /
-    // 501; state-based lattice step of 31538 slices
+    // 501; FP64 state-based 530 / 514, 1077 / 1016; state-based lattice step of 31538 slices
     // 228.9 / 209.6, 7657: 64.8 / 62.6, but 4219: 38.1 / 39.8, hence its limit of two rounds
     // of its force loop.  (The general FP32 kernel keeps resident blocks: 107.6 / 110.0.)
     const bool on_demand = (blocks_per_sm <= 0 || blocks_per_sm >= full) &&
@@ -833,9 +815,7 @@ pd_status vv_force_pass(pd_handle* h)
         a.peek = 1;
         a.vout = (double*)h->vpeek;
         if (h->model == 1)
-            e = h->dw ? launch_osb_dw_step(a, dw_args(h), osbdw_args(h), h->grid, h->block,
-                                           h->stream)
-                      : launch_osb_step(a, osb_args(h), h->grid, h->block, h->stream);
+            e = launch_osb_w3_step(a, w3_args(h), osbw3_args(h), h->grid, h->block, h->stream);
         else
             e = h->dw && !h->w3
                     ? launch_step_dw(a, dw_args(h), h->sc_mode, h->grid, h->block, h->stream)
@@ -1041,7 +1021,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
     std::vector<uint8_t> cls;
     std::string msg = bc_classes(n, d.type, d.disp, d.force, d.no_fail, table, cls, h->has_nofail);
     if (!msg.empty()) return fail(PD_ERR_ARG, "%s", msg.c_str());
-    h->w3 = cfg->precision != PD_PREC_F32 && h->model == 0 &&
+    h->w3 = cfg->precision != PD_PREC_F32 &&
             (h->kr < 1.0 || (h->kr == 1.0 && !h->has_nofail));
     // The literal FP64 step is bound by each SM's FP64 pipe, so its slices have to be
     // spread evenly: one warp per block (a 962-slice model fills 121 SMs with 8 slices
@@ -1154,16 +1134,10 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
                 ALLOC(h->osb32_mvol, float, np);
                 ALLOC(h->osb32_ab, float2, np);
             }
-        } else if (h->dw) {
-            ALLOC(h->osb_mvol, double, np);
-            ALLOC(h->osb_theta, double, np);
-            ALLOC(h->osbdw_ab, float4, np);
         } else {
-            ALLOC(h->osb_len, double, nbr.size());
             ALLOC(h->osb_mvol, double, np);
-            ALLOC(h->osb_theta, double, np);
-            ALLOC(h->osb_alpha, double, np);
-            ALLOC(h->osb_beta, double, np);
+            ALLOC(h->osb_ab64, double2, np);
+            ALLOC(h->osb_ab, float4, np);
         }
     }
     // bilinear softening: every bond starts intact, mu = 1 (FP64 and double-word with
@@ -1372,8 +1346,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
         if (e != cudaSuccess) return cuda_fail(e, "bond lengths");
     }
     if (h->model == 1 && !f32) {
-        e = h->dw ? launch_osb_dw_setup(args_f64(h, 0), osbdw_args(h), h->stream)
-                  : launch_osb_setup(args_f64(h, 0), osb_args(h), h->x64, h->stream);
+        e = launch_osb_w3_setup(args_f64(h, 0), osbw3_args(h), h->x64, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "state-based set-up");
     }
     if ((st = upload_weights(h)) != PD_OK) return st;
@@ -1425,8 +1398,8 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
     if (!cfg->block_threads && (h->w3 || (h->lattice && h->model == 1))) {
         int sms = 0;
         PD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device), "sm count");
-        bool small = h->n_slices <= 64LL * sms;
-        if (h->w3) {
+        bool small = h->n_slices <= 64LL * sms || h->w3;
+        if (h->w3 && h->model == 0) {
             const int team = w3_team(h, sms);
             small = team != 8 && (team > 1 || h->n_slices > 16LL * sms);
         }
@@ -2511,7 +2484,9 @@ pd_status pd_autotune(pd_handle* h, int32_t trial_steps, int32_t* block_threads,
             if (var >= 2) break;  // the tile step's grid does not depend on bps
             int occ = 0;
             const void* fn = step_kernel_fn(h);
-            const size_t smem = h->w3 ? step_f64_smem(h->team, h->Q * (32 / kW3Seg), block) : 0;
+            const size_t smem = h->w3 && h->model == 0
+                                    ? step_f64_smem(h->team, h->Q * (32 / kW3Seg), block)
+                                    : 0;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem);
             if (bps >= occ) break;  // larger requests are capped to the same grid
         }

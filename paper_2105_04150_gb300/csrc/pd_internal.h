@@ -383,31 +383,22 @@ struct DwArgs {
     int32_t uniform_w;         // 1: every node has weight w_const
 };
 
-// Ordinary state-based (linear solid) arrays, FP64 handles with model 1
-struct OsbArgs {
-    double* len;               // per slot |xi|
+// Ordinary state-based (linear solid) arrays, FP64 and double-word handles with model 1
+// (pd_step_osb_w3.cu)
+struct OsbW3Args {
     const double* vol;         // per node V
     double* mvol;              // per node weighted volume m_i
-    double* theta;             // per node dilation of the current step
-    double* alpha;             // per node 3 K theta / m - beta theta / 3 (current step)
-    double* beta;              // per node 15 G / m
+    double2* ab64;             // per node {alpha, beta} of the current step
+    float4* ab;                // per node {alpha h, l, alpha - beta h, l} in units of
+                               // (K + G) / (V_ref U^2)
     double K, G;               // bulk and shear modulus
 };
 
-// Ordinary state-based arrays of PD_PREC_DW handles (pd_step_osb_dw.cu; lengths
-// in horizon units)
-struct OsbDwArgs {
-    const float2* len;         // per slot |xi| / delta (the double-word step's)
-    const double* vol;         // per node V
-    double* mvol;              // per node m~ = sum |xi~|^2 V_j
-    double* theta;             // per node dilation of the current step
-    float4* ab;                // per node {alpha~ h, l, beta~ h, l} (double-words)
-    double K, G;
-};
-
-cudaError_t launch_osb_dw_setup(const StepArgsF64& a, const OsbDwArgs& o, cudaStream_t s);
-cudaError_t launch_osb_dw_step(const StepArgsF64& a, const DwArgs& d, const OsbDwArgs& o, int grid,
+cudaError_t launch_osb_w3_setup(const StepArgsF64& a, const OsbW3Args& o, const double* x64,
+                                cudaStream_t s);
+cudaError_t launch_osb_w3_step(const StepArgsF64& a, const W3Args& d, const OsbW3Args& o, int grid,
                                int block, cudaStream_t s);
+const void* osb_w3_force_kernel(bool uniform_w);
 
 // Shared-memory tile step of single bond-based lattice models
 // (pd_step_f32_lat_tma.cu): a block per box of BZ x BY x BX nodes, the box's
@@ -679,11 +670,6 @@ cudaError_t launch_gather_damage(int precision, const void* dmg, const int32_t* 
 // record buffers) and wsum_inv (a slot is a real member iff its init_bits bit is set)
 // state-based model: per-slot |xi| and weighted volumes (once), and one step
 // (dilation kernel, then force + integration kernel)
-cudaError_t launch_osb_setup(const StepArgsF64& a, const OsbArgs& o, const double* x64,
-                             cudaStream_t s);
-cudaError_t launch_osb_step(const StepArgsF64& a, const OsbArgs& o, int grid, int block,
-                            cudaStream_t s);
-const void* osb_force_kernel();
 cudaError_t launch_osb32_setup(const StepArgsF32& a, const OsbArgs32& o, cudaStream_t s);
 // the two state-based launches, each on a grid sized by its own occupancy
 cudaError_t launch_osb32_step(const StepArgsF32& a, const OsbArgs32& o, int sc_mode, int grid,

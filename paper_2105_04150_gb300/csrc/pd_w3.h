@@ -224,6 +224,40 @@ __device__ __forceinline__ Own2 own_pairs(const Rec& r)
     return o;
 }
 
+// xi and eta of one bond: the (x, y) components and z
+struct Pair {
+    Dw2 xi, et;
+    Dw xz, ez;
+};
+__device__ __forceinline__ Pair pair_of(const Own2& o, const Rec& j, float2 ts2, float2 tsz)
+{
+    Pair p;
+    p.xi = diff3_2(make_float2(j.a0.x, j.a0.y), make_float2(j.b0.x, j.b0.y), o.xh, o.xm,
+                   add2(make_float2(k_of(j.a1.z), k_of(j.a1.w)), o.xk), ts2);
+    const float2 dt = add2(make_float2(ut_of(j.a1.z), ut_of(j.a1.w)), o.ut);
+    {
+        const float2 dh = add2(make_float2(j.a0.z, j.a0.w), o.uh);
+        const float2 dm = add2(make_float2(j.b0.z, j.b0.w), o.um);
+        const float2 s = add2(dh, dm);
+        p.et = Dw2{s, add2(dt, sub2(dm, sub2(s, dh)))};
+    }
+    const Dw2 zz = diff3_2(make_float2(j.a1.x, j.a1.y), make_float2(j.b1.x, j.b1.y), o.zh, o.zm,
+                           add2(make_float2(k_of(j.b1.z), ut_of(j.b1.z)), o.zt), tsz);
+    p.xz = Dw{zz.h.x, zz.l.x};
+    p.ez = Dw{zz.h.y, zz.l.y};
+    return p;
+}
+
+// eta . v
+__device__ __forceinline__ Dw eta_dot(const Pair& p, Dw2 v, Dw vz)
+{
+    const Dw2 n2 = dw_mul2(p.et, v);
+    const Dw nz = dw_mul(p.ez, vz);
+    Dw num = two_sum(n2.h.x, n2.h.y);
+    num.l += n2.l.x + n2.l.y;
+    return dw_add(num, nz);
+}
+
 // y = xi + eta and num = eta . (2 xi + eta) of one bond
 struct Kin {
     Dw2 y;   // x, y components
@@ -232,38 +266,32 @@ struct Kin {
 };
 __device__ __forceinline__ Kin kin(const Own2& o, const Rec& j, float2 ts2, float2 tsz)
 {
-    const Dw2 xi = diff3_2(make_float2(j.a0.x, j.a0.y), make_float2(j.b0.x, j.b0.y), o.xh, o.xm,
-                           add2(make_float2(k_of(j.a1.z), k_of(j.a1.w)), o.xk), ts2);
-    const float2 dt = add2(make_float2(ut_of(j.a1.z), ut_of(j.a1.w)), o.ut);
-    Dw2 et;
-    {
-        const float2 dh = add2(make_float2(j.a0.z, j.a0.w), o.uh);
-        const float2 dm = add2(make_float2(j.b0.z, j.b0.w), o.um);
-        const float2 s = add2(dh, dm);
-        et = Dw2{s, add2(dt, sub2(dm, sub2(s, dh)))};
-    }
-    const Dw2 zz = diff3_2(make_float2(j.a1.x, j.a1.y), make_float2(j.b1.x, j.b1.y), o.zh, o.zm,
-                           add2(make_float2(k_of(j.b1.z), ut_of(j.b1.z)), o.zt), tsz);
-    const Dw xz{zz.h.x, zz.l.x}, ez{zz.h.y, zz.l.y};
+    const Pair p = pair_of(o, j, ts2, tsz);
     Kin k;
-    k.y = dw_add2(xi, et);
-    k.yz = dw_add(xz, ez);
-    const Dw2 n2 = dw_mul2(et, dw_add2(xi, k.y));
-    const Dw nz = dw_mul(ez, dw_add(xz, k.yz));
-    Dw num = two_sum(n2.h.x, n2.h.y);
-    num.l += n2.l.x + n2.l.y;
-    k.num = dw_add(num, nz);
+    k.y = dw_add2(p.xi, p.et);
+    k.yz = dw_add(p.xz, p.ez);
+    k.num = eta_dot(p, dw_add2(p.xi, k.y), dw_add(p.xz, k.yz));
     return k;
 }
 
-// x = |y|^2 / |xi|^2 - 1 of two bonds and (1 / |xi|) z = -s / |y| (see bond_geo)
-struct Coef2 {
-    float2 x;  // leading words
-    Dw2 c;
+// num alone: without y, 24 operations less
+struct KinNum {
+    Dw num;
 };
-__device__ __forceinline__ Coef2 coef2(Dw a, Dw b, const float4 il)
+__device__ __forceinline__ KinNum kin_num(const Own2& o, const Rec& j, float2 ts2, float2 tsz)
 {
-    const Dw2 num{make_float2(a.h, b.h), make_float2(a.l, b.l)};
+    const Pair p = pair_of(o, j, ts2, tsz);
+    const Dw2 x2{add2(p.xi.h, p.xi.h), add2(p.xi.l, p.xi.l)};
+    return {eta_dot(p, dw_add2(x2, p.et), dw_add(Dw{p.xz.h + p.xz.h, p.xz.l + p.xz.l}, p.ez))};
+}
+
+// x = |y|^2 / |xi|^2 - 1 and z = |xi| / |y| - 1 of two bonds (see bond_geo)
+struct Stretch2 {
+    float2 x;  // leading words
+    Dw2 z;
+};
+__device__ __forceinline__ Stretch2 stretch2(Dw2 num, const float4 il)
+{
     const Dw2 iL{make_float2(il.x, il.y), make_float2(il.z, il.w)};
     const Dw2 x = dw_mul2(dw_mul2(num, iL), iL);
     const float2 x1 = add2(both(1.0f), x.h);
@@ -276,8 +304,18 @@ __device__ __forceinline__ Coef2 coef2(Dw a, Dw b, const float4 il)
     const Dw2 p{ph, add2(sub2(zz, fma2(both(-2.0f), z0, ph)), e)};
     const Dw2 xp = dw_mul2(x, p);
     const float2 R = add2(add2(add2(ph, x.h), xp.h), add2(add2(p.l, x.l), xp.l));
-    const Dw2 z{z0, mul2(R, fma2(z0, both(-0.5f), both(-0.5f)))};
-    return {x.h, dw_mul2(z, iL)};
+    return {x.h, Dw2{z0, mul2(R, fma2(z0, both(-0.5f), both(-0.5f)))}};
+}
+
+// x of two bonds and (1 / |xi|) z = -s / |y|
+struct Coef2 {
+    float2 x;  // leading words
+    Dw2 c;
+};
+__device__ __forceinline__ Coef2 coef2(Dw a, Dw b, const float4 il)
+{
+    const Stretch2 t = stretch2(Dw2{make_float2(a.h, b.h), make_float2(a.l, b.l)}, il);
+    return {t.x, dw_mul2(t.z, Dw2{make_float2(il.x, il.y), make_float2(il.z, il.w)})};
 }
 
 }  // namespace w3
