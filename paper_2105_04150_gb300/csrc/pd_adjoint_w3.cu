@@ -23,6 +23,9 @@
 // (whose s has an absolute error of 3e-16).  Bonds with |eta| / L past 2^-6 or past
 // kW3XMax, or whose w leaves FP32's range, are evaluated literally in FP64.
 //
+// PD_PREC_DW handles (F64 false) take K d = y q (A + B) / L^3 - (z / L) d in double-word
+// arithmetic as a whole, to 2^-44 of each bond's term: no FP64 operation and no e.
+//
 // The FP64 pipe needs few warps and a model of this use is small (the recorded run
 // is kept in memory), so a slice is shared by a block of four warps, each taking
 // every fourth slot; their sums are added in a fixed order.
@@ -158,7 +161,7 @@ __device__ __forceinline__ Dw dot3(const Dw (&a)[3], const Dw (&b)[3])
     return dw_add(s, dw_mul(a[2], b[2]));
 }
 
-template <bool UW>
+template <bool UW, bool F64>
 __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_constant__ AdjW3Args a)
 {
     __shared__ double sd[kTeam][3][32];
@@ -203,12 +206,14 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         dwa::ld_rec(a.rec + 4 * j, in.nb.a0, in.nb.a1);
         dwa::ld_rec(a.rec + 4 * j + 2, in.nb.b0, in.nb.b1);
         dwa::ld_rec(a.wdw + 2 * j, in.v0, in.v1);
-        in.wj = ld_d4(a.w64 + 4 * j);
+        if (F64) in.wj = ld_d4(a.w64 + 4 * j);
         in.il2 = __ldg(a.il + (row >> 1) * 32 + lane);
-        const double* ep = a.e + row * 96 + lane;  // x, y, z rows
-        in.e0 = __ldg(ep);
-        in.e1 = __ldg(ep + 32);
-        in.e2 = __ldg(ep + 64);
+        if (F64) {
+            const double* ep = a.e + row * 96 + lane;  // x, y, z rows
+            in.e0 = __ldg(ep);
+            in.e1 = __ldg(ep + 32);
+            in.e2 = __ldg(ep + 64);
+        }
         in.gc = a.gc[row * 32 + lane];
     };
     uint32_t word = 0u;
@@ -240,27 +245,37 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             }
         }
         // the undeformed part in FP64
-        double d0, d1, d2;
-        if (UW) {
-            d0 = in.wj.x - wm.x;
-            d1 = in.wj.y - wm.y;
-            d2 = in.wj.z - wm.z;
-        } else {
-            const double vj = (double)rj.x + (double)rj.y;
-            d0 = vm * in.wj.x - vj * wm.x;
-            d1 = vm * in.wj.y - vj * wm.y;
-            d2 = vm * in.wj.z - vj * wm.z;
+        double e0 = 0.0, e1 = 0.0, e2 = 0.0, ed = 0.0;
+        if (F64) {
+            double d0, d1, d2;
+            if (UW) {
+                d0 = in.wj.x - wm.x;
+                d1 = in.wj.y - wm.y;
+                d2 = in.wj.z - wm.z;
+            } else {
+                const double vj = (double)rj.x + (double)rj.y;
+                d0 = vm * in.wj.x - vj * wm.x;
+                d1 = vm * in.wj.y - vj * wm.y;
+                d2 = vm * in.wj.z - vj * wm.z;
+            }
+            e0 = in.e0;
+            e1 = in.e1;
+            e2 = in.e2;
+            ed = fma(e0, d0, fma(e1, d1, e2 * d2));
         }
-        const double e0 = in.e0, e1 = in.e1, e2 = in.e2;
-        double ed = fma(e0, d0, fma(e1, d1, e2 * d2));
         if (b + kTeam < Wg) {
             load(b + kTeam, jn);
             jc = jn;
             if (((b + kTeam) & 31) < kTeam) word = a.bits[(g * Q + ((b + kTeam) >> 5)) * 32 + lane];
             if (b + 2 * kTeam < Wg) jn = __ldg(col + (b + 2 * kTeam) * 32);
         }
-        const Dw A = dot3(geo.xi, d), B = dot3(geo.et, d);
-        const Dw AB = dw_add(A, B);
+        Dw B{0.0f, 0.0f}, AB;
+        if (F64) {
+            B = dot3(geo.et, d);
+            AB = dw_add(dot3(geo.xi, d), B);
+        } else {
+            AB = dot3(geo.y, d);
+        }
         const float eta = fmaxf(fmaxf(fabsf(geo.et[0].h), fabsf(geo.et[1].h)), fabsf(geo.et[2].h));
         const bool ok = fabsf(geo.x.h) < kW3XMax && eta * il.x < 0x1.0p-6f && fabsf(AB.h) < 1e30f;
         if (!alive) continue;
@@ -285,17 +300,22 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
                 const float2 cv = __ldg(a.cb + slot);
                 i3 = dw_mul(i3, Dw{cv.x, cv.y});
                 zc = dw_mul(zc, Dw{cv.x, cv.y});
-                ed *= __ldg(a.cbond + slot);
+                if (F64) ed *= __ldg(a.cbond + slot);
             }
-            acc[0] = fma(ed, e0, acc[0]);
-            acc[1] = fma(ed, e1, acc[1]);
-            acc[2] = fma(ed, e2, acc[2]);
-            const Dw al = dw_mul(dw_add(B, qAB), i3), be = dw_mul(dw_add(AB, qAB), i3);
+            const Dw be = dw_mul(dw_add(AB, qAB), i3);
+            Dw al{0.0f, 0.0f};
+            if (F64) {
+                acc[0] = fma(ed, e0, acc[0]);
+                acc[1] = fma(ed, e1, acc[1]);
+                acc[2] = fma(ed, e2, acc[2]);
+                al = dw_mul(dw_add(B, qAB), i3);
+            }
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const Dw zd = dw_mul(zc, d[k]);
-                const Dw f = dw_add(dw_add(dw_mul(geo.xi[k], al), dw_mul(geo.et[k], be)),
-                                    Dw{-zd.h, -zd.l});
+                const Dw v = F64 ? dw_add(dw_mul(geo.xi[k], al), dw_mul(geo.et[k], be))
+                                 : dw_mul(geo.y[k], be);
+                const Dw f = dw_add(v, Dw{-zd.h, -zd.l});
                 cor[k] = dw_add(cor[k], f);
             }
         } else {
@@ -437,7 +457,11 @@ cudaError_t launch_adj_prep_w3(const AdjW3Args& a, double dt, double ws, int64_t
 
 cudaError_t launch_adj_step_w3(const AdjW3Args& a, cudaStream_t s)
 {
-    const void* fn = a.uniform_w ? (const void*)k_adj_step_w3<true> : (const void*)k_adj_step_w3<false>;
+    const void* fn = a.e != nullptr
+                         ? a.uniform_w ? (const void*)k_adj_step_w3<true, true>
+                                       : (const void*)k_adj_step_w3<false, true>
+                     : a.uniform_w ? (const void*)k_adj_step_w3<true, false>
+                                   : (const void*)k_adj_step_w3<false, false>;
     void* args[] = {const_cast<AdjW3Args*>(&a)};
     return launch_pdl(fn, dim3((unsigned)((a.n + 31) / 32)), dim3(32 * kTeam), args, 0, s);
 }

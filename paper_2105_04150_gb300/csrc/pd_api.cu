@@ -2167,16 +2167,20 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         if ((e = h->alloc(&T.partial, (size_t)T.n_partial)) != cudaSuccess)
             return cuda_fail(e, "cudaMalloc reduction scratch");
     }
-    if (!T.e) {
+    if (!T.wmax) {
         for (int k = 0; k < 2; ++k)
             if ((e = h->alloc(&T.rrec[k], (size_t)(4 * h->n_pad))) != cudaSuccess ||
                 (e = h->alloc(&T.wrec[k], (size_t)(2 * h->n_pad))) != cudaSuccess ||
                 (e = h->alloc(&T.w64[k], (size_t)(4 * h->n_pad))) != cudaSuccess)
                 return cuda_fail(e, "cudaMalloc adjoint records");
-        if ((e = h->alloc(&T.wmax, 1)) != cudaSuccess ||
-            (e = h->alloc(&T.e, (size_t)(3 * slots))) != cudaSuccess)
+        if (!h->dw) {
+            if ((e = h->alloc(&T.e, (size_t)(3 * slots))) != cudaSuccess)
+                return cuda_fail(e, "cudaMalloc adjoint records");
+            PD_CUDA(launch_adj_e(h->rec[0], h->nbr, h->n_slices, h->Q, T.e, h->stream),
+                    "bond vectors");
+        }
+        if ((e = h->alloc(&T.wmax, 1)) != cudaSuccess)
             return cuda_fail(e, "cudaMalloc adjoint records");
-        PD_CUDA(launch_adj_e(h->rec[0], h->nbr, h->n_slices, h->Q, T.e, h->stream), "bond vectors");
     }
     // seed: dL/du^N, dL/dv^N in library order
     auto to_lib = [&](const double* src, double* dst) -> pd_status {
