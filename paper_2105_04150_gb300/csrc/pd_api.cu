@@ -773,7 +773,12 @@ pd_status upload_weights(pd_handle* h)
     PD_CUDA(launch_set_weights(h->precision, w0, w1, h->vol, h->nbr, h->bits0, h->sw, h->n, h->Q,
                                wscale, h->wsum_inv, h->stream),
             "set weights");
-    if (h->w3)
+    if (h->w3 && h->dw)
+        PD_CUDA(launch_damage_intact_dw(h->uniform_vol && !h->batch, w3_args(h).w_ref, h->rec[0],
+                                        h->nbr, h->bits0, h->sw, (const double*)h->wsum_inv, h->n,
+                                        h->Q, h->phi0, h->stream),
+                "intact damage");
+    else if (h->w3)
         PD_CUDA(launch_damage(64, w0, h->nbr, h->bits0, h->sw, h->wsum_inv, nullptr, h->n, h->Q,
                               nullptr, h->phi0, h->stream),
                 "intact damage");
@@ -2054,7 +2059,7 @@ pd_status pd_damage(pd_handle* h, double* phi)
     if (h->damage_fresh)  // written by the last step kernel (fused)
         PD_CUDA(launch_gather_damage(h->precision, h->damage, h->gid, h->n, dst, h->stream),
                 "damage");
-    else if (h->w3)
+    else if (h->w3 && !h->dw)
         PD_CUDA(launch_damage_lost(h->uniform_vol, h->rec[0], h->nbr, h->bits, h->bits0,
                                    (const double*)h->wsum_inv, h->phi0, h->gid, h->n, h->Q, dst,
                                    h->stream),

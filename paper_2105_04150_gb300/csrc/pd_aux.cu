@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "pd_dw.h"
 #include "pd_internal.h"
 
 namespace pd {
@@ -192,6 +193,38 @@ __global__ void k_damage(const void* __restrict__ wrec, const int32_t* __restric
     }
 }
 
+// The damage of intact families on double-word handles: zero up to the rounding of
+// the weight sum as those handles form it (the count times w, or a double-word sum in
+// slot order), which is kept as k_damage's is for FP64 handles.
+__global__ void k_damage_intact_dw(bool uniform_w, double w_const, const double* __restrict__ rec,
+                                   const int32_t* __restrict__ nbr,
+                                   const uint32_t* __restrict__ bits0,
+                                   const int32_t* __restrict__ sw,
+                                   const double* __restrict__ wsum_inv, int64_t n, int Q,
+                                   double* __restrict__ phi)
+{
+    const int64_t W = 32LL * Q;
+    GRID_STRIDE(p, ((n + 31) >> 5) << 5)
+    {
+        const int64_t g = p >> 5;
+        const int lane = (int)(p & 31);
+        int count = 0;
+        dwa::Dw ws{0.0f, 0.0f};
+        for (int m = 0; m < sw[g]; ++m) {
+            if (!((bits0[(g * Q + (m >> 5)) * 32 + lane] >> (m & 31)) & 1u)) continue;
+            ++count;
+            const double w = rec[8 * (int64_t)nbr[(g * W + m) * 32 + lane] + 3];
+            const float wh = (float)w;
+            const dwa::Dw t = dwa::two_sum(ws.h, wh);
+            ws.h = t.h;
+            ws.l += t.l + (float)(w - (double)wh);
+        }
+        const double sum = uniform_w ? w_const * (double)count : (double)ws.h + (double)ws.l;
+        const double wi = wsum_inv[p];
+        if (p < n) phi[p] = wi > 0.0 ? fmax(0.0, 1.0 - sum * wi) : 0.0;
+    }
+}
+
 __global__ void k_damage_lost(bool uniform_w, const double* __restrict__ rec,
                               const int32_t* __restrict__ nbr, const uint32_t* __restrict__ bits,
                               const uint32_t* __restrict__ bits0,
@@ -344,6 +377,16 @@ cudaError_t launch_damage(int precision, const void* wrec, const int32_t* nbr,
     else
         k_damage<double><<<g, 256, 0, s>>>(wrec, nbr, bits, sw, (const double*)wsum_inv, gid, n,
                                            Q, (const double*)integ, phi_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_damage_intact_dw(bool uniform_w, double w_const, const double* rec,
+                                    const int32_t* nbr, const uint32_t* bits0, const int32_t* sw,
+                                    const double* wsum_inv, int64_t n, int Q, double* phi,
+                                    cudaStream_t s)
+{
+    k_damage_intact_dw<<<grid_for(((n + 31) >> 5) << 5, 256), 256, 0, s>>>(
+        uniform_w, w_const, rec, nbr, bits0, sw, wsum_inv, n, Q, phi);
     return cudaGetLastError();
 }
 

@@ -650,6 +650,10 @@ cudaError_t launch_damage(int precision, const void* wrec, const int32_t* nbr,
                           const int32_t* gid, int64_t n, int Q, const void* integ,
                           double* phi_out, cudaStream_t s);
 // the same for the FP64 step's handles, as its kernel writes it (damage_lost)
+cudaError_t launch_damage_intact_dw(bool uniform_w, double w_const, const double* rec,
+                                    const int32_t* nbr, const uint32_t* bits0, const int32_t* sw,
+                                    const double* wsum_inv, int64_t n, int Q, double* phi,
+                                    cudaStream_t s);
 cudaError_t launch_damage_lost(bool uniform_w, const double* rec, const int32_t* nbr,
                                const uint32_t* bits, const uint32_t* bits0, const double* wsum_inv,
                                const double* phi0, const int32_t* gid, int64_t n, int Q,
