@@ -650,7 +650,7 @@ pd_status encode_lat_tma(pd_handle* h, int shape)
 // whatever the model's size, so a model with fewer slices than the chip holds warps
 // (16 per SM) shares each among 8, 4 or 2 as long as that fills the chip only once.
 // Past that, two warps per slice where they leave a last wave that one would not fill.
-// us per step with 1 / 2 / 4 / 8 warps: 125 slices 45.6 / 29.3 / 18.0 / 12.5, 422
+// us per step with 1 / 2 / 4 / 8 warps (blocks of 256): 125 slices 45.6 / 29.3 / 18.0 / 12.5, 422
 // slices 45 / 29 / 26 / 30, 1000: 46 / 45 / 48 / 53, 2695: 120 / 110 / 126 / 130, 4160:
 // 159 / 181 / 175 / 200, 6075: 241 / 228 / 250 / 286, 9000: 320 / 329 / 371 / 421 (the
 // barrier and the shared sums).

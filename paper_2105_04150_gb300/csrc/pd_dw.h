@@ -1,5 +1,5 @@
-// Double-word arithmetic for the FP64-grade kernels (pd_step_f64.cu, pd_adjoint_w3.cu,
-// pd_step_dw.cu, pd_step_osb_dw.cu), device code only.
+// Double-word arithmetic for the FP64-grade kernels (pd_step_f64.cu, pd_step_osb_w3.cu,
+// pd_adjoint_w3.cu, pd_step_dw.cu), device code only.
 //
 // A double-word is an unevaluated sum h + l of two FP32 numbers (Dekker 1971;
 // Knuth's two-sum; the products and error bounds of Joldes, Muller & Popescu,

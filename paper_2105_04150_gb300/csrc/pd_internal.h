@@ -29,9 +29,9 @@
 // FP64 path:
 //   rec[2] 8 doubles per node {x, y, z, w, ux, uy, uz, 0}, double buffered
 //   v      double velocity, 3 per node
-//   Bond-based handles without softening (and PD_PREC_DW ones) add 64-byte three-word
-//   copies of the records for the neighbours and U / |xi| per slot, see W3Args; the other
-//   PD_PREC_DW handles 64-byte double-word copies and |xi| per slot, see DwArgs.
+//   Handles without softening add 64-byte three-word copies of the records for the
+//   neighbours and U / |xi| per slot, see W3Args; PD_PREC_DW handles with softening
+//   64-byte double-word copies and |xi| per slot, see DwArgs.
 #pragma once
 
 #include <algorithm>
@@ -369,7 +369,7 @@ struct W3Args {
     int32_t max_seg;           // segments of the largest family
 };
 
-// Double-word (FP64-grade) step of FP64 handles created with PD_PREC_DW
+// Double-word (FP64-grade) step of PD_PREC_DW handles with softening
 // (pd_step_dw.cu): neighbour records and per-slot reference lengths
 struct DwArgs {
     const float4* rec[2];      // 4 float4 per node, double buffered like the FP64 records

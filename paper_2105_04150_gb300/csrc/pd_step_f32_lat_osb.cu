@@ -1,6 +1,6 @@
 // Ordinary state-based model (the linear peridynamic solid, section
 // "State-based Peridynamics"; the FP64 form and the formulas are in
-// pd_step_osb.cu) on a regular lattice: the two loops of the step as stencil
+// pd_step_osb_w3.cu) on a regular lattice: the two loops of the step as stencil
 // kernels over the lattice layout of pd_step_f32_lat.cu (no neighbour ids,
 // xi = kappa o, FP64 displacement published to the bond arithmetic rounded to
 // FP32).  Lengths in horizon units; with m~_i = sum_j |xi~|^2 V_j the weighted

@@ -8,7 +8,7 @@ namespace pd {
 namespace {
 // ---------------------------------------------------------------------------
 // Ordinary state-based model in FP32 (the FP64 form and the formulas are in
-// pd_step_osb.cu).  Lengths in horizon units: e = |y| - |xi| comes out of the
+// pd_step_osb_w3.cu).  Lengths in horizon units: e = |y| - |xi| comes out of the
 // cancellation-free bond terms as num |xi| / den (den = |xi| (|xi| + |y|)), so
 // the dilation's |xi| e = num |xi|^2 / den needs no length at all and the force
 // forms |xi| from |xi|^2 with one reciprocal square root: no per-slot length
