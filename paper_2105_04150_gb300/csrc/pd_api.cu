@@ -546,6 +546,7 @@ W3Args w3_args(pd_handle* h)
     d.x_grid = h->w3_x_grid;
     d.dt_rho = h->dt / h->rho;
     d.x_hi = h->frozen ? kW3XMax : w3_x_hi(h->sc_lo);
+    d.wide = h->dw ? 1 : 0;
     d.uniform_w = h->uniform_vol ? 1 : 0;
     d.team = h->team;
     d.max_seg = h->Q * (32 / kW3Seg);
@@ -567,8 +568,8 @@ cudaError_t publish64(pd_handle* h, int b)
 const void* step_kernel_fn(pd_handle* h)
 {
     if (h->precision == 32) return f32_kernel(h);
-    if (h->model == 1) return osb_w3_force_kernel(h->uniform_vol);
-    if (h->w3) return step_f64_kernel(h->uniform_vol, h->team > 1);
+    if (h->model == 1) return osb_w3_force_kernel(h->uniform_vol, h->dw);
+    if (h->w3) return step_f64_kernel(h->uniform_vol, h->team > 1, h->dw);
     if (h->dw)
         return step_dw_kernel(h->sc_mode, h->uniform_vol && !h->batch,
                               h->integrator == PD_INTEGRATOR_VV);

@@ -344,6 +344,7 @@ constexpr int kW3Seg = 16;             // slots of a family whose forces are sum
 constexpr int kW3TeamSegs = 256 / kW3Seg;  // largest family, in segments, that a team takes
 constexpr float kW3XMax = 0x1.0p-6f;   // largest |x|, x = |y|^2 / |xi|^2 - 1, of the double-word
                                        // bond arithmetic (see pd_w3.h)
+constexpr float kW3EtaMax = 0x1.0p-7f; // FP64 handles: largest |eta_c| / |xi| of it (see pd_w3.h)
 constexpr int kW3UGrid = -22;          // exponent of the displacements' grid below 4 U
 // the record's x at which the literal evaluation takes over: a band below the stretch
 // s_lo at which a bond can first break or soften, never past kW3XMax
@@ -364,6 +365,7 @@ struct W3Args {
     double dt_rho;             // dt / rho
     int32_t x_grid;            // exponent of the positions' grid (batches: per instance)
     float x_hi;                // w3_x_hi (batches: per instance); kW3XMax while frozen
+    int32_t wide;              // 1: PD_PREC_DW, whose bonds have no bound on eta (see pd_w3.h)
     int32_t uniform_w;         // 1: every node has weight w_ref
     int32_t team;              // warps per slice
     int32_t max_seg;           // segments of the largest family
@@ -398,7 +400,7 @@ cudaError_t launch_osb_w3_setup(const StepArgsF64& a, const OsbW3Args& o, const 
                                 cudaStream_t s);
 cudaError_t launch_osb_w3_step(const StepArgsF64& a, const W3Args& d, const OsbW3Args& o, int grid,
                                int block, cudaStream_t s);
-const void* osb_w3_force_kernel(bool uniform_w);
+const void* osb_w3_force_kernel(bool uniform_w, bool wide);
 
 // Shared-memory tile step of single bond-based lattice models
 // (pd_step_f32_lat_tma.cu): a block per box of BZ x BY x BX nodes, the box's
@@ -593,7 +595,7 @@ const void* step_f32_kernel_lat_batch_r80(int sc_mode, bool per_bond_c);
 cudaError_t launch_step_f32_soft(const StepArgsF32& a, int sc_mode, int grid, int block,
                                  cudaStream_t s);
 const void* step_f32_kernel_soft(int sc_mode, bool uniform_w, bool per_bond_c);
-const void* step_f64_kernel(bool uniform_w, bool team);
+const void* step_f64_kernel(bool uniform_w, bool team, bool wide);
 // literal FP64 step of the models with softening (pd_step_f64_soft.cu)
 cudaError_t launch_step_f64_soft(const StepArgsF64& a, int grid, int block, cudaStream_t s);
 const void* step_f64_soft_kernel(int sc_mode);

@@ -112,7 +112,7 @@ __device__ __noinline__ uint32_t literal_segment(const StepArgsF64& a, int cur, 
 // prefetch to L1 has no effect), so the walk is software-pipelined across segments:
 // a record's registers are free after kin(), and the next chunk's loads go out
 // there, behind them the coefficients and forces of the current one.
-template <bool UW, bool TEAM>
+template <bool UW, bool TEAM, bool WIDE>
 __device__ __forceinline__ void walk(const StepArgsF64& a, const W3Args& d, int cur,
                                      const Own2& own, float x_hi, float ts, int64_t i, int64_t g,
                                      int rank, int team, int Wg, Sums* S)
@@ -147,12 +147,16 @@ __device__ __forceinline__ void walk(const StepArgsF64& a, const W3Args& d, int 
         const bool more = mn < Wg;
         const int b = m & (kSeg - 1);
         if (b == 0) word = (bw[(m >> 5) * 32] >> (m & 31)) & ((1u << kSeg) - 1u);
-        const Kin bA = kin(own, A, both(ts), make_float2(ts, 1.0f));
+        // (a turned bond's x becomes infinite; held until literal_of as one more word, its
+        // eta costs a 220k-node step 253 instead of 241 us, 237 without the bound)
+        Kin bA = kin(own, A, both(ts), make_float2(ts, 1.0f));
+        if (!WIDE && turned(bA.e, il.x)) bA.num.h = INFINITY;
         if (more) {
             dwa::ld_rec(R + 4 * (int64_t)n0, A.a0, A.a1);
             dwa::ld_rec(R + 4 * (int64_t)n0 + 2, A.b0, A.b1);
         }
-        const Kin bB = kin(own, B, both(ts), make_float2(ts, 1.0f));
+        Kin bB = kin(own, B, both(ts), make_float2(ts, 1.0f));
+        if (!WIDE && turned(bB.e, il.y)) bB.num.h = INFINITY;
         const float4 ilc = il;
         const int32_t c0 = j0, c1 = j1;
         const int mc = m;
@@ -172,9 +176,8 @@ __device__ __forceinline__ void walk(const StepArgsF64& a, const W3Args& d, int 
             }
         }
         Coef2 cf = coef2(bA.num, bB.num, ilc);
-        // literal evaluation: near or past s_c, past kW3XMax, or not a number
-        const bool litA = !(cf.x.x < x_hi) || !(cf.x.x > -kW3XMax);
-        const bool litB = !(cf.x.y < x_hi) || !(cf.x.y > -kW3XMax);
+        const uint32_t live = (word >> b) & 3u;
+        const uint32_t lit = literal_of<WIDE>(cf.x, x_hi, live);
         if (d.cb != nullptr) {  // per-bond stiffness (a uniform branch)
             const float2* cb = d.cb + (g * 32LL * Q + mc) * 32 + lane;
             const float2 cA = __ldg(cb), cB = __ldg(cb + 32);
@@ -184,10 +187,9 @@ __device__ __forceinline__ void walk(const StepArgsF64& a, const W3Args& d, int 
             const float2 wA = __ldg(d.wrel + c0), wB = __ldg(d.wrel + c1);
             cf.c = dw_mul2(cf.c, Dw2{make_float2(wA.x, wB.x), make_float2(wA.y, wB.y)});
         }
-        const uint32_t wb = word >> b;
-        pend |= (((litA ? 1u : 0u) | (litB ? 2u : 0u)) & wb) << b;
-        add_force(F, cf.c.h.x, cf.c.l.x, bA, (wb & 1u) && !litA);
-        add_force(F, cf.c.h.y, cf.c.l.y, bB, (wb & 2u) && !litB);
+        pend |= lit << b;
+        add_force(F, cf.c.h.x, cf.c.l.x, bA, (live & ~lit) & 1u);
+        add_force(F, cf.c.h.y, cf.c.l.y, bB, (live & ~lit) & 2u);
 
         if (b == kSeg - 2 || !more) {  // the segment's end
             const int m_lo = mc & ~(kSeg - 1);
@@ -214,7 +216,7 @@ __device__ __forceinline__ void walk(const StepArgsF64& a, const W3Args& d, int 
     }
 }
 
-template <bool UW, bool TEAM>
+template <bool UW, bool TEAM, bool WIDE>
 __global__ void __launch_bounds__(256, 2)
     k_step_f64(const __grid_constant__ StepArgsF64 a, const __grid_constant__ W3Args d)
 {
@@ -277,7 +279,7 @@ __global__ void __launch_bounds__(256, 2)
                 for (int k = 0; k < 3; ++k) S->lit[k][lane] = 0.0;
                 S->info[lane] = 0;
             }
-            walk<UW, TEAM>(a, d, cur, own, x_hi, ts, i, g, rank, team, Wg, S);
+            walk<UW, TEAM, WIDE>(a, d, cur, own, x_hi, ts, i, g, rank, team, Wg, S);
             if (rank == 0) nd = load_node(a, d, cur, i);  // (node arrays are padded)
         }
         if (TEAM) __syncthreads();
@@ -378,18 +380,20 @@ int step_f64_carveout(int team, int max_seg, int block)
     return (int)std::min<size_t>(100, 1 + 100 * resident / (228 << 10));
 }
 
-const void* step_f64_kernel(bool uniform_w, bool team)
+const void* step_f64_kernel(bool uniform_w, bool team, bool wide)
 {
-    static const void* const k[4] = {
-        (const void*)k_step_f64<false, false>, (const void*)k_step_f64<false, true>,
-        (const void*)k_step_f64<true, false>, (const void*)k_step_f64<true, true>};
-    return k[(uniform_w ? 2 : 0) + (team ? 1 : 0)];
+    static const void* const k[8] = {
+        (const void*)k_step_f64<false, false, false>, (const void*)k_step_f64<false, true, false>,
+        (const void*)k_step_f64<true, false, false>,  (const void*)k_step_f64<true, true, false>,
+        (const void*)k_step_f64<false, false, true>,  (const void*)k_step_f64<false, true, true>,
+        (const void*)k_step_f64<true, false, true>,   (const void*)k_step_f64<true, true, true>};
+    return k[(wide ? 4 : 0) + (uniform_w ? 2 : 0) + (team ? 1 : 0)];
 }
 
 cudaError_t launch_step_f64(const StepArgsF64& a, const W3Args& d, int grid, int block,
                             cudaStream_t s)
 {
-    const void* fn = step_f64_kernel(d.uniform_w != 0, d.team > 1);
+    const void* fn = step_f64_kernel(d.uniform_w != 0, d.team > 1, d.wide != 0);
     void* args[] = {const_cast<StepArgsF64*>(&a), const_cast<W3Args*>(&d)};
     return launch_pdl(fn, dim3(grid), dim3(block), args, step_f64_smem(d.team, d.max_seg, block), s,
                       step_f64_carveout(d.team, d.max_seg, block));

@@ -169,11 +169,16 @@ __device__ __forceinline__ Stretch2 w_of(Dw2 num, const float4 il)
     return {x.h, Dw2{w0, mul2(R, fma2(x.h, both(0.125f), both(-0.25f)))}};
 }
 
-// live bonds past the double-word form's range (or not numbers)
-__device__ __forceinline__ uint32_t literal_of(float2 x, float x_hi, uint32_t live)
+// literal_of with the turned bonds of FP64 handles (here the infinite x of pd_step_f64.cu
+// is the slower form: 494 against 473 us a step of 220k nodes)
+template <bool WIDE>
+__device__ __forceinline__ uint32_t literal_or_turned(float2 x, float eA, float eB, const float4 il,
+                                                      float x_hi, uint32_t live)
 {
-    const bool A = !(x.x < x_hi) || !(x.x > -kW3XMax);
-    const bool B = !(x.y < x_hi) || !(x.y > -kW3XMax);
+    if (WIDE) return literal_of<true>(x, x_hi, live);
+    const float2 t = mul2(make_float2(eA, eB), make_float2(il.x, il.y));
+    const bool A = !(x.x < x_hi) || !(t.x < kW3EtaMax);
+    const bool B = !(x.y < x_hi) || !(t.y < kW3EtaMax);
     return ((A ? 1u : 0u) | (B ? 2u : 0u)) & live;
 }
 
@@ -218,7 +223,7 @@ __device__ __noinline__ double literal_dilation(const StepArgsF64& a, const OsbW
     return sum;
 }
 
-template <bool UW>
+template <bool UW, bool WIDE>
 __global__ void __launch_bounds__(256, 2)
     k_osb_w3_dilation(const __grid_constant__ StepArgsF64 a, const __grid_constant__ W3Args d,
                       const __grid_constant__ OsbW3Args o)
@@ -246,7 +251,7 @@ __global__ void __launch_bounds__(256, 2)
             [&](int32_t c0, int32_t c1, const KinNum& A, const KinNum& B, const float4 il, uint32_t live) {
                 const Dw2 num{make_float2(A.num.h, B.num.h), make_float2(A.num.l, B.num.l)};
                 const Stretch2 t = w_of(num, il);
-                const uint32_t pend = literal_of(t.x, un.x_hi, live);
+                const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il, un.x_hi, live);
                 const Dw2 hn{mul2(num.h, both(0.5f)), mul2(num.l, both(0.5f))};
                 Dw2 e = dw_add2(hn, dw_mul2(hn, t.z));
                 if (!UW) {
@@ -297,7 +302,7 @@ __device__ __noinline__ void literal_force(const StepArgsF64& a, const OsbW3Args
     }
 }
 
-template <bool UW>
+template <bool UW, bool WIDE>
 __global__ void __launch_bounds__(256, 2)
     k_osb_w3_force(const __grid_constant__ StepArgsF64 a, const __grid_constant__ W3Args d,
                    const __grid_constant__ OsbW3Args o)
@@ -329,7 +334,7 @@ __global__ void __launch_bounds__(256, 2)
                 const float4 p0 = __ldg(o.ab + c0), p1 = __ldg(o.ab + c1);
                 const Stretch2 t = stretch2(
                     Dw2{make_float2(A.num.h, B.num.h), make_float2(A.num.l, B.num.l)}, il);
-                const uint32_t pend = literal_of(t.x, kW3XMax, live);
+                const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il, kW3XMax, live);
                 const Dw2 al = dw_add2(Dw2{both(own_ab.x), both(own_ab.y)},
                                        Dw2{make_float2(p0.x, p1.x), make_float2(p0.y, p1.y)});
                 const Dw2 ga = dw_add2(Dw2{both(own_ab.z), both(own_ab.w)},
@@ -376,17 +381,22 @@ cudaError_t launch_osb_w3_step(const StepArgsF64& a, const W3Args& d, const OsbW
                                int block, cudaStream_t s)
 {
     void* args[] = {const_cast<StepArgsF64*>(&a), const_cast<W3Args*>(&d), const_cast<OsbW3Args*>(&o)};
-    const void* dil = d.uniform_w ? (const void*)k_osb_w3_dilation<true>
-                                  : (const void*)k_osb_w3_dilation<false>;
+    static const void* const dil_k[4] = {
+        (const void*)k_osb_w3_dilation<false, false>, (const void*)k_osb_w3_dilation<true, false>,
+        (const void*)k_osb_w3_dilation<false, true>, (const void*)k_osb_w3_dilation<true, true>};
+    const void* dil = dil_k[(d.wide ? 2 : 0) + (d.uniform_w ? 1 : 0)];
     const cudaError_t e = launch_pdl(dil, dim3(grid), dim3(block), args, 0, s);
     return e != cudaSuccess
                ? e
-               : launch_pdl(osb_w3_force_kernel(d.uniform_w != 0), dim3(grid), dim3(block), args, 0, s);
+               : launch_pdl(osb_w3_force_kernel(d.uniform_w != 0, d.wide != 0), dim3(grid), dim3(block), args, 0, s);
 }
 
-const void* osb_w3_force_kernel(bool uniform_w)
+const void* osb_w3_force_kernel(bool uniform_w, bool wide)
 {
-    return uniform_w ? (const void*)k_osb_w3_force<true> : (const void*)k_osb_w3_force<false>;
+    static const void* const k[4] = {
+        (const void*)k_osb_w3_force<false, false>, (const void*)k_osb_w3_force<true, false>,
+        (const void*)k_osb_w3_force<false, true>, (const void*)k_osb_w3_force<true, true>};
+    return k[(wide ? 2 : 0) + (uniform_w ? 1 : 0)];
 }
 
 }  // namespace pd

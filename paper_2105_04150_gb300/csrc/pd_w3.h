@@ -49,6 +49,13 @@ using dwa::two_sum;
 // to the literal FP64 evaluation of Eq. 4, which has the smaller error there: its
 // stretch carries an absolute rounding error of about 3e-16, i.e. 3e-16 / s of the
 // bond's force, against the 1e-14 of the form below.
+// num = eta . (2 xi + eta) cancels when a bond rotates: its terms of size |eta| |xi|
+// carry 2^-47 each, so s an absolute error (rms, on random lattice bonds) of 2.4e-17,
+// 1.2e-16, 7e-16 and 4.2e-15 at 0.01, 0.05, 0.3 and pi/2 rad, where the literal form
+// keeps 1.1e-16 throughout.  So bonds of FP64 handles with a component of eta past
+// kW3EtaMax |xi| (a rotation of about half a degree, or a compression of 0.8 to 1.4 %)
+// are literal.  PD_PREC_DW, about 1e-13 of the force and no less than 46 bits of |y|, has
+// no such bound.
 
 struct Own {
     float xh[3], xm[3], xk[3], uh[3], um[3], ut[3];
@@ -258,11 +265,18 @@ __device__ __forceinline__ Dw eta_dot(const Pair& p, Dw2 v, Dw vz)
     return dw_add(num, nz);
 }
 
+// the largest |component| of eta
+__device__ __forceinline__ float eta_max(const Pair& p)
+{
+    return fmaxf(fmaxf(fabsf(p.et.h.x), fabsf(p.et.h.y)), fabsf(p.ez.h));
+}
+
 // y = xi + eta and num = eta . (2 xi + eta) of one bond
 struct Kin {
     Dw2 y;   // x, y components
     Dw yz;
     Dw num;
+    float e;  // eta_max
 };
 __device__ __forceinline__ Kin kin(const Own2& o, const Rec& j, float2 ts2, float2 tsz)
 {
@@ -271,18 +285,21 @@ __device__ __forceinline__ Kin kin(const Own2& o, const Rec& j, float2 ts2, floa
     k.y = dw_add2(p.xi, p.et);
     k.yz = dw_add(p.xz, p.ez);
     k.num = eta_dot(p, dw_add2(p.xi, k.y), dw_add(p.xz, k.yz));
+    k.e = eta_max(p);
     return k;
 }
 
 // num alone: without y, 24 operations less
 struct KinNum {
     Dw num;
+    float e;
 };
 __device__ __forceinline__ KinNum kin_num(const Own2& o, const Rec& j, float2 ts2, float2 tsz)
 {
     const Pair p = pair_of(o, j, ts2, tsz);
     const Dw2 x2{add2(p.xi.h, p.xi.h), add2(p.xi.l, p.xi.l)};
-    return {eta_dot(p, dw_add2(x2, p.et), dw_add(Dw{p.xz.h + p.xz.h, p.xz.l + p.xz.l}, p.ez))};
+    return {eta_dot(p, dw_add2(x2, p.et), dw_add(Dw{p.xz.h + p.xz.h, p.xz.l + p.xz.l}, p.ez)),
+            eta_max(p)};
 }
 
 // x = |y|^2 / |xi|^2 - 1 and z = |xi| / |y| - 1 of two bonds (see bond_geo)
@@ -305,6 +322,20 @@ __device__ __forceinline__ Stretch2 stretch2(Dw2 num, const float4 il)
     const Dw2 xp = dw_mul2(x, p);
     const float2 R = add2(add2(add2(ph, x.h), xp.h), add2(add2(p.l, x.l), xp.l));
     return {x.h, Dw2{z0, mul2(R, fma2(z0, both(-0.5f), both(-0.5f)))}};
+}
+
+// eta past kW3EtaMax (il: the slot's U / |xi|)
+__device__ __forceinline__ bool turned(float e, float il) { return e * il >= kW3EtaMax; }
+
+// Which of two live bonds are to be evaluated literally: near or past s_c or past kW3XMax
+// (x_hi), past -kW3XMax, or not a number.  FP64 handles (not WIDE) take turned bonds out
+// elsewhere, which bounds the compression too.
+template <bool WIDE>
+__device__ __forceinline__ uint32_t literal_of(float2 x, float x_hi, uint32_t live)
+{
+    const bool A = !(x.x < x_hi) || (WIDE && !(x.x > -kW3XMax));
+    const bool B = !(x.y < x_hi) || (WIDE && !(x.y > -kW3XMax));
+    return ((A ? 1u : 0u) | (B ? 2u : 0u)) & live;
 }
 
 // x of two bonds and (1 / |xi|) z = -s / |y|
