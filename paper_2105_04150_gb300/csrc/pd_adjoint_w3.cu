@@ -29,6 +29,8 @@
 // The FP64 pipe needs few warps and a model of this use is small (the recorded run
 // is kept in memory), so a slice is shared by a block of four warps, each taking
 // every fourth slot; their sums are added in a fixed order.
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 #include "pd_internal.h"
@@ -161,9 +163,42 @@ __device__ __forceinline__ Dw dot3(const Dw (&a)[3], const Dw (&b)[3])
     return dw_add(s, dw_mul(a[2], b[2]));
 }
 
+// v in FP64 by integer operations: the conversion instruction takes a turn of the FP64
+// pipe (a step forth and back of a 100k plate 499 us with it, 488 without; 454 with a
+// double-word sum).  Denormal numbers become 0.
+__device__ __forceinline__ double wide_of(float v)
+{
+    const uint32_t b = __float_as_uint(v);
+    const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20));
+    return (b & 0x7f800000u) != 0u ? __hiloint2double((int)hi, (int)(b << 29)) : 0.0;
+}
+
+// The running sum of a slot's dL/dc terms: FP64, or on double-word handles a double-word,
+// renormalised with each term (without that its low word grows with the number of terms
+// and so does its rounding: 2.8e-13 of the sum, rms, after 1500 terms of one sign).
+__device__ __forceinline__ double add_term(double sum, Dw t)
+{
+    return sum + (wide_of(t.h) + wide_of(t.l));
+}
+__device__ __forceinline__ float2 add_term(float2 sum, Dw t)
+{
+    const Dw s = two_sum(sum.x, t.h);
+    const float l = sum.y + (s.l + t.l);
+    const float h = __fadd_rn(s.h, l);
+    return make_float2(h, __fsub_rn(l, __fsub_rn(h, s.h)));
+}
+__device__ __forceinline__ double add_term(double sum, double t) { return sum + t; }
+__device__ __forceinline__ float2 add_term(float2 sum, double t)
+{
+    const float h = (float)t;
+    return add_term(sum, Dw{h, (float)(t - (double)h)});
+}
+
 template <bool UW, bool F64>
 __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_constant__ AdjW3Args a)
 {
+    using Sum = std::conditional_t<F64, double, float2>;
+    Sum* const gc = reinterpret_cast<Sum*>(a.gc);
     __shared__ double sd[kTeam][3][32];
     __shared__ float sf[kTeam][6][32];
     const int lane = threadIdx.x & 31, rank = threadIdx.x >> 5;
@@ -199,7 +234,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         float4 v0, v1;
         float4 il2;
         double e0, e1, e2;
-        float2 gc;
+        Sum gc;
     } in;
     auto load = [&](int b, int64_t j) {
         const int64_t row = g * 32LL * Q + b;  // of 32 slots
@@ -214,7 +249,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             in.e1 = __ldg(ep + 32);
             in.e2 = __ldg(ep + 64);
         }
-        in.gc = a.gc[row * 32 + lane];
+        in.gc = gc[row * 32 + lane];
     };
     uint32_t word = 0u;
     int32_t jc = 0, jn = 0;
@@ -228,7 +263,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         const bool alive = (word >> (b & 31)) & 1u;
         const int64_t j = jc, slot = slot0 + b * 32;
         const float2 il = b & 1 ? make_float2(in.il2.y, in.il2.w) : make_float2(in.il2.x, in.il2.z);
-        const float2 old = in.gc;
+        const Sum old = in.gc;
         float2 rj = make_float2(1.0f, 0.0f);
         if (!UW) rj = __ldg(a.wrel + j);
         const Geo geo = bond_geo(own, in.nb, il, ts);
@@ -279,7 +314,6 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         const float eta = fmaxf(fmaxf(fabsf(geo.et[0].h), fabsf(geo.et[1].h)), fabsf(geo.et[2].h));
         const bool ok = fabsf(geo.x.h) < kW3XMax && eta * il.x < 0x1.0p-6f && fabsf(AB.h) < 1e30f;
         if (!alive) continue;
-        Dw gs;  // the bond's dL/dc in units of V_ref / unit_scale
         if (ok) {
             const Dw iL{il.x, il.y};
             const Dw zL = dw_mul(geo.z, iL);
@@ -293,9 +327,9 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             Dw i3 = dw_mul(iL, dw_mul(iL, iL));
             Dw zc = zL;
             const Dw yw = dot3(geo.y, wd);
-            gs = dw_mul(zL, yw);
+            Dw gs = dw_mul(zL, yw);  // -dL/dc of the bond in units of V_ref / unit_scale
             if (!UW) gs = dw_mul(gs, Dw{rj.x, rj.y});
-            gs = Dw{-gs.h, -gs.l};
+            gc[slot] = add_term(old, Dw{-gs.h, -gs.l});
             if (a.cbond != nullptr) {  // per-bond stiffness (a uniform branch)
                 const float2 cv = __ldg(a.cb + slot);
                 i3 = dw_mul(i3, Dw{cv.x, cv.y});
@@ -320,16 +354,12 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             }
         } else {
             double f[3];
-            const double gd = literal_adj(a, m, j, slot, f) * us;
+            gc[slot] = add_term(old, literal_adj(a, m, j, slot, f) * us);
             const double cij = a.cbond != nullptr ? __ldg(a.cbond + slot) : 1.0;
             acc[0] += cij * f[0];
             acc[1] += cij * f[1];
             acc[2] += cij * f[2];
-            gs.h = (float)gd;
-            gs.l = (float)(gd - (double)gs.h);
         }
-        const Dw t = two_sum(old.x, gs.h);
-        a.gc[slot] = make_float2(t.h, old.y + (t.l + gs.l));
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -418,15 +448,16 @@ __global__ void k_adj_e(const double* __restrict__ x64, const int32_t* __restric
     }
 }
 
-// the double-word per-slot accumulators become FP64, times scale / unit_scale, in place
-__global__ void k_adj_merge_w3(double* gc, int64_t count, double scale,
+// the per-slot sums (double-words unless f64) become FP64, times scale / unit_scale, in place
+__global__ void k_adj_merge_w3(double* gc, int64_t count, double scale, bool f64,
                                const unsigned long long* __restrict__ wmax)
 {
     const double s = scale / unit_scale(wmax);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count;
          e += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(gc[e]);
-        gc[e] = s * ((double)__uint_as_float((uint32_t)b) + (double)__uint_as_float((uint32_t)(b >> 32)));
+        gc[e] = s * (f64 ? gc[e]
+                         : (double)__uint_as_float((uint32_t)b) + (double)__uint_as_float((uint32_t)(b >> 32)));
     }
 }
 
@@ -466,10 +497,10 @@ cudaError_t launch_adj_step_w3(const AdjW3Args& a, cudaStream_t s)
     return launch_pdl(fn, dim3((unsigned)((a.n + 31) / 32)), dim3(32 * kTeam), args, 0, s);
 }
 
-cudaError_t launch_adj_merge_w3(double* gc, int64_t count, double scale,
+cudaError_t launch_adj_merge_w3(double* gc, int64_t count, double scale, bool f64,
                                 const unsigned long long* wmax, cudaStream_t s)
 {
-    k_adj_merge_w3<<<grid_of(count), 256, 0, s>>>(gc, count, scale, wmax);
+    k_adj_merge_w3<<<grid_of(count), 256, 0, s>>>(gc, count, scale, f64, wmax);
     return cudaGetLastError();
 }
 
