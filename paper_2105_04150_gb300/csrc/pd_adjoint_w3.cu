@@ -21,7 +21,8 @@
 // of the whole; it runs on the FP32 pipe beside the FP64 one.  dL/dc needs the
 // stretch, which is more accurate in double-words than in the literal FP64 form
 // (whose s has an absolute error of 3e-16).  Bonds with |eta| / L past 2^-6 or past
-// kW3XMax, or whose w leaves FP32's range, are evaluated literally in FP64.
+// kW3XMax, or whose w leaves FP32's range (kWTiny), are evaluated literally in FP64.  The
+// per-slot sums of dL/dc over the steps are FP64: two additions a bond.
 //
 // PD_PREC_DW handles (F64 false) take K d = y q (A + B) / L^3 - (z / L) d in double-word
 // arithmetic as a whole, to 2^-44 of each bond's term: no FP64 operation and no e.
@@ -29,8 +30,6 @@
 // The FP64 pipe needs few warps and a model of this use is small (the recorded run
 // is kept in memory), so a slice is shared by a block of four warps, each taking
 // every fourth slot; their sums are added in a fixed order.
-#include <type_traits>
-
 #include <cuda_runtime.h>
 
 #include "pd_internal.h"
@@ -74,17 +73,24 @@ __global__ void k_adj_scale(const double* __restrict__ ub, const double* __restr
     if (m > 0.0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
 }
 
-// power of two that brings that component to [1, 2) (1 without seeds)
+// power of two that brings that component to [1, 2), as far as it is a finite number (1
+// without seeds)
 __device__ __forceinline__ double unit_scale(const unsigned long long* m)
 {
     const double v = __longlong_as_double((long long)*m);
-    return v > 0.0 && v < 1e300 ? scalbn(1.0, -ilogb(v)) : 1.0;
+    return v > 0.0 && v < 1e300 ? scalbn(1.0, min(-ilogb(v), 1000)) : 1.0;
 }
+
+// Largest component of a node's w, in that unit, below which FP32 does not hold its
+// products: |s / |y|| |w| has to keep its low word, 2^-24 of it, above 2^-126.  Bonds of such
+// nodes (far from the seeds) are evaluated literally.
+constexpr double kWTiny = 0x1.0p-48;
 
 // The records of a reverse step for node p, from its ubar, vbar and u^n: w = ws (vbar + dt
 // ubar) with the controlled components of ubar and vbar zeroed (as k_adj_mask), the
 // three-word record of x (its words from `fwd`) and u^n, w in FP64 ({w, 0}) and w as
-// double-words in units of 1 / unit_scale ({wh, wl.x} {wl.y, wl.z, 0, 0}).
+// double-words in units of 1 / unit_scale ({wh, wl.x} {wl.y, wl.z, tiny, 0}; tiny is 1 for a
+// w below kWTiny that is not zero).
 __device__ __forceinline__ void adj_records(const AdjW3Args& a, int64_t p, uint32_t mask,
                                             const double (&ub)[3], const double (&vb)[3],
                                             const double* un, double dt, double ws, double us,
@@ -92,7 +98,7 @@ __device__ __forceinline__ void adj_records(const AdjW3Args& a, int64_t p, uint3
 {
     const float tin[3] = {fwd.a1.z, fwd.a1.w, fwd.b1.z};
     float uh[3], um[3], t[3], wh[3], wl[3];
-    double w[3];
+    double w[3], w_max = 0.0;
     for (int k = 0; k < 3; ++k) {
         const bool ctl = (mask >> k) & 1u;
         const double u = ctl ? 0.0 : ub[k];
@@ -102,6 +108,7 @@ __device__ __forceinline__ void adj_records(const AdjW3Args& a, int64_t p, uint3
         float ut;
         split3(un[3 * p + k] * a.scale, kW3UGrid, uh[k], um[k], ut);
         t[k] = pack_t(__float_as_uint(tin[k]) & 0x7ffu, ut);
+        w_max = fmax(w_max, fabs(w[k]));
         const double v1 = w[k] * us;
         wh[k] = (float)v1;
         wl[k] = (float)(v1 - (double)wh[k]);
@@ -114,7 +121,7 @@ __device__ __forceinline__ void adj_records(const AdjW3Args& a, int64_t p, uint3
     dwa::st_rec(rec + 4 * p + 2, make_float4(fwd.b0.x, fwd.b0.y, um[0], um[1]),
                 make_float4(fwd.b1.x, um[2], t[2], 0.0f));
     dwa::st_rec(wdw + 2 * p, make_float4(wh[0], wh[1], wh[2], wl[0]),
-                make_float4(wl[1], wl[2], 0.0f, 0.0f));
+                make_float4(wl[1], wl[2], w_max > 0.0 && w_max * us < kWTiny ? 1.0f : 0.0f, 0.0f));
 }
 
 __global__ void k_adj_prep_w3(const __grid_constant__ AdjW3Args a, double dt, double ws, int64_t n_pad)
@@ -163,9 +170,8 @@ __device__ __forceinline__ Dw dot3(const Dw (&a)[3], const Dw (&b)[3])
     return dw_add(s, dw_mul(a[2], b[2]));
 }
 
-// v in FP64 by integer operations: the conversion instruction takes a turn of the FP64
-// pipe (a step forth and back of a 100k plate 499 us with it, 488 without; 454 with a
-// double-word sum).  Denormal numbers become 0.
+// v in FP64 by integer operations: a conversion instruction takes a turn of the FP64 pipe
+// (2 % of the sweep of a 100k plate).  Denormal numbers become 0.
 __device__ __forceinline__ double wide_of(float v)
 {
     const uint32_t b = __float_as_uint(v);
@@ -173,32 +179,9 @@ __device__ __forceinline__ double wide_of(float v)
     return (b & 0x7f800000u) != 0u ? __hiloint2double((int)hi, (int)(b << 29)) : 0.0;
 }
 
-// The running sum of a slot's dL/dc terms: FP64, or on double-word handles a double-word,
-// renormalised with each term (without that its low word grows with the number of terms
-// and so does its rounding: 2.8e-13 of the sum, rms, after 1500 terms of one sign).
-__device__ __forceinline__ double add_term(double sum, Dw t)
-{
-    return sum + (wide_of(t.h) + wide_of(t.l));
-}
-__device__ __forceinline__ float2 add_term(float2 sum, Dw t)
-{
-    const Dw s = two_sum(sum.x, t.h);
-    const float l = sum.y + (s.l + t.l);
-    const float h = __fadd_rn(s.h, l);
-    return make_float2(h, __fsub_rn(l, __fsub_rn(h, s.h)));
-}
-__device__ __forceinline__ double add_term(double sum, double t) { return sum + t; }
-__device__ __forceinline__ float2 add_term(float2 sum, double t)
-{
-    const float h = (float)t;
-    return add_term(sum, Dw{h, (float)(t - (double)h)});
-}
-
 template <bool UW, bool F64>
 __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_constant__ AdjW3Args a)
 {
-    using Sum = std::conditional_t<F64, double, float2>;
-    Sum* const gc = reinterpret_cast<Sum*>(a.gc);
     __shared__ double sd[kTeam][3][32];
     __shared__ float sf[kTeam][6][32];
     const int lane = threadIdx.x & 31, rank = threadIdx.x >> 5;
@@ -220,6 +203,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
     float4 w0, w1;
     dwa::ld_rec(a.wdw + 2 * m, w0, w1);
     const Dw wd[3] = {{w0.x, w0.w}, {w0.y, w1.x}, {w0.z, w1.y}};
+    const float tiny = w1.z;
     float2 rm = make_float2(1.0f, 0.0f);
     if (!UW) rm = __ldg(a.wrel + m);
     const double vm = UW ? 1.0 : (double)rm.x + (double)rm.y;
@@ -234,7 +218,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         float4 v0, v1;
         float4 il2;
         double e0, e1, e2;
-        Sum gc;
+        double gc;  // the sum of the steps before
     } in;
     auto load = [&](int b, int64_t j) {
         const int64_t row = g * 32LL * Q + b;  // of 32 slots
@@ -249,7 +233,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             in.e1 = __ldg(ep + 32);
             in.e2 = __ldg(ep + 64);
         }
-        in.gc = gc[row * 32 + lane];
+        in.gc = a.gc[row * 32 + lane];
     };
     uint32_t word = 0u;
     int32_t jc = 0, jn = 0;
@@ -263,11 +247,12 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         const bool alive = (word >> (b & 31)) & 1u;
         const int64_t j = jc, slot = slot0 + b * 32;
         const float2 il = b & 1 ? make_float2(in.il2.y, in.il2.w) : make_float2(in.il2.x, in.il2.z);
-        const Sum old = in.gc;
+        const double old = in.gc;
         float2 rj = make_float2(1.0f, 0.0f);
         if (!UW) rj = __ldg(a.wrel + j);
         const Geo geo = bond_geo(own, in.nb, il, ts);
         const Dw wn[3] = {{in.v0.x, in.v0.w}, {in.v0.y, in.v1.x}, {in.v0.z, in.v1.y}};
+        const bool far = tiny + in.v1.z != 0.0f;
         Dw d[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -312,7 +297,8 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             AB = dot3(geo.y, d);
         }
         const float eta = fmaxf(fmaxf(fabsf(geo.et[0].h), fabsf(geo.et[1].h)), fabsf(geo.et[2].h));
-        const bool ok = fabsf(geo.x.h) < kW3XMax && eta * il.x < 0x1.0p-6f && fabsf(AB.h) < 1e30f;
+        const bool ok = fabsf(geo.x.h) < kW3XMax && eta * il.x < 0x1.0p-6f && fabsf(AB.h) < 1e30f &&
+                        !far;
         if (!alive) continue;
         if (ok) {
             const Dw iL{il.x, il.y};
@@ -329,7 +315,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             const Dw yw = dot3(geo.y, wd);
             Dw gs = dw_mul(zL, yw);  // -dL/dc of the bond in units of V_ref / unit_scale
             if (!UW) gs = dw_mul(gs, Dw{rj.x, rj.y});
-            gc[slot] = add_term(old, Dw{-gs.h, -gs.l});
+            a.gc[slot] = old + (wide_of(-gs.h) + wide_of(-gs.l));
             if (a.cbond != nullptr) {  // per-bond stiffness (a uniform branch)
                 const float2 cv = __ldg(a.cb + slot);
                 i3 = dw_mul(i3, Dw{cv.x, cv.y});
@@ -354,7 +340,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             }
         } else {
             double f[3];
-            gc[slot] = add_term(old, literal_adj(a, m, j, slot, f) * us);
+            a.gc[slot] = old + literal_adj(a, m, j, slot, f) * us;
             const double cij = a.cbond != nullptr ? __ldg(a.cbond + slot) : 1.0;
             acc[0] += cij * f[0];
             acc[1] += cij * f[1];
@@ -448,17 +434,14 @@ __global__ void k_adj_e(const double* __restrict__ x64, const int32_t* __restric
     }
 }
 
-// the per-slot sums (double-words unless f64) become FP64, times scale / unit_scale, in place
-__global__ void k_adj_merge_w3(double* gc, int64_t count, double scale, bool f64,
+// the per-slot sums times scale / unit_scale
+__global__ void k_adj_merge_w3(double* gc, int64_t count, double scale,
                                const unsigned long long* __restrict__ wmax)
 {
     const double s = scale / unit_scale(wmax);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(gc[e]);
-        gc[e] = s * (f64 ? gc[e]
-                         : (double)__uint_as_float((uint32_t)b) + (double)__uint_as_float((uint32_t)(b >> 32)));
-    }
+         e += (int64_t)gridDim.x * blockDim.x)
+        gc[e] *= s;
 }
 
 }  // namespace
@@ -497,10 +480,10 @@ cudaError_t launch_adj_step_w3(const AdjW3Args& a, cudaStream_t s)
     return launch_pdl(fn, dim3((unsigned)((a.n + 31) / 32)), dim3(32 * kTeam), args, 0, s);
 }
 
-cudaError_t launch_adj_merge_w3(double* gc, int64_t count, double scale, bool f64,
+cudaError_t launch_adj_merge_w3(double* gc, int64_t count, double scale,
                                 const unsigned long long* wmax, cudaStream_t s)
 {
-    k_adj_merge_w3<<<grid_of(count), 256, 0, s>>>(gc, count, scale, f64, wmax);
+    k_adj_merge_w3<<<grid_of(count), 256, 0, s>>>(gc, count, scale, wmax);
     return cudaGetLastError();
 }
 

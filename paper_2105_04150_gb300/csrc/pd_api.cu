@@ -2318,7 +2318,7 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         }
     }
     if (ke == cudaSuccess)
-        ke = launch_adj_merge_w3(T.gc, slots, dt_rho * h->vol0, !h->dw, T.wmax, h->stream);
+        ke = launch_adj_merge_w3(T.gc, slots, dt_rho * h->vol0, T.wmax, h->stream);
     h->frozen = false;
     h->drop_graph();
     // restore the final state u^N, v^N

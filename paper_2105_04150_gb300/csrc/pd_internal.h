@@ -517,8 +517,7 @@ struct AdjW3Args {
     const double* ilen;        // per slot 1 / |xi|
     const double* e;           // per slot xi / |xi|^(3/2), rows of 32 lanes per component
     const float4* il;          // W3Args::il
-    double* gc;                // per-slot sum of dL/dc; double-words without e, and merged
-                               // to FP64 in place
+    double* gc;                // per-slot sum of dL/dc
     double* gl;                // per-node accumulator of force . w
     const uint8_t* bcc;
     const BcClass* bct;
@@ -538,7 +537,7 @@ cudaError_t launch_adj_e(const double* x64, const int32_t* nbr, int64_t n_slices
 cudaError_t launch_adj_prep_w3(const AdjW3Args& a, double dt, double ws, int64_t n_pad,
                                cudaStream_t s);
 cudaError_t launch_adj_step_w3(const AdjW3Args& a, cudaStream_t s);
-cudaError_t launch_adj_merge_w3(double* gc, int64_t count, double scale, bool f64,
+cudaError_t launch_adj_merge_w3(double* gc, int64_t count, double scale,
                                 const unsigned long long* wmax, cudaStream_t s);
 
 cudaError_t launch_adj_mask(const double* ub, const double* vb, const uint8_t* bcc,

@@ -5,11 +5,8 @@ and swept by itself with the gradient that the step after it left, so they are t
 of the long sweep bit for bit (the scale of the double-words is a power of two).  Their
 sum in long double is compared with the long sweep's dL/dc.
 
-PD_PREC_F64 sums in FP64, one rounding of at most 2^-53 of the running sum a step, and
-scales the result by dt/rho V and 1/scale (each single term too): (N + 8) 2^-53 sum |g_k|.
-PD_PREC_DW sums in double-words: the two sums of low words round, each by at most half an
-ulp of 2^-24 of the running sum or twice that, 1.3 2^-48 sum |g_k| rms a step, and the
-steps' roundings are independent: 1.3 sqrt(N) 2^-48 sum |g_k| rms over the bonds."""
+The sum is an FP64 one, one rounding of at most 2^-53 of the running sum a step, and the
+result is scaled by dt/rho V and 1/scale (each single term too): (N + 8) 2^-53 sum |g_k|."""
 import numpy as np
 import pytest
 
@@ -63,7 +60,4 @@ def test_stiffness_gradient_is_the_sum_of_its_steps(precision, jitter):
     assert np.array_equal(du, du1) and np.array_equal(dv, dv1)
     assert (abs_total > 0).all()
     rel = np.abs(np.asarray(g - total, np.float64)) / abs_total
-    if precision == pdgb.PD_PREC_F64:
-        assert rel.max() <= (N + 8) * 2.0 ** -53
-    else:
-        assert np.sqrt(np.mean(rel ** 2)) <= 1.3 * np.sqrt(N) * 2.0 ** -48
+    assert rel.max() <= (N + 8) * 2.0 ** -53
