@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
                 s += sd[r][k][lane];
                 c = dw_add(c, Dw{sf[r][2 * k][lane], sf[r][2 * k + 1][lane]});
             }
-            s += ((double)c.h + (double)c.l) * (a.scale / us);
+            s = fma(s, a.inv_c_ref, ((double)c.h + (double)c.l) * (a.scale / us));
             ub[k] = a.ubm[3 * m + k] + (a.dt_rho * a.w_ref) * s;
             vb[k] = a.damp * w3[k];
             a.ub_out[3 * m + k] = ub[k];

@@ -139,6 +139,7 @@ struct pd_handle {
     float4* rec3[2] = {nullptr, nullptr};
     float4* il3 = nullptr;
     float2 *cb3 = nullptr, *wrel3 = nullptr;
+    double c_ref = 1.0;     // unit of cb3
     double* phi0 = nullptr; // per node the damage of an intact family
     int32_t* fam3 = nullptr;  // per node its bonds
     double w3_scale = 1.0;  // 1 / U, a power of two (batches: per instance in itab)
@@ -541,7 +542,7 @@ W3Args w3_args(pd_handle* h)
     d.wrel = h->wrel3;
     d.phi0 = h->phi0;
     d.fam = h->fam3;
-    d.w_ref = ((h->per_bond_c || h->model == 1) ? 1.0 : h->c) * h->vol0;
+    d.w_ref = (h->per_bond_c ? h->c_ref : h->model == 1 ? 1.0 : h->c) * h->vol0;
     d.scale = h->w3_scale;
     d.x_grid = h->w3_x_grid;
     d.dt_rho = h->dt / h->rho;
@@ -775,7 +776,7 @@ pd_status upload_weights(pd_handle* h)
                                wscale, h->wsum_inv, h->stream),
             "set weights");
     if (h->w3 && h->dw)
-        PD_CUDA(launch_damage_intact_dw(h->uniform_vol && !h->batch, w3_args(h).w_ref, h->rec[0],
+        PD_CUDA(launch_damage_intact_dw(h->uniform_vol && !h->batch, wscale * h->vol0, h->rec[0],
                                         h->nbr, h->bits0, h->sw, (const double*)h->wsum_inv, h->n,
                                         h->Q, h->phi0, h->stream),
                 "intact damage");
@@ -2237,7 +2238,8 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         A.bcc = h->bcc;
         A.bct = h->bct;
         A.scale = h->w3_scale;
-        A.w_ref = (h->per_bond_c ? 1.0 : h->c) * h->vol0;
+        A.w_ref = (h->per_bond_c ? h->c_ref : h->c) * h->vol0;
+        A.inv_c_ref = h->per_bond_c ? 1.0 / h->c_ref : 1.0;
         A.inv_vref = 1.0 / h->vol0;
         A.dt_rho = dt_rho;
         A.n = h->n;
@@ -2560,7 +2562,15 @@ pd_status pd_set_params(pd_handle* h, double c, double sc, double load, double d
                     cudaError_t e = h->alloc(&dst, slots);
                     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc c_bond");
                 }
-                PD_CUDA(launch_dw_split((const double*)h->cbond, (int64_t)slots, dst, h->stream),
+                double unit = 1.0;
+                if (h->w3) {
+                    const double top = *std::max_element(cb.begin(), cb.end());
+                    if (top > 0.0)
+                        unit = std::ldexp(1.0, std::max(-1000, std::min(1000, std::ilogb(top))));
+                    h->c_ref = unit;
+                }
+                PD_CUDA(launch_dw_split((const double*)h->cbond, (int64_t)slots, 1.0 / unit, dst,
+                                        h->stream),
                         "double-word c_bond");
             }
         }

@@ -356,11 +356,13 @@ inline float w3_x_hi(double s_lo)
 struct W3Args {
     const float4* rec[2];      // 4 float4 per node, double buffered like the FP64 records
     const float4* il;          // per pair of slots U / |xi| as double-words {h, h', l, l'}
-    const float2* cb;          // per slot stiffness c_ij as a double-word, or nullptr
+    const float2* cb;          // per slot c_ij / c_ref as a double-word, or nullptr (c_ref: a
+                               // power of two near the largest c_ij, which FP32 need not hold)
     const float2* wrel;        // per node w / w_ref as a double-word (non-uniform weights)
     const double* phi0;        // per node the damage of an intact family (rounding only)
     const int32_t* fam;        // per node the bonds of the intact family
-    double w_ref;              // weight of the first node (batches: per instance)
+    double w_ref;              // weight of the first node (batches: per instance), with
+                               // stiffnesses per bond c_ref V
     double scale;              // 1 / U (batches: per instance)
     double dt_rho;             // dt / rho
     int32_t x_grid;            // exponent of the positions' grid (batches: per instance)
@@ -513,7 +515,7 @@ struct AdjW3Args {
     const double* vol;
     const float2* wrel;        // per node V / V_ref as a double-word (non-uniform volumes)
     const double* cbond;       // per-slot stiffness, or nullptr for the constant c
-    const float2* cb;          // the same as double-words
+    const float2* cb;          // W3Args::cb
     const double* ilen;        // per slot 1 / |xi|
     const double* e;           // per slot xi / |xi|^(3/2), rows of 32 lanes per component
     const float4* il;          // W3Args::il
@@ -522,7 +524,8 @@ struct AdjW3Args {
     const uint8_t* bcc;
     const BcClass* bct;
     double scale;              // 1 / U
-    double w_ref;              // V_ref, times the constant c without per-bond stiffness
+    double w_ref;              // V_ref times the constant c, or c_ref
+    double inv_c_ref;          // 1 / c_ref (1 with the constant c)
     double inv_vref;           // 1 / V_ref
     double dt_rho;             // dt / rho
     double damp;               // 1 - dt eta / rho
@@ -619,8 +622,9 @@ cudaError_t launch_dw_publish(const double* rec64, float4* rec, int64_t n_pad, c
 // every slot's |xi| / delta (1 where there is no bond)
 cudaError_t launch_dw_len(const double* x64, const int32_t* nbr, int64_t n, int Q,
                           double inv_delta, float2* len, cudaStream_t s);
-// double-word copy of an FP64 per-slot array
-cudaError_t launch_dw_split(const double* in, int64_t count, float2* out, cudaStream_t s);
+// double-word copy of an FP64 per-slot array, times scale
+cudaError_t launch_dw_split(const double* in, int64_t count, double scale, float2* out,
+                            cudaStream_t s);
 
 // ---- helper kernels (pd_aux.cu) ---------------------------------------------
 cudaError_t launch_advance(int64_t* step_ctr, int64_t k, cudaStream_t s);

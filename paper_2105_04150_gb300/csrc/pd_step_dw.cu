@@ -463,12 +463,14 @@ __global__ void k_dw_len(const double* __restrict__ x64, const int32_t* __restri
     }
 }
 
-__global__ void k_dw_split(const double* __restrict__ in, int64_t count, float2* __restrict__ out)
+__global__ void k_dw_split(const double* __restrict__ in, int64_t count, double scale,
+                           float2* __restrict__ out)
 {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count;
          k += (int64_t)gridDim.x * blockDim.x) {
-        const float h = (float)in[k];
-        out[k] = make_float2(h, (float)(in[k] - (double)h));
+        const double v = in[k] * scale;
+        const float h = (float)v;
+        out[k] = make_float2(h, (float)(v - (double)h));
     }
 }
 
@@ -526,9 +528,10 @@ cudaError_t launch_dw_len(const double* x64, const int32_t* nbr, int64_t n, int 
     return cudaGetLastError();
 }
 
-cudaError_t launch_dw_split(const double* in, int64_t count, float2* out, cudaStream_t s)
+cudaError_t launch_dw_split(const double* in, int64_t count, double scale, float2* out,
+                            cudaStream_t s)
 {
-    k_dw_split<<<grid_of(count), 256, 0, s>>>(in, count, out);
+    k_dw_split<<<grid_of(count), 256, 0, s>>>(in, count, scale, out);
     return cudaGetLastError();
 }
 
