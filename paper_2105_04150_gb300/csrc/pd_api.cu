@@ -2061,7 +2061,7 @@ pd_status pd_damage(pd_handle* h, double* phi)
     if (h->damage_fresh)  // written by the last step kernel (fused)
         PD_CUDA(launch_gather_damage(h->precision, h->damage, h->gid, h->n, dst, h->stream),
                 "damage");
-    else if (h->w3 && !h->dw)
+    else if (h->w3)  // as the step writes it
         PD_CUDA(launch_damage_lost(h->uniform_vol, h->rec[0], h->nbr, h->bits, h->bits0,
                                    (const double*)h->wsum_inv, h->phi0, h->gid, h->n, h->Q, dst,
                                    h->stream),
