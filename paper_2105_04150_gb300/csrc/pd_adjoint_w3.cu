@@ -303,11 +303,11 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         if (ok) {
             const Dw iL{il.x, il.y};
             const Dw zL = dw_mul(geo.z, iL);
-            // q - 1 = z (3 + 3z + z^2)
+            // q - 1 = z (3 + 3z + z^2); the low word of z, 2^-22 of it, enters z^2 too
             const float p = __fmul_rn(3.0f, geo.z.h), zz = __fmul_rn(geo.z.h, geo.z.h);
             const float s1 = __fadd_rn(3.0f, p), s2 = __fadd_rn(s1, zz);
             const Dw t3{s2, ((p - (s1 - 3.0f)) + (zz - (s2 - s1))) +
-                                fmaf(3.0f, geo.z.l, fmaf(3.0f, geo.z.h, -p)) +
+                                fmaf(fmaf(2.0f, geo.z.h, 3.0f), geo.z.l, fmaf(3.0f, geo.z.h, -p)) +
                                 fmaf(geo.z.h, geo.z.h, -zz)};
             const Dw qAB = dw_mul(dw_mul(geo.z, t3), AB);
             Dw i3 = dw_mul(iL, dw_mul(iL, iL));
