@@ -546,7 +546,7 @@ W3Args w3_args(pd_handle* h)
     d.scale = h->w3_scale;
     d.x_grid = h->w3_x_grid;
     d.dt_rho = h->dt / h->rho;
-    d.x_hi = h->frozen ? kW3XMax : w3_x_hi(h->sc_lo);
+    d.x_hi = w3_x_hi(h->frozen ? 1.0 : h->sc_lo, h->dw);
     d.wide = h->dw ? 1 : 0;
     d.uniform_w = h->uniform_vol ? 1 : 0;
     d.team = h->team;
@@ -1314,7 +1314,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
             } else {
                 itab[k].w3_scale = s;
                 itab[k].w3_x_grid = g;
-                itab[k].w3_x_hi = w3_x_hi(itab[k].sc_lo);
+                itab[k].w3_x_hi = w3_x_hi(itab[k].sc_lo, h->dw);
             }
         }
         fam.assign(np, 0);

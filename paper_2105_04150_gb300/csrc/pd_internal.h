@@ -343,15 +343,16 @@ struct StepArgsF64 {
 constexpr int kW3Seg = 16;             // slots of a family whose forces are summed together
 constexpr int kW3TeamSegs = 256 / kW3Seg;  // largest family, in segments, that a team takes
 constexpr float kW3XMax = 0x1.0p-6f;   // largest |x|, x = |y|^2 / |xi|^2 - 1, of the double-word
-                                       // bond arithmetic (see pd_w3.h)
+                                       // bond arithmetic on FP64 handles (see pd_w3.h)
+constexpr float kW3XWide = 0.5f;       // on PD_PREC_DW handles
 constexpr float kW3EtaMax = 0x1.0p-7f; // FP64 handles: largest |eta_c| / |xi| of it (see pd_w3.h)
 constexpr int kW3UGrid = -22;          // exponent of the displacements' grid below 4 U
 // the record's x at which the literal evaluation takes over: a band below the stretch
-// s_lo at which a bond can first break or soften, never past kW3XMax
-inline float w3_x_hi(double s_lo)
+// s_lo at which a bond can first break or soften, never past kW3XMax (kW3XWide)
+inline float w3_x_hi(double s_lo, bool wide)
 {
     const double f = (1.0 - 0x1.0p-20) * s_lo;
-    return (float)std::min((double)kW3XMax, f * (2.0 + f));
+    return (float)std::min((double)(wide ? kW3XWide : kW3XMax), f * (2.0 + f));
 }
 struct W3Args {
     const float4* rec[2];      // 4 float4 per node, double buffered like the FP64 records
@@ -366,7 +367,7 @@ struct W3Args {
     double scale;              // 1 / U (batches: per instance)
     double dt_rho;             // dt / rho
     int32_t x_grid;            // exponent of the positions' grid (batches: per instance)
-    float x_hi;                // w3_x_hi (batches: per instance); kW3XMax while frozen
+    float x_hi;                // w3_x_hi (batches: per instance); its bound while frozen
     int32_t wide;              // 1: PD_PREC_DW, whose bonds have no bound on eta (see pd_w3.h)
     int32_t uniform_w;         // 1: every node has weight w_ref
     int32_t team;              // warps per slice

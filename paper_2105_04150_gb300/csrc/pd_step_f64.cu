@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(256, 2)
                 const InstParams& ip = a.itab[a.inst[i]];
                 w_ref = ip.w_ref;
                 scale = ip.w3_scale;
-                x_hi = a.frozen ? kW3XMax : ip.w3_x_hi;
+                if (!a.frozen) x_hi = ip.w3_x_hi;
                 grid = ip.w3_x_grid;
             }
             const float ts = pow2(grid - 33);

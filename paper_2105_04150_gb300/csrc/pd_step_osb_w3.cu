@@ -151,14 +151,15 @@ __device__ __forceinline__ void osb_walk(const StepArgsF64& a, const W3Args& d, 
 }
 
 // x and w = z / (2 + z) of two bonds: seeded as -x / (1 + r)^2, r = sqrt(1 + x), and
-// corrected by one Newton step on f(w) = x (1 + w)^2 + 4 w = 0, whose leading terms cancel
-// exactly.
+// corrected by one Newton step on f(w) = x (1 + w)^2 + 4 w = 0, f' = 4 r, whose leading
+// terms cancel exactly for |x| <= 1/2.
 __device__ __forceinline__ Stretch2 w_of(Dw2 num, const float4 il)
 {
     const Dw2 iL{make_float2(il.x, il.y), make_float2(il.z, il.w)};
     const Dw2 x = dw_mul2(dw_mul2(num, iL), iL);
     const float2 x1 = add2(both(1.0f), x.h);
-    const float2 r1 = fma2(x1, make_float2(dwa::rsqrt_seed(x1.x), dwa::rsqrt_seed(x1.y)), both(1.0f));
+    const float2 ir = make_float2(dwa::rsqrt_seed(x1.x), dwa::rsqrt_seed(x1.y));
+    const float2 r1 = fma2(x1, ir, both(1.0f));
     const float2 den = mul2(r1, r1), nx = mul2(x.h, both(-1.0f));
     const float2 w0 = mul2(nx, make_float2(dwa::rcp_seed(den.x), dwa::rcp_seed(den.y)));
     const float2 ww = mul2(w0, w0), ph = fma2(both(2.0f), w0, ww);
@@ -166,7 +167,7 @@ __device__ __forceinline__ Stretch2 w_of(Dw2 num, const float4 il)
     const Dw2 p{ph, add2(sub2(ww, fma2(both(-2.0f), w0, ph)), e)};
     const Dw2 xp = dw_mul2(x, p);
     const float2 R = add2(add2(fma2(both(4.0f), w0, x.h), xp.h), add2(x.l, xp.l));
-    return {x.h, Dw2{w0, mul2(R, fma2(x.h, both(0.125f), both(-0.25f)))}};
+    return {x.h, Dw2{w0, mul2(R, mul2(ir, both(-0.25f)))}};
 }
 
 // literal_of with the turned bonds of FP64 handles (here the infinite x of pd_step_f64.cu
@@ -194,7 +195,7 @@ __device__ __forceinline__ Unit unit_of(const StepArgsF64& a, const W3Args& d, i
         const InstParams& ip = a.itab[a.inst[i]];
         u.w_ref = ip.w_ref;
         u.scale = ip.w3_scale;
-        u.x_hi = a.frozen ? kW3XMax : ip.w3_x_hi;
+        u.x_hi = a.frozen ? d.x_hi : ip.w3_x_hi;
         u.ts = pow2(ip.w3_x_grid - 33);
     }
     return u;
@@ -334,7 +335,8 @@ __global__ void __launch_bounds__(256, 2)
                 const float4 p0 = __ldg(o.ab + c0), p1 = __ldg(o.ab + c1);
                 const Stretch2 t = stretch2(
                     Dw2{make_float2(A.num.h, B.num.h), make_float2(A.num.l, B.num.l)}, il);
-                const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il, kW3XMax, live);
+                const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il,
+                                                                WIDE ? kW3XWide : kW3XMax, live);
                 const Dw2 al = dw_add2(Dw2{both(own_ab.x), both(own_ab.y)},
                                        Dw2{make_float2(p0.x, p1.x), make_float2(p0.y, p1.y)});
                 const Dw2 ga = dw_add2(Dw2{both(own_ab.z), both(own_ab.w)},

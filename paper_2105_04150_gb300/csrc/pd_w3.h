@@ -12,9 +12,9 @@
 // bits.  So h + m + t holds 57 bits of the largest position and 2^-59 U of a
 // displacement, or every bit of an FP64 displacement above 4 U.
 // The words of two bonded nodes lie on grids at most a factor 2 apart, so their
-// differences dh and dm are exact FP32 operations (|dh| <= 2.02 = the largest
-// component difference of a bond that is stretched by less than kW3XMax, and
-// |dm| <= 1.75 2^g), and dh + dm + dt, renormalised with one fast two-sum (dh is
+// differences dh and dm are exact FP32 operations (|dh| <= 2.23, the largest component of
+// eta of a bond with |y|^2 <= 1.5 |xi|^2 however it turned, below the 4 that 24 bits of a
+// grid of 2^-22 hold, and |dm| <= 1.75 2^g), and dh + dm + dt, renormalised with one fast two-sum (dh is
 // zero or its exponent no smaller than dm's), is the difference of the two values.
 // The difference of two plain double-words costs more (a two-sum for the leading
 // words, whose grids differ) and keeps only 2^-48 of |v|.
@@ -45,10 +45,15 @@ using dwa::dw_add;
 using dwa::dw_mul;
 using dwa::two_sum;
 
-// Bonds with |x| = ||y|^2 / |xi|^2 - 1| past kW3XMax (a stretch of 0.78 %) are left
-// to the literal FP64 evaluation of Eq. 4, which has the smaller error there: its
-// stretch carries an absolute rounding error of about 3e-16, i.e. 3e-16 / s of the
-// bond's force, against the 1e-14 of the form below.
+// Range of the arithmetic: |x| = ||y|^2 / |xi|^2 - 1| <= 1/2 (kW3XWide: there the leading
+// terms of the Newton residuals cancel exactly), the whole of it on PD_PREC_DW handles,
+// whose contract is about 1e-13 of the bond's force.  (Up to 0.78 % only, the bonds past it
+// in FP64, a step of a body at 2 % strain took 6.7 times as long: 220k nodes 1621 instead
+// of 242 us, state-based 4280 / 488.)
+// On FP64 handles bonds past kW3XMax (a stretch of 0.78 %) are left to the literal FP64
+// evaluation of Eq. 4, which has the smaller error there: its stretch carries an absolute
+// rounding error of about 3e-16, i.e. 3e-16 / s of the bond's force, against the 1e-14 of
+// the form below.
 // num = eta . (2 xi + eta) cancels when a bond rotates: its terms of size |eta| |xi|
 // carry 2^-47 each, so s an absolute error (rms, on random lattice bonds) of 2.4e-17,
 // 1.2e-16, 7e-16 and 4.2e-15 at 0.01, 0.05, 0.3 and pi/2 rad, where the literal form
@@ -327,14 +332,14 @@ __device__ __forceinline__ Stretch2 stretch2(Dw2 num, const float4 il)
 // eta past kW3EtaMax (il: the slot's U / |xi|)
 __device__ __forceinline__ bool turned(float e, float il) { return e * il >= kW3EtaMax; }
 
-// Which of two live bonds are to be evaluated literally: near or past s_c or past kW3XMax
-// (x_hi), past -kW3XMax, or not a number.  FP64 handles (not WIDE) take turned bonds out
+// Which of two live bonds are to be evaluated literally: near or past s_c, past the bound
+// on x (x_hi; -kW3XWide), or not a number.  FP64 handles (not WIDE) take turned bonds out
 // elsewhere, which bounds the compression too.
 template <bool WIDE>
 __device__ __forceinline__ uint32_t literal_of(float2 x, float x_hi, uint32_t live)
 {
-    const bool A = !(x.x < x_hi) || (WIDE && !(x.x > -kW3XMax));
-    const bool B = !(x.y < x_hi) || (WIDE && !(x.y > -kW3XMax));
+    const bool A = !(x.x < x_hi) || (WIDE && !(x.x > -kW3XWide));
+    const bool B = !(x.y < x_hi) || (WIDE && !(x.y > -kW3XWide));
     return ((A ? 1u : 0u) | (B ? 2u : 0u)) & live;
 }
 
