@@ -792,6 +792,25 @@ __device__ __forceinline__ double rsqrt_nr(double x)
     y = fma(0.5 * y, fma(-t, y, 1.0), y);
     return y;
 }
+
+// rsqrt_nr with the halvings and the seed's conversion to FP64 as integer operations on
+// the exponent field (the same bits; they keep three operations a bond off the FP64 pipe)
+__device__ __forceinline__ double half_of(double y)
+{
+    return __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y));
+}
+__device__ __forceinline__ double rsqrt_nr_int(double x)
+{
+    const float xf = (float)x;
+    if (!(xf > 0x1.0p-100f) || xf > 0x1.0p100f) return rsqrt_nr(x);
+    const uint32_t b = __float_as_uint(rsqrtf(xf));  // in [2^-50, 2^50]
+    double y = __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
+    double t = x * y;
+    y = fma(half_of(y), fma(-t, y, 1.0), y);
+    t = x * y;
+    y = fma(half_of(y), fma(-t, y, 1.0), y);
+    return y;
+}
 #endif
 cudaError_t launch_set_weights(int precision, void* wrec0, void* wrec1, const double* vol,
                                const int32_t* nbr, const uint32_t* init_bits, const int32_t* sw,

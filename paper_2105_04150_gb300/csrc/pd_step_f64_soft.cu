@@ -45,25 +45,6 @@ __device__ __noinline__ bool pair_no_fail(const uint8_t* __restrict__ bcc,
     return ((bct[bcc[i]].mask | bct[bcc[j]].mask) & 8u) != 0u;
 }
 
-// rsqrt_nr with the halvings and the seed's conversion to FP64 as integer operations on
-// the exponent field (the same bits; they keep three operations a bond off the FP64 pipe)
-__device__ __forceinline__ double half_of(double y)
-{
-    return __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y));
-}
-__device__ __forceinline__ double rsqrt_nr_int(double x)
-{
-    const float xf = (float)x;
-    if (!(xf > 0x1.0p-100f) || xf > 0x1.0p100f) return rsqrt_nr(x);
-    const uint32_t b = __float_as_uint(rsqrtf(xf));  // in [2^-50, 2^50]
-    double y = __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
-    double t = x * y;
-    y = fma(half_of(y), fma(-t, y, 1.0), y);
-    t = x * y;
-    y = fma(half_of(y), fma(-t, y, 1.0), y);
-    return y;
-}
-
 template <int SCM>
 __global__ void __launch_bounds__(256) k_step_f64_soft(const StepArgsF64 a)
 {

@@ -1,0 +1,81 @@
+"""The literal FP64 bonds of the state-based step: their cost and their break decisions.
+
+Cost: 61 FP64 operations a bond in the two loops, against the 30 of the literal bond-based
+step of softening models, which both are bound by: a ratio of 2.03.  2.2 leaves room for the
+rest of the loops.  (With a square root for |xi| in each loop it was 2.5.)
+
+Decisions: a line of nodes stretched evenly by 2^-6 has s = 2^-6 in every bond, to a few
+2^-53; an s_c that differs by more than that decides all of them, whether it is told by the
+high words of the two numbers or not."""
+import time
+
+import numpy as np
+import pytest
+
+import paper_2105_04150_gb300 as pdgb
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _need_gpu():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    pdgb.build()
+
+
+def _time(w, u, n):
+    m = pdgb.Model.from_workload(w, precision=pdgb.PD_PREC_F64)
+    best = float("inf")
+    for _ in range(4):
+        m.set_state(u, np.zeros_like(u), 0)
+        m.step(1)
+        m.sync()
+        t = time.perf_counter()
+        m.step(n)
+        m.sync()
+        best = min(best, time.perf_counter() - t)
+    m.close()
+    return best
+
+
+def test_cost_of_a_strained_body():
+    t = {}
+    for kind in ("soft", "state"):
+        w = workloads.tensile_bar(180, 35, 35, rate=0.0, sc=0.5)
+        w.bc_type[:] = 0
+        if kind == "soft":
+            w.kr = 2.0
+        else:
+            w.state_based = (w.bulk_modulus, 0.6 * w.bulk_modulus)
+        t[kind] = _time(w, 2e-2 * (w.coords - w.coords.mean(0)), 4)
+    assert t["state"] <= 2.2 * t["soft"]
+
+
+@pytest.mark.parametrize("precision", [pdgb.PD_PREC_F64, pdgb.PD_PREC_DW])
+@pytest.mark.parametrize("off", [1e-13, 5e-7, 1.5e-6, 1e-3, 0.5])
+@pytest.mark.parametrize("no_fail", [False, True])
+def test_break_decisions(precision, off, no_fail):
+    s = 2.0 ** -6
+    for sign in (-1, 1):
+        w = workloads.tensile_bar(40, 1, 1, rate=0.0, sc=s * (1 + sign * off))
+        w.bc_type[:] = 0
+        w.state_based = (w.bulk_modulus, 0.6 * w.bulk_modulus)
+        if no_fail:
+            w.no_fail = (np.arange(w.n) < 10).astype(np.uint8)
+        u = s * w.coords
+        m = pdgb.Model.from_workload(w, precision=precision)
+        off_, idx = m.family()
+        rows = np.repeat(np.arange(w.n), np.diff(off_))
+        m.set_state(u, np.zeros((w.n, 3)), 0)
+        m.step(1)
+        mu = m.bonds()
+        m.close()
+        if sign > 0:
+            assert (mu == 1).all()
+        elif no_fail:
+            assert np.array_equal(mu == 1, (rows < 10) | (idx < 10))
+        else:
+            assert (mu == 0).all()
