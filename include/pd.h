@@ -409,6 +409,9 @@ pd_status pd_set_params(pd_handle* h, double c, double sc, double load, double d
  *   only F_i; an undirected bond's sensitivity is the sum of its two entries),
  *   dL_dload (host scalar), dL_du0 / dL_dv0 (n*3, host or device).  The handle's
  *   state is left at u^N, v^N.  PD_ERR_STATE without a recorded forward.
+ *   Device memory, allocated by the first call and kept in the handle: 384 B per
+ *   node (padded to a multiple of 32), 32 B per SELL slot (8 B on PD_PREC_DW), and
+ *   once dL_dc is asked for 8 B per node and 12 B per directed bond.
  */
 pd_status pd_adjoint_forward(pd_handle* h, int64_t n_steps, int64_t checkpoint_every);
 pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dLdv,

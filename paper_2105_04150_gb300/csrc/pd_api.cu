@@ -181,13 +181,14 @@ struct pd_handle {
                *fin_v = nullptr;
         int64_t cap_ck = 0, cap_seg = 0;
         double *ub[2] = {nullptr, nullptr}, *vb[2] = {nullptr, nullptr}, *ubm = nullptr,
-               *w = nullptr, *gc = nullptr, *gl = nullptr, *partial = nullptr, *out = nullptr;
+               *gc = nullptr, *gl = nullptr, *partial = nullptr, *out = nullptr;
         int n_partial = 0;
         // the reverse sweep's records (pd_adjoint_w3.cu), double buffered: u^n, w in
         // double-words and in FP64; xi / |xi|^(3/2) per slot, the seeds' largest component
         float4 *rrec[2] = {nullptr, nullptr}, *wrec[2] = {nullptr, nullptr};
         double *w64[2] = {nullptr, nullptr}, *e = nullptr;
         unsigned long long* wmax = nullptr;
+        bool e_done = false;
         // dL/dc in canonical order: the family on the device, and the result
         int64_t* fam_off = nullptr;
         int32_t* fam_idx = nullptr;
@@ -2159,35 +2160,30 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
     const int64_t np3 = 3 * h->n_pad;
     const int64_t slots = h->n_slices * 32LL * h->Q * 32;
     cudaError_t e;
-    if (!T.w) {
-        if ((e = h->alloc(&T.ub[0], (size_t)np3)) != cudaSuccess ||
-            (e = h->alloc(&T.ub[1], (size_t)np3)) != cudaSuccess ||
-            (e = h->alloc(&T.vb[0], (size_t)np3)) != cudaSuccess ||
-            (e = h->alloc(&T.vb[1], (size_t)np3)) != cudaSuccess ||
-            (e = h->alloc(&T.ubm, (size_t)np3)) != cudaSuccess ||
-            (e = h->alloc(&T.w, (size_t)np3)) != cudaSuccess ||
-            (e = h->alloc(&T.gc, (size_t)slots)) != cudaSuccess ||
-            (e = h->alloc(&T.gl, (size_t)h->n_pad)) != cudaSuccess ||
-            (e = h->alloc(&T.out, 1)) != cudaSuccess)
-            return cuda_fail(e, "cudaMalloc adjoint buffers");
-        T.n_partial = sum_partials_needed(h->n);
-        if ((e = h->alloc(&T.partial, (size_t)T.n_partial)) != cudaSuccess)
-            return cuda_fail(e, "cudaMalloc reduction scratch");
+    // kept in the handle; what an earlier call that ran out of memory got is used again
+    auto need = [&](auto*& ptr, int64_t count) {
+        if (e == cudaSuccess && !ptr) e = h->alloc(&ptr, (size_t)count);
+    };
+    T.n_partial = sum_partials_needed(h->n);
+    e = cudaSuccess;
+    for (int k = 0; k < 2; ++k) {
+        need(T.ub[k], np3);
+        need(T.vb[k], np3);
+        need(T.rrec[k], 4 * h->n_pad);
+        need(T.wrec[k], 2 * h->n_pad);
+        need(T.w64[k], 4 * h->n_pad);
     }
-    if (!T.wmax) {
-        for (int k = 0; k < 2; ++k)
-            if ((e = h->alloc(&T.rrec[k], (size_t)(4 * h->n_pad))) != cudaSuccess ||
-                (e = h->alloc(&T.wrec[k], (size_t)(2 * h->n_pad))) != cudaSuccess ||
-                (e = h->alloc(&T.w64[k], (size_t)(4 * h->n_pad))) != cudaSuccess)
-                return cuda_fail(e, "cudaMalloc adjoint records");
-        if (!h->dw) {
-            if ((e = h->alloc(&T.e, (size_t)(3 * slots))) != cudaSuccess)
-                return cuda_fail(e, "cudaMalloc adjoint records");
-            PD_CUDA(launch_adj_e(h->rec[0], h->nbr, h->n_slices, h->Q, T.e, h->stream),
-                    "bond vectors");
-        }
-        if ((e = h->alloc(&T.wmax, 1)) != cudaSuccess)
-            return cuda_fail(e, "cudaMalloc adjoint records");
+    need(T.ubm, np3);
+    need(T.gc, slots);
+    need(T.gl, h->n_pad);
+    need(T.out, 1);
+    need(T.partial, T.n_partial);
+    if (!h->dw) need(T.e, 3 * slots);
+    need(T.wmax, 1);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc adjoint buffers");
+    if (!h->dw && !T.e_done) {
+        PD_CUDA(launch_adj_e(h->rec[0], h->nbr, h->n_slices, h->Q, T.e, h->stream), "bond vectors");
+        T.e_done = true;
     }
     // seed: dL/du^N, dL/dv^N in library order
     auto to_lib = [&](const double* src, double* dst) -> pd_status {
