@@ -43,7 +43,7 @@ import workloads  # noqa: E402
 # position+weight 16 B read, FP64 displacement 24 B read + 24 B written, FP32
 # velocity 12 B read + 12 B written, damage 4 B written, BC class 1 B.
 BYTES_PER_BOND = 4.125
-BYTES_PER_NODE = {32: 93.0, 64: 136.0}
+BYTES_PER_NODE = 93.0
 # Algorithmic FP64 work per bond (Eqs. 4-5 as written): xi, eta, y (9), |xi|^2 and
 # |y|^2 (10), two square roots and the stretch's division (3), c V s / |y| (3), the
 # force accumulation (6 as 3 fused multiply-adds) = 31 flops, counting a square
@@ -84,11 +84,19 @@ DW_FP32_OPS_PER_BOND = 192.0
 # scalar (20) and the force and its sum (36) = 391
 W3_OSB_FP32_OPS_PER_BOND = 391.0
 FP32_PEAK_TOPS = 35.1
-# per node: the double-word record 64 B read + 64 B written, the FP64 record
-# (x, w copied, u) 56 B read + 56 B written, FP64 velocity 24 + 24 B, damage
-# 8 B, wsum_inv 8 B, BC class 1 B; per bond 8 B of double-word |xi| on top
-BYTES_PER_NODE[48] = 305.0
-DW_BYTES_PER_BOND = BYTES_PER_BOND + 8.0
+# Softening steps.  Double-word, per node: the double-word record 64 B read + 64 B
+# written, the FP64 record (x, w copied, u) 56 B read + 56 B written, FP64 velocity
+# 24 + 24 B, damage 8 B, inverse weight sum 8 B, BC class 1 B; FP64: its record 64 B read
+# + 64 B written and the rest of that.  Per bond 8 B of |xi| as a double-word or 1/|xi| in
+# FP64 and the FP64 integrity 8 B (FP32 models: 4 B).
+SOFT_BYTES_PER_NODE = {32: BYTES_PER_NODE, 48: 305.0, 64: 193.0}
+SOFT_BYTES_PER_BOND = {32: BYTES_PER_BOND + 4.0, 48: BYTES_PER_BOND + 16.0,
+                       64: BYTES_PER_BOND + 16.0}
+# State-based models, per node and step besides the bond-based step's (each array once):
+# FP32: weighted volume, dilation and (alpha', beta') 16 B; FP64 and double-word: alpha and
+# gamma 16 B, alpha and beta 16 B, m 8 B
+OSB_BYTES_PER_NODE = 16.0
+W3_OSB_BYTES_PER_NODE = 40.0
 STEP_SRC = {32: ["pd_step_f32.cu"], 64: ["pd_step_f64.cu", "pd_w3.h"],
             48: ["pd_step_f64.cu", "pd_w3.h"],
             "lat": ["pd_step_f32_lat.cu"], "lat_tma": ["pd_step_f32_lat_tma.cu", "pd_step_f32_lat.cu"]}
@@ -106,13 +114,28 @@ L2_BYTES = 129e6
 FLUSH_BYTES = int(4 * L2_BYTES)
 
 
-def step_footprint(n_nodes, n_bonds, precision, lattice, osb=False):
+def three_word(precision, kr):
+    """Whether a model runs the three-word step: FP64 and double-word without softening
+    (kr = 1 is the PMB law; no workload here has no-fail nodes with it)."""
+    return precision != 32 and kr <= 1.0
+
+
+def model_bytes(precision, osb=False, kr=0.0):
+    """(bytes per directed bond, bytes per node) of the general step's arrays, each once."""
+    if three_word(precision, kr):
+        return W3_BYTES_PER_BOND, W3_BYTES_PER_NODE + (W3_OSB_BYTES_PER_NODE if osb else 0.0)
+    if kr:
+        return SOFT_BYTES_PER_BOND[precision], SOFT_BYTES_PER_NODE[precision]
+    return BYTES_PER_BOND, BYTES_PER_NODE + (OSB_BYTES_PER_NODE if osb else 0.0)
+
+
+def step_footprint(n_nodes, n_bonds, precision, lattice, osb=False, kr=0.0):
     """Bytes of device memory one step touches (node state, and the family where
     the kernel streams one)."""
     if lattice:
         return n_nodes * (LAT_OSB_FOOTPRINT_PER_NODE if osb else LAT_FOOTPRINT_PER_NODE)
-    per_bond = BYTES_PER_BOND if precision == 32 else W3_BYTES_PER_BOND
-    return n_bonds * per_bond + n_nodes * BYTES_PER_NODE[precision]
+    per_bond, per_node = model_bytes(precision, osb, kr)
+    return n_bonds * per_bond + n_nodes * per_node
 
 
 def l2_flush_buffer(torch, device):
@@ -214,7 +237,8 @@ def describe(w, n_bonds, precision, integrator="ec", lattice=None):
         "l2_policy": (f"L2 flushed between timed steps: a {FLUSH_BYTES / 1e6:.0f} MB write, then "
                       f"a read of it, on the launching stream between per-step CUDA-event "
                       f"intervals (step "
-                      f"footprint {step_footprint(w.n, n_bonds, precision, lattice, osb) / 1e6:.0f}"
+                      f"footprint "
+                      f"{step_footprint(w.n, n_bonds, precision, lattice, osb, w.kr) / 1e6:.0f}"
                       f" MB, L2 {L2_BYTES / 1e6:.0f} MB)"),
     }
 
@@ -541,21 +565,14 @@ def run_ours(args):
         return
     ms_step = ms_max / args.steps
     value = whole_job(n_bonds * args.steps, ms_max, world)
-    # softening adds the per-bond integrity read every step (FP32 4 B, FP64 8 B)
-    per_bond = BYTES_PER_BOND + ((4.0 if args.precision == 32 else 8.0) if args.kr else 0.0)
-    if args.precision == 48:
-        per_bond = DW_BYTES_PER_BOND + (8.0 if args.kr else 0.0)
     osb = args.state_based is not None
-    w3 = args.precision != 32 and not args.kr
-    alg_bytes = n_bonds * per_bond + w.n * BYTES_PER_NODE[args.precision]
-    if w3 and osb:  # the family twice; alpha and gamma 16 B, alpha and beta 16 B, m 8 B
-        alg_bytes = n_bonds * 2 * W3_BYTES_PER_BOND + w.n * (W3_BYTES_PER_NODE + 64 + 88)
-    elif w3:
-        alg_bytes = n_bonds * W3_BYTES_PER_BOND + w.n * W3_BYTES_PER_NODE
-    if osb and args.precision == 32:
-        # two passes over the family (ids and flags twice), and per node the
-        # weighted volume, dilation and (alpha', beta') besides the step's node data
-        alg_bytes = n_bonds * 2 * BYTES_PER_BOND + w.n * (BYTES_PER_NODE[32] + 16)
+    w3 = three_word(args.precision, w.kr)
+    per_bond, per_node = model_bytes(args.precision, osb, w.kr)
+    if osb:  # two passes over the family
+        per_bond *= 2
+    if w3 and osb:  # and over the three-word records, u and v
+        per_node += 64 + 48
+    alg_bytes = n_bonds * per_bond + w.n * per_node
     peak, peak_kind = hbm_peak()
     achieved = alg_bytes / (ms_step * 1e-3) / 1e9
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
@@ -753,9 +770,10 @@ def measure_batch(args, steps, warmup, with_cpu, with_e2e):
     ms_ll, lay_ll = loop_graph_ms(pdgb, torch, ws, args.precision, False, stream, GL, reps)
     # roofline: the step's algorithmic bytes over all instances (FP32), or the FP32
     # operations of the double-word arithmetic (FP64 and double-word)
-    w3 = args.precision != 32
-    alg_bytes = n_bonds * (W3_BYTES_PER_BOND if w3 else BYTES_PER_BOND) + n_nodes * (
-        W3_BYTES_PER_NODE if w3 else BYTES_PER_NODE[32])
+    kr = ws[0].kr
+    w3 = three_word(args.precision, kr)
+    per_bond, per_node = model_bytes(args.precision, kr=kr)
+    alg_bytes = n_bonds * per_bond + n_nodes * per_node
     peak, peak_kind = hbm_peak()
     achieved = alg_bytes / (ms_b * 1e-3) / 1e9
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
@@ -816,7 +834,7 @@ def measure_batch(args, steps, warmup, with_cpu, with_e2e):
                    "layout": "lattice stencil kernel" if lat else "sliced ELL",
                    "autotuned_launch": {"block_threads": block, "blocks_per_sm": bps},
                    "l2_policy": f"inputs larger than L2 (step footprint "
-                                f"{step_footprint(n_nodes, n_bonds, args.precision, lat) / 1e6:.0f}"
+                                f"{step_footprint(n_nodes, n_bonds, args.precision, lat, kr=kr) / 1e6:.0f}"
                                 f" MB over all instances, L2 {L2_BYTES / 1e6:.0f} MB)"},
         "instance_steps_per_s": n_inst / (ms_b * 1e-3),
         "loop": {"ms_per_step": ms_l, "instance_steps_per_s": n_inst / (ms_l * 1e-3),
