@@ -96,7 +96,10 @@ typedef struct {
                              pd_info_t.layout); 1 = always the general sliced-ELL step */
     int32_t lat_variant;  /* compiled variant of the stencil step (lattice handles; the
                              same results bit for bit, pd_autotune searches them):
-                             0 = default, records read through L1 (64 registers);
+                             0 = default, records read through L1 (64 registers; models
+                             of up to 456 slices of 32 nodes, single bond-based ones, run
+                             four warps per slice in blocks of their own, on which
+                             block_threads and blocks_per_sm have no effect);
                              1 = the same for 3 resident blocks (80 registers);
                              2, 3, 4 = records staged in shared memory by one TMA
                              bulk tensor copy per block of 16x2x8, 8x4x8 or 32x2x4

@@ -434,10 +434,11 @@ cudaError_t launch_f64(pd_handle* h, const StepArgsF64& a)
 // The lattice step's form with four warps per slice, a block (and 62 KB of terms) each: as
 // long as all blocks are resident at once, three per SM.  us per step, one warp / four:
 // 16 slices 8.7 / 5.8, 125: 9.7 / 7.1, 422: 10.2 / 7.9, 1000: 10.1 / 16.7.
-bool lat_team(const pd_handle* h)
+bool lat_team_model(const pd_handle* h)  // with lat_variant 0
 {
-    return h->lattice && !h->batch && h->model == 0 && h->lat_var == 0 && h->n_slices <= 3 * 152;
+    return h->lattice && !h->batch && h->model == 0 && h->n_slices <= 3 * kSms;
 }
+bool lat_team(const pd_handle* h) { return h->lat_var == 0 && lat_team_model(h); }
 
 // the FP32 step kernel build for this handle (bilinear softening or not)
 cudaError_t launch_f32(pd_handle* h, const StepArgsF32& a)
@@ -2465,7 +2466,7 @@ pd_status pd_autotune(pd_handle* h, int32_t trial_steps, int32_t* block_threads,
     const int n_var = !(h->lattice && h->model == 0) ? 1 : h->batch ? 2 : 2 + kLatTmaShapes;
     for (int var = 0; var < n_var && st == PD_OK; ++var)
     for (int block : {128, 256}) {
-        if (var >= 2 && block != 256) continue;
+        if ((var >= 2 || (var == 0 && lat_team_model(h))) && block != 256) continue;
         for (int bps = 1; bps <= 16 && st == PD_OK; ++bps) {
             h->lat_var = var;
             h->block = block;
@@ -2489,7 +2490,8 @@ pd_status pd_autotune(pd_handle* h, int32_t trial_steps, int32_t* block_threads,
                 best_bps = bps;
                 best_var = var;
             }
-            if (var >= 2) break;  // the tile step's grid does not depend on bps
+            // the tile step's grid, and that of four warps per slice, do not depend on bps
+            if (var >= 2 || lat_team(h)) break;
             int occ = 0;
             const void* fn = step_kernel_fn(h);
             const size_t smem = h->w3 && h->model == 0

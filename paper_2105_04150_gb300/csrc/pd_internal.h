@@ -44,6 +44,8 @@
 
 namespace pd {
 
+constexpr int kSms = 152;  // of a GB300
+
 // Programmatic dependent launch: a kernel launched with launch_pdl starts while its
 // predecessor in the stream runs (once all of that one's blocks have let it), and reads
 // what the predecessor writes only after pdl_begin, which waits for its completion.  It
@@ -76,7 +78,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_begin(bool early = false)
 {
     pdl_wait();
-    if (early && gridDim.x <= 152u) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (early && gridDim.x <= (unsigned)kSms) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 #endif
 
