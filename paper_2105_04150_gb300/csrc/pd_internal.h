@@ -46,6 +46,24 @@ namespace pd {
 
 constexpr int kSms = 152;  // of a GB300
 
+#ifdef __CUDACC__
+// A slot's integrity: an ordinary load, since the kernels that read it write it too (the
+// read-only path is for memory that nothing writes while the kernel runs, and a kernel
+// launched programmatically runs while its predecessor does).
+__device__ __forceinline__ double ld_integ(const double* p)
+{
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_integ(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+#endif
+
 // Programmatic dependent launch: a kernel launched with launch_pdl starts while its
 // predecessor in the stream runs (once all of that one's blocks have let it), and reads
 // what the predecessor writes only after pdl_begin, which waits for its completion.  It

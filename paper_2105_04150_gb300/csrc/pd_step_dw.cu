@@ -200,9 +200,8 @@ __device__ __noinline__ BondDw resolve_dw(const StepArgsF64& a, const DwArgs& d,
 // returns mu - 1 for the damage weight
 __device__ __forceinline__ double soften(BondDw& b, const double* integ, int64_t slot)
 {
-    const unsigned long long bits = __ldg(reinterpret_cast<const unsigned long long*>(integ) + slot);
-    if (bits == 0x3FF0000000000000ull) return 0.0;  // mu = 1
-    const double mu = __longlong_as_double(bits);
+    const double mu = ld_integ(integ + slot);
+    if (__double_as_longlong(mu) == 0x3FF0000000000000ll) return 0.0;  // mu = 1
     const float mh = (float)mu;
     b.coef = dw_mul(b.coef, Dw{mh, (float)(mu - (double)mh)});
     return mu - 1.0;

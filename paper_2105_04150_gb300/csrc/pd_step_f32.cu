@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(256, PD_F32_MIN_BLOCKS)
                 if (cb != nullptr) wj *= ld_f32(cb + (g * W + m0 + u) * 32 + lane);
                 float mj = 1.0f;
                 if (kSoft) {
-                    mj = ld_f32(a.integ + (g * W + m0 + u) * 32 + lane);
+                    mj = ld_integ(a.integ + (g * W + m0 + u) * 32 + lane);
                     wj *= mj;
                 }
                 float coef = bond_coef(bd, wj);

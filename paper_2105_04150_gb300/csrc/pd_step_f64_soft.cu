@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(256) k_step_f64_soft(const StepArgsF64 a)
                     // s_0 of the bond, the smallest the slice's bonds can have when
                     // s_c is drawn per bond: below it, by the high words (an integer
                     // comparison; not-a-numbers and ties go on), nothing changes
-                    double mu = __ldg(a.integ + slot);
+                    double mu = ld_integ(a.integ + slot);
                     if (__double2hiint(s) >= s0_hi) {
                         double sc = a.sc;
                         if (a.inst != nullptr) {  // batch: instance parameters, local ids
