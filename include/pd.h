@@ -48,12 +48,14 @@ typedef enum {
     PD_ERR_STATE = 8              /* call not valid in the handle's current state */
 } pd_status;
 
-#define PD_PREC_F64 64   /* FP64 state, integration and results.  On bond-based models
-                            without softening the bonds with |s| below 0.78 % are
-                            evaluated from exact differences in double-word arithmetic,
-                            with a smaller error than the literal FP64 form of Eq. 4
-                            (about 1e-14 of the bond's force, against 3e-16 / s); the
-                            others and every break are literal FP64 */
+#define PD_PREC_F64 64   /* FP64 state, integration and results.  On models without
+                            softening, bond-based and state-based, a bond with |s| up
+                            to about 0.8 % that has not turned (no component of eta past
+                            |xi| / 128, about half a degree) is evaluated from exact
+                            differences in double-word arithmetic, with a smaller error
+                            than the literal FP64 form of Eq. 4 (about 1e-14 of the
+                            bond's force, against 3e-16 / s); the others, every break
+                            and softening models are literal FP64 */
 #define PD_PREC_F32 32   /* FP32 bond arithmetic; an FP64 re-test of bonds whose
                             stretch is near s_c.  Each node's displacement is
                             accumulated in FP64 on lattice models (layout
@@ -63,16 +65,17 @@ typedef enum {
                             high word and a bf16 rounding of the low word) */
 #define PD_PREC_DW 48    /* FP64-grade step from FP32 double-word arithmetic: node
                             state (u, v) and integration in FP64 exactly as with
-                            PD_PREC_F64.  Bond-based models without softening run
-                            PD_PREC_F64's step and adjoint (the same results); on
-                            softening and state-based models every bond quantity (xi,
-                            eta, y, the stretch of Eq. 4, |y|, the force of Eq. 5) is
-                            carried as an unevaluated sum of two FP32 numbers (~48-bit
-                            significand, bond-force relative error ~1e-13), and the
-                            break test decided against the FP64 s_c, where PD_PREC_F64
-                            is literal FP64.  Everything PD_PREC_F64 offers: both
-                            integrators, per-bond stiffness, softening, batches, the
-                            state-based model and the adjoint.
+                            PD_PREC_F64; every bond quantity (xi, eta, y, the stretch of
+                            Eq. 4, |y|, the force of Eq. 5) an unevaluated sum of two
+                            FP32 numbers (about 46 bits, bond-force relative error
+                            ~1e-13), the break test decided against the FP64 s_c.
+                            Without softening this is PD_PREC_F64's step (the same
+                            results) with the double-word form kept at every rotation
+                            and up to |y|^2 / |xi|^2 = 1 +- 1/2, where PD_PREC_F64 goes
+                            over to literal FP64, 6 to 7 times slower; the reverse sweep
+                            is in double-words as a whole.  Everything PD_PREC_F64
+                            offers: both integrators, per-bond stiffness, softening,
+                            batches, the state-based model and the adjoint.
                             pd_get_info reports 48. */
 #define PD_MAX_FAMILY 1024
 #define PD_MAX_BC_CLASSES 256
@@ -395,8 +398,9 @@ pd_status pd_set_params(pd_handle* h, double c, double sc, double load, double d
  * (u^0, v^0); then dL_dv0 is the derivative with respect to that velocity and
  * dLdv refers to the full-step velocity v^N that pd_get_state reports.  The
  * reverse sweep of pd_adjoint_backward forms each bond's undeformed part in FP64 and
- * the remainder in double-word arithmetic (FP64-grade); the one of
- * pd_adjoint_backward_static is literal FP64 (the same outputs to ~1e-10).
+ * the remainder in double-word arithmetic, on PD_PREC_DW handles the whole of it, and
+ * sums dL_dc over the steps in FP64 (FP64-grade); the one of pd_adjoint_backward_static
+ * is literal FP64 (the same outputs to ~1e-10).
  *
  * pd_adjoint_forward - advance n_steps (>= 1) from the current state with the
  *   bond flags frozen (no bond breaks, so the run is a smooth function of the

@@ -21,7 +21,7 @@
 // of the whole; it runs on the FP32 pipe beside the FP64 one.  dL/dc needs the
 // stretch, which is more accurate in double-words than in the literal FP64 form
 // (whose s has an absolute error of 3e-16).  Bonds with |eta| / L past 2^-6 or past
-// kW3XMax, or whose w leaves FP32's range (kWTiny), are evaluated literally in FP64: 0.35 ms
+// kW3XMax, or whose w differ in bucket, are evaluated literally in FP64: 0.35 ms
 // a step of a 16k plate at 2 % strain, 0.08 at rest (all of it literal before: 0.60).  The
 // per-slot sums of dL/dc over the steps are FP64: two additions a bond.
 //
@@ -83,16 +83,36 @@ __device__ __forceinline__ double unit_scale(const unsigned long long* m)
     return v > 0.0 && v < 1e300 ? scalbn(1.0, min(-ilogb(v), 1000)) : 1.0;
 }
 
-// Largest component of a node's w, in that unit, below which FP32 does not hold its
-// products: |s / |y|| |w| has to keep its low word, 2^-24 of it, above 2^-126.  Bonds of such
-// nodes (far from the seeds) are evaluated literally.
-constexpr double kWTiny = 0x1.0p-48;
+// Far from a local seed w is smaller by any number of orders of magnitude, over most of the
+// body for as long as no wave has reached it.  So a node's double-words are in a unit of its
+// own, 2^(-104 B) of that one, its bucket B chosen so that its largest component lies above
+// 2^-64 in it, where FP32 holds its products with s / |y|, low words included (in buckets
+// past 0 up to 2^40, well inside FP32).  Bonds between buckets are evaluated literally.
+// (All bonds of nodes past bucket 0 literally: 1313 ms for the gradient of 2000 steps of a
+// 100k plate with a loss of two nodes, 1192 so; 1160 without regard to the range.)
+// The record holds the bucket as the float whose bits are (896 - 104 B) << 20, the exponent
+// offset from FP32 to FP64 of such a word (wide_of), and not-a-number, which equals no
+// bucket, past bucket 8.
+__device__ __forceinline__ float w_bucket(double w_max)
+{
+    const int e = (int)((uint32_t)__double2hiint(w_max) >> 20) - 1023;
+    const int B = e >= -63 || w_max == 0.0 ? 0 : 1 + (-64 - e) / 104;
+    return __uint_as_float(B <= 8 ? (896u - 104u * (uint32_t)B) << 20 : 0x7fc00000u);
+}
+// 2^(104 B) and its reciprocal
+__device__ __forceinline__ double bucket_up(float b)
+{
+    return __hiloint2double((int)(((1023u + 896u) << 20) - __float_as_uint(b)), 0);
+}
+__device__ __forceinline__ double bucket_down(float b)
+{
+    return __hiloint2double((int)(((1023u - 896u) << 20) + __float_as_uint(b)), 0);
+}
 
 // The records of a reverse step for node p, from its ubar, vbar and u^n: w = ws (vbar + dt
 // ubar) with the controlled components of ubar and vbar zeroed (as k_adj_mask), the
 // three-word record of x (its words from `fwd`) and u^n, w in FP64 ({w, 0}) and w as
-// double-words in units of 1 / unit_scale ({wh, wl.x} {wl.y, wl.z, tiny, 0}; tiny is 1 for a
-// w below kWTiny that is not zero).
+// double-words in units of 2^(-104 B) / unit_scale ({wh, wl.x} {wl.y, wl.z, B, 0}).
 __device__ __forceinline__ void adj_records(const AdjW3Args& a, int64_t p, uint32_t mask,
                                             const double (&ub)[3], const double (&vb)[3],
                                             const double* un, double dt, double ws, double us,
@@ -100,7 +120,7 @@ __device__ __forceinline__ void adj_records(const AdjW3Args& a, int64_t p, uint3
 {
     const float tin[3] = {fwd.a1.z, fwd.a1.w, fwd.b1.z};
     float uh[3], um[3], t[3], wh[3], wl[3];
-    double w[3], w_max = 0.0;
+    double w[3];
     for (int k = 0; k < 3; ++k) {
         const bool ctl = (mask >> k) & 1u;
         const double u = ctl ? 0.0 : ub[k];
@@ -110,8 +130,13 @@ __device__ __forceinline__ void adj_records(const AdjW3Args& a, int64_t p, uint3
         float ut;
         split3(un[3 * p + k] * a.scale, kW3UGrid, uh[k], um[k], ut);
         t[k] = pack_t(__float_as_uint(tin[k]) & 0x7ffu, ut);
-        w_max = fmax(w_max, fabs(w[k]));
-        const double v1 = w[k] * us;
+    }
+    const double w_max = fmax(fabs(w[0]), fmax(fabs(w[1]), fabs(w[2]))), v_max = w_max * us;
+    float bucket = w_bucket(v_max);
+    if (v_max == 0.0 && w_max > 0.0) bucket = __uint_as_float(0x7fc00000u);
+    const double up = bucket == bucket ? bucket_up(bucket) : 1.0;
+    for (int k = 0; k < 3; ++k) {
+        const double v1 = w[k] * us * up;
         wh[k] = (float)v1;
         wl[k] = (float)(v1 - (double)wh[k]);
     }
@@ -123,7 +148,7 @@ __device__ __forceinline__ void adj_records(const AdjW3Args& a, int64_t p, uint3
     dwa::st_rec(rec + 4 * p + 2, make_float4(fwd.b0.x, fwd.b0.y, um[0], um[1]),
                 make_float4(fwd.b1.x, um[2], t[2], 0.0f));
     dwa::st_rec(wdw + 2 * p, make_float4(wh[0], wh[1], wh[2], wl[0]),
-                make_float4(wl[1], wl[2], w_max > 0.0 && w_max * us < kWTiny ? 1.0f : 0.0f, 0.0f));
+                make_float4(wl[1], wl[2], bucket, 0.0f));
 }
 
 __global__ void k_adj_prep_w3(const __grid_constant__ AdjW3Args a, double dt, double ws, int64_t n_pad)
@@ -172,12 +197,12 @@ __device__ __forceinline__ Dw dot3(const Dw (&a)[3], const Dw (&b)[3])
     return dw_add(s, dw_mul(a[2], b[2]));
 }
 
-// v in FP64 by integer operations: a conversion instruction takes a turn of the FP64 pipe
-// (2 % of the sweep of a 100k plate).  Denormal numbers become 0.
-__device__ __forceinline__ double wide_of(float v)
+// v 2^(-104 B) in FP64 by integer operations: a conversion instruction takes a turn of the
+// FP64 pipe (2 % of the sweep of a 100k plate).  Denormal numbers become 0.
+__device__ __forceinline__ double wide_of(float v, float bucket)
 {
     const uint32_t b = __float_as_uint(v);
-    const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20));
+    const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + __float_as_uint(bucket));
     return (b & 0x7f800000u) != 0u ? __hiloint2double((int)hi, (int)(b << 29)) : 0.0;
 }
 
@@ -205,7 +230,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
     float4 w0, w1;
     dwa::ld_rec(a.wdw + 2 * m, w0, w1);
     const Dw wd[3] = {{w0.x, w0.w}, {w0.y, w1.x}, {w0.z, w1.y}};
-    const float tiny = w1.z;
+    const float bucket = w1.z;
     float2 rm = make_float2(1.0f, 0.0f);
     if (!UW) rm = __ldg(a.wrel + m);
     const double vm = UW ? 1.0 : (double)rm.x + (double)rm.y;
@@ -220,7 +245,8 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         float4 v0, v1;
         float4 il2;
         double e0, e1, e2;
-        double gc;  // the sum of the steps before
+        double gc;  // the sum of the steps before (FP64 handles load it where it is used: held
+                    // from here, the registers run out, 507 instead of 451 us a step)
     } in;
     auto load = [&](int b, int64_t j) {
         const int64_t row = g * 32LL * Q + b;  // of 32 slots
@@ -235,7 +261,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             in.e1 = __ldg(ep + 32);
             in.e2 = __ldg(ep + 64);
         }
-        in.gc = a.gc[row * 32 + lane];
+        if (!F64) in.gc = a.gc[row * 32 + lane];
     };
     uint32_t word = 0u;
     int32_t jc = 0, jn = 0;
@@ -254,7 +280,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         if (!UW) rj = __ldg(a.wrel + j);
         const Geo geo = bond_geo(own, in.nb, il, ts);
         const Dw wn[3] = {{in.v0.x, in.v0.w}, {in.v0.y, in.v1.x}, {in.v0.z, in.v1.y}};
-        const bool far = tiny + in.v1.z != 0.0f;
+        const bool same = in.v1.z == bucket;
         Dw d[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -300,7 +326,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
         }
         const float eta = fmaxf(fmaxf(fabsf(geo.et[0].h), fabsf(geo.et[1].h)), fabsf(geo.et[2].h));
         const bool ok = fabsf(geo.x.h) < (F64 ? kW3XMax : kW3XWide) &&
-                        (!F64 || eta * il.x < 0x1.0p-6f) && fabsf(AB.h) < 1e30f && !far;
+                        (!F64 || eta * il.x < 0x1.0p-6f) && fabsf(AB.h) < 1e30f && same;
         if (!alive) continue;
         if (ok) {
             const Dw iL{il.x, il.y};
@@ -317,7 +343,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             const Dw yw = dot3(geo.y, wd);
             Dw gs = dw_mul(zL, yw);  // -dL/dc of the bond in units of V_ref / unit_scale
             if (!UW) gs = dw_mul(gs, Dw{rj.x, rj.y});
-            a.gc[slot] = old + (wide_of(-gs.h) + wide_of(-gs.l));
+            a.gc[slot] = (F64 ? a.gc[slot] : old) + (wide_of(-gs.h, bucket) + wide_of(-gs.l, bucket));
             if (a.cbond != nullptr) {  // per-bond stiffness (a uniform branch)
                 const float2 cv = __ldg(a.cb + slot);
                 i3 = dw_mul(i3, Dw{cv.x, cv.y});
@@ -342,7 +368,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             }
         } else {
             double f[3];
-            a.gc[slot] = old + literal_adj(a, m, j, slot, f) * us;
+            a.gc[slot] = (F64 ? a.gc[slot] : old) + literal_adj(a, m, j, slot, f) * us;
             const double cij = a.cbond != nullptr ? __ldg(a.cbond + slot) : 1.0;
             acc[0] += cij * f[0];
             acc[1] += cij * f[1];
@@ -367,7 +393,9 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
                 s += sd[r][k][lane];
                 c = dw_add(c, Dw{sf[r][2 * k][lane], sf[r][2 * k + 1][lane]});
             }
-            s = fma(s, a.inv_c_ref, ((double)c.h + (double)c.l) * (a.scale / us));
+            // (a node past the buckets has nothing in c)
+            const double unit = bucket == bucket ? (a.scale / us) * bucket_down(bucket) : 0.0;
+            s = fma(s, a.inv_c_ref, ((double)c.h + (double)c.l) * unit);
             ub[k] = a.ubm[3 * m + k] + (a.dt_rho * a.w_ref) * s;
             vb[k] = a.damp * w3[k];
             a.ub_out[3 * m + k] = ub[k];
