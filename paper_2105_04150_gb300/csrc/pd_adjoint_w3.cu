@@ -15,8 +15,8 @@
 //   A = xi.d, B = eta.d,
 //
 // e is a constant of the slot, stored (24 bytes streamed cost less than the five
-// operations that form it: 0.34 ms a step of the 100k plate with xi and 1 / L^3; 0.32 now,
-// the FP64 pipe 60 % busy).  The second line is smaller than the first by |eta| / L, 1e-4 to 1e-2, so the
+// operations that form it: 0.34 ms a step of the 100k plate with xi and 1 / L^3, 0.31 so,
+// the FP64 pipe 69 % busy).  The second line is smaller than the first by |eta| / L, 1e-4 to 1e-2, so the
 // double-word arithmetic of pd_w3.h (relative 1e-14) gives it to FP64's rounding
 // of the whole; it runs on the FP32 pipe beside the FP64 one.  dL/dc needs the
 // stretch, which is more accurate in double-words than in the literal FP64 form
@@ -26,8 +26,8 @@
 // per-slot sums of dL/dc over the steps are FP64: two additions a bond.
 //
 // PD_PREC_DW handles (F64 false) take K d = y q (A + B) / L^3 - (z / L) d in double-word
-// arithmetic as a whole, to 2^-44 of each bond's term: no FP64 operation and no e, and the
-// whole range of pd_w3.h, at any rotation.
+// arithmetic as a whole, to 2^-44 of each bond's term: no FP64 operation but the two of
+// dL/dc and no e, and the whole range of pd_w3.h, at any rotation.
 //
 // The FP64 pipe needs few warps and a model of this use is small (the recorded run
 // is kept in memory), so a slice is shared by a block of four warps, each taking

@@ -19,8 +19,9 @@
 //   t |y|^-1 = (alpha_i + alpha_j) + (gamma_i + gamma_j) z,  gamma = alpha - beta,
 // so neither loop needs |xi|, a root or a division of its own.  alpha and gamma are
 // published per node as double-words in units of (K + G) / (V_ref U^2).  Bonds past
-// kW3XMax, and in the dilation loop those in or above the band below the smallest s_c,
-// are evaluated (and decided) literally in FP64 after their flag word.
+// kW3XMax or turned past kW3EtaMax (on PD_PREC_DW handles: past kW3XWide), and in the
+// dilation loop those in or above the band below the smallest s_c, are evaluated (and
+// decided) literally in FP64 after their flag word.
 #include <algorithm>
 
 #include <cuda_runtime.h>
