@@ -55,7 +55,9 @@ typedef enum {
                             differences in double-word arithmetic, with a smaller error
                             than the literal FP64 form of Eq. 4 (about 1e-14 of the
                             bond's force, against 3e-16 / s); the others, every break
-                            and softening models are literal FP64 */
+                            and softening models are literal FP64 (bodies longer than
+                            1000 horizons: the stretches shrink with the length, so
+                            that the error stays below the literal form's) */
 #define PD_PREC_F32 32   /* FP32 bond arithmetic; an FP64 re-test of bonds whose
                             stretch is near s_c.  Each node's displacement is
                             accumulated in FP64 on lattice models (layout

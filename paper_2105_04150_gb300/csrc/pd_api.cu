@@ -143,7 +143,7 @@ struct pd_handle {
     double* phi0 = nullptr; // per node the damage of an intact family
     int32_t* fam3 = nullptr;  // per node its bonds
     double w3_scale = 1.0;  // 1 / U, a power of two (batches: per instance in itab)
-    int w3_x_grid = kW3UGrid;  // exponent of the positions' grid
+    int w3_x_grid = kW3UGrid;  // exponent of the positions' grid (batches: the largest)
     int team = 1;           // warps per slice
     int integrator = PD_INTEGRATOR_EC;
     int64_t ramp_steps = 0;
@@ -548,7 +548,9 @@ W3Args w3_args(pd_handle* h)
     d.scale = h->w3_scale;
     d.x_grid = h->w3_x_grid;
     d.dt_rho = h->dt / h->rho;
-    d.x_hi = w3_x_hi(h->frozen ? 1.0 : h->sc_lo, h->dw);
+    d.x_hi = w3_x_hi(h->frozen ? 1.0 : h->sc_lo, h->dw, h->w3_x_grid);
+    d.x_max = w3_x_max(h->dw, h->w3_x_grid);
+    d.eta_max = w3_eta_max(h->w3_x_grid);
     d.wide = h->dw ? 1 : 0;
     d.uniform_w = h->uniform_vol ? 1 : 0;
     d.team = h->team;
@@ -1316,7 +1318,8 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
             } else {
                 itab[k].w3_scale = s;
                 itab[k].w3_x_grid = g;
-                itab[k].w3_x_hi = w3_x_hi(itab[k].sc_lo, h->dw);
+                itab[k].w3_x_hi = w3_x_hi(itab[k].sc_lo, h->dw, g);
+                h->w3_x_grid = k == 0 ? g : std::max(h->w3_x_grid, g);
             }
         }
         fam.assign(np, 0);
@@ -2223,6 +2226,8 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         A.Q = h->Q;
         A.uniform_w = h->uniform_vol ? 1 : 0;
         A.x_grid = h->w3_x_grid;
+        A.x_max = w3_x_max(h->dw, h->w3_x_grid);
+        A.eta_max = (float)std::min(0x1.0p-6, w3_s_grid(h->w3_x_grid));
         A.vol = h->vol;
         A.wrel = h->wrel3;
         A.cbond = h->per_bond_c ? (const double*)h->cbond : nullptr;

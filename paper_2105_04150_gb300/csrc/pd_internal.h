@@ -35,6 +35,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cuda.h>  // CUtensorMap
 #include <cuda_runtime.h>
@@ -367,12 +368,24 @@ constexpr float kW3XMax = 0x1.0p-6f;   // largest |x|, x = |y|^2 / |xi|^2 - 1, o
 constexpr float kW3XWide = 0.5f;       // on PD_PREC_DW handles
 constexpr float kW3EtaMax = 0x1.0p-7f; // FP64 handles: largest |eta_c| / |xi| of it (see pd_w3.h)
 constexpr int kW3UGrid = -22;          // exponent of the displacements' grid below 4 U
+// FP64 handles: stretch up to which the grid of the positions (x_grid: 2^(g - 33) a word's
+// unit, about 1.4 of that s in the stretch of a short bond) adds no more to it than the
+// literal form rounds, 2^-53: below kW3XMax only in bodies longer than 1024 U
+inline double w3_s_grid(int x_grid) { return std::ldexp(1.0, -21 - x_grid); }
+inline float w3_x_max(bool wide, int x_grid)
+{
+    return wide ? kW3XWide : (float)std::min((double)kW3XMax, 2.0 * w3_s_grid(x_grid));
+}
+inline float w3_eta_max(int x_grid)
+{
+    return (float)std::min((double)kW3EtaMax, w3_s_grid(x_grid));
+}
 // the record's x at which the literal evaluation takes over: a band below the stretch
-// s_lo at which a bond can first break or soften, never past kW3XMax (kW3XWide)
-inline float w3_x_hi(double s_lo, bool wide)
+// s_lo at which a bond can first break or soften, never past w3_x_max
+inline float w3_x_hi(double s_lo, bool wide, int x_grid)
 {
     const double f = (1.0 - 0x1.0p-20) * s_lo;
-    return (float)std::min((double)(wide ? kW3XWide : kW3XMax), f * (2.0 + f));
+    return (float)std::min((double)w3_x_max(wide, x_grid), f * (2.0 + f));
 }
 struct W3Args {
     const float4* rec[2];      // 4 float4 per node, double buffered like the FP64 records
@@ -388,6 +401,7 @@ struct W3Args {
     double dt_rho;             // dt / rho
     int32_t x_grid;            // exponent of the positions' grid (batches: per instance)
     float x_hi;                // w3_x_hi (batches: per instance); its bound while frozen
+    float x_max, eta_max;      // w3_x_max, w3_eta_max (batches: the smallest)
     int32_t wide;              // 1: PD_PREC_DW, whose bonds have no bound on eta (see pd_w3.h)
     int32_t uniform_w;         // 1: every node has weight w_ref
     int32_t team;              // warps per slice
@@ -547,6 +561,8 @@ struct AdjW3Args {
     double scale;              // 1 / U
     double w_ref;              // V_ref times the constant c, or c_ref
     double inv_c_ref;          // 1 / c_ref (1 with the constant c)
+    float x_max, eta_max;      // bounds on |x| and, on FP64 handles, |eta_c| / |xi| of the
+                               // double-word form
     double inv_vref;           // 1 / V_ref
     double dt_rho;             // dt / rho
     double damp;               // 1 - dt eta / rho

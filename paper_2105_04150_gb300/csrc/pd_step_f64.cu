@@ -152,13 +152,13 @@ __device__ __forceinline__ void walk(const StepArgsF64& a, const W3Args& d, int 
         // (a turned bond's x becomes infinite; held until literal_of as one more word, its
         // eta costs a 220k-node step 253 instead of 241 us, 237 without the bound)
         Kin bA = kin(own, A, both(ts), make_float2(ts, 1.0f));
-        if (!WIDE && turned(bA.e, il.x)) bA.num.h = INFINITY;
+        if (!WIDE && turned(bA.e, il.x, d.eta_max)) bA.num.h = INFINITY;
         if (more) {
             dwa::ld_rec(R + 4 * (int64_t)n0, A.a0, A.a1);
             dwa::ld_rec(R + 4 * (int64_t)n0 + 2, A.b0, A.b1);
         }
         Kin bB = kin(own, B, both(ts), make_float2(ts, 1.0f));
-        if (!WIDE && turned(bB.e, il.y)) bB.num.h = INFINITY;
+        if (!WIDE && turned(bB.e, il.y, d.eta_max)) bB.num.h = INFINITY;
         const float4 ilc = il;
         const int32_t c0 = j0, c1 = j1;
         const int mc = m;

@@ -197,12 +197,12 @@ __device__ __forceinline__ Stretch2 w_of(Dw2 num, const float4 il)
 // is the slower form: 494 against 473 us a step of 220k nodes)
 template <bool WIDE>
 __device__ __forceinline__ uint32_t literal_or_turned(float2 x, float eA, float eB, const float4 il,
-                                                      float x_hi, uint32_t live)
+                                                      float x_hi, float eta_max, uint32_t live)
 {
     if (WIDE) return literal_of<true>(x, x_hi, live);
     const float2 t = mul2(make_float2(eA, eB), make_float2(il.x, il.y));
-    const bool A = !(x.x < x_hi) || !(t.x < kW3EtaMax);
-    const bool B = !(x.y < x_hi) || !(t.y < kW3EtaMax);
+    const bool A = !(x.x < x_hi) || !(t.x < eta_max);
+    const bool B = !(x.y < x_hi) || !(t.y < eta_max);
     return ((A ? 1u : 0u) | (B ? 2u : 0u)) & live;
 }
 
@@ -276,7 +276,8 @@ __global__ void __launch_bounds__(256, 2)
             [&](int32_t c0, int32_t c1, const KinNum& A, const KinNum& B, const float4 il, uint32_t live) {
                 const Dw2 num{make_float2(A.num.h, B.num.h), make_float2(A.num.l, B.num.l)};
                 const Stretch2 t = w_of(num, il);
-                const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il, un.x_hi, live);
+                const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il, un.x_hi,
+                                                                d.eta_max, live);
                 const Dw2 hn{mul2(num.h, both(0.5f)), mul2(num.l, both(0.5f))};
                 Dw2 e = dw_add2(hn, dw_mul2(hn, t.z));
                 if (!UW) {
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(256, 2)
                 const Stretch2 t = stretch2(
                     Dw2{make_float2(A.num.h, B.num.h), make_float2(A.num.l, B.num.l)}, il);
                 const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il,
-                                                                WIDE ? kW3XWide : kW3XMax, live);
+                                                                d.x_max, d.eta_max, live);
                 const Dw2 al = dw_add2(Dw2{both(own_ab.x), both(own_ab.y)},
                                        Dw2{make_float2(p0.x, p1.x), make_float2(p0.y, p1.y)});
                 const Dw2 ga = dw_add2(Dw2{both(own_ab.z), both(own_ab.w)},

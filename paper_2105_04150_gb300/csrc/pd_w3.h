@@ -61,6 +61,10 @@ using dwa::two_sum;
 // kW3EtaMax |xi| (a rotation of about half a degree, or a compression of 0.8 to 1.4 %)
 // are literal.  PD_PREC_DW, about 1e-13 of the force and no less than 46 bits of |y|, has
 // no such bound.
+// The positions' grid adds 1.4 2^(g - 33) of s, nothing that shows while the largest position
+// is below 1024 U; in longer bodies, near whose origin FP64 coordinates are finer than the
+// grid, both bounds of FP64 handles shrink with it (w3_s_grid: without that a line of 66,000
+// horizons had 50 times the literal form's error there at a stretch of 0.7 %).
 
 struct Own {
     float xh[3], xm[3], xk[3], uh[3], um[3], ut[3];
@@ -329,8 +333,8 @@ __device__ __forceinline__ Stretch2 stretch2(Dw2 num, const float4 il)
     return {x.h, Dw2{z0, mul2(R, fma2(z0, both(-0.5f), both(-0.5f)))}};
 }
 
-// eta past kW3EtaMax (il: the slot's U / |xi|)
-__device__ __forceinline__ bool turned(float e, float il) { return e * il >= kW3EtaMax; }
+// eta past eta_max |xi| (il: the slot's U / |xi|)
+__device__ __forceinline__ bool turned(float e, float il, float eta_max) { return e * il >= eta_max; }
 
 // Which of two live bonds are to be evaluated literally: near or past s_c, past the bound
 // on x (x_hi; -kW3XWide), or not a number.  FP64 handles (not WIDE) take turned bonds out
