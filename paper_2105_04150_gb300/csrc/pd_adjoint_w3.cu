@@ -20,7 +20,7 @@
 // double-word arithmetic of pd_w3.h (relative 1e-14) gives it to FP64's rounding
 // of the whole; it runs on the FP32 pipe beside the FP64 one.  dL/dc needs the
 // stretch, which is more accurate in double-words than in the literal FP64 form
-// (whose s has an absolute error of 3e-16).  Bonds with |eta| / L past 2^-6 or past
+// (whose s has an absolute error of 3e-16).  Bonds with |eta| / L past kW3EtaMax or past
 // kW3XMax, or whose w differ in bucket, are evaluated literally in FP64: 0.35 ms
 // a step of a 16k plate at 2 % strain, 0.08 at rest (all of it literal before: 0.60).  The
 // per-slot sums of dL/dc over the steps are FP64: two additions a bond.
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
                 const Dw v = F64 ? dw_add(dw_mul(geo.xi[k], al), dw_mul(geo.et[k], be))
                                  : dw_mul(geo.y[k], be);
                 const Dw f = dw_add(v, Dw{-zd.h, -zd.l});
-                cor[k] = dw_add(cor[k], f);
+                cor[k] = renorm(dw_add(cor[k], f));
             }
         } else {
             double f[3];

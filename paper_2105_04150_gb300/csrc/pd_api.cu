@@ -548,8 +548,8 @@ W3Args w3_args(pd_handle* h)
     d.scale = h->w3_scale;
     d.x_grid = h->w3_x_grid;
     d.dt_rho = h->dt / h->rho;
-    d.x_hi = w3_x_hi(h->frozen ? 1.0 : h->sc_lo, h->dw, h->w3_x_grid);
-    d.x_max = w3_x_max(h->dw, h->w3_x_grid);
+    d.x_max = w3_x_max(h->dw, h->model == 1, h->w3_x_grid);
+    d.x_hi = w3_x_hi(h->frozen ? 1.0 : h->sc_lo, d.x_max);
     d.eta_max = w3_eta_max(h->w3_x_grid);
     d.wide = h->dw ? 1 : 0;
     d.uniform_w = h->uniform_vol ? 1 : 0;
@@ -1318,7 +1318,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
             } else {
                 itab[k].w3_scale = s;
                 itab[k].w3_x_grid = g;
-                itab[k].w3_x_hi = w3_x_hi(itab[k].sc_lo, h->dw, g);
+                itab[k].w3_x_hi = w3_x_hi(itab[k].sc_lo, w3_x_max(h->dw, h->model == 1, g));
                 h->w3_x_grid = k == 0 ? g : std::max(h->w3_x_grid, g);
             }
         }
@@ -1345,7 +1345,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
             return st;
     }
     if (!f32) {
-        e = launch_inv_len(h->x64, h->nbr, h->sw, n, h->Q, h->ilen, h->stream);
+        e = launch_inv_len(h->x64, h->nbr, h->sw, n, h->Q, h->w3, h->ilen, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "bond lengths");
     }
     if (h->w3) {
@@ -2226,8 +2226,8 @@ pd_status pd_adjoint_backward(pd_handle* h, const double* dLdu, const double* dL
         A.Q = h->Q;
         A.uniform_w = h->uniform_vol ? 1 : 0;
         A.x_grid = h->w3_x_grid;
-        A.x_max = w3_x_max(h->dw, h->w3_x_grid);
-        A.eta_max = (float)std::min(0x1.0p-6, w3_s_grid(h->w3_x_grid));
+        A.x_max = w3_x_max(h->dw, false, h->w3_x_grid);
+        A.eta_max = w3_eta_max(h->w3_x_grid);
         A.vol = h->vol;
         A.wrel = h->wrel3;
         A.cbond = h->per_bond_c ? (const double*)h->cbond : nullptr;

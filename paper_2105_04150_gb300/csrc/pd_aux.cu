@@ -274,7 +274,7 @@ __global__ void k_wsum(const void* __restrict__ wrec, const int32_t* __restrict_
 }
 
 __global__ void k_inv_len(const double* __restrict__ x64, const int32_t* __restrict__ nbr,
-                          const int32_t* __restrict__ sw, int64_t n, int Q,
+                          const int32_t* __restrict__ sw, int64_t n, int Q, bool rounded,
                           double* __restrict__ ilen)
 {
     const int64_t W = 32LL * Q;
@@ -291,6 +291,16 @@ __global__ void k_inv_len(const double* __restrict__ x64, const int32_t* __restr
                 const double ex = x64[3 * j] - x64[3 * p], ey = x64[3 * j + 1] - x64[3 * p + 1],
                              ez = x64[3 * j + 2] - x64[3 * p + 2];
                 v = 1.0 / sqrt(ex * ex + ey * ey + ez * ez);
+                if (rounded) {
+                    // to rounding: a Newton step on v^2 L^2 = 1, its residual in FP64 pairs
+                    const double xx = ex * ex, yy = ey * ey, zz = ez * ez;
+                    const double a = xx + yy, b = a - xx, q = a + zz, c = q - a;
+                    const double ql = ((xx - (a - b)) + (yy - b)) + ((a - (q - c)) + (zz - c)) +
+                                      fma(ex, ex, -xx) + fma(ey, ey, -yy) + fma(ez, ez, -zz);
+                    const double vv = v * v, t = q * vv;
+                    const double r = ((1.0 - t) - fma(q, vv, -t)) - fma(q, fma(v, v, -vv), ql * vv);
+                    v = fma(0.5 * v, r, v);
+                }
             }
             ilen[slot] = v;
         }
@@ -485,9 +495,9 @@ cudaError_t launch_fill(int precision, void* dst, int64_t n, double v, cudaStrea
 }
 
 cudaError_t launch_inv_len(const double* x64, const int32_t* nbr, const int32_t* sw, int64_t n,
-                           int Q, double* ilen, cudaStream_t s)
+                           int Q, bool rounded, double* ilen, cudaStream_t s)
 {
-    k_inv_len<<<grid_for(((n + 31) >> 5) << 5, 256), 256, 0, s>>>(x64, nbr, sw, n, Q, ilen);
+    k_inv_len<<<grid_for(((n + 31) >> 5) << 5, 256), 256, 0, s>>>(x64, nbr, sw, n, Q, rounded, ilen);
     return cudaGetLastError();
 }
 

@@ -363,29 +363,33 @@ struct StepArgsF64 {
 // displacements in units of U, a power of two no smaller than the longest bond
 constexpr int kW3Seg = 16;             // slots of a family whose forces are summed together
 constexpr int kW3TeamSegs = 256 / kW3Seg;  // largest family, in segments, that a team takes
-constexpr float kW3XMax = 0x1.0p-6f;   // largest |x|, x = |y|^2 / |xi|^2 - 1, of the double-word
-                                       // bond arithmetic on FP64 handles (see pd_w3.h)
-constexpr float kW3XWide = 0.5f;       // on PD_PREC_DW handles
-constexpr float kW3EtaMax = 0x1.0p-7f; // FP64 handles: largest |eta_c| / |xi| of it (see pd_w3.h)
+// bounds of the double-word bond arithmetic (see pd_w3.h): on FP64 handles largest |x|,
+// x = |y|^2 / |xi|^2 - 1, of the bond-based step and its adjoint and of the state-based
+// step, and largest |eta_c| / |xi|; on PD_PREC_DW handles largest |x|
+constexpr float kW3XMax = 0x1.4p-7f;
+constexpr float kW3XMaxOsb = 0x1.8p-8f;
+constexpr float kW3EtaMax = 0x1.0p-6f;
+constexpr float kW3XWide = 0.5f;
 constexpr int kW3UGrid = -22;          // exponent of the displacements' grid below 4 U
 // FP64 handles: stretch up to which the grid of the positions (x_grid: 2^(g - 33) a word's
 // unit, about 1.4 of that s in the stretch of a short bond) adds no more to it than the
-// literal form rounds, 2^-53: below kW3XMax only in bodies longer than 1024 U
+// literal form rounds, 2^-53: below the bounds above only in bodies longer than 512 U
 inline double w3_s_grid(int x_grid) { return std::ldexp(1.0, -21 - x_grid); }
-inline float w3_x_max(bool wide, int x_grid)
+inline float w3_x_max(bool wide, bool osb, int x_grid)
 {
-    return wide ? kW3XWide : (float)std::min((double)kW3XMax, 2.0 * w3_s_grid(x_grid));
+    return wide ? kW3XWide
+                : (float)std::min((double)(osb ? kW3XMaxOsb : kW3XMax), 2.0 * w3_s_grid(x_grid));
 }
 inline float w3_eta_max(int x_grid)
 {
     return (float)std::min((double)kW3EtaMax, w3_s_grid(x_grid));
 }
 // the record's x at which the literal evaluation takes over: a band below the stretch
-// s_lo at which a bond can first break or soften, never past w3_x_max
-inline float w3_x_hi(double s_lo, bool wide, int x_grid)
+// s_lo at which a bond can first break or soften, never past x_max
+inline float w3_x_hi(double s_lo, float x_max)
 {
     const double f = (1.0 - 0x1.0p-20) * s_lo;
-    return (float)std::min((double)w3_x_max(wide, x_grid), f * (2.0 + f));
+    return (float)std::min((double)x_max, f * (2.0 + f));
 }
 struct W3Args {
     const float4* rec[2];      // 4 float4 per node, double buffered like the FP64 records
@@ -725,7 +729,7 @@ const void* osb32_dilation_kernel(int sc_mode, bool uniform_w);
 const void* osb32_force_kernel(int sc_mode, bool uniform_w);
 // per slot 1 / |x_j - x_i| from the FP64 reference positions (0 for unused slots)
 cudaError_t launch_inv_len(const double* x64, const int32_t* nbr, const int32_t* sw, int64_t n,
-                           int Q, double* ilen, cudaStream_t s);
+                           int Q, bool rounded, double* ilen, cudaStream_t s);
 // step_ctr[0] is the device step counter; step_ctr[1] the step at which the
 // state was last set (velocity-Verlet forms a^n afresh there)
 

@@ -179,7 +179,7 @@ __device__ __forceinline__ void walk(const StepArgsF64& a, const W3Args& d, int 
         }
         Coef2 cf = coef2(bA.num, bB.num, ilc);
         const uint32_t live = (word >> b) & 3u;
-        const uint32_t lit = literal_of<WIDE>(cf.x, x_hi, live);
+        const uint32_t lit = literal_of(cf.x, x_hi, d.x_max, live);
         if (d.cb != nullptr) {  // per-bond stiffness (a uniform branch)
             const float2* cb = d.cb + (g * 32LL * Q + mc) * 32 + lane;
             const float2 cA = __ldg(cb), cB = __ldg(cb + 32);
@@ -192,6 +192,8 @@ __device__ __forceinline__ void walk(const StepArgsF64& a, const W3Args& d, int 
         pend |= lit << b;
         add_force(F, cf.c.h.x, cf.c.l.x, bA, (live & ~lit) & 1u);
         add_force(F, cf.c.h.y, cf.c.l.y, bB, (live & ~lit) & 2u);
+        F.xy = renorm2(F.xy);  // (240 -> 242 us a step; without it 1.6 times the error at 0.6 %)
+        F.z = renorm(F.z);
 
         if (b == kSeg - 2 || !more) {  // the segment's end
             const int m_lo = mc & ~(kSeg - 1);

@@ -19,7 +19,7 @@
 //   t |y|^-1 = (alpha_i + alpha_j) + (gamma_i + gamma_j) z,  gamma = alpha - beta,
 // so neither loop needs |xi|, a root or a division of its own.  alpha and gamma are
 // published per node as double-words in units of (K + G) / (V_ref U^2).  Bonds past
-// kW3XMax or turned past kW3EtaMax (on PD_PREC_DW handles: past kW3XWide), and in the
+// kW3XMaxOsb or turned past kW3EtaMax (on PD_PREC_DW handles: past kW3XWide), and in the
 // dilation loop those in or above the band below the smallest s_c, are evaluated (and
 // decided) literally in FP64 after their flag word.
 #include <algorithm>
@@ -197,13 +197,14 @@ __device__ __forceinline__ Stretch2 w_of(Dw2 num, const float4 il)
 // is the slower form: 494 against 473 us a step of 220k nodes)
 template <bool WIDE>
 __device__ __forceinline__ uint32_t literal_or_turned(float2 x, float eA, float eB, const float4 il,
-                                                      float x_hi, float eta_max, uint32_t live)
+                                                      float x_hi, const W3Args& d, uint32_t live)
 {
-    if (WIDE) return literal_of<true>(x, x_hi, live);
-    const float2 t = mul2(make_float2(eA, eB), make_float2(il.x, il.y));
-    const bool A = !(x.x < x_hi) || !(t.x < eta_max);
-    const bool B = !(x.y < x_hi) || !(t.y < eta_max);
-    return ((A ? 1u : 0u) | (B ? 2u : 0u)) & live;
+    uint32_t lit = literal_of(x, x_hi, d.x_max, live);
+    if (!WIDE) {
+        const float2 t = mul2(make_float2(eA, eB), make_float2(il.x, il.y));
+        lit |= ((t.x < d.eta_max ? 0u : 1u) | (t.y < d.eta_max ? 0u : 2u)) & live;
+    }
+    return lit;
 }
 
 // The unit, grid and weight of the slice's node (batches: its instance's)
@@ -276,8 +277,7 @@ __global__ void __launch_bounds__(256, 2)
             [&](int32_t c0, int32_t c1, const KinNum& A, const KinNum& B, const float4 il, uint32_t live) {
                 const Dw2 num{make_float2(A.num.h, B.num.h), make_float2(A.num.l, B.num.l)};
                 const Stretch2 t = w_of(num, il);
-                const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il, un.x_hi,
-                                                                d.eta_max, live);
+                const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il, un.x_hi, d, live);
                 const Dw2 hn{mul2(num.h, both(0.5f)), mul2(num.l, both(0.5f))};
                 Dw2 e = dw_add2(hn, dw_mul2(hn, t.z));
                 if (!UW) {
@@ -363,8 +363,7 @@ __global__ void __launch_bounds__(256, 2)
                 const float4 p0 = __ldg(o.ab + c0), p1 = __ldg(o.ab + c1);
                 const Stretch2 t = stretch2(
                     Dw2{make_float2(A.num.h, B.num.h), make_float2(A.num.l, B.num.l)}, il);
-                const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il,
-                                                                d.x_max, d.eta_max, live);
+                const uint32_t pend = literal_or_turned<WIDE>(t.x, A.e, B.e, il, d.x_max, d, live);
                 const Dw2 al = dw_add2(Dw2{both(own_ab.x), both(own_ab.y)},
                                        Dw2{make_float2(p0.x, p1.x), make_float2(p0.y, p1.y)});
                 const Dw2 ga = dw_add2(Dw2{both(own_ab.z), both(own_ab.w)},
@@ -377,6 +376,8 @@ __global__ void __launch_bounds__(256, 2)
                 const uint32_t ok = live & ~pend;
                 add_force(F, c.h.x, c.l.x, A, ok & 1u);
                 add_force(F, c.h.y, c.l.y, B, ok & 2u);
+                F.xy = renorm2(F.xy);  // (472 -> 475 us; a third of the error at 0.6 %)
+                F.z = renorm(F.z);
                 return pend;
             },
             [&](int q, uint32_t word, uint32_t pend) {

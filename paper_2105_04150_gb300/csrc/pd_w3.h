@@ -50,20 +50,20 @@ using dwa::two_sum;
 // whose contract is about 1e-13 of the bond's force.  (Up to 0.78 % only, the bonds past it
 // in FP64, a step of a body at 2 % strain took 6.7 times as long: 220k nodes 1621 instead
 // of 242 us, state-based 4280 / 488.)
-// On FP64 handles bonds past kW3XMax (a stretch of 0.78 %) are left to the literal FP64
-// evaluation of Eq. 4, which has the smaller error there: its stretch carries an absolute
-// rounding error of about 3e-16, i.e. 3e-16 / s of the bond's force, against the 1e-14 of
-// the form below.
-// num = eta . (2 xi + eta) cancels when a bond rotates: its terms of size |eta| |xi|
-// carry 2^-47 each, so s an absolute error (rms, on random lattice bonds) of 2.4e-17,
-// 1.2e-16, 7e-16 and 4.2e-15 at 0.01, 0.05, 0.3 and pi/2 rad, where the literal form
-// keeps 1.1e-16 throughout.  So bonds of FP64 handles with a component of eta past
-// kW3EtaMax |xi| (a rotation of about half a degree, or a compression of 0.8 to 1.4 %)
-// are literal.  PD_PREC_DW, about 1e-13 of the force and no less than 46 bits of |y|, has
-// no such bound.
+// FP64 handles leave the double-word form where the literal FP64 evaluation of Eq. 4 has the
+// smaller error.  That one rounds s at an absolute 1.1e-16 rms at any stretch and rotation;
+// this one has a relative error, of the bond and of the force sum (renormalised with every
+// pair of bonds), that reaches it at a stretch of 0.5 % (force of an irregular body against
+// the exact sum, in the literal form's rms error: 0.66 at 0.4 %, 1.04 at 0.6 %) and, the
+// state-based force having the coherent error of the dilation, at 0.35 %: kW3XMax and
+// kW3XMaxOsb.  And num = eta . (2 xi + eta) cancels when a bond turns: its terms of size
+// |eta| |xi| carry 2^-47 each, so s an absolute error (rms, on random lattice bonds) of
+// 2.4e-17, 1.2e-16, 7e-16 and 4.2e-15 at 0.01, 0.05, 0.3 and pi/2 rad.  So bonds with a
+// component of eta past kW3EtaMax |xi| (about 1 to 1.5 degrees) are literal too.
+// PD_PREC_DW, about 1e-13 of the force and no less than 46 bits of |y|, has no such bounds.
 // The positions' grid adds 1.4 2^(g - 33) of s, nothing that shows while the largest position
-// is below 1024 U; in longer bodies, near whose origin FP64 coordinates are finer than the
-// grid, both bounds of FP64 handles shrink with it (w3_s_grid: without that a line of 66,000
+// is below 512 U; in longer bodies, near whose origin FP64 coordinates are finer than the
+// grid, the bounds of FP64 handles shrink with it (w3_s_grid: without that a line of 66,000
 // horizons had 50 times the literal form's error there at a stretch of 0.7 %).
 
 struct Own {
@@ -122,6 +122,13 @@ __device__ __forceinline__ uint32_t t_int(float xt, int g)
 __device__ __forceinline__ float pack_t(uint32_t k, float ut)
 {
     return __uint_as_float(((__float_as_uint(ut) + 0x400u) & ~0x7ffu) | k);
+}
+
+// the same number with |l| at most half an ulp of h (fast two-sum)
+__device__ __forceinline__ Dw renorm(Dw a)
+{
+    const float s = __fadd_rn(a.h, a.l);
+    return {s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
 }
 
 // the difference j - i of one component as a double-word: dh + dm + dt ts
@@ -210,6 +217,12 @@ __device__ __forceinline__ Dw2 dw_mul2(Dw2 a, Dw2 b)
     const float2 p = mul2(a.h, b.h);
     const float2 e = make_float2(fmaf(a.h.x, b.h.x, -p.x), fmaf(a.h.y, b.h.y, -p.y));
     return {p, fma2(a.h, b.l, fma2(a.l, b.h, e))};
+}
+// the same numbers with |l| at most half an ulp of h (fast two-sum)
+__device__ __forceinline__ Dw2 renorm2(Dw2 a)
+{
+    const float2 s = add2(a.h, a.l);
+    return {s, sub2(a.l, sub2(s, a.h))};
 }
 // the difference of two records' pairs, as diff3
 __device__ __forceinline__ Dw2 diff3_2(float2 jh, float2 jm, float2 nh, float2 nm, float2 dt,
@@ -336,14 +349,12 @@ __device__ __forceinline__ Stretch2 stretch2(Dw2 num, const float4 il)
 // eta past eta_max |xi| (il: the slot's U / |xi|)
 __device__ __forceinline__ bool turned(float e, float il, float eta_max) { return e * il >= eta_max; }
 
-// Which of two live bonds are to be evaluated literally: near or past s_c, past the bound
-// on x (x_hi; -kW3XWide), or not a number.  FP64 handles (not WIDE) take turned bonds out
-// elsewhere, which bounds the compression too.
-template <bool WIDE>
-__device__ __forceinline__ uint32_t literal_of(float2 x, float x_hi, uint32_t live)
+// Which of two live bonds are to be evaluated literally: near or past s_c or past x_max
+// (x_hi), past -x_max, or not a number.  (Turned bonds of FP64 handles: elsewhere.)
+__device__ __forceinline__ uint32_t literal_of(float2 x, float x_hi, float x_max, uint32_t live)
 {
-    const bool A = !(x.x < x_hi) || (WIDE && !(x.x > -kW3XWide));
-    const bool B = !(x.y < x_hi) || (WIDE && !(x.y > -kW3XWide));
+    const bool A = !(x.x < x_hi) || !(x.x > -x_max);
+    const bool B = !(x.y < x_hi) || !(x.y > -x_max);
     return ((A ? 1u : 0u) | (B ? 2u : 0u)) & live;
 }
 
