@@ -1319,6 +1319,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
                 itab[k].w3_scale = s;
                 itab[k].w3_x_grid = g;
                 itab[k].w3_x_hi = w3_x_hi(itab[k].sc_lo, w3_x_max(h->dw, h->model == 1, g));
+                itab[k].w3_il_max = h->dw ? INFINITY : w3_il_max(g);
                 h->w3_x_grid = k == 0 ? g : std::max(h->w3_x_grid, g);
             }
         }
@@ -1350,6 +1351,7 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
     }
     if (h->w3) {
         e = launch_w3_ilen(h->ilen, h->nbr, h->sw, n, h->Q, h->w3_scale,
+                           h->dw ? INFINITY : w3_il_max(h->w3_x_grid),
                            h->batch ? h->inst : nullptr, h->itab, h->il3, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "bond lengths");
     }

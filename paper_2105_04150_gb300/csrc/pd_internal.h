@@ -129,6 +129,7 @@ struct InstParams {
     double w_ref, w3_scale;
     float w3_x_hi;
     int32_t w3_x_grid;
+    float w3_il_max, pad1;     // infinite on PD_PREC_DW handles
 };
 
 // Regular-lattice stencil.  On a cubic lattice of spacing dx with
@@ -380,6 +381,14 @@ inline float w3_x_max(bool wide, bool osb, int x_grid)
     return wide ? kW3XWide
                 : (float)std::min((double)(osb ? kW3XMaxOsb : kW3XMax), 2.0 * w3_s_grid(x_grid));
 }
+// FP64 handles: the largest U / |xi| of a bond in double-words.  The words' differences are
+// exact to 2^-60 U (displacements) and 0.4 2^(g - 33) U (positions), which a bond's stretch
+// gets by U / |xi|, the positions' with |eta| / |xi|: no more than half of the literal form's
+// rounding.  8 to 64 times shorter bonds than U, meshes with close nodes, are literal.
+inline float w3_il_max(int x_grid)
+{
+    return (float)std::ldexp(1.0, std::max(3, std::min(6, -12 - x_grid)));
+}
 inline float w3_eta_max(int x_grid)
 {
     return (float)std::min((double)kW3EtaMax, w3_s_grid(x_grid));
@@ -394,6 +403,7 @@ inline float w3_x_hi(double s_lo, float x_max)
 struct W3Args {
     const float4* rec[2];      // 4 float4 per node, double buffered like the FP64 records
     const float4* il;          // per pair of slots U / |xi| as double-words {h, h', l, l'}
+                               // (not a number: literal, see w3_il_max)
     const float2* cb;          // per slot c_ij / c_ref as a double-word, or nullptr (c_ref: a
                                // power of two near the largest c_ij, which FP32 need not hold)
     const float2* wrel;        // per node w / w_ref as a double-word (non-uniform weights)
@@ -652,8 +662,8 @@ cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, d
                               int x_grid, const int32_t* inst, const InstParams* itab,
                               cudaStream_t s);
 cudaError_t launch_w3_ilen(const double* ilen, const int32_t* nbr, const int32_t* sw, int64_t n,
-                           int Q, double scale, const int32_t* inst, const InstParams* itab,
-                           float4* il, cudaStream_t s);
+                           int Q, double scale, float il_max, const int32_t* inst,
+                           const InstParams* itab, float4* il, cudaStream_t s);
 cudaError_t launch_step_dw(const StepArgsF64& a, const DwArgs& d, int sc_mode, int grid, int block,
                            cudaStream_t s);
 const void* step_dw_kernel(int sc_mode, bool uniform_w, bool vv);

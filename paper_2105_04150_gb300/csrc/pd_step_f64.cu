@@ -335,12 +335,12 @@ __global__ void k_w3_publish(const double* __restrict__ rec64, float4* __restric
     }
 }
 
-// U / |xi| of every slot as a double-word (1 where there is no bond), by pairs of slots:
-// {h, h', l, l'} of slots m and m + 1
+// U / |xi| of every slot as a double-word (1 where there is no bond, not a number past il_max,
+// so that x is not and the bond literal), by pairs of slots: {h, h', l, l'} of slots m and m + 1
 __global__ void k_w3_ilen(const double* __restrict__ ilen, const int32_t* __restrict__ nbr,
                           const int32_t* __restrict__ sw, int64_t n, int Q, double scale,
-                          const int32_t* __restrict__ inst, const InstParams* __restrict__ itab,
-                          float4* __restrict__ il)
+                          float il_max, const int32_t* __restrict__ inst,
+                          const InstParams* __restrict__ itab, float4* __restrict__ il)
 {
     const int64_t W = 32LL * Q;
     const int64_t total = ((n + 31) >> 5) << 5;
@@ -348,12 +348,13 @@ __global__ void k_w3_ilen(const double* __restrict__ ilen, const int32_t* __rest
          p += (int64_t)gridDim.x * blockDim.x) {
         const int64_t g = p >> 5;
         const double U = 1.0 / (inst != nullptr ? itab[inst[p]].w3_scale : scale);  // a power of two
+        const float top = inst != nullptr ? itab[inst[p]].w3_il_max : il_max;
         for (int m = 0; m < W; m += 2) {
             float h[2], l[2];
             for (int k = 0; k < 2; ++k) {
                 const int64_t slot = (g * W + m + k) * 32 + (p & 31);
                 const double v = m + k < sw[g] && nbr[slot] != p ? ilen[slot] * U : 1.0;
-                h[k] = (float)v;
+                h[k] = v <= (double)top ? (float)v : __uint_as_float(0x7fc00000u);
                 l[k] = (float)(v - (double)h[k]);
             }
             il[(g * W / 2 + m / 2) * 32 + (p & 31)] = make_float4(h[0], h[1], l[0], l[1]);
@@ -412,11 +413,11 @@ cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, d
 }
 
 cudaError_t launch_w3_ilen(const double* ilen, const int32_t* nbr, const int32_t* sw, int64_t n,
-                           int Q, double scale, const int32_t* inst, const InstParams* itab,
-                           float4* il, cudaStream_t s)
+                           int Q, double scale, float il_max, const int32_t* inst,
+                           const InstParams* itab, float4* il, cudaStream_t s)
 {
-    k_w3_ilen<<<grid_of(((n + 31) >> 5) << 5), 256, 0, s>>>(ilen, nbr, sw, n, Q, scale, inst, itab,
-                                                            il);
+    k_w3_ilen<<<grid_of(((n + 31) >> 5) << 5), 256, 0, s>>>(ilen, nbr, sw, n, Q, scale, il_max, inst,
+                                                            itab, il);
     return cudaGetLastError();
 }
 
