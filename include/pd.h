@@ -49,15 +49,15 @@ typedef enum {
 } pd_status;
 
 #define PD_PREC_F64 64   /* FP64 state, integration and results.  On models without
-                            softening, bond-based and state-based, a bond with |s| up
-                            to about 0.8 % that has not turned (no component of eta past
-                            |xi| / 128, about half a degree) is evaluated from exact
-                            differences in double-word arithmetic, with a smaller error
-                            than the literal FP64 form of Eq. 4 (about 1e-14 of the
-                            bond's force, against 3e-16 / s); the others, every break
-                            and softening models are literal FP64 (bodies longer than
-                            1000 horizons: the stretches shrink with the length, so
-                            that the error stays below the literal form's) */
+                            softening most bonds are evaluated from exact differences in
+                            double-word arithmetic, with a smaller error than the literal
+                            FP64 form of Eq. 4 (about 1e-14 of the bond's force, against
+                            3e-16 / s).  Bonds for which that does not hold (|s| past
+                            0.49 %, on state-based models 0.29 %; a component of eta past
+                            |xi| / 64, a rotation of about one degree; bonds 64 times
+                            shorter than the longest; in bodies hundreds of horizons
+                            long these bounds shrink), every break and softening models
+                            are literal FP64 */
 #define PD_PREC_F32 32   /* FP32 bond arithmetic; an FP64 re-test of bonds whose
                             stretch is near s_c.  Each node's displacement is
                             accumulated in FP64 on lattice models (layout

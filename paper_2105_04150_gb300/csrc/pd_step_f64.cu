@@ -7,20 +7,20 @@
 // kernel that forms Eq. 4 literally in FP64 (about 41 FP64 operations a bond) is
 // bound by that pipe: 1.88 ms per step of a 180x35x35 notched beam, and 0.29 ms of a
 // 4000-node bar, whose 125 warps each walk a whole family alone.  With the arithmetic
-// and the split below they take 0.25 and 0.0125 ms, 198 warp instructions a bond (277
-// without the paired instructions, 0.285 ms), 58 % of the issue slots with the FMA
+// and the split below they take 0.25 and 0.0125 ms, 202 warp instructions a bond (277
+// without the paired instructions, 0.285 ms), 59 % of the issue slots with the FMA
 // pipe occupied twice by each pair and 16 warps per SM (128 registers).
 // Here the FP64 differences x_j - x_i and u_j - u_i come exactly from three-word
 // FP32 records, and the stretch without cancellation in double-word arithmetic
 // (pd_w3.h): no FP64 operation on the bonds of the bulk.  The literal form rounds
 // s = |y| / |xi| - 1 at an absolute 3e-16, 3e-12 of the force at a stretch of
 // 1e-4; this one has a relative error of about 1e-14 of the force, so it is the more
-// accurate of the two up to stretches of about 1 % (velocities of the beam after 5
+// accurate of the two up to stretches of about 0.5 % (velocities of the beam after 5
 // steps: 6e-13 relative to the exact step instead of 1.2e-11).  The other bonds are decided and
 // evaluated literally in FP64 after their segment (literal_bond): those past kW3XMax,
-// those turned past kW3EtaMax (a body all of whose bonds are takes 1.63 ms, 1.71 in the
-// kernel it replaced; on PD_PREC_DW handles, WIDE, only those past kW3XWide are) and those
-// in or above the band below the smallest s_c, so that every break is an
+// turned past kW3EtaMax or far shorter than U (a body all of whose bonds are takes 1.63
+// ms, 1.71 in the kernel it replaced; on PD_PREC_DW handles, WIDE, only those past kW3XWide
+// are) and those in or above the band below the smallest s_c, so that every break is an
 // FP64 decision on Eq. 4.  Models with softening take the literal kernel of
 // pd_step_f64_soft.cu for every bond.
 //
