@@ -139,6 +139,7 @@ struct pd_handle {
     float4* rec3[2] = {nullptr, nullptr};
     float4* il3 = nullptr;
     float2 *cb3 = nullptr, *wrel3 = nullptr;
+    double3 w3_origin{0.0, 0.0, 0.0};  // of the records' positions
     double c_ref = 1.0;     // unit of cb3
     double* phi0 = nullptr; // per node the damage of an intact family
     int32_t* fam3 = nullptr;  // per node its bonds
@@ -565,7 +566,7 @@ cudaError_t publish64(pd_handle* h, int b)
         return launch_dw_publish(h->rec[b], h->recdw[b], h->n_pad, h->dw_origin, 1.0 / h->delta,
                                  h->stream);
     if (h->w3)
-        return launch_w3_publish(h->rec[b], h->rec3[b], h->n_pad, h->w3_scale, h->w3_x_grid,
+        return launch_w3_publish(h->rec[b], h->rec3[b], h->n_pad, h->w3_scale, h->w3_x_grid, h->w3_origin,
                                  h->batch ? h->inst : nullptr, h->itab, h->stream);
     return cudaSuccess;
 }
@@ -1277,47 +1278,68 @@ pd_status build_device(pd_handle* h, const ModelDesc& d, const pd_config* cfg)
     std::vector<int32_t> fam;
     if (h->w3) {
         // U: a power of two no smaller than the longest bond (of each instance), and the
-        // FP32 grid of the largest coordinate in that unit
-        std::vector<double> len2(std::max<size_t>(1, itab.size()), 0.0), far(len2);
-        const int nl = (int)len2.size();
+        // FP32 grid of the largest position in that unit
+        struct Box {
+            double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+            double len2 = 0.0;
+            void add(const Box& b)
+            {
+                for (int a = 0; a < 3; ++a) {
+                    lo[a] = std::min(lo[a], b.lo[a]);
+                    hi[a] = std::max(hi[a], b.hi[a]);
+                }
+                len2 = std::max(len2, b.len2);
+            }
+        };
+        std::vector<Box> box(std::max<size_t>(1, itab.size()));
+        const int nl = (int)box.size();
         const int64_t* off = h->off.data();
         const int32_t* idx = h->idx.data();
 #pragma omp parallel
         {
-            std::vector<double> mine(nl, 0.0), wide(nl, 0.0);
+            std::vector<Box> mine(nl);
 #pragma omp for schedule(static)
             for (int64_t i = 0; i < n; ++i) {
-                double m = 0.0;
+                Box o;
                 for (int64_t k = off[i]; k < off[i + 1]; ++k) {
                     double q = 0.0;
                     for (int a = 0; a < 3; ++a) {
                         const double e = d.coords[3 * (int64_t)idx[k] + a] - d.coords[3 * i + a];
                         q += e * e;
                     }
-                    m = std::max(m, q);
+                    o.len2 = std::max(o.len2, q);
                 }
-                const int b = d.inst.empty() ? 0 : d.inst[i];
-                mine[b] = std::max(mine[b], m);
-                for (int a = 0; a < 3; ++a)
-                    wide[b] = std::max(wide[b], std::fabs(d.coords[3 * i + a]));
+                for (int a = 0; a < 3; ++a) o.lo[a] = o.hi[a] = d.coords[3 * i + a];
+                mine[d.inst.empty() ? 0 : d.inst[i]].add(o);
             }
 #pragma omp critical
-            for (int k = 0; k < nl; ++k) {
-                len2[k] = std::max(len2[k], mine[k]);
-                far[k] = std::max(far[k], wide[k]);
-            }
+            for (int k = 0; k < nl; ++k) box[k].add(mine[k]);
         }
         for (int k = 0; k < nl; ++k) {
-            const double L = len2[k] > 0.0 ? std::sqrt(len2[k]) : d.unit;
+            const Box& B = box[k];
+            const double L = B.len2 > 0.0 ? std::sqrt(B.len2) : d.unit;
             const double s = std::ldexp(1.0, -(std::ilogb(L) + 1));
-            const double X = far[k] * s;
+            // An axis along which the body lies away from the origin, by no less than its own
+            // extent, is counted from its near end: exact (Sterbenz), and the grid is then
+            // that of the extent
+            double o[3], X = 0.0;
+            for (int a = 0; a < 3; ++a) {
+                o[a] = B.lo[a] > 0.0 && B.hi[a] <= 2.0 * B.lo[a]   ? B.lo[a]
+                       : B.hi[a] < 0.0 && B.lo[a] >= 2.0 * B.hi[a] ? B.hi[a]
+                                                                   : 0.0;
+                X = std::max({X, std::fabs(B.lo[a] - o[a]), std::fabs(B.hi[a] - o[a])});
+            }
+            X *= s;
+            const double3 origin = make_double3(o[0], o[1], o[2]);
             const int g = std::min(100, std::max(kW3UGrid, (X > 0.0 ? std::ilogb(X) : 0) - 23));
             if (itab.empty()) {
                 h->w3_scale = s;
                 h->w3_x_grid = g;
+                h->w3_origin = origin;
             } else {
                 itab[k].w3_scale = s;
                 itab[k].w3_x_grid = g;
+                itab[k].w3_origin = origin;
                 itab[k].w3_x_hi = w3_x_hi(itab[k].sc_lo, w3_x_max(h->dw, h->model == 1, g));
                 itab[k].w3_il_max = h->dw ? INFINITY : w3_il_max(g);
                 h->w3_x_grid = k == 0 ? g : std::max(h->w3_x_grid, g);

@@ -130,6 +130,7 @@ struct InstParams {
     float w3_x_hi;
     int32_t w3_x_grid;
     float w3_il_max, pad1;     // infinite on PD_PREC_DW handles
+    double3 w3_origin;
 };
 
 // Regular-lattice stencil.  On a cubic lattice of spacing dx with
@@ -659,8 +660,8 @@ size_t step_f64_smem_max();  // over every team, family and block size
 int step_f64_carveout(int team, int max_seg, int block);
 // three-word records of every node from its FP64 record, and U / |xi| of every slot
 cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, double scale,
-                              int x_grid, const int32_t* inst, const InstParams* itab,
-                              cudaStream_t s);
+                              int x_grid, double3 origin, const int32_t* inst,
+                              const InstParams* itab, cudaStream_t s);
 cudaError_t launch_w3_ilen(const double* ilen, const int32_t* nbr, const int32_t* sw, int64_t n,
                            int Q, double scale, float il_max, const int32_t* inst,
                            const InstParams* itab, float4* il, cudaStream_t s);

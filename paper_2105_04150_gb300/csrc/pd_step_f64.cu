@@ -313,18 +313,20 @@ __global__ void __launch_bounds__(256, 2)
 
 // Records of every node from its FP64 record
 __global__ void k_w3_publish(const double* __restrict__ rec64, float4* __restrict__ rec,
-                             int64_t n_pad, double scale, int x_grid, const int32_t* __restrict__ inst,
-                             const InstParams* __restrict__ itab)
+                             int64_t n_pad, double scale, int x_grid, double3 origin,
+                             const int32_t* __restrict__ inst, const InstParams* __restrict__ itab)
 {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_pad;
          p += (int64_t)gridDim.x * blockDim.x) {
         const double* r = rec64 + 8 * p;
         const double sc = inst != nullptr ? itab[inst[p]].w3_scale : scale;
         const int g = inst != nullptr ? itab[inst[p]].w3_x_grid : x_grid;
+        const double3 o = inst != nullptr ? itab[inst[p]].w3_origin : origin;
+        const double o3[3] = {o.x, o.y, o.z};
         float xh[3], xm[3], uh[3], um[3], t[3];
         for (int k = 0; k < 3; ++k) {
             float xt, ut;
-            split3(r[k] * sc, g, xh[k], xm[k], xt);
+            split3((r[k] - o3[k]) * sc, g, xh[k], xm[k], xt);
             split3(r[4 + k] * sc, kW3UGrid, uh[k], um[k], ut);
             t[k] = pack_t(t_int(xt, g), ut);
         }
@@ -405,10 +407,10 @@ cudaError_t launch_step_f64(const StepArgsF64& a, const W3Args& d, int grid, int
 }
 
 cudaError_t launch_w3_publish(const double* rec64, float4* rec, int64_t n_pad, double scale,
-                              int x_grid, const int32_t* inst, const InstParams* itab,
-                              cudaStream_t s)
+                              int x_grid, double3 origin, const int32_t* inst,
+                              const InstParams* itab, cudaStream_t s)
 {
-    k_w3_publish<<<grid_of(n_pad), 256, 0, s>>>(rec64, rec, n_pad, scale, x_grid, inst, itab);
+    k_w3_publish<<<grid_of(n_pad), 256, 0, s>>>(rec64, rec, n_pad, scale, x_grid, origin, inst, itab);
     return cudaGetLastError();
 }
 

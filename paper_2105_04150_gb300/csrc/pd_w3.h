@@ -6,8 +6,9 @@
 //   h  v rounded to FP32, to a multiple of a grid 2^g
 //   m  the remainder v - h rounded to a multiple of 2^(g - 23)
 //   t  what is left, |t| <= 1.25 2^(g - 24)
-// Positions have one grid for the whole model (each instance of a batch), that of
-// its largest |x|; t is kept as an 11-bit integer (in units of 2^(g - 33)).
+// Positions, counted along each axis from the body's near end where it lies away from the
+// origin (an exact difference), have one grid for the whole model (each instance of a
+// batch), that of its largest |x|; t is kept as an 11-bit integer (in units of 2^(g - 33)).
 // Displacements have g = -22 below 4 and their own FP32 grid above; t is kept to 13
 // bits.  So h + m + t holds 57 bits of the largest position and 2^-59 U of a
 // displacement, or every bit of an FP64 displacement above 4 U.

@@ -6,6 +6,8 @@ One step from v = 0 of a line of nodes moved off their lattice, the force of the
 the origin against the same sums in long double; the literal form's rms error of a bond's
 s is at most 2.2 2^-53 (test_rotation_gpu.py derives it), of the node's force that of
 sum_j c V_j 2.2 2^-53 y / |y|."""
+import time
+
 import numpy as np
 import pytest
 
@@ -89,3 +91,51 @@ def test_stiffness_gradient_near_the_origin(n, strain):
     s = r / L - 1
     err = np.asarray(gc[:len(rows)] - f * s * d, np.float64) / f
     assert np.sqrt(np.mean(err ** 2)) <= RMS_S + 4 * 2.0 ** -53 * abs(strain)
+
+
+@pytest.mark.parametrize("offset", [(1e6, 1e6, 1e6), (-3e5, 0.0, 0.0), (0.0, 5e7, 2e3)])
+@pytest.mark.parametrize("batch", [False, True])
+def test_a_body_far_from_the_origin(offset, batch):
+    # a body of ordinary length anywhere (offsets in spacings): the same cost and, against the
+    # sums with its own coordinates in long double, the same bound
+    t = {}
+    for off3 in ((0.0, 0.0, 0.0), offset):
+        w = workloads.tensile_bar(100, 20, 20, rate=0.0, sc=0.5)
+        rng = np.random.default_rng(12)
+        w.bc_type[:] = 0
+        w.coords = w.coords + rng.uniform(-0.2, 0.2, w.coords.shape) * w.dx + np.array(off3) * w.dx
+        A = 2e-3 * (np.eye(3) + rng.uniform(-0.2, 0.2, (3, 3)))
+        u = (w.coords - w.coords.mean(0)) @ A.T
+        v0 = np.zeros_like(u)
+        if batch:
+            m = pdgb.Model.batch([w], precision=pdgb.PD_PREC_F64)
+        else:
+            m = pdgb.Model.from_workload(w, precision=pdgb.PD_PREC_F64)
+        m.set_state(u, v0, 0)
+        m.step(1)
+        got = m.state()[1] * (w.density / w.dt)
+        best = float("inf")
+        for _ in range(4):
+            m.set_state(u, v0, 0)
+            m.step(2)
+            m.sync()
+            s = time.perf_counter()
+            m.step(10)
+            m.sync()
+            best = min(best, time.perf_counter() - s)
+        m.close()
+        t[off3] = best
+    off, idx = oracle.cut_family(w.coords, w.horizon, w.cuts_array())
+    rows = np.repeat(np.arange(w.n), np.diff(off))
+    ld = np.longdouble
+    xi = w.coords[idx].astype(ld) - w.coords[rows].astype(ld)
+    y = xi + (u[idx].astype(ld) - u[rows].astype(ld))
+    L, r = np.sqrt((xi * xi).sum(1)), np.sqrt((y * y).sum(1))
+    d = y / r[:, None]
+    cV = oracle.micromodulus(w.bulk_modulus, w.horizon) * w.volumes[idx]
+    exact, var = np.zeros((w.n, 3), ld), np.zeros((w.n, 3))
+    np.add.at(exact, rows, (cV * (r / L - 1))[:, None] * d)
+    np.add.at(var, rows, (cV ** 2)[:, None] * np.asarray(d, np.float64) ** 2)
+    err = np.asarray(got - exact, np.float64)
+    assert np.sqrt(np.mean(err ** 2)) <= RMS_S * np.sqrt(np.mean(var))
+    assert t[offset] <= 1.5 * t[0.0, 0.0, 0.0]
