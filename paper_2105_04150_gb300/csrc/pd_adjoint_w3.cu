@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(32 * kTeam, 4) k_adj_step_w3(const __grid_cons
             AB = dot3(geo.y, d);
         }
         const float eta = fmaxf(fmaxf(fabsf(geo.et[0].h), fabsf(geo.et[1].h)), fabsf(geo.et[2].h));
-        const bool ok = fabsf(geo.x.h) < a.x_max && (!F64 || eta * il.x < a.eta_max) && fabsf(AB.h) < 1e30f && same;
+        const bool ok = fabsf(geo.x) < a.x_max && (!F64 || eta * il.x < a.eta_max) && fabsf(AB.h) < 1e30f && same;
         if (!alive) continue;
         if (ok) {
             const Dw iL{il.x, il.y};

@@ -190,7 +190,7 @@ __device__ __forceinline__ Stretch2 w_of(Dw2 num, const float4 il)
     const Dw2 p{ph, add2(sub2(ww, fma2(both(-2.0f), w0, ph)), e)};
     const Dw2 xp = dw_mul2(x, p);
     const float2 R = add2(add2(fma2(both(4.0f), w0, x.h), xp.h), add2(x.l, xp.l));
-    return {x.h, Dw2{w0, mul2(R, mul2(ir, both(-0.25f)))}};
+    return {add2(x.h, x.l) /* see stretch2 */, Dw2{w0, mul2(R, mul2(ir, both(-0.25f)))}};
 }
 
 // literal_of with the turned bonds of FP64 handles (here the infinite x of pd_step_f64.cu

@@ -144,7 +144,7 @@ __device__ __forceinline__ Dw diff3(float jh, float jm, float ih, float im, floa
 struct Geo {
     Dw xi[3], et[3];  // xi = x_j - x_i, eta = u_j - u_i
     Dw y[3];          // xi + eta
-    Dw x;             // |y|^2 / |xi|^2 - 1
+    float x;          // |y|^2 / |xi|^2 - 1
     Dw z;             // |xi| / |y| - 1
 };
 
@@ -175,15 +175,16 @@ __device__ __forceinline__ Geo bond_geo(const Own& o, const Rec& j, const float2
     num = dw_add(num, nm[2]);
     const Dw iL{il.x, il.y};
     const Dw x = dw_mul(dw_mul(num, iL), iL);
-    const float x1 = 1.0f + x.h;
+    const float xs = x.h + x.l;  // (see stretch2)
+    const float x1 = 1.0f + xs;
     const float r = x1 * dwa::rsqrt_seed(x1);
-    const float z0 = -x.h * dwa::rcp_seed(fmaf(r, r, r));
+    const float z0 = -xs * dwa::rcp_seed(fmaf(r, r, r));
     // p = 2 z0 + z0^2 as a double-word
     const float zz = __fmul_rn(z0, z0), ph = fmaf(2.0f, z0, zz);
     const Dw p{ph, (zz - fmaf(-2.0f, z0, ph)) + fmaf(z0, z0, -zz)};
     const Dw xp = dw_mul(x, p);
     const float R = __fadd_rn(__fadd_rn(ph, x.h), xp.h) + ((p.l + x.l) + xp.l);
-    out.x = x;
+    out.x = xs;
     out.z = Dw{z0, R * fmaf(z0, -0.5f, -0.5f)};
     return out;
 }
@@ -325,9 +326,14 @@ __device__ __forceinline__ KinNum kin_num(const Own2& o, const Rec& j, float2 ts
             eta_max(p)};
 }
 
-// x = |y|^2 / |xi|^2 - 1 and z = |xi| / |y| - 1 of two bonds (see bond_geo)
+// x = |y|^2 / |xi|^2 - 1 and z = |xi| / |y| - 1 of two bonds (see bond_geo).  x is the sum of
+// both words: in a turned bond num's low word is 2^-24 of terms that cancel, so its leading
+// word alone misses num by 1e-5 of it at one degree and a stretch of 1e-4, and by more at
+// more, past the margin of the comparison with x_hi (bonds above s_c did not break).  As the
+// seed of z too the sum lengthens the chain (242 -> 245 us a step); Newton's step does not
+// need it.
 struct Stretch2 {
-    float2 x;  // leading words
+    float2 x;
     Dw2 z;
 };
 __device__ __forceinline__ Stretch2 stretch2(Dw2 num, const float4 il)
@@ -344,7 +350,7 @@ __device__ __forceinline__ Stretch2 stretch2(Dw2 num, const float4 il)
     const Dw2 p{ph, add2(sub2(zz, fma2(both(-2.0f), z0, ph)), e)};
     const Dw2 xp = dw_mul2(x, p);
     const float2 R = add2(add2(add2(ph, x.h), xp.h), add2(add2(p.l, x.l), xp.l));
-    return {x.h, Dw2{z0, mul2(R, fma2(z0, both(-0.5f), both(-0.5f)))}};
+    return {add2(x.h, x.l), Dw2{z0, mul2(R, fma2(z0, both(-0.5f), both(-0.5f)))}};
 }
 
 // eta past eta_max |xi| (il: the slot's U / |xi|)
@@ -361,7 +367,7 @@ __device__ __forceinline__ uint32_t literal_of(float2 x, float x_hi, float x_max
 
 // x of two bonds and (1 / |xi|) z = -s / |y|
 struct Coef2 {
-    float2 x;  // leading words
+    float2 x;
     Dw2 c;
 };
 __device__ __forceinline__ Coef2 coef2(Dw a, Dw b, const float4 il)

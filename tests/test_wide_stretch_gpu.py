@@ -103,51 +103,59 @@ def test_state_based_step(strain, angle, jitter):
     assert (np.abs(vg - vo).max(1) <= tol).all()
 
 
-def _step_time(m, u, n):
-    best = float("inf")
-    for _ in range(5):
-        m.set_state(u, np.zeros_like(u), 0)
-        m.step(2)
-        m.sync()
-        t = time.perf_counter()
-        m.step(n)
-        m.sync()
-        best = min(best, time.perf_counter() - t)
-    return best
+def _ratio(run, limit):
+    """Largest time of run[1:] over that of run[0], the least of up to 12 turns each, in turn,
+    until it is within the limit (others may use the device)."""
+    best = [float("inf")] * len(run)
+    for _ in range(12):
+        for k, r in enumerate(run):
+            best[k] = min(best[k], r())
+        if _ >= 2 and max(best[1:]) <= limit * best[0]:
+            break
+    return max(best[1:]) / best[0]
 
 
 @pytest.mark.parametrize("state_based", [False, True])
 def test_a_strained_or_turned_body_costs_what_a_resting_one_does(state_based):
     # (all of its bonds in FP64 would take 6 to 9 times as long)
-    t = {}
+    runs, models = [], []
     for strain, angle in ((1e-4, 0.0), (2e-2, 0.0), (0.15, 0.0), (2e-2, 0.5)):
         w, u = _state((120, 25, 25), strain, angle)
         if state_based:
             w.state_based = (w.bulk_modulus, 0.6 * w.bulk_modulus)
         m = pdgb.Model.from_workload(w, precision=pdgb.PD_PREC_DW)
-        t[strain, angle] = _step_time(m, u, 6)
+        models.append(m)
+
+        def run(m=m, u=u):
+            m.set_state(u, np.zeros_like(u), 0)
+            m.step(2)
+            m.sync()
+            t = time.perf_counter()
+            m.step(6)
+            m.sync()
+            return time.perf_counter() - t
+        runs.append(run)
+    assert _ratio(runs, 1.5) <= 1.5
+    for m in models:
         m.close()
-    rest = t.pop((1e-4, 0.0))
-    for v in t.values():
-        assert v <= 1.5 * rest
 
 
 def test_the_reverse_sweep_of_a_strained_body_costs_what_a_resting_one_does():
-    t = {}
+    runs, models = [], []
     for strain, angle in ((1e-4, 0.0), (2e-2, 0.0), (2e-2, 0.5)):
         w, u = _state((100, 40, 4), strain, angle)
         m = pdgb.Model.from_workload(w, precision=pdgb.PD_PREC_DW)
+        models.append(m)
         g = np.random.default_rng(0).normal(size=u.shape)
-        best = float("inf")
-        for _ in range(4):
+
+        def run(m=m, u=u, g=g):
             m.set_state(u, np.zeros_like(u), 0)
             pdgb.pd_adjoint_forward(m.h, 40)
             m.sync()
-            s = time.perf_counter()
+            t = time.perf_counter()
             pdgb.pd_adjoint_backward(m.h, g, None, want_c=False)
-            best = min(best, time.perf_counter() - s)
+            return time.perf_counter() - t
+        runs.append(run)
+    assert _ratio(runs, 1.5) <= 1.5
+    for m in models:
         m.close()
-        t[strain, angle] = best
-    rest = t.pop((1e-4, 0.0))
-    for v in t.values():
-        assert v <= 1.5 * rest
