@@ -280,7 +280,8 @@ __global__ void __launch_bounds__(256, PD_DW_MIN_BLOCKS)
                 scale_coef(bA, __ldg(d.cb + (g * W + m0) * 32 + lane));
                 scale_coef(bB, __ldg(d.cb + (g * W + m0 + 1) * 32 + lane));
             }
-            const bool candA = bA.s.h >= fast_lo, candB = bB.s.h >= fast_lo;
+            // (both words: in a turned bond the low one is 2^-24 of terms that cancel in s)
+            const bool candA = bA.s.h + bA.s.l >= fast_lo, candB = bB.s.h + bB.s.l >= fast_lo;
             const bool okA = (wb & 1u) && !candA, okB = ((wb >> 1) & 1u) && !candB;
             {
                 const double dA = soften(bA, a.integ, (g * W + m0) * 32 + lane);
